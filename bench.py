@@ -301,7 +301,7 @@ def model_bytes(N, npw, nocc, s):
 
 def src_hash():
     h = hashlib.sha256()
-    for f in ("fft.cuh", "kernels_fft.cu", "kernels_linalg.cu", "gw_common.cuh", "kernels_cg.cu", "pcg.cuh"):
+    for f in ("fft.cuh", "kernels_fft.cu", "kernels_linalg.cu", "gw_common.cuh", "kernels_cg.cu", "col.cuh", "col_kernel.cuh"):
         with open(os.path.join(ROOT, "paper_1408_3036_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

@@ -292,10 +292,10 @@ gw_status gw_grad_vloc_basis(gw_ctx* ctx, const double* phi, const double* basis
  *   out[6] CUDA kernels launched by the library since it was loaded,
  *   out[7] iterations run by persistent CG launches (each launch counts the
  *          iterations of its slowest column)
- *   out[8] CTAs of the last persistent CG launch, out[9] its cluster size
- *          (0: the grid-wide cooperative kernel)
+ *   out[8] CTAs of the last one-launch CG or SQMR pass, out[9] the cluster
+ *          size of the last CG pass (0: the grid-wide cooperative kernel)
  *   out[10] CUDA-graph replays of SQMR iterations in the last SQMR solve
- *   out[11] threads per CTA of the last persistent CG launch (256 or 512)
+ *   out[11] threads per CTA of the last one-launch CG pass (256 or 512)
  *   n: entries wanted (<= 12)
  */
 gw_status gw_stats(const gw_ctx* ctx, double* out, int n);
@@ -371,11 +371,13 @@ typedef enum {
 gw_status gw_set_imaginary_route(gw_ctx* ctx, int route);
 
 /*
- * gw_set_graphs -- on (default 1): the ten launches of one simplified-QMR
- * iteration (the transform passes of H, the projector, the four update
- * steps) are captured once per solve into a CUDA graph and replayed every
- * iteration; 0: launched one by one.  Same arithmetic either way; a stream
- * that cannot be captured falls back to direct launches.
+ * gw_set_graphs -- 1: the ten launches of one simplified-QMR iteration (the
+ * transform passes of H, the projector, the four update steps) are captured
+ * once per solve into a CUDA graph and replayed every iteration; 0: launched
+ * one by one.  Same arithmetic either way; a stream that cannot be captured
+ * falls back to direct launches.  A context on which it was never called runs
+ * a whole simplified-QMR pass in one launch, one thread-block cluster per
+ * column, where that fits, and replays graphs elsewhere.
  */
 gw_status gw_set_graphs(gw_ctx* ctx, int on);
 
@@ -393,12 +395,14 @@ gw_status gw_set_graphs(gw_ctx* ctx, int on);
  */
 gw_status gw_set_solver(gw_ctx* ctx, double tol, double tol_inner, int max_iter, int max_outer);
 
-/* Kernel of the CG passes at omega = 0 (gw_set_cg_kernel). */
+/* Kernel of the CG passes at omega = 0 (gw_set_cg_kernel).  A context on which
+ * it was never called takes the cluster form where it fits. */
 typedef enum {
-  GW_CG_PERSISTENT = 0,    /* one cooperative persistent launch per pass (default) */
+  GW_CG_PERSISTENT = 0,    /* one cooperative persistent launch per pass */
   GW_CG_MULTI_LAUNCH = 1,  /* one launch per transform pass, projector and update, per iteration */
-  GW_CG_CLUSTER = 2        /* one thread-block cluster per column (falls back to the persistent
-                              kernel when a column's planes do not fit in a cluster) */
+  GW_CG_CLUSTER = 2        /* one thread-block cluster per pair of columns that are real in real
+                              space (the persistent kernel for other columns, and when the grid
+                              size has no radices there or a pair does not fit in a cluster) */
 } gw_cg_kernel;
 
 /*

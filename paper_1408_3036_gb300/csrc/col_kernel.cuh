@@ -1,0 +1,1330 @@
+// Column solver (Eq. P2 inside the FP64 refinement): one thread-block cluster
+// of Q = 1, 2, 4, 8 or 16 CTAs runs the whole inner pass of one unit,
+//   COL_CG_PAIR   two columns that are real in real space, conjugate gradients
+//   COL_QMR       one complex column, simplified QMR (bilinear form)
+//   COL_QMR_PAIR  two real columns with real shifts, simplified QMR
+// with everything an iteration exchanges in (distributed) shared memory; units
+// do not wait for one another, and no iteration returns to the host.
+//
+// Work split.  The CTA of rank r owns a contiguous range of mirror pairs of
+// disc pencils {(i0, i1), (-i0, -i1)} -- so G and -G live in the same CTA --
+// and the slabs i2 = r nzl .. (r + 1) nzl.  One application of H:
+//   scatter, z-IFFT of the own pencils, values sent to the slab owners
+//   per slab: y-IFFT of the planes |n0| <= nm, x-IFFT, * V(r)/N_g, x-FFT,
+//     y-FFT, the disc values sent back to the pencil owners
+//   z-FFT, gather, kinetic part
+// so that only the disc's values (npen N) cross the cluster, twice.
+//
+// Transforms.  N = N1 N2, both radices in registers: step 1 takes
+// x[n1 N2 + n2] over n1 and leaves k1 in its place (times w_N^(k1 n2)), step 2
+// takes n2 over N2 contiguous slots and leaves X[k1 + N1 k2] at slot
+// k1 N2 + k2.  The way back runs the transposed steps from that slot order to
+// natural order, so every pass is in place, no pass only reorders, and the
+// second x step, the product with V and the first step back are one pass.
+//
+// Half-sphere storage.  A half entry h stands for G and -G (h = 0: G = 0).
+// A real column has c(-G) = conj c(G): one complex value per half entry and
+// real projector coefficients; a pair shares the transform as u_0 + i u_1.  A
+// complex column keeps both values.  The projector rows are real in real space
+// too, so <C|y> = sum_h conj(c) y(G) + c y(-G) takes 4 real products per row
+// and half entry for either kind, half of what the full sphere takes, and half
+// of the rows' bytes.
+//
+// Scalars of the recurrences come from ordered sums that every CTA of the
+// cluster forms from the same partial sums: all CTAs decide alike.
+//
+// What bounds it: the latency of one unit's iteration (barriers of the
+// cluster, shared-memory passes of the transforms; FP64 the FP64 pipe).
+// Measured on a GB300, one application, before (launches per step, or the
+// grid-wide task queue of kernels_cg.cu) and after: 48^3 grid, 12053 plane
+// waves, 16 CG columns, FP32 3.64 -> 2.32 ms, FP64 15.8 -> 12.5 ms; 45^3, 2007
+// plane waves, 22 complex columns 11.7 -> 4.1 ms; 32^3, 2109 plane waves, 69
+// rows, 1104 complex columns 398 -> 92 ms; 64^3, 38401 plane waves, 64 rows,
+// 256 complex columns 1082 -> 553 ms.
+#pragma once
+
+#include <cooperative_groups.h>
+
+#include <algorithm>
+#include <cmath>
+#include <map>
+#include <mutex>
+#include <tuple>
+
+#include "col.cuh"
+#include "fft.cuh"
+#include "linalg.cuh"
+
+namespace gw {
+namespace col {
+
+namespace cgr = cooperative_groups;
+
+constexpr int kTPB = 512;
+constexpr int kNW = kTPB / 32;
+constexpr size_t kSmemMax = 226 * 1024;
+constexpr int kNearWait = 32;        // SQMR iterations granted within a factor 2 of the target norm (see below)
+constexpr int kQmrWindow = 1000;     // SQMR stagnation window (as the multi-launch solver's)
+
+template <typename T> struct alignas(16) V4 { T x, y, z, w; };
+
+// --- scalar sums: FP64, or a float pair whose additions are error-free
+// transformations (Knuth's TwoSum; products split through an FMA)
+template <typename T> struct AccOf { using type = double; };
+template <> struct AccOf<float> { using type = float2; };
+template <typename T> using Acc = typename AccOf<T>::type;
+__device__ __forceinline__ double add_(double a, double b) { return a + b; }
+__device__ __forceinline__ float2 add_(float2 a, float2 b) {
+  const float s = __fadd_rn(a.x, b.x);
+  const float bb = __fsub_rn(s, a.x);
+  const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
+  const float t = __fadd_rn(e, __fadd_rn(a.y, b.y));
+  const float h = __fadd_rn(s, t);
+  return make_float2(h, __fsub_rn(t, __fsub_rn(h, s)));
+}
+__device__ __forceinline__ double scale_(double a, double c) { return a * c; }
+__device__ __forceinline__ float2 scale_(float2 a, float c) {
+  const float p = __fmul_rn(a.x, c);
+  const float e = fmaf(a.y, c, fmaf(a.x, c, -p));
+  const float h = __fadd_rn(p, e);
+  return make_float2(h, __fsub_rn(e, __fsub_rn(h, p)));
+}
+__device__ __forceinline__ void fma_(double& acc, double a, double b) { acc += a * b; }
+__device__ __forceinline__ void fma_(float2& acc, float a, float b) {
+  const float p = __fmul_rn(a, b);
+  acc = add_(acc, make_float2(p, fmaf(a, b, -p)));
+}
+__device__ __forceinline__ double of_(double x) { return x; }
+__device__ __forceinline__ float2 of_(float x) { return make_float2(x, 0.f); }
+__device__ __forceinline__ double val_(double a) { return a; }
+__device__ __forceinline__ float val_(float2 a) { return __fadd_rn(a.x, a.y); }
+__device__ __forceinline__ double dbl_(double a) { return a; }
+__device__ __forceinline__ double dbl_(float2 a) { return (double)a.x + (double)a.y; }
+__device__ __forceinline__ double shx_(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ float2 shx_(float2 a, int o) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
+}
+
+// --- R-point transforms in registers
+template <typename T, int S> __device__ __forceinline__ cpx<T> rot(cpx<T> a, T c, T s) {   // a (c + S i s)
+  return S > 0 ? mk<T>(a.x * c - a.y * s, a.y * c + a.x * s) : mk<T>(a.x * c + a.y * s, a.y * c - a.x * s);
+}
+template <typename T, int S, int R> __device__ __forceinline__ void dft(cpx<T>* v) {
+  using V = cpx<T>;
+  if constexpr (R <= 5) {
+    if constexpr (R > 1) butterfly<T, S>(v, R);
+  } else if constexpr (R == 9) {
+    const T c1 = (T)0.76604444311897803520, s1 = (T)0.64278760968653932632;   // exp(2 pi i / 9)
+    const T c2 = (T)0.17364817766693034885, s2 = (T)0.98480775301220805937;
+    const T c4 = (T)-0.93969262078590838405, s4 = (T)0.34202014332566873304;
+    V a[3][3];
+#pragma unroll
+    for (int n2 = 0; n2 < 3; ++n2) {
+#pragma unroll
+      for (int n1 = 0; n1 < 3; ++n1) a[n2][n1] = v[3 * n1 + n2];
+      butterfly<T, S>(a[n2], 3);
+    }
+    a[1][1] = rot<T, S>(a[1][1], c1, s1);
+    a[1][2] = rot<T, S>(a[1][2], c2, s2);
+    a[2][1] = rot<T, S>(a[2][1], c2, s2);
+    a[2][2] = rot<T, S>(a[2][2], c4, s4);
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+      V b[3] = {a[0][k1], a[1][k1], a[2][k1]};
+      butterfly<T, S>(b, 3);
+#pragma unroll
+      for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = b[k2];
+    }
+  } else {                                   // 6, 8, 10: two interleaved transforms of R / 2 points
+    constexpr int H = R / 2;
+    V e[H], o[H];
+#pragma unroll
+    for (int k = 0; k < H; ++k) { e[k] = v[2 * k]; o[k] = v[2 * k + 1]; }
+    butterfly<T, S>(e, H);
+    butterfly<T, S>(o, H);
+    if constexpr (R == 6) {
+      const T h = (T)0.86602540378443864676;
+      o[1] = rot<T, S>(o[1], (T)0.5, h);
+      o[2] = rot<T, S>(o[2], (T)-0.5, h);
+    } else if constexpr (R == 8) {
+      const T h = (T)0.70710678118654752440;
+      const V p = o[1], q = o[3];
+      o[1] = S > 0 ? mk<T>((p.x - p.y) * h, (p.x + p.y) * h) : mk<T>((p.x + p.y) * h, (p.y - p.x) * h);
+      o[2] = mul_i(o[2], S);
+      o[3] = S > 0 ? mk<T>(-(q.x + q.y) * h, (q.x - q.y) * h) : mk<T>((q.y - q.x) * h, -(q.x + q.y) * h);
+    } else {
+      const T c1 = (T)0.80901699437494742410, s1 = (T)0.58778525229247312917;   // exp(2 pi i / 10)
+      const T c2 = (T)0.30901699437494742410, s2 = (T)0.95105651629515357212;
+      o[1] = rot<T, S>(o[1], c1, s1);
+      o[2] = rot<T, S>(o[2], c2, s2);
+      o[3] = rot<T, S>(o[3], -c2, s2);
+      o[4] = rot<T, S>(o[4], -c1, s1);
+    }
+#pragma unroll
+    for (int k = 0; k < H; ++k) { v[k] = cadd(e[k], o[k]); v[k + H] = csub(e[k], o[k]); }
+  }
+}
+// v[k] *= w_N^(S k m)  (stw holds exp(-2 pi i k / N); k m < N)
+template <typename T, int S, int R> __device__ __forceinline__ void twid(cpx<T>* v, const cpx<T>* stw, int m) {
+#pragma unroll
+  for (int k = 1; k < R; ++k) {
+    cpx<T> w = stw[k * m];
+    if (S > 0) w.y = -w.y;
+    v[k] = cmul(v[k], w);
+  }
+}
+template <int R> struct IC { static constexpr int value = R; };
+template <class F> __device__ __forceinline__ void radix1(int r, F f) {
+  switch (r) {
+    case 3: f(IC<3>()); break;
+    case 4: f(IC<4>()); break;
+    case 5: f(IC<5>()); break;
+    case 6: f(IC<6>()); break;
+    default: f(IC<8>());
+  }
+}
+template <class F> __device__ __forceinline__ void radix2(int r, F f) {
+  switch (r) {
+    case 4: f(IC<4>()); break;
+    case 5: f(IC<5>()); break;
+    case 6: f(IC<6>()); break;
+    case 8: f(IC<8>()); break;
+    case 9: f(IC<9>()); break;
+    default: f(IC<10>());
+  }
+}
+
+// --- shared memory of one CTA (byte offsets)
+struct Lay {
+  size_t Z, R, T, X, C, K, kin, hpos, rt, own, zm, zs, tw, coefp, coef, sc, total;
+};
+__host__ __device__ inline size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
+__host__ __device__ inline int splits(int nproj) { return nproj >= kNW ? 1 : (nproj > 0 ? kNW / nproj : 1); }
+
+template <typename T>
+__host__ __device__ inline Lay layout(int kind, const ColShape& sh, int N, int P, int npair, int ldz, int nhl,
+                                      int nproj) {
+  const size_t sv = sizeof(cpx<T>), s4 = 4 * sizeof(T);
+  const int Q = 1 << sh.lq, nzl = (N + Q - 1) / Q, nv = kind == COL_CG_PAIR ? 4 : 2;
+  const size_t tile = (size_t)sh.nsb * N * (N | 1) * sv, temp = (size_t)nhl * s4;
+  Lay L;
+  L.Z = 0;
+  L.R = up16(L.Z + (size_t)N * ldz * sv);
+  L.T = up16(L.R + (size_t)nzl * (2 * npair) * sv);
+  L.X = up16(L.T + (tile > temp ? tile : temp));
+  L.C = up16(L.X + (sh.vec_smem ? 4 * (size_t)nhl * s4 : 0));
+  L.K = up16(L.C + (sh.c_smem ? (size_t)nproj * nhl * sv : 0));
+  L.kin = up16(L.K + (size_t)nhl * (kind == COL_QMR ? 1 : 2) * sizeof(T));
+  L.hpos = up16(L.kin + (size_t)nhl * sizeof(T));
+  L.rt = up16(L.hpos + (size_t)nhl * sizeof(unsigned));
+  L.own = up16(L.rt + (size_t)N * P * sizeof(unsigned short));
+  L.zm = up16(L.own + (size_t)2 * npair);
+  L.zs = up16(L.zm + (size_t)ldz);
+  L.tw = up16(L.zs + (size_t)N);
+  L.coefp = up16(L.tw + (size_t)N * sv);
+  L.coef = up16(L.coefp + (size_t)Q * splits(nproj) * nproj * nv * sizeof(T));
+  L.sc = up16(L.coef + (size_t)nproj * nv * sizeof(T));
+  L.total = up16(L.sc + (size_t)3 * Q * kNW * 4 * sizeof(Acc<T>));
+  return L;
+}
+
+// Per-column state of the recurrences (every CTA keeps its own equal copy).
+template <typename T> struct CgCol {
+  T gam, gprev, alpha, stop, rmin, rbest, al, bt;
+  int it, itb, active, flag;
+};
+struct QmrCol {
+  double2 rho, alpha, beta, qc;
+  double dc, theta, tau, stop, qbest;
+  int it, itb, near, active, flag, upd;
+};
+
+template <typename T, int KIND>
+__global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
+  using V = cpx<T>;
+  using W4 = V4<T>;
+  using SA = Acc<T>;
+  constexpr bool PAIR = KIND != COL_QMR;
+  constexpr bool CG = KIND == COL_CG_PAIR;
+  constexpr int NV = CG ? 4 : 2;
+  constexpr int NC = PAIR ? 2 : 1;
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ int s_pb[kColMaxQ + 1];
+  __shared__ CgCol<T> s_cg[2];
+  __shared__ QmrCol s_q[2];
+  __shared__ int s_any;
+  cgr::cluster_group cl = cgr::this_cluster();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int Q = 1 << a.sh.lq, rank = Q > 1 ? (int)cl.block_rank() : 0;
+  int unit = blockIdx.x >> a.sh.lq;
+  if (a.order) unit = a.order[unit];
+  const int c0 = PAIR ? 2 * unit : unit, nc = min(NC, a.ncol - c0);
+  bool on[2] = {false, false};
+  for (int c = 0; c < nc; ++c) on[c] = !a.outer_active || a.outer_active[c0 + c];
+  if (!on[0] && !on[1]) {                         // the whole cluster leaves together
+    if (rank == 0 && tid < nc) { a.iters[c0 + tid] = 0; a.flags[c0 + tid] = 0; }
+    return;
+  }
+  const int N = a.N, N1 = a.N1, N2 = a.N2, P = a.P, LD = N | 1, ldz = a.ldz, ldr = 2 * a.npair;
+  const int nproj = a.nproj, nsplit = splits(nproj);
+  const Lay L = layout<T>(KIND, a.sh, N, P, a.npair, ldz, a.nhl, nproj);
+  V* Z = reinterpret_cast<V*>(sm + L.Z);          // [N][ldz] own pencils
+  V* R = reinterpret_cast<V*>(sm + L.R);          // [nzl][ldr] own slabs, disc values
+  V* Tt = reinterpret_cast<V*>(sm + L.T);         // [nsb][N][LD] slab tiles
+  W4* Tm = reinterpret_cast<W4*>(sm + L.T);       // [nhl] A u (shares the tiles' place)
+  T* Kt = reinterpret_cast<T*>(sm + L.K);
+  T* kin = reinterpret_cast<T*>(sm + L.kin);
+  unsigned* hpos = reinterpret_cast<unsigned*>(sm + L.hpos);
+  unsigned short* rt = reinterpret_cast<unsigned short*>(sm + L.rt);
+  unsigned char* own = sm + L.own;
+  signed char* zm = reinterpret_cast<signed char*>(sm + L.zm);
+  unsigned char* zs = sm + L.zs;
+  V* stw = reinterpret_cast<V*>(sm + L.tw);
+  T* coefp = reinterpret_cast<T*>(sm + L.coefp);  // [Q][nsplit][nproj][NV]
+  T* coef = reinterpret_cast<T*>(sm + L.coef);    // [nproj][NV]
+  SA* sc = reinterpret_cast<SA*>(sm + L.sc);      // [3][Q][kNW][4]
+  const int nsc = Q * kNW * 4;
+
+  auto at = [&](auto* p, int q) { return Q > 1 ? cl.map_shared_rank(p, q) : p; };
+  auto csync = [&]() { if (Q > 1) cl.sync(); else __syncthreads(); };
+
+  // ---- tables
+  if (tid <= Q) s_pb[tid] = a.split[a.sh.lq * (kColMaxQ + 1) + tid];
+  __syncthreads();
+  const int p0 = s_pb[rank], npl = s_pb[rank + 1] - p0, nrl = 2 * npl;
+  const int h0 = a.hstart[p0], nh = a.hstart[p0 + npl] - h0;
+  const int nzl = (N + Q - 1) >> a.sh.lq, z0 = rank * nzl, nsl = max(0, min(nzl, N - z0));
+  FastDiv dnr;
+  dnr.set((unsigned)max(nrl, 1));
+  auto owner = [&](int j) { int o = 0; while (o + 1 < Q && j >= s_pb[o + 1]) ++o; return o; };
+  for (int k = tid; k < N; k += kTPB) {
+    stw[k] = a.tw[k];
+    zs[k] = (unsigned char)((k % N1) * N2 + k / N1);
+  }
+  for (int k = tid; k < 2 * a.npair; k += kTPB) {
+    const int j = k >> 1, m = k & 1, o = owner(j);
+    own[2 * s_pb[o] + (m ? s_pb[o + 1] - s_pb[o] : 0) + (j - s_pb[o])] = (unsigned char)o;
+  }
+  for (int k = tid; k < N * P; k += kTPB) {
+    const unsigned d = a.disc[k];
+    unsigned v = 0xffffu;
+    if (d != 0xffffu) {
+      const int j = d >> 1, o = owner(j);
+      v = (unsigned)(2 * s_pb[o] + ((d & 1) ? s_pb[o + 1] - s_pb[o] : 0) + (j - s_pb[o]));
+    }
+    rt[k] = (unsigned short)v;
+  }
+  for (int k = tid; k < nrl; k += kTPB) {
+    const int j = p0 + (k < npl ? k : k - npl);
+    zm[k] = (signed char)((j == 0 && k >= npl) ? -1 : (int)a.zmax[j]);
+  }
+  T rtk[2] = {(T)0, (T)0};
+  T Ex[2] = {(T)0, (T)0}, Ey = (T)0;
+  for (int c = 0; c < nc; ++c) {
+    rtk[c] = (a.tk && a.tk[c0 + c] != 0.0) ? (T)(1.0 / a.tk[c0 + c]) : (T)0;
+    Ex[c] = (T)a.E[c0 + c].x;
+    if (!PAIR) Ey = (T)a.E[c0].y;
+  }
+  // solver vectors: CG r, p, s, x; SQMR r, q, d, x
+  const size_t xs = a.sh.vec_smem ? (size_t)a.nhl : (size_t)a.nh;
+  W4* X = a.sh.vec_smem ? reinterpret_cast<W4*>(sm + L.X)
+                        : reinterpret_cast<W4*>(a.vecs + (size_t)unit * a.sh.vec_elems) + h0;
+  const V* C = a.Ch + h0;
+  size_t ldc = (size_t)a.nh;
+  if (a.sh.c_smem) {
+    V* Cs = reinterpret_cast<V*>(sm + L.C);
+    for (int v = warp; v < nproj; v += kNW)
+      for (int e = lane; e < nh; e += 32) Cs[(size_t)v * a.nhl + e] = C[(size_t)v * ldc + e];
+    C = Cs;
+    ldc = (size_t)a.nhl;
+  }
+  for (int e = tid; e < nh; e += kTPB) {
+    const int h = h0 + e;
+    const T k = a.kin[h];
+    kin[e] = k;
+    hpos[e] = a.hpos[h];
+    if (PAIR) {
+      Kt[2 * e] = (rtk[0] != (T)0) ? tpa<T>(k * rtk[0]) : (T)1;
+      Kt[2 * e + 1] = (rtk[1] != (T)0) ? tpa<T>(k * rtk[1]) : (T)1;
+    } else {
+      Kt[e] = (rtk[0] != (T)0) ? tpa<T>(k * rtk[0]) : (T)1;
+    }
+    const int g = a.gp[h], m = a.gm[h];
+    W4 r = {(T)0, (T)0, (T)0, (T)0};
+    if (PAIR) {
+      double2 b[2] = {make_double2(0, 0), make_double2(0, 0)};
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        if (on[c]) {
+          const double2 u = a.b64[(size_t)(c0 + c) * a.npw + g], w = a.b64[(size_t)(c0 + c) * a.npw + m];
+          b[c] = make_double2(0.5 * (u.x + w.x), 0.5 * (u.y - w.y));
+        }
+      r = {(T)b[0].x, (T)b[0].y, (T)b[1].x, (T)b[1].y};
+    } else {
+      const double2 u = a.b64[(size_t)c0 * a.npw + g], w = a.b64[(size_t)c0 * a.npw + m];
+      r = {(T)u.x, (T)u.y, (T)w.x, (T)w.y};
+      if (h == 0) r.z = r.w = (T)0;
+    }
+    const W4 zero = {(T)0, (T)0, (T)0, (T)0};
+    X[e] = r;
+    X[xs + e] = zero;
+    X[2 * xs + e] = zero;
+    X[3 * xs + e] = zero;
+  }
+  if (tid < 2) {
+    s_cg[tid] = CgCol<T>{};
+    s_q[tid] = QmrCol{};
+  }
+  csync();                                        // every CTA of the cluster has started
+
+  const T one = (T)1, two = (T)2;
+  auto mirror_row = [&](int j) { return j == 0 ? 0 : npl + (j - p0); };   // local row of a pair's second pencil
+
+  // u (both halves of the pair, or the complex column) into the own pencils
+  auto scatter = [&](int e, const W4& u) {
+    const unsigned hp = hpos[e];
+    const int j = (int)(hp >> 8), z = (int)(hp & 255u);
+    V g, m;
+    if (PAIR) {
+      g = mk<T>(u.x - u.w, u.y + u.z);
+      m = mk<T>(u.x + u.w, u.z - u.y);
+    } else {
+      g = mk<T>(u.x, u.y);
+      m = mk<T>(u.z, u.w);
+    }
+    Z[z * ldz + (j - p0)] = g;
+    if (h0 + e != 0) Z[(N - z) % N * ldz + mirror_row(j)] = m;
+  };
+
+  // z-IFFT of the own pencils, sent to the slab owners
+  auto z_inverse = [&]() {
+    radix1(N1, [&](auto RR) {
+      constexpr int R1 = decltype(RR)::value;
+      for (int t = tid; t < nrl * N2; t += kTPB) {
+        const int n2 = dnr.div(t), row = t - n2 * nrl;
+        const int zmx = zm[row];
+        V v[R1];
+#pragma unroll
+        for (int n1 = 0; n1 < R1; ++n1) {
+          const int z = n1 * N2 + n2;
+          v[n1] = (z <= zmx || z >= N - zmx) ? Z[z * ldz + row] : mk<T>(0, 0);
+        }
+        dft<T, 1, R1>(v);
+        twid<T, 1, R1>(v, stw, n2);
+#pragma unroll
+        for (int k = 0; k < R1; ++k) Z[(k * N2 + n2) * ldz + row] = v[k];
+      }
+    });
+    __syncthreads();
+    radix2(N2, [&](auto RR) {
+      constexpr int R2 = decltype(RR)::value;
+      for (int t = tid; t < nrl * N1; t += kTPB) {
+        const int k1 = dnr.div(t), row = t - k1 * nrl;
+        V v[R2];
+#pragma unroll
+        for (int k = 0; k < R2; ++k) v[k] = Z[(k1 * R2 + k) * ldz + row];
+        dft<T, 1, R2>(v);
+#pragma unroll
+        for (int k = 0; k < R2; ++k) {
+          const int z = k1 + N1 * k;
+          const int o = a.dnz.div(z);
+          at(R, o)[(z - o * nzl) * ldr + 2 * p0 + row] = v[k];
+        }
+      }
+    });
+  };
+
+  // the slabs: returns true when the unit has stopped (CG: decided while the
+  // first step runs)
+  auto slabs = [&](bool check) {
+    const int absent = N - P;                     // planes without entries: nm < i0 < N - nm
+    for (int sb = 0; sb < max(nsl, 1); sb += a.sh.nsb) {
+      const int ns = min(a.sh.nsb, nsl - sb);
+      radix1(N1, [&](auto RR) {
+        constexpr int R1 = decltype(RR)::value;
+        for (int t = tid; t < ns * N2 * P; t += kTPB) {
+          const int q = a.dP.div(t), p = t - q * P, s = a.dN2.div(q), n2 = q - s * N2;
+          const V* src = R + (size_t)(sb + s) * ldr;
+          V v[R1];
+#pragma unroll
+          for (int n1 = 0; n1 < R1; ++n1) {
+            const unsigned row = rt[(n1 * N2 + n2) * P + p];
+            v[n1] = row != 0xffffu ? src[row] : mk<T>(0, 0);
+          }
+          dft<T, 1, R1>(v);
+          twid<T, 1, R1>(v, stw, n2);
+          V* d = Tt + (s * N + (p <= a.nm ? p : p + absent)) * LD + n2;
+#pragma unroll
+          for (int k = 0; k < R1; ++k) d[k * N2] = v[k];
+        }
+      });
+      __syncthreads();
+      if (check && sb == 0 && !s_any) return true;
+      radix2(N2, [&](auto RR) {
+        constexpr int R2 = decltype(RR)::value;
+        for (int t = tid; t < ns * N1 * P; t += kTPB) {
+          const int q = a.dP.div(t), p = t - q * P, s = a.dN1.div(q), k1 = q - s * N1;
+          V* d = Tt + (s * N + (p <= a.nm ? p : p + absent)) * LD + k1 * R2;
+          V v[R2];
+#pragma unroll
+          for (int k = 0; k < R2; ++k) v[k] = d[k];
+          dft<T, 1, R2>(v);
+#pragma unroll
+          for (int k = 0; k < R2; ++k) d[k] = v[k];
+        }
+      });
+      __syncthreads();
+      radix1(N1, [&](auto RR) {
+        constexpr int R1 = decltype(RR)::value;
+        for (int t = tid; t < ns * N2 * N; t += kTPB) {
+          const int q = a.dN.div(t), y = t - q * N, s = a.dN2.div(q), n2 = q - s * N2;
+          V* d = Tt + (s * N + n2) * LD + y;
+          V v[R1];
+#pragma unroll
+          for (int n1 = 0; n1 < R1; ++n1) {
+            const int x = n1 * N2 + n2;
+            v[n1] = (x <= a.nm || x >= N - a.nm) ? d[n1 * N2 * LD] : mk<T>(0, 0);
+          }
+          dft<T, 1, R1>(v);
+          twid<T, 1, R1>(v, stw, n2);
+#pragma unroll
+          for (int k = 0; k < R1; ++k) d[k * N2 * LD] = v[k];
+        }
+      });
+      __syncthreads();
+      radix2(N2, [&](auto RR) {
+        constexpr int R2 = decltype(RR)::value;
+        for (int t = tid; t < ns * N1 * N; t += kTPB) {
+          const int q = a.dN.div(t), y = t - q * N, s = a.dN1.div(q), k1 = q - s * N1;
+          V* d = Tt + (s * N + k1 * R2) * LD + y;
+          const T* vp = a.Vp + ((size_t)(z0 + sb + s) * N + k1) * N + y;
+          T pot[R2];
+          V v[R2];
+#pragma unroll
+          for (int k = 0; k < R2; ++k) pot[k] = vp[k * N1 * N];
+#pragma unroll
+          for (int k = 0; k < R2; ++k) v[k] = d[k * LD];
+          dft<T, 1, R2>(v);
+#pragma unroll
+          for (int k = 0; k < R2; ++k) v[k] = mk<T>(v[k].x * pot[k], v[k].y * pot[k]);
+          dft<T, -1, R2>(v);
+          twid<T, -1, R2>(v, stw, k1);
+#pragma unroll
+          for (int k = 0; k < R2; ++k) d[k * LD] = v[k];
+        }
+      });
+      __syncthreads();
+      radix1(N1, [&](auto RR) {
+        constexpr int R1 = decltype(RR)::value;
+        for (int t = tid; t < ns * N2 * N; t += kTPB) {
+          const int q = a.dN.div(t), y = t - q * N, s = a.dN2.div(q), n2 = q - s * N2;
+          V* d = Tt + (s * N + n2) * LD + y;
+          V v[R1];
+#pragma unroll
+          for (int k = 0; k < R1; ++k) v[k] = d[k * N2 * LD];
+          dft<T, -1, R1>(v);
+#pragma unroll
+          for (int n1 = 0; n1 < R1; ++n1) {
+            const int x = n1 * N2 + n2;
+            if (x <= a.nm || x >= N - a.nm) d[n1 * N2 * LD] = v[n1];
+          }
+        }
+      });
+      __syncthreads();
+      radix2(N2, [&](auto RR) {
+        constexpr int R2 = decltype(RR)::value;
+        for (int t = tid; t < ns * N1 * P; t += kTPB) {
+          const int q = a.dP.div(t), p = t - q * P, s = a.dN1.div(q), k1 = q - s * N1;
+          V* d = Tt + (s * N + (p <= a.nm ? p : p + absent)) * LD + k1 * R2;
+          V v[R2];
+#pragma unroll
+          for (int k = 0; k < R2; ++k) v[k] = d[k];
+          dft<T, -1, R2>(v);
+          twid<T, -1, R2>(v, stw, k1);
+#pragma unroll
+          for (int k = 0; k < R2; ++k) d[k] = v[k];
+        }
+      });
+      __syncthreads();
+      radix1(N1, [&](auto RR) {
+        constexpr int R1 = decltype(RR)::value;
+        for (int t = tid; t < ns * N2 * P; t += kTPB) {
+          const int q = a.dP.div(t), p = t - q * P, s = a.dN2.div(q), n2 = q - s * N2;
+          const V* d = Tt + (s * N + (p <= a.nm ? p : p + absent)) * LD + n2;
+          V v[R1];
+#pragma unroll
+          for (int k = 0; k < R1; ++k) v[k] = d[k * N2];
+          dft<T, -1, R1>(v);
+          const int z = z0 + sb + s;
+#pragma unroll
+          for (int n1 = 0; n1 < R1; ++n1) {
+            const unsigned row = rt[(n1 * N2 + n2) * P + p];
+            if (row != 0xffffu) {
+              const int o = own[row];
+              at(Z, o)[z * ldz + ((int)row - 2 * s_pb[o])] = v[n1];
+            }
+          }
+        }
+      });
+      __syncthreads();
+    }
+    return false;
+  };
+
+  // z-FFT of the own pencils, in place (frequency z at slot zs[z])
+  auto z_forward = [&]() {
+    radix1(N1, [&](auto RR) {
+      constexpr int R1 = decltype(RR)::value;
+      for (int t = tid; t < nrl * N2; t += kTPB) {
+        const int n2 = dnr.div(t), row = t - n2 * nrl;
+        V v[R1];
+#pragma unroll
+        for (int n1 = 0; n1 < R1; ++n1) v[n1] = Z[(n1 * N2 + n2) * ldz + row];
+        dft<T, -1, R1>(v);
+        twid<T, -1, R1>(v, stw, n2);
+#pragma unroll
+        for (int k = 0; k < R1; ++k) Z[(k * N2 + n2) * ldz + row] = v[k];
+      }
+    });
+    __syncthreads();
+    radix2(N2, [&](auto RR) {
+      constexpr int R2 = decltype(RR)::value;
+      for (int t = tid; t < nrl * N1; t += kTPB) {
+        const int k1 = dnr.div(t), row = t - k1 * nrl;
+        V v[R2];
+#pragma unroll
+        for (int k = 0; k < R2; ++k) v[k] = Z[(k1 * R2 + k) * ldz + row];
+        dft<T, -1, R2>(v);
+#pragma unroll
+        for (int k = 0; k < R2; ++k) Z[(k1 * R2 + k) * ldz + row] = v[k];
+      }
+    });
+    __syncthreads();
+  };
+
+  // (V u) + (kin - E) u at one half entry
+  auto gather = [&](int e, const W4& u) {
+    const unsigned hp = hpos[e];
+    const int j = (int)(hp >> 8), z = (int)(hp & 255u);
+    const V y1 = Z[zs[z] * ldz + (j - p0)], y2 = Z[zs[(N - z) % N] * ldz + mirror_row(j)];
+    const T k = kin[e];
+    W4 t;
+    if (PAIR) {
+      t.x = (T)0.5 * (y1.x + y2.x) + (k - Ex[0]) * u.x;
+      t.y = (T)0.5 * (y1.y - y2.y) + (k - Ex[0]) * u.y;
+      t.z = (T)0.5 * (y1.y + y2.y) + (k - Ex[1]) * u.z;
+      t.w = (T)0.5 * (y2.x - y1.x) + (k - Ex[1]) * u.w;
+    } else {
+      const T dr = k - Ex[0], di = -Ey;
+      t.x = y1.x + dr * u.x - di * u.y;
+      t.y = y1.y + dr * u.y + di * u.x;
+      t.z = y2.x + dr * u.z - di * u.w;
+      t.w = y2.y + dr * u.w + di * u.z;
+      if (h0 + e == 0) t.z = t.w = (T)0;
+    }
+    return t;
+  };
+  // the four real vectors whose products with Re C and Im C are the coefficients
+  auto abcd = [&](int e, const W4& y) {
+    if (PAIR) {
+      const T f = (h0 + e == 0) ? one : two;
+      return W4{f * y.x, f * y.y, f * y.z, f * y.w};
+    }
+    return W4{y.x + y.z, y.y - y.w, y.y + y.w, y.z - y.x};
+  };
+
+  // projector coefficients of Tm (and, CG, of u = K r): partial sums over the
+  // own entries to every CTA; a warp takes RG rows (and one of the nsplit parts
+  // of the entries) at a time
+  auto dots_rows = [&](auto RR) {
+    constexpr int RG = decltype(RR)::value;
+    const int ngr = (nproj + RG - 1) / RG;
+    for (int w = warp; w < ngr * nsplit; w += kNW) {
+      const int gr = w / nsplit, part = w - gr * nsplit, v0 = gr * RG;
+      T acc[RG][NV];
+#pragma unroll
+      for (int q = 0; q < RG; ++q)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) acc[q][k] = (T)0;
+#pragma unroll 2
+      for (int e = lane + 32 * part; e < nh; e += 32 * nsplit) {
+        V c[RG];
+#pragma unroll
+        for (int q = 0; q < RG; ++q) c[q] = C[(size_t)min(v0 + q, nproj - 1) * ldc + e];
+        const W4 y = abcd(e, Tm[e]);
+        W4 u = {(T)0, (T)0, (T)0, (T)0};
+        if (CG) {
+          const W4 r = X[e];
+          const T k0 = Kt[2 * e], k1 = Kt[2 * e + 1];
+          u = abcd(e, W4{k0 * r.x, k0 * r.y, k1 * r.z, k1 * r.w});
+        }
+#pragma unroll
+        for (int q = 0; q < RG; ++q) {
+          acc[q][0] += c[q].x * y.x + c[q].y * y.y;
+          acc[q][1] += c[q].x * y.z + c[q].y * y.w;
+          if (CG) {
+            acc[q][NV - 2] += c[q].x * u.x + c[q].y * u.y;
+            acc[q][NV - 1] += c[q].x * u.z + c[q].y * u.w;
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < RG; ++q)
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) acc[q][k] += __shfl_xor_sync(0xffffffffu, acc[q][k], o);
+      if (lane < Q) {
+        T* d = at(coefp, lane);
+#pragma unroll
+        for (int q = 0; q < RG; ++q)
+          if (v0 + q < nproj)
+#pragma unroll
+            for (int k = 0; k < NV; ++k)
+              d[((size_t)(rank * nsplit + part) * nproj + v0 + q) * NV + k] = acc[q][k];
+      }
+    }
+  };
+  auto dots = [&]() {
+    if (nproj >= 4 * kNW) dots_rows(IC<4>());
+    else if (nproj >= 2 * kNW) dots_rows(IC<2>());
+    else dots_rows(IC<1>());
+  };
+  auto coef_sum = [&](int first) {                // threads from `first` on
+    for (int j = tid - first; j >= 0 && j < nproj * NV; j += kTPB - first) {
+      T s = (T)0;
+      for (int q = 0; q < Q * nsplit; ++q) s += coefp[(size_t)q * nproj * NV + j];
+      coef[j] = s;
+    }
+  };
+  // y - sum_v C_v coef_v at one half entry
+  auto project = [&](int e, W4 y) {
+    T a1 = (T)0, a2 = (T)0, a3 = (T)0, a4 = (T)0;
+    int v = 0;
+    for (; v + 8 <= nproj; v += 8) {
+      V c[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) c[q] = C[(size_t)(v + q) * ldc + e];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const T k0 = coef[(v + q) * NV], k1 = coef[(v + q) * NV + 1];
+        a1 += c[q].x * k0;
+        a4 += c[q].y * k0;
+        a3 += c[q].x * k1;
+        a2 += c[q].y * k1;
+      }
+    }
+    for (; v < nproj; ++v) {
+      const V c = C[(size_t)v * ldc + e];
+      const T k0 = coef[v * NV], k1 = coef[v * NV + 1];
+      a1 += c.x * k0;
+      a4 += c.y * k0;
+      a3 += c.x * k1;
+      a2 += c.y * k1;
+    }
+    if (PAIR) {
+      y.x -= a1; y.y -= a4; y.z -= a3; y.w -= a2;
+    } else {
+      y.x -= a1 - a2; y.y -= a3 + a4;
+      if (h0 + e != 0) { y.z -= a1 + a2; y.w -= a3 - a4; }
+    }
+    return y;
+  };
+
+  // NS sums of this thread's values to every CTA (slot k), and their ordered
+  // total in every lane of the calling warp after the cluster barrier
+  auto send_sums = [&](auto NN, SA* v, int slot) {
+    constexpr int NS = decltype(NN)::value;
+#pragma unroll
+    for (int k = 0; k < NS; ++k)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v[k] = add_(v[k], shx_(v[k], o));
+    if (lane < Q) {
+      SA* d = at(sc, lane) + slot * nsc + (rank * kNW + warp) * 4;
+#pragma unroll
+      for (int k = 0; k < NS; ++k) d[k] = v[k];
+    }
+  };
+  auto take_sum = [&](int slot, int k) {          // one warp
+    const SA* s = sc + slot * nsc + k;
+    SA t = of_((T)0);
+    for (int q = lane; q < Q * kNW; q += 32) t = add_(t, s[q * 4]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t = add_(t, shx_(t, o));
+    return t;
+  };
+
+  if constexpr (CG) {
+    // Chronopoulos and Gear's one-reduction form (see kernels_cg.cu): u = K r,
+    // w = P_c (H - E) u, gamma = r^H u, delta = u^H w
+    for (int k = 0;; ++k) {
+      // r after k updates: u into the pencils, gamma and |r|^2
+      SA v4[4] = {of_((T)0), of_((T)0), of_((T)0), of_((T)0)};
+      {
+        T g0 = (T)0, r0 = (T)0, g1 = (T)0, r1 = (T)0;
+        const T al0 = s_cg[0].al, al1 = s_cg[1].al, bt0 = s_cg[0].bt, bt1 = s_cg[1].bt;
+        const bool a0 = k == 0 || s_cg[0].active, a1 = k == 0 || s_cg[1].active;
+        for (int e = tid; e < nh; e += kTPB) {
+          const T k0 = Kt[2 * e], k1 = Kt[2 * e + 1];
+          W4 r = X[e];
+          if (k > 0) {
+            W4 p = X[xs + e], s = X[2 * xs + e], x = X[3 * xs + e];
+            const W4 w = project(e, Tm[e]);
+            if (a0) {
+              p.x = k0 * r.x + bt0 * p.x; p.y = k0 * r.y + bt0 * p.y;
+              s.x = w.x + bt0 * s.x;      s.y = w.y + bt0 * s.y;
+              x.x += al0 * p.x;           x.y += al0 * p.y;
+              r.x -= al0 * s.x;           r.y -= al0 * s.y;
+            }
+            if (a1) {
+              p.z = k1 * r.z + bt1 * p.z; p.w = k1 * r.w + bt1 * p.w;
+              s.z = w.z + bt1 * s.z;      s.w = w.w + bt1 * s.w;
+              x.z += al1 * p.z;           x.w += al1 * p.w;
+              r.z -= al1 * s.z;           r.w -= al1 * s.w;
+            }
+            X[e] = r;
+            X[xs + e] = p;
+            X[2 * xs + e] = s;
+            X[3 * xs + e] = x;
+          }
+          const T f = (h0 + e == 0) ? one : two;
+          const T n0 = f * (r.x * r.x + r.y * r.y), n1 = f * (r.z * r.z + r.w * r.w);
+          r0 += n0;
+          g0 += k0 * n0;
+          r1 += n1;
+          g1 += k1 * n1;
+          W4 u = {(T)0, (T)0, (T)0, (T)0};
+          if (a0) { u.x = k0 * r.x; u.y = k0 * r.y; }
+          if (a1) { u.z = k1 * r.z; u.w = k1 * r.w; }
+          scatter(e, u);
+        }
+        v4[0] = of_(g0); v4[1] = of_(r0); v4[2] = of_(g1); v4[3] = of_(r1);
+      }
+      send_sums(IC<4>(), v4, 0);
+      __syncthreads();
+      z_inverse();
+      csync();
+      // while the slabs' first step runs: gamma, |r|^2 and the stopping tests
+      if (warp == 0) {
+        SA g[2], q[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) { g[c] = take_sum(0, 2 * c); q[c] = take_sum(0, 2 * c + 1); }
+        int act = 0;
+        if (lane < 2) {
+          CgCol<T>& st = s_cg[lane];
+          const T gam = val_(lane ? g[1] : g[0]), rr = val_(lane ? q[1] : q[0]);
+          if (k == 0) {
+            const T s1 = (T)a.tol2 * rr, s2 = (a.rr_abs && lane < nc) ? (T)a.rr_abs[c0 + lane] : (T)0;
+            st.stop = s1 > s2 ? s1 : s2;
+            st.rmin = rr;
+            st.rbest = rr;
+            st.active = (lane < nc && on[lane] && rr > (T)0) ? 1 : 0;
+          }
+          if (st.active) {
+            st.rmin = rr < st.rmin ? rr : st.rmin;
+            if (rr < (T)0.25 * st.rbest) { st.rbest = rr; st.itb = k; }
+            int stop = 0;
+            if (!isfinite(rr)) { st.flag = 2; stop = 1; }
+            else if (rr <= st.stop) { st.flag = 0; stop = 1; }
+            else if (rr > (T)1e4 * st.rmin) { st.flag = 3; stop = 1; }
+            else if (k >= a.maxit) { st.flag = 1; stop = 1; }
+            else if (k - st.itb > max(kCgStagWindow, 2 * st.itb)) { st.flag = 4; stop = 1; }
+            st.it = k;
+            st.gprev = st.gam;
+            st.gam = gam;
+            if (stop) st.active = 0;
+          }
+          act = st.active;
+        }
+        const unsigned any = __ballot_sync(0xffffffffu, act != 0);
+        if (lane == 0) s_any = any != 0u;
+      }
+      if (slabs(true)) break;
+      csync();
+      z_forward();
+      {
+        T d0 = (T)0, d1 = (T)0;
+        for (int e = tid; e < nh; e += kTPB) {
+          const T k0 = Kt[2 * e], k1 = Kt[2 * e + 1];
+          const W4 r = X[e];
+          const W4 u = {k0 * r.x, k0 * r.y, k1 * r.z, k1 * r.w};
+          const W4 w = gather(e, u);
+          Tm[e] = w;
+          const T f = (h0 + e == 0) ? one : two;
+          d0 += f * (u.x * w.x + u.y * w.y);
+          d1 += f * (u.z * w.z + u.w * w.w);
+        }
+        v4[0] = of_(d0);
+        v4[1] = of_(d1);
+      }
+      send_sums(IC<2>(), v4, 1);
+      __syncthreads();
+      dots();
+      csync();
+      coef_sum(32);
+      SA uw0 = of_((T)0), uw1 = of_((T)0);
+      if (warp == 0) { uw0 = take_sum(1, 0); uw1 = take_sum(1, 1); }
+      __syncthreads();
+      if (warp == 0) {
+        // delta = u^H w - sum_v <C_v|u> <C_v|w>, alpha, beta
+        SA t0 = of_((T)0), t1 = of_((T)0);
+        for (int v = lane; v < nproj; v += 32) {
+          const T* c = coef + v * NV;
+          t0 = add_(t0, of_(c[0] * c[NV - 2]));
+          t1 = add_(t1, of_(c[1] * c[NV - 1]));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) { t0 = add_(t0, shx_(t0, o)); t1 = add_(t1, shx_(t1, o)); }
+        int act = 0;
+        if (lane < 2) {
+          CgCol<T>& st = s_cg[lane];
+          if (st.active) {
+            const T delta = val_(add_(lane ? uw1 : uw0, scale_(lane ? t1 : t0, (T)-1)));
+            T den = delta, bt = (T)0;
+            if (k > 0) {
+              bt = st.gam / st.gprev;
+              den = delta - bt * st.gam / st.alpha;
+            }
+            if (!(den > (T)0) || !isfinite(den) || !(st.gam > (T)0)) {
+              st.flag = 2;
+              st.active = 0;
+            } else {
+              st.alpha = st.gam / den;
+              st.al = st.alpha;
+              st.bt = bt;
+            }
+          }
+          act = st.active;
+        }
+        const unsigned any = __ballot_sync(0xffffffffu, act != 0);
+        if (lane == 0) s_any = any != 0u;
+      }
+      __syncthreads();
+      if (!s_any) break;
+    }
+  } else {
+    // simplified QMR (kernels_linalg.cu has the recurrences):
+    //   t = P_c (H - E) q; alpha = rho / [q, t]; r -= alpha t;
+    //   theta, tau from |r|; d = dc d + qc q; x += d; rho' = [r, K r]; q = K r + beta q
+    auto kk = [&](int e, int c) { return PAIR ? Kt[2 * e + c] : Kt[e]; };
+    // r^H r and [r, K r] of one entry into v (PAIR: rr0, rr1, rho0, rho1; else rr, rho)
+    auto norms = [&](int e, const W4& r, SA* v) {
+      if (PAIR) {
+        const T f = (h0 + e == 0) ? one : two;
+        const T k0 = f * kk(e, 0), k1 = f * kk(e, 1);
+        fma_(v[0], f * r.x, r.x); fma_(v[0], f * r.y, r.y);
+        fma_(v[1], f * r.z, r.z); fma_(v[1], f * r.w, r.w);
+        fma_(v[2], k0 * r.x, r.x); fma_(v[2], k0 * r.y, r.y);
+        fma_(v[3], k1 * r.z, r.z); fma_(v[3], k1 * r.w, r.w);
+      } else {
+        const T k = kk(e, 0);
+        fma_(v[0], r.x, r.x); fma_(v[0], r.y, r.y); fma_(v[0], r.z, r.z); fma_(v[0], r.w, r.w);
+        if (h0 + e == 0) {
+          fma_(v[1], k * r.x, r.x); fma_(v[1], -k * r.y, r.y);
+          fma_(v[2], two * k * r.x, r.y);
+        } else {
+          const T k2 = two * k;
+          fma_(v[1], k2 * r.x, r.z); fma_(v[1], -k2 * r.y, r.w);
+          fma_(v[2], k2 * r.x, r.w); fma_(v[2], k2 * r.y, r.z);
+        }
+      }
+    };
+    // totals of the four slots of `norms` for column c: |r|^2, rho
+    auto take_norms = [&](int slot, int c, double* rr, double2* rho) {
+      if (PAIR) {
+        const double a0 = dbl_(take_sum(slot, 0)), a1 = dbl_(take_sum(slot, 1));
+        const double b0 = dbl_(take_sum(slot, 2)), b1 = dbl_(take_sum(slot, 3));
+        *rr = c ? a1 : a0;
+        *rho = make_double2(c ? b1 : b0, 0.0);
+      } else {
+        *rr = dbl_(take_sum(slot, 0));
+        const double x = dbl_(take_sum(slot, 1));
+        *rho = make_double2(x, dbl_(take_sum(slot, 2)));
+      }
+    };
+    auto cdiv_ = [](double2 p, double2 q) {
+      if (PAIR) return make_double2(p.x / q.x, 0.0);
+      const double den = q.x * q.x + q.y * q.y;
+      return make_double2((p.x * q.x + p.y * q.y) / den, (p.y * q.x - p.x * q.y) / den);
+    };
+    {
+      SA v[4] = {of_((T)0), of_((T)0), of_((T)0), of_((T)0)};
+      for (int e = tid; e < nh; e += kTPB) {
+        const W4 r = X[e];
+        norms(e, r, v);
+        const T k0 = kk(e, 0), k1 = kk(e, NC - 1);
+        const W4 q = {k0 * r.x, k0 * r.y, k1 * r.z, k1 * r.w};
+        X[xs + e] = q;
+        scatter(e, q);
+      }
+      send_sums(IC<4>(), v, 0);
+      csync();
+      if (warp == 0) {
+        double rr;
+        double2 rho;
+        take_norms(0, lane, &rr, &rho);
+        int act = 0;
+        if (lane < nc) {
+          QmrCol& st = s_q[lane];
+          st.tau = sqrt(rr);
+          st.rho = rho;
+          st.stop = fmax(a.tol2 * rr, a.rr_abs ? a.rr_abs[c0 + lane] : 0.0);
+          st.qbest = rr;
+          st.near = -1;
+          st.active = act = (on[lane] && rr > 0.0) ? 1 : 0;
+        }
+        const unsigned any = __ballot_sync(0xffffffffu, act != 0);
+        if (lane == 0) s_any = any != 0u;
+      }
+      __syncthreads();
+    }
+    while (s_any) {
+      z_inverse();
+      csync();
+      slabs(false);
+      csync();
+      z_forward();
+      for (int e = tid; e < nh; e += kTPB) Tm[e] = gather(e, X[xs + e]);
+      __syncthreads();
+      dots();
+      csync();
+      coef_sum(0);
+      __syncthreads();
+      // t = P_c t and [q, t]
+      SA v[4] = {of_((T)0), of_((T)0), of_((T)0), of_((T)0)};
+      for (int e = tid; e < nh; e += kTPB) {
+        const W4 t = project(e, Tm[e]);
+        Tm[e] = t;
+        const W4 q = X[xs + e];
+        if (PAIR) {
+          const T f = (h0 + e == 0) ? one : two;
+          fma_(v[0], f * q.x, t.x); fma_(v[0], f * q.y, t.y);
+          fma_(v[1], f * q.z, t.z); fma_(v[1], f * q.w, t.w);
+        } else if (h0 + e == 0) {
+          fma_(v[0], q.x, t.x); fma_(v[0], -q.y, t.y);
+          fma_(v[1], q.x, t.y); fma_(v[1], q.y, t.x);
+        } else {
+          fma_(v[0], q.z, t.x); fma_(v[0], -q.w, t.y); fma_(v[0], q.x, t.z); fma_(v[0], -q.y, t.w);
+          fma_(v[1], q.z, t.y); fma_(v[1], q.w, t.x); fma_(v[1], q.x, t.w); fma_(v[1], q.y, t.z);
+        }
+      }
+      send_sums(IC<2>(), v, 1);
+      csync();
+      if (warp == 0) {
+        const double s0 = dbl_(take_sum(1, 0)), s1 = dbl_(take_sum(1, 1));
+        if (lane < nc) {
+          QmrCol& st = s_q[lane];
+          const double2 sg = PAIR ? make_double2(lane ? s1 : s0, 0.0) : make_double2(s0, s1);
+          const double2 rho = st.rho;
+          if (!st.active) {
+            // a stopped column of a pair: q = 0, nothing to update
+          } else if (!(sg.x * sg.x + sg.y * sg.y > 1e-300 * (rho.x * rho.x + rho.y * rho.y)) || !isfinite(sg.x) ||
+              !isfinite(sg.y)) {
+            st.alpha = make_double2(0.0, 0.0);
+            st.flag = 2;                          // serious breakdown: [q, A q] = 0
+          } else {
+            st.alpha = cdiv_(rho, sg);
+          }
+        }
+      }
+      __syncthreads();
+      // r -= alpha t
+      {
+        const bool a0 = s_q[0].active, a1 = PAIR ? s_q[1].active : a0;
+        const T ax = (T)s_q[0].alpha.x, ay = (T)(PAIR ? s_q[1].alpha.x : s_q[0].alpha.y);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = of_((T)0);
+        for (int e = tid; e < nh; e += kTPB) {
+          W4 r = X[e];
+          const W4 t = Tm[e];
+          if (PAIR) {
+            if (a0) { r.x -= ax * t.x; r.y -= ax * t.y; }
+            if (a1) { r.z -= ay * t.z; r.w -= ay * t.w; }
+          } else {
+            r.x -= ax * t.x - ay * t.y;
+            r.y -= ax * t.y + ay * t.x;
+            r.z -= ax * t.z - ay * t.w;
+            r.w -= ax * t.w + ay * t.z;
+          }
+          X[e] = r;
+          norms(e, r, v);
+        }
+      }
+      send_sums(IC<4>(), v, 2);
+      csync();
+      if (warp == 0) {
+        double rr;
+        double2 rn;
+        take_norms(2, lane, &rr, &rn);
+        int act = 0;
+        if (lane < nc) {
+          QmrCol& st = s_q[lane];
+          st.upd = st.active;
+          if (st.active) {
+            const double th = sqrt(rr) / st.tau;
+            const double c2 = 1.0 / (1.0 + th * th);
+            st.dc = c2 * st.theta * st.theta;
+            st.qc = make_double2(c2 * st.alpha.x, c2 * st.alpha.y);
+            st.tau = st.tau * th * sqrt(c2);
+            st.theta = th;
+            const double2 rho = st.rho;
+            st.beta = (rho.x * rho.x + rho.y * rho.y > 0.0) ? cdiv_(rn, rho) : make_double2(0.0, 0.0);
+            st.rho = rn;
+            const int it = ++st.it;
+            const double qb = st.tau * st.tau;
+            if (qb < 0.25 * st.qbest) { st.qbest = qb; st.itb = it; }
+            if (st.near < 0 && qb <= 4.0 * st.stop) st.near = it;
+            bool stop = false;
+            if (st.flag == 2 || !isfinite(st.tau)) { st.flag = 2; stop = true; }
+            else if (qb <= st.stop) { st.flag = 0; stop = true; }
+            else if (!(rn.x * rn.x + rn.y * rn.y > 0.0)) { st.flag = 2; stop = true; }
+            else if (it >= a.maxit) { st.flag = 1; stop = true; }
+            else if (it - st.itb > max(kQmrWindow, 2 * st.itb)) { st.flag = 4; stop = true; }
+            // tau never grows; within a factor 2 of the target and still short
+            // of it after kNearWait iterations, it has reached the floor of
+            // the working precision (FP32 passes stop a little above 1e-5
+            // now and then): the FP64 residual of the refinement decides
+            else if (st.near >= 0 && it - st.near > kNearWait) { st.flag = 4; stop = true; }
+            if (stop) st.active = 0;
+          }
+          act = st.active;
+        }
+        const unsigned any = __ballot_sync(0xffffffffu, act != 0);
+        if (lane == 0) s_any = any != 0u;
+      }
+      __syncthreads();
+      // d = dc d + qc q; x += d; q = K r + beta q, into the pencils
+      {
+        const int l = PAIR ? 1 : 0;
+        const bool u0 = s_q[0].upd, u1 = s_q[l].upd, a0 = s_q[0].active, a1 = s_q[l].active, any = s_any;
+        const T d0 = (T)s_q[0].dc, d1 = (T)s_q[l].dc;
+        const T qx = (T)s_q[0].qc.x, qy = (T)(PAIR ? s_q[1].qc.x : s_q[0].qc.y);
+        const T bx = (T)s_q[0].beta.x, by = (T)(PAIR ? s_q[1].beta.x : s_q[0].beta.y);
+        for (int e = tid; e < nh; e += kTPB) {
+          W4 q = X[xs + e], d = X[2 * xs + e], x = X[3 * xs + e];
+          const T k0 = kk(e, 0), k1 = kk(e, NC - 1);
+          if (PAIR) {
+            if (u0) { d.x = d0 * d.x + qx * q.x; d.y = d0 * d.y + qx * q.y; x.x += d.x; x.y += d.y; }
+            if (u1) { d.z = d1 * d.z + qy * q.z; d.w = d1 * d.w + qy * q.w; x.z += d.z; x.w += d.w; }
+          } else {
+            d.x = d0 * d.x + (qx * q.x - qy * q.y);
+            d.y = d0 * d.y + (qx * q.y + qy * q.x);
+            d.z = d0 * d.z + (qx * q.z - qy * q.w);
+            d.w = d0 * d.w + (qx * q.w + qy * q.z);
+            x.x += d.x; x.y += d.y; x.z += d.z; x.w += d.w;
+          }
+          X[2 * xs + e] = d;
+          X[3 * xs + e] = x;
+          if (!any) continue;
+          const W4 r = X[e];
+          if (PAIR) {
+            q.x = a0 ? k0 * r.x + bx * q.x : (T)0;
+            q.y = a0 ? k0 * r.y + bx * q.y : (T)0;
+            q.z = a1 ? k1 * r.z + by * q.z : (T)0;
+            q.w = a1 ? k1 * r.w + by * q.w : (T)0;
+          } else {
+            q = W4{k0 * r.x + bx * q.x - by * q.y, k0 * r.y + bx * q.y + by * q.x,
+                   k0 * r.z + bx * q.z - by * q.w, k0 * r.w + bx * q.w + by * q.z};
+          }
+          X[xs + e] = q;
+          scatter(e, q);
+        }
+        __syncthreads();
+      }
+    }
+  }
+
+  // ---- the solution of the pass, added to x64 (own entries)
+  for (int e = tid; e < nh; e += kTPB) {
+    const int h = h0 + e, g = a.gp[h], m = a.gm[h];
+    const W4 x = X[3 * xs + e];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      if (c >= nc || !on[c]) continue;
+      double2* o = a.x64 + (size_t)(c0 + c) * a.npw;
+      const double ux = c ? (double)x.z : (double)x.x, uy = c ? (double)x.w : (double)x.y;
+      double2 y = o[g];
+      o[g] = make_double2(y.x + ux, y.y + uy);
+      if (h == 0) continue;
+      y = o[m];
+      o[m] = PAIR ? make_double2(y.x + ux, y.y - uy) : make_double2(y.x + (double)x.z, y.y + (double)x.w);
+    }
+  }
+  if (rank == 0 && tid < nc) {
+    a.iters[c0 + tid] = CG ? s_cg[tid].it : s_q[tid].it;
+    a.flags[c0 + tid] = CG ? s_cg[tid].flag : s_q[tid].flag;
+  }
+  csync();                                        // no CTA leaves while others may reach its memory
+}
+
+template <typename T, int KIND> struct Fn { static const void* get() { return (const void*)k_col_solve<T, KIND>; } };
+
+template <typename T> const void* kernel_of(int kind) {
+  if (kind == COL_CG_PAIR) return Fn<T, COL_CG_PAIR>::get();
+  if (kind == COL_QMR) return Fn<T, COL_QMR>::get();
+  return Fn<T, COL_QMR_PAIR>::get();
+}
+
+inline cudaLaunchConfig_t config(cudaLaunchAttribute* at, int q, int grid, size_t smem, cudaStream_t s) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(kTPB);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = q;
+  at->val.clusterDim.y = 1;
+  at->val.clusterDim.z = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return c;
+}
+
+// Kernel attributes (once per function and process) and the clusters of size q
+// that run at once (0: this size does not run here).
+template <typename T> int active_clusters(int kind, int lq, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, size_t>, int> known;
+  static bool ready[3] = {false, false, false};
+  std::lock_guard<std::mutex> lock(mu);
+  const void* f = kernel_of<T>(kind);
+  if (!ready[kind]) {
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess ||
+        cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    ready[kind] = true;
+  }
+  auto it = known.find({kind, lq, smem});
+  if (it != known.end()) return it->second;
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t c = config(&at, 1 << lq, 1 << lq, smem, nullptr);
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, f, &c) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  known[{kind, lq, smem}] = n;
+  return n;
+}
+
+}  // namespace col
+
+template <typename T>
+bool col_shape(const ColPlan& p, int kind, int N, int nproj, int nunit, int cta_div, ColShape* out) {
+  if (!p.ok || nunit < 1 || nproj > kMaxOcc) return false;
+  // An iteration of one unit takes a fixed time (barriers, reductions, scalar
+  // steps) and its work over Q CTAs; microseconds, fitted to sweeps over Q
+  // (45^3 grid, 11 rows, FP32 SQMR: 107, 57, 38, 26, 25 for Q = 1 .. 16; 48^3,
+  // 16 rows, CG pair: 55, 30, 22 for Q = 4 .. 16, FP64 424, 222 for Q = 8, 16;
+  // 16^3, 4 rows, FP64: 88, 57, 42, 35, 36).  Units beyond the clusters that
+  // run at once wait for a free one: whole rounds for CG (columns alike, but the
+  // last few pairs of a cell are its fastest); for SQMR the slowest columns,
+  // which start first, take about twice the mean.  The order of the sums, and
+  // with it the last bits, depends on Q: FP64 results do not depend on how many
+  // contexts share the GPU, so there Q does not either.
+  const bool f32 = sizeof(T) == 4;
+  const double share = f32 ? std::max(cta_div, 1) : 1.0;
+  const double fixed = f32 ? 11.0 : 27.0;
+  const double work = (f32 ? 1.0e-3 : 1.5e-2) * N * N * N + (f32 ? 0.9e-3 : 1.66e-2) * nproj * p.nh;
+  double best = 1e300;
+  for (int lq = 0; lq < kColNQ; ++lq) {
+    const int Q = 1 << lq, ldz = 2 * p.maxpair[lq], nhl = p.maxh[lq];
+    if (Q > N || Q > p.npair) continue;
+    ColShape s;
+    s.lq = lq;
+    const int nzl = (N + Q - 1) / Q;
+    auto fits = [&](int nsb, bool vec, bool c) {
+      s.nsb = nsb;
+      s.vec_smem = vec;
+      s.c_smem = c;
+      s.smem = col::layout<T>(kind, s, N, p.P, p.npair, ldz, nhl, nproj).total;
+      return s.smem <= col::kSmemMax;
+    };
+    // slabs together first (threads busy), then the vectors, then the rows
+    int nsb = nzl;
+    while (nsb > 1 && !fits(nsb, false, false)) --nsb;
+    if (!fits(nsb, false, false)) continue;
+    while (nsb > 1 && !fits(nsb, true, false) && (size_t)(nsb - 1) * N * N >= 8 * (size_t)col::kTPB) --nsb;
+    const bool vec = fits(nsb, true, false);
+    const bool c = fits(nsb, vec, true);
+    fits(nsb, vec, c);
+    s.vec_elems = vec ? 0 : 16 * (size_t)p.nh;
+    const int act = col::active_clusters<T>(kind, lq, s.smem);
+    if (act < 1) continue;
+    const double load = (double)nunit * share / act;
+    const double rounds = kind != COL_CG_PAIR ? std::max(1.0, 0.5 * load)
+                                              : load <= 1.25 ? std::max(1.0, load) : std::ceil(load);
+    const double t = rounds * (fixed + lq + work / Q);
+    if (t < best) { best = t; *out = s; }
+  }
+  return best < 1e300;
+}
+
+template <typename T>
+cudaError_t launch_col_solve(cudaStream_t s, int kind, const ColArgs<T>& a) {
+  const int Q = 1 << a.sh.lq;
+  if (col::active_clusters<T>(kind, a.sh.lq, a.sh.smem) < 1) return cudaErrorNotSupported;
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t c = col::config(&at, Q, a.nunit * Q, a.sh.smem, s);
+  ColArgs<T> arg = a;
+  void* args[] = {&arg};
+  ++g_launches;
+  return cudaLaunchKernelExC(&c, col::kernel_of<T>(kind), args);
+}
+
+namespace col {
+template <typename T>
+__global__ void k_col_perm_v(int N, int N1, int N2, const T* __restrict__ v, T* __restrict__ out) {
+  const int n = N * N * N;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int c = i % N, x = (i / N) % N, z = i / (N * N);
+    const int y = c / N2 + N1 * (c % N2);
+    out[i] = v[((size_t)x * N + y) * N + z];
+  }
+}
+template <typename T>
+__global__ void k_col_perm_rows(int nh, int npw, int rows, const int* __restrict__ gp, const cpx<T>* __restrict__ C,
+                                cpx<T>* __restrict__ out) {
+  const size_t n = (size_t)nh * rows;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const size_t v = i / nh;
+    out[i] = C[v * npw + gp[i - v * nh]];
+  }
+}
+template <typename T>
+__global__ void k_col_perm_kin(int nh, const int* __restrict__ gp, const T* __restrict__ kin, T* __restrict__ out) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nh; i += gridDim.x * blockDim.x) out[i] = kin[gp[i]];
+}
+}  // namespace col
+
+// vloc_s / kin (fixed per cell) and C (per occupied block) in the solver's
+// orders; a null input leaves that part alone.
+template <typename T>
+cudaError_t launch_col_permute(cudaStream_t s, const ColPlan& p, int N, int npw, const T* vloc_s, const cpx<T>* C,
+                               int nproj, const T* kin, ColPrec<T>& out) {
+  if (vloc_s) {
+    ++g_launches;
+    col::k_col_perm_v<T><<<std::min((N * N * N + 255) / 256, 152 * 8), 256, 0, s>>>(N, p.N1, p.N2, vloc_s, out.Vp);
+  }
+  if (kin) {
+    ++g_launches;
+    col::k_col_perm_kin<T><<<(p.nh + 255) / 256, 256, 0, s>>>(p.nh, p.gp, kin, out.kin);
+  }
+  if (C && nproj > 0) {
+    const size_t n = (size_t)p.nh * nproj;
+    ++g_launches;
+    col::k_col_perm_rows<T><<<(int)std::min<size_t>((n + 255) / 256, 152 * 16), 256, 0, s>>>(p.nh, npw, nproj, p.gp, C,
+                                                                                              out.Ch);
+  }
+  return cudaGetLastError();
+}
+
+#define GW_COL_INST(T)                                                                                     \
+  template bool col_shape<T>(const ColPlan&, int, int, int, int, int, ColShape*);                               \
+  template cudaError_t launch_col_solve<T>(cudaStream_t, int, const ColArgs<T>&);                          \
+  template cudaError_t launch_col_permute<T>(cudaStream_t, const ColPlan&, int, int, const T*, const cpx<T>*, int, \
+                                             const T*, ColPrec<T>&);
+
+}  // namespace gw

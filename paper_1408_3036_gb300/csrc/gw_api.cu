@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "gw.h"
+#include "col.cuh"
 #include "gw_common.cuh"
 #include "linalg.cuh"
 #include "tune.h"
@@ -44,9 +45,13 @@ struct gw_ctx {
   size_t work_cols = 0;
   double tol = 1e-13, tol_mixed = 1e-10, tol_inner = 1e-5;   // backward errors (FP64 / mixed), inner
   double anorm = 1.0;           // bound on |H - E| used by the backward error
-  int cg_kernel = GW_CG_PERSISTENT;   // kernel of the CG passes (gw_set_cg_kernel)
+  int cg_kernel = -1;                 // kernel of the CG passes (gw_set_cg_kernel; -1: chosen by size)
+  ColPlan col;                        // column solver (col_kernel.cuh): tables, and the data in its orders
+  ColPrec<double> col64;
+  ColPrec<float> col32;
   int maxplane = 0;                   // most sphere entries in one plane i0
-  bool use_graphs = true;             // SQMR iterations replayed from a captured CUDA graph
+  int use_graphs = -1;                // SQMR: 1 iterations replayed from a captured CUDA graph, 0 launched one
+                                      // by one, -1 the column solver where it fits, else replayed
   int imag_route = GW_IMAG_SQMR;      // solver of purely imaginary frequencies (gw_set_imaginary_route)
   double recycle_w0 = 0.0;            // > 0: recycled bases augmented with x(i w0)
   bool use_tc = false;                // tensor-core projector coefficients where they apply (opt-in)
@@ -63,7 +68,7 @@ struct gw_ctx {
   struct PcgPending {           // that launch, until the caller's next synchronisation (pcg_finish)
     bool on = false;
     int ncol = 0, used = 0, tune_tpb = 0;
-    bool fp64 = false;
+    bool fp64 = false, qmr = false;
     std::string tune_key;
   } pcg_pend;
   int pcg_cluster = 0;          // cluster size of the last persistent launch (0: grid-wide kernel)
@@ -242,7 +247,7 @@ enum ProfClass { PC_ZSCAT = 0, PC_YINV = 1, PC_XH = 2, PC_YFWD = 3, PC_ZGATH = 4
 // (counts: tasks run, and tasks skipped / waits)
 
 int prof_begin(gw_ctx* ctx, int cls) {
-  if (!(ctx->prof_mask & (1u << cls))) return -1;
+  if (cls >= PC_N || !(ctx->prof_mask & (1u << cls))) return -1;
   if (ctx->ev_next + 2 > ctx->ev_pool.size()) {
     for (int i = 0; i < 256; ++i) {
       cudaEvent_t e;
@@ -272,6 +277,9 @@ void prof_end(gw_ctx* ctx, int cls, int a) {
 template <typename T> Prec<T>& prec_of(gw_ctx* ctx);
 template <> Prec<double>& prec_of<double>(gw_ctx* ctx) { return ctx->P64; }
 template <> Prec<float>& prec_of<float>(gw_ctx* ctx) { return ctx->P32; }
+template <typename T> ColPrec<T>& col_of(gw_ctx* ctx);
+template <> ColPrec<double>& col_of<double>(gw_ctx* ctx) { return ctx->col64; }
+template <> ColPrec<float>& col_of<float>(gw_ctx* ctx) { return ctx->col32; }
 template <typename T> const char* tname();
 template <> const char* tname<double>() { return "64"; }
 template <> const char* tname<float>() { return "32"; }
@@ -480,6 +488,74 @@ gw_status cg_solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, 
   return GW_OK;
 }
 
+// Iteration counts, flags and the error word (if any) of a one-launch pass
+// come back into pinned memory and are read at the caller's next
+// synchronisation (pcg_finish): no stream synchronisation of its own per pass.
+gw_status pcg_read_back(gw_ctx* ctx, int ncol, const int* iters, const int* flags, const unsigned* ctl) {
+  if (ctx->pcg_pin_n < (size_t)(2 * ncol + 1)) {
+    if (ctx->pcg_pin) CK(cudaFreeHost(ctx->pcg_pin));
+    ctx->pcg_pin = nullptr;
+    ctx->pcg_pin_n = 0;
+    CK(cudaMallocHost(&ctx->pcg_pin, (size_t)(2 * ncol + 1) * sizeof(int)));
+    ctx->pcg_pin_n = (size_t)(2 * ncol + 1);
+  }
+  CK(cudaMemcpyAsync(ctx->pcg_pin, iters, ncol * sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+  CK(cudaMemcpyAsync(ctx->pcg_pin + ncol, flags, ncol * sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+  ctx->pcg_pin[2 * ncol] = 0;
+  if (ctl) CK(cudaMemcpyAsync(ctx->pcg_pin + 2 * ncol, ctl + 2, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->st));
+  ctx->pcg_pend.on = true;
+  ctx->pcg_pend.ncol = ncol;
+  return GW_OK;
+}
+
+// One inner pass by the column solver (col_kernel.cuh): x64 += the solution.
+// *ran = false (nothing done) when the cell's transform length has no radices
+// there or no cluster holds a unit.
+template <typename T>
+gw_status col_solve(gw_ctx* ctx, int kind, int ncol, const double2* b64, const double2* E, const int* outer_active,
+                    double2* x64, double tol, const double* rr_abs, const double* tk, bool* ran) {
+  *ran = false;
+  const ColPlan& p = ctx->col;
+  if (!p.ok) return GW_OK;
+  const std::string t = tname<T>();
+  ColArgs<T> a;
+  a.nunit = kind == COL_QMR ? ncol : (ncol + 1) / 2;
+  if (!col_shape<T>(p, kind, ctx->N, nproj(ctx), a.nunit, ctx->cta_div, &a.sh)) return GW_OK;
+  auto& P = prec_of<T>(ctx);
+  auto& c = col_of<T>(ctx);
+  a.N = ctx->N; a.N1 = p.N1; a.N2 = p.N2; a.P = p.P; a.nm = p.nm; a.npair = p.npair; a.nh = p.nh;
+  a.npw = ctx->npw; a.nproj = nproj(ctx); a.ncol = ncol; a.maxit = ctx->max_iter;
+  a.ldz = 2 * p.maxpair[a.sh.lq];
+  a.nhl = p.maxh[a.sh.lq];
+  const int nzl = (a.N + (1 << a.sh.lq) - 1) >> a.sh.lq;
+  a.dN.set(a.N); a.dP.set(a.P); a.dN1.set(a.N1); a.dN2.set(a.N2); a.dnz.set(nzl);
+  a.tw = P.tw; a.Vp = c.Vp; a.Ch = c.Ch; a.kin = c.kin;
+  a.split = p.split; a.hstart = p.hstart; a.gp = p.gp; a.gm = p.gm; a.hpos = p.hpos; a.disc = p.disc; a.zmax = p.zmax;
+  a.b64 = b64; a.x64 = x64; a.outer_active = outer_active; a.E = E; a.rr_abs = rr_abs; a.tk = tk; a.order = nullptr;
+  a.tol2 = tol * tol;
+  a.vecs = nullptr;
+  if (a.sh.vec_elems) TRY(getbuf(ctx, "col_vecs" + t, a.sh.vec_elems * (size_t)a.nunit, &a.vecs));
+  TRY(getbuf(ctx, "pcg_iters", ncol, &a.iters));
+  TRY(getbuf(ctx, "pcg_flags", ncol, &a.flags));
+  const int pa = prof_begin(ctx, kind == COL_CG_PAIR ? PC_PCG : PC_N);
+  CK(launch_col_solve<T>(ctx->st, kind, a));
+  prof_end(ctx, PC_PCG, pa);
+  TRY(pcg_read_back(ctx, ncol, a.iters, a.flags, nullptr));
+  ctx->pcg_pend.used = a.nunit << a.sh.lq;
+  ctx->pcg_pend.fp64 = std::is_same<T, double>::value;
+  ctx->pcg_pend.qmr = kind != COL_CG_PAIR;
+  ctx->pcg_pend.tune_key.clear();
+  ctx->pcg_pend.tune_tpb = 0;
+  if (kind == COL_CG_PAIR) {
+    ctx->pcg_cluster = 1 << a.sh.lq;
+    ctx->pcg_tpb = 512;
+  } else {
+    ctx->graph_replays = 0;
+  }
+  *ran = true;
+  return GW_OK;
+}
+
 // ---------------------------------------------------------------------------
 // the same CG pass as cg_solve in one cooperative launch (kernels_cg.cu)
 // ---------------------------------------------------------------------------
@@ -497,99 +573,68 @@ gw_status cg_solve_persistent(gw_ctx* ctx, int ncol, const double2* b64, const d
   TRY(getbuf(ctx, "pcg_flags", ncol, &flags));
   int used = 0;
   const int pa = prof_begin(ctx, PC_PCG);
-  cudaError_t le = cudaErrorNotSupported;
   unsigned* ctl = nullptr;
   std::string tune_key;
   int tune_tpb = 0;
-  if (ctx->cg_kernel == GW_CG_CLUSTER) {
-    // opt-in: one thread-block cluster per column when the column's planes
-    // fit in the cluster's shared memory
-    cpx<T>*r, *p, *Ap;
-    TRY(getbuf(ctx, "cg_r" + t, (size_t)ncol * npw, &r));
-    TRY(getbuf(ctx, "cg_p" + t, (size_t)ncol * npw, &p));
-    TRY(getbuf(ctx, "cg_Ap" + t, (size_t)ncol * npw, &Ap));
-    int q = 0;
-    le = launch_cg_cluster<T>(ctx->st, ctx->geo, ctx->plan, prec_of<T>(ctx), nproj(ctx), npw, ncol, b64, outer_active,
-                              E, rr_abs, tk, tol * tol, ctx->max_iter, x, r, p, Ap, iters, flags, rr_out, &q, nullptr);
-    used = ncol * q;
-    ctx->pcg_cluster = q;
+  ctx->pcg_cluster = 0;
+  // real-in-real-space columns in packed pairs
+  const PcgSizes z = pcg_sizes(nproj(ctx), npw, ncol, sym ? 2 : 1, ctx->geo.nplanes, ctx->N,
+                               (int)sizeof(cpx<T>));
+  cpx<T>*r, *p, *sv, *Y, *grid;
+  unsigned char* rec;
+  double* apart;
+  PcgCol* cst;
+  TRY(getbuf(ctx, "cg_r" + t, (size_t)ncol * npw, &r));
+  TRY(getbuf(ctx, "cg_p" + t, (size_t)ncol * npw, &p));
+  TRY(getbuf(ctx, "cg_Ap" + t, (size_t)ncol * npw, &sv));
+  TRY(getbuf(ctx, "pcg_Y" + t, z.Y, &Y));
+  TRY(getbuf(ctx, "g_cg" + t, z.grid, &grid));
+  TRY(getbuf(ctx, "pcg_rec", z.rec_total, &rec));
+  TRY(getbuf(ctx, "pcg_apart", z.apart, &apart));
+  TRY(getbuf(ctx, "pcg_cst", z.cst, &cst));
+  TRY(getbuf(ctx, "pcg_ctl", z.ctl, &ctl));
+  T* cin;
+  TRY(getbuf(ctx, "pcg_cin" + t, (size_t)4 * ncol, &cin));
+  CK(cudaMemsetAsync(ctl, 0, z.ctl * sizeof(unsigned), ctx->st));
+  unsigned long long* ptask = nullptr;
+  if (ctx->prof_mask & (1u << PC_TASKS)) {
+    if (!ctx->ptask) {
+      TRY(getbuf(ctx, "pcg_ptask", 36, &ctx->ptask));
+      CK(cudaMemsetAsync(ctx->ptask, 0, 36 * sizeof(unsigned long long), ctx->st));
+    }
+    ptask = ctx->ptask;
   }
-  if (le == cudaErrorNotSupported) {
+  // CTA width: 256 (two per SM) or 512 (one per SM), tuned per shape
+  char key[160];
+  std::snprintf(key, sizeof(key), "pcg1_tpb:%s:N%d:npw%d:nproj%d:ncol%d:W%d:div%d", tname<T>(), ctx->N, npw,
+                nproj(ctx), ncol, z.W, ctx->cta_div);
+  const int tpb = tune_pick(key, {256, 512}, ctx->tune && ctx->cta_div == 1);
+  if (!ctx->tune_ev[0]) {
+    CK(cudaEventCreate(&ctx->tune_ev[0]));
+    CK(cudaEventCreate(&ctx->tune_ev[1]));
+  }
+  const bool timing = ctx->tune && ctx->cta_div == 1 && !tune_known(key);
+  if (timing) CK(cudaEventRecord(ctx->tune_ev[0], ctx->st));
+  const cudaError_t le = launch_cg_persistent<T>(
+      ctx->st, ctx->geo, ctx->plan, prec_of<T>(ctx), nproj(ctx), npw, ncol, z, ctx->maxplane, b64, outer_active, E,
+      rr_abs, tk, tol * tol, ctx->max_iter, x, r, p, sv, Y, grid, rec, apart, cst, ctl, cin, iters, flags, rr_out,
+      &used, ctx->cta_div, ctx->wait_limit, ptask, tpb);
+  if (timing && le == cudaSuccess) CK(cudaEventRecord(ctx->tune_ev[1], ctx->st));
+  ctx->pcg_tpb = tpb;
+  tune_key = key;
+  tune_tpb = timing ? tpb : 0;
+  if (le == cudaErrorNotSupported) {      // shared memory beyond one SM: the multi-launch CG
     cudaGetLastError();
-    ctx->pcg_cluster = 0;
-    // the grid-wide task-queue kernel: real-in-real-space columns in packed pairs
-    const PcgSizes z = pcg_sizes(nproj(ctx), npw, ncol, sym ? 2 : 1, ctx->geo.nplanes, ctx->N,
-                                 (int)sizeof(cpx<T>));
-    cpx<T>*r, *p, *sv, *Y, *grid;
-    unsigned char* rec;
-    double* apart;
-    PcgCol* cst;
-    TRY(getbuf(ctx, "cg_r" + t, (size_t)ncol * npw, &r));
-    TRY(getbuf(ctx, "cg_p" + t, (size_t)ncol * npw, &p));
-    TRY(getbuf(ctx, "cg_Ap" + t, (size_t)ncol * npw, &sv));
-    TRY(getbuf(ctx, "pcg_Y" + t, z.Y, &Y));
-    TRY(getbuf(ctx, "g_cg" + t, z.grid, &grid));
-    TRY(getbuf(ctx, "pcg_rec", z.rec_total, &rec));
-    TRY(getbuf(ctx, "pcg_apart", z.apart, &apart));
-    TRY(getbuf(ctx, "pcg_cst", z.cst, &cst));
-    TRY(getbuf(ctx, "pcg_ctl", z.ctl, &ctl));
-    T* cin;
-    TRY(getbuf(ctx, "pcg_cin" + t, (size_t)4 * ncol, &cin));
-    CK(cudaMemsetAsync(ctl, 0, z.ctl * sizeof(unsigned), ctx->st));
-    unsigned long long* ptask = nullptr;
-    if (ctx->prof_mask & (1u << PC_TASKS)) {
-      if (!ctx->ptask) {
-        TRY(getbuf(ctx, "pcg_ptask", 36, &ctx->ptask));
-        CK(cudaMemsetAsync(ctx->ptask, 0, 36 * sizeof(unsigned long long), ctx->st));
-      }
-      ptask = ctx->ptask;
-    }
-    // CTA width: 256 (two per SM) or 512 (one per SM), tuned per shape
-    char key[160];
-    std::snprintf(key, sizeof(key), "pcg1_tpb:%s:N%d:npw%d:nproj%d:ncol%d:W%d:div%d", tname<T>(), ctx->N, npw,
-                  nproj(ctx), ncol, z.W, ctx->cta_div);
-    const int tpb = tune_pick(key, {256, 512}, ctx->tune && ctx->cta_div == 1);
-    if (!ctx->tune_ev[0]) {
-      CK(cudaEventCreate(&ctx->tune_ev[0]));
-      CK(cudaEventCreate(&ctx->tune_ev[1]));
-    }
-    const bool timing = ctx->tune && ctx->cta_div == 1 && !tune_known(key);
-    if (timing) CK(cudaEventRecord(ctx->tune_ev[0], ctx->st));
-    le = launch_cg_persistent<T>(ctx->st, ctx->geo, ctx->plan, prec_of<T>(ctx), nproj(ctx), npw, ncol, z,
-                                 ctx->maxplane, b64, outer_active, E, rr_abs, tk, tol * tol, ctx->max_iter, x, r, p,
-                                 sv, Y, grid, rec, apart, cst, ctl, cin, iters, flags, rr_out, &used, ctx->cta_div,
-                                 ctx->wait_limit, ptask, tpb);
-    if (timing && le == cudaSuccess) CK(cudaEventRecord(ctx->tune_ev[1], ctx->st));
-    ctx->pcg_tpb = tpb;
-    tune_key = key;
-    tune_tpb = timing ? tpb : 0;
-    if (le == cudaErrorNotSupported) {      // shared memory beyond one SM: the multi-launch CG
-      cudaGetLastError();
-      prof_end(ctx, PC_PCG, pa);
-      *ran = false;
-      return GW_OK;
-    }
+    prof_end(ctx, PC_PCG, pa);
+    *ran = false;
+    return GW_OK;
   }
   CK(le);
   prof_end(ctx, PC_PCG, pa);
-  // Iteration counts, flags and the error word come back into pinned memory
-  // and are read at the caller's next synchronisation (pcg_finish): no stream
-  // synchronisation of its own per pass.
-  if (ctx->pcg_pin_n < (size_t)(2 * ncol + 1)) {
-    if (ctx->pcg_pin) CK(cudaFreeHost(ctx->pcg_pin));
-    ctx->pcg_pin = nullptr;
-    ctx->pcg_pin_n = 0;
-    CK(cudaMallocHost(&ctx->pcg_pin, (size_t)(2 * ncol + 1) * sizeof(int)));
-    ctx->pcg_pin_n = (size_t)(2 * ncol + 1);
-  }
-  CK(cudaMemcpyAsync(ctx->pcg_pin, iters, ncol * sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-  CK(cudaMemcpyAsync(ctx->pcg_pin + ncol, flags, ncol * sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-  ctx->pcg_pin[2 * ncol] = 0;
-  if (ctl) CK(cudaMemcpyAsync(ctx->pcg_pin + 2 * ncol, ctl + 2, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->st));
-  ctx->pcg_pend.on = true;
-  ctx->pcg_pend.ncol = ncol;
+  TRY(pcg_read_back(ctx, ncol, iters, flags, ctl));
   ctx->pcg_pend.used = used;
   ctx->pcg_pend.fp64 = std::is_same<T, double>::value;
+  ctx->pcg_pend.qmr = false;
   ctx->pcg_pend.tune_key = tune_key;
   ctx->pcg_pend.tune_tpb = tune_tpb;
   (void)it_sum;
@@ -613,10 +658,12 @@ gw_status pcg_finish(gw_ctx* ctx, long long* it_sum, int* it_max) {
     *it_max = std::max(*it_max, its[c]);
     imax = std::max(imax, its[c]);
     if (fl[c] == 2 && ctx->pcg_pend.fp64)
-      return fail(ctx, GW_E_BREAKDOWN, "CG breakdown: (H - E) is not positive definite on P_c");
+      return fail(ctx, GW_E_BREAKDOWN, ctx->pcg_pend.qmr ? "SQMR serious breakdown: [q, A q] = 0"
+                                                         : "CG breakdown: (H - E) is not positive definite on P_c");
   }
-  ctx->pcg_iters += imax;       // iterations of the whole launch (bounded by the slowest column)
   ctx->pcg_launch_blocks = ctx->pcg_pend.used;
+  if (ctx->pcg_pend.qmr) return GW_OK;
+  ctx->pcg_iters += imax;       // iterations of the whole launch (bounded by the slowest column)
   if (ctx->pcg_pend.tune_tpb && imax > 0) {
     float ms = 0.f;
     if (cudaEventElapsedTime(&ms, ctx->tune_ev[0], ctx->tune_ev[1]) == cudaSuccess)
@@ -714,7 +761,7 @@ gw_status qmr_solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E,
   cudaGraphExec_t& exec = guard.e;
   unsigned long long per_iter = 0;
   ctx->graph_replays = 0;
-  if (ctx->use_graphs) {
+  if (ctx->use_graphs != 0) {
     const unsigned long long l0 = g_launches;
     if (cudaStreamBeginCapture(ctx->st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
       iteration();
@@ -767,27 +814,42 @@ gw_status qmr_solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E,
 // states).  Each inner solve stops at tol_inner relative to its own right-hand
 // side, or at a tenth of the final target, whichever is larger.
 // ---------------------------------------------------------------------------
-// One inner solve in precision U: simplified QMR, or CG (one persistent launch
-// when the columns fit, else the multi-launch form).
+// One inner solve in precision U, its solution added to x64: the column solver
+// where it takes the unit (real columns in pairs; complex columns with
+// simplified QMR), else the persistent or the multi-launch kernels through the
+// buffer d.
 template <typename U>
 gw_status inner_solve(gw_ctx* ctx, bool qmr, int ncol, const double2* r64, const double2* E, const int* oact,
-                      cpx<U>* d, double tol_in, const double* rra, const double* tk, bool sym, long long* it_sum,
-                      int* it_max, const double* w2 = nullptr) {
-  if (w2) return cg_solve<U>(ctx, ncol, r64, E, oact, d, tol_in, rra, tk, it_sum, it_max, w2);
-  if (qmr) return qmr_solve<U>(ctx, ncol, r64, E, oact, d, tol_in, rra, tk, it_sum, it_max);
-  if (ncol <= kPersistentMaxCols && ctx->cg_kernel != GW_CG_MULTI_LAUNCH) {
-    bool ran = false;
-    TRY(cg_solve_persistent<U>(ctx, ncol, r64, E, oact, d, tol_in, rra, tk, sym, it_sum, it_max, &ran));
+                      cpx<U>* d, double2* x64, double tol_in, const double* rra, const double* tk, bool sym,
+                      bool real_shift, long long* it_sum, int* it_max, const double* w2 = nullptr) {
+  const bool col = !w2 && (qmr ? ctx->use_graphs < 0 && !ctx->use_tc
+                               : sym && (ctx->cg_kernel < 0 || ctx->cg_kernel == GW_CG_CLUSTER));
+  bool ran = false;
+  if (col) {
+    const int kind = !qmr ? COL_CG_PAIR : sym && real_shift ? COL_QMR_PAIR : COL_QMR;
+    TRY(col_solve<U>(ctx, kind, ncol, r64, E, oact, x64, tol_in, rra, tk, &ran));
     if (ran) return GW_OK;
   }
-  return cg_solve<U>(ctx, ncol, r64, E, oact, d, tol_in, rra, tk, it_sum, it_max);
+  if (w2) {
+    TRY(cg_solve<U>(ctx, ncol, r64, E, oact, d, tol_in, rra, tk, it_sum, it_max, w2));
+  } else if (qmr) {
+    TRY(qmr_solve<U>(ctx, ncol, r64, E, oact, d, tol_in, rra, tk, it_sum, it_max));
+  } else {
+    if (ncol <= kPersistentMaxCols && ctx->cg_kernel != GW_CG_MULTI_LAUNCH)
+      TRY(cg_solve_persistent<U>(ctx, ncol, r64, E, oact, d, tol_in, rra, tk, sym, it_sum, it_max, &ran));
+    if (!ran) TRY(cg_solve<U>(ctx, ncol, r64, E, oact, d, tol_in, rra, tk, it_sum, it_max));
+  }
+  if (sym) launch_add_conv_sym<U>(ctx->st, ctx->npw, ncol, d, x64, oact, ctx->geo.sph_neg);
+  else launch_add_conv<U>(ctx->st, ctx->npw, ncol, d, x64, oact);
+  return GW_OK;
 }
 
 // w2 (optional, device [ncol]): solve the squared system of Eq. P2+,
 // (P_c (H - E) P_c)^2 x + w2 x = b, by CG (w2max: the largest w2, for |A|).
 template <typename T>
 gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, double2* x64, bool qmr = false,
-                const double* tk = nullptr, const double* w2 = nullptr, double w2max = 0.0, int sym_hint = -1) {
+                const double* tk = nullptr, const double* w2 = nullptr, double w2max = 0.0, int sym_hint = -1,
+                bool real_shift = false) {
   const int npw = ctx->npw;
   const bool mixed = !std::is_same<T, double>::value;
   ctx->pcg_pend.on = false;
@@ -822,7 +884,7 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
   // when it knows (sym_hint 0 or 1), else decided from the data, to the FP64
   // rounding of the right-hand sides.
   bool sym = false;
-  if (!qmr && sym_hint >= 0) {
+  if (sym_hint >= 0) {
     sym = sym_hint != 0;             // known to the caller (real fields and states)
   } else if (!qmr) {
     double* symv;
@@ -864,15 +926,11 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
     }
     if (esc) {
       if (!d64) TRY(getbuf(ctx, "sv_d64", (size_t)ncol * npw, &d64));
-      TRY(inner_solve<double>(ctx, qmr, ncol, r64, E, oact, reinterpret_cast<cpx<double>*>(d64),
-                              std::max(1e2 * ctx->tol, 1e-11), rra, tk, sym, &it_sum, &it_max, w2));
-      if (sym) launch_add_conv_sym<double>(ctx->st, npw, ncol, reinterpret_cast<cpx<double>*>(d64), x64, oact,
-                                           ctx->geo.sph_neg);
-      else launch_add_conv<double>(ctx->st, npw, ncol, reinterpret_cast<cpx<double>*>(d64), x64, oact);
+      TRY(inner_solve<double>(ctx, qmr, ncol, r64, E, oact, reinterpret_cast<cpx<double>*>(d64), x64,
+                              std::max(1e2 * ctx->tol, 1e-11), rra, tk, sym, real_shift, &it_sum, &it_max, w2));
     } else {
-      TRY(inner_solve<T>(ctx, qmr, ncol, r64, E, oact, d, tol_in, rra, tk, sym, &it_sum, &it_max, w2));
-      if (sym) launch_add_conv_sym<T>(ctx->st, npw, ncol, d, x64, oact, ctx->geo.sph_neg);
-      else launch_add_conv<T>(ctx->st, npw, ncol, d, x64, oact);
+      TRY(inner_solve<T>(ctx, qmr, ncol, r64, E, oact, d, x64, tol_in, rra, tk, sym, real_shift, &it_sum, &it_max,
+                         w2));
     }
     if (ctx->ndef > 0)                // the deflated components, exactly
       launch_proj_update<double>(ctx->st, ctx->P64.C + (size_t)ctx->nocc * npw, ctx->ndef, npw, x64, ncol, oact,
@@ -1192,6 +1250,25 @@ gw_status chi0_core(gw_ctx* ctx, const void* y, bool y_cplx, int nb, const std::
     }
     if (pass == 0) nstd = (int)src.size();
   }
+  {
+    // highest shift first: those columns take the most iterations, so they
+    // start first, and columns solved as a pair are alike
+    std::vector<int> ord(nstd), at(nstd), src0(src);
+    std::vector<double2> E0(E);
+    std::vector<double> tk0(tk);
+    for (int j = 0; j < nstd; ++j) ord[j] = j;
+    std::stable_sort(ord.begin(), ord.end(), [&](int p, int q) { return E0[p].x > E0[q].x; });
+    for (int j = 0; j < nstd; ++j) {
+      src[j] = src0[ord[j]];
+      E[j] = E0[ord[j]];
+      tk[j] = tk0[ord[j]];
+      at[ord[j]] = j;
+    }
+    for (int k = 0; k < nsol; ++k) {
+      if (s0[k] >= 0 && s0[k] < nstd) s0[k] = at[s0[k]];
+      if (s1[k] >= 0 && s1[k] < nstd) s1[k] = at[s1[k]];
+    }
+  }
   const int ncol = (int)src.size(), nsq = ncol - nstd;
   int *dsrc, *ds0, *ds1;
   double2* dE;
@@ -1206,8 +1283,13 @@ gw_status chi0_core(gw_ctx* ctx, const void* y, bool y_cplx, int nb, const std::
   TRY(getbuf(ctx, "xcol", (size_t)ncol * npw, &xcol));
   launch_gather_rows<double, double>(ctx->st, npw, ncol, rhs64, dsrc, bcol);
   gw_status sv = GW_OK;
-  // real fields at omega = 0: right-hand sides real in real space by construction
-  if (nstd > 0) SOFT(sv, (solve<S>(ctx, nstd, bcol, dE, xcol, qmr, dtk, nullptr, 0.0, (!qmr && !y_cplx) ? 1 : -1)));
+  // real fields: right-hand sides real in real space by construction, and at
+  // real frequencies solutions too
+  bool real_w = true;
+  for (int j = 0; j < nstd; ++j) real_w = real_w && E[j].y == 0.0;
+  const bool real_cols = !y_cplx && real_w;
+  if (nstd > 0)
+    SOFT(sv, (solve<S>(ctx, nstd, bcol, dE, xcol, qmr, dtk, nullptr, 0.0, real_cols ? 1 : -1, real_cols)));
   if (nsq > 0) {
     // Eq. P2+: ((H - e_v)^2 + w^2) y = 2 (H - e_v) b gives y = x^- + x^+ at
     // omega = i w; solved for x = y / 2 from the right-hand side P_c (H - e_v) b
@@ -1799,6 +1881,90 @@ gw_status grad_from_basis(gw_ctx* ctx, const double* phi, const double* Q, const
 }
 
 // host sphere, pencils, planes
+// Tables of the column solver: the disc pencils as mirror pairs in the order
+// (n1, then n0 as the planes are counted), the half entries in that order.
+gw_status build_col_plan(gw_ctx* ctx, const std::vector<int4>& pencils, const std::vector<int>& i2s,
+                         const std::vector<int>& pen, const std::vector<int>& negs,
+                         const std::vector<uint8_t>& disc, size_t nplanes) {
+  ColPlan& p = ctx->col;
+  const int N = ctx->N;
+  p.ok = false;
+  if (!col_radices(N, &p.N1, &p.N2)) return GW_OK;
+  p.P = (int)nplanes;
+  p.nm = p.P / 2;
+  auto plane = [&](int i0) { return i0 <= p.nm ? i0 : i0 - (N - p.P); };
+  for (const int4& q : pencils) {           // the planes are |n0| <= nm
+    const int n0 = 2 * q.x < N ? q.x : q.x - N;
+    if (std::abs(n0) > p.nm) return GW_OK;
+  }
+  std::vector<int> where(N * N, -1);
+  for (size_t k = 0; k < pencils.size(); ++k) where[pencils[k].x * N + pencils[k].y] = (int)k;
+  // first pencils of the pairs: (0, 0), then n1 = 0 with n0 > 0, then n1 > 0
+  std::vector<int> rep;
+  rep.push_back(where[0]);
+  for (int i1 = 0; 2 * i1 < N; ++i1)
+    for (int q = 0; q < p.P; ++q) {
+      const int i0 = q <= p.nm ? q : q + (N - p.P);
+      if (i1 == 0 && (q == 0 || q > p.nm)) continue;
+      if (disc[i0 * N + i1]) rep.push_back(where[i0 * N + i1]);
+    }
+  if (2 * rep.size() - 1 != pencils.size()) return GW_OK;
+  p.npair = (int)rep.size();
+  std::vector<int> hstart(1, 0), gp, gm;
+  std::vector<unsigned> hpos;
+  std::vector<unsigned short> dsc((size_t)N * p.P, 0xffff);
+  std::vector<unsigned char> zmax(p.npair);
+  for (int j = 0; j < p.npair; ++j) {
+    const int4 q = pencils[rep[j]];
+    const int m0 = (N - q.x) % N, m1 = (N - q.y) % N;
+    dsc[(size_t)q.y * p.P + plane(q.x)] = (unsigned short)(2 * j);
+    if (j > 0) dsc[(size_t)m1 * p.P + plane(m0)] = (unsigned short)(2 * j + 1);
+    int zm = 0;
+    for (int s = q.z; s < q.z + q.w; ++s) {
+      const int z = i2s[s], n2 = 2 * z < N ? z : z - N;
+      zm = std::max(zm, std::abs(n2));
+      if (j == 0 && n2 < 0) continue;          // (0, 0): -G lies in the same pencil
+      gp.push_back(s);
+      gm.push_back(negs[s]);
+      hpos.push_back((unsigned)j << 8 | (unsigned)z);
+    }
+    if (2 * zm + 1 != q.w) return GW_OK;       // the pencil's entries are |n2| <= zm
+    zmax[j] = (unsigned char)zm;
+    hstart.push_back((int)gp.size());
+  }
+  p.nh = (int)gp.size();
+  if (2 * p.nh - 1 != ctx->npw || gp[0] != gm[0]) return GW_OK;
+  // equal shares of entries (solver vectors, projector) and pencils (transforms)
+  std::vector<int> split(kColNQ * (kColMaxQ + 1), p.npair);
+  auto cost = [&](int j) { return (long)hstart[j] + (long)j * N / 8; };
+  for (int lq = 0; lq < kColNQ; ++lq) {
+    const int Q = 1 << lq;
+    int* s = &split[lq * (kColMaxQ + 1)];
+    s[0] = 0;
+    p.maxpair[lq] = p.maxh[lq] = 0;
+    if (Q > p.npair) continue;
+    for (int r = 1; r < Q; ++r) {
+      int j = s[r - 1] + 1;
+      while (j < p.npair - (Q - r) && cost(j) * Q < cost(p.npair) * r) ++j;
+      s[r] = j;
+    }
+    s[Q] = p.npair;
+    for (int r = 0; r < Q; ++r) {
+      p.maxpair[lq] = std::max(p.maxpair[lq], s[r + 1] - s[r]);
+      p.maxh[lq] = std::max(p.maxh[lq], hstart[s[r + 1]] - hstart[s[r]]);
+    }
+  }
+  TRY(upload(ctx, "col_split", split, &p.split));
+  TRY(upload(ctx, "col_hstart", hstart, &p.hstart));
+  TRY(upload(ctx, "col_gp", gp, &p.gp));
+  TRY(upload(ctx, "col_gm", gm, &p.gm));
+  TRY(upload(ctx, "col_hpos", hpos, &p.hpos));
+  TRY(upload(ctx, "col_disc", dsc, &p.disc));
+  TRY(upload(ctx, "col_zmax", zmax, &p.zmax));
+  p.ok = true;
+  return GW_OK;
+}
+
 gw_status build_geometry(gw_ctx* ctx) {
   const int N = ctx->N;
   const double gg = 2.0 * M_PI / ctx->L;
@@ -1893,7 +2059,7 @@ gw_status build_geometry(gw_ctx* ctx) {
   TRY(upload(ctx, "geo_plane_pen", plane_pen, &g.plane_pen));
   TRY(upload(ctx, "geo_i1", i1s, &g.sph_i1));
   TRY(upload(ctx, "geo_neg", negs, &g.sph_neg));
-  return GW_OK;
+  return build_col_plan(ctx, pencils, i2s, pen, negs, disc, plane_sph.size() - 1);
 }
 
 template <typename T>
@@ -1913,6 +2079,12 @@ gw_status upload_prec(gw_ctx* ctx, const std::vector<double>& vloc, const std::v
   TRY(upload(ctx, "p_kin" + t, kin, &P.kin));
   TRY(upload(ctx, "p_v" + t, vs, &P.vloc_s));
   TRY(upload(ctx, "p_sqv" + t, sq, &P.sqv_s));
+  if (ctx->col.ok) {
+    auto& c = col_of<T>(ctx);
+    TRY(getbuf(ctx, "col_V" + t, (size_t)N3, &c.Vp));
+    TRY(getbuf(ctx, "col_kin" + t, (size_t)ctx->col.nh, &c.kin));
+    CK(launch_col_permute<T>(ctx->st, ctx->col, N, ctx->npw, P.vloc_s, nullptr, 0, P.kin, c));
+  }
   return GW_OK;
 }
 
@@ -2078,6 +2250,13 @@ gw_status upload_projector(gw_ctx* ctx, const std::vector<zc>& cdef) {
   }
   TRY(upload(ctx, "occ_C64", c64, &ctx->P64.C));
   TRY(upload(ctx, "occ_C32", c32, &ctx->P32.C));
+  if (ctx->col.ok) {
+    const int r = (int)(n / ctx->npw);
+    TRY(getbuf(ctx, "col_C64", (size_t)r * ctx->col.nh, &ctx->col64.Ch));
+    TRY(getbuf(ctx, "col_C32", (size_t)r * ctx->col.nh, &ctx->col32.Ch));
+    CK(launch_col_permute<double>(ctx->st, ctx->col, ctx->N, ctx->npw, nullptr, ctx->P64.C, r, nullptr, ctx->col64));
+    CK(launch_col_permute<float>(ctx->st, ctx->col, ctx->N, ctx->npw, nullptr, ctx->P32.C, r, nullptr, ctx->col32));
+  }
   // the rows split into TF32 hi / lo parts for the tensor-core projector
   // coefficients (up to 64 rows); without a tensor-map encoder the CUDA-core
   // dots remain

@@ -58,7 +58,6 @@
 #include "fft.cuh"
 #include "gw_common.cuh"
 #include "linalg.cuh"
-#include "pcg.cuh"
 
 namespace gw {
 

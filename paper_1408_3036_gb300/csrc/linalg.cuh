@@ -230,14 +230,6 @@ cudaError_t launch_cg_persistent(cudaStream_t s, const Geometry& g, const FftPla
                                  T* cin, int* iters, int* flags, double* rr_out, int* grid_used, int cta_div,
                                  unsigned long long spin_limit, unsigned long long* ptask = nullptr,
                                  int tpb = 256);
-// One thread-block cluster per column (kernels_cgc.cu); cudaErrorNotSupported
-// when the column's planes do not fit in the shared memory of a cluster.
-template <typename T>
-cudaError_t launch_cg_cluster(cudaStream_t s, const Geometry& g, const FftPlan& pl, const Prec<T>& P, int nocc,
-                              int npw, int ncol, const double2* b64, const int* outer_active, const double2* E,
-                              const double* rr_abs, const double* tk, double tol_in2, int maxit, cpx<T>* x,
-                              cpx<T>* r, cpx<T>* p, cpx<T>* Ap, int* iters, int* flags, double* rr_out,
-                              int* q_used, unsigned long long* ptime = nullptr);
 constexpr int kPersistentMaxCols = 256;
 constexpr int kPcgChunkMin = 64;   // smallest chunk (sphere entries) of the persistent CG's update phase
 // A CG pass whose |r|^2 has not dropped 4x for max(kCgStagWindow, 2 k_best)
