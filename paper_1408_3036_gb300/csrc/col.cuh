@@ -47,6 +47,7 @@ struct ColShape {
   int lq = 0, nsb = 1;           // log2 of the cluster size; slabs transformed together
   bool vec_smem = false;         // solver vectors in shared memory (else in vecs)
   bool c_smem = false;           // projector rows in shared memory
+  bool v_smem = false;           // the slabs' potential in shared memory
   size_t smem = 0;
   size_t vec_elems = 0;          // T entries of the global vectors of one unit (0 with vec_smem)
 };

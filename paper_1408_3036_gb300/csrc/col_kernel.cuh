@@ -35,12 +35,17 @@
 //
 // What bounds it: the latency of one unit's iteration (barriers of the
 // cluster, shared-memory passes of the transforms; FP64 the FP64 pipe).
+// FP32 at 48^3, 16 rows, Q = 16: 41k cycles an iteration, of which the slabs'
+// seven passes 19k, z passes 6k, projector 6k, three cluster barriers 4k;
+// FP64 390k, of which the transforms 280k (FP64 instructions issue once in 64
+// cycles and scheduler here, so sums are halved across the lanes instead of
+// repeated in them, and scalar steps share one division).
 // Measured on a GB300, one application, before (launches per step, or the
 // grid-wide task queue of kernels_cg.cu) and after: 48^3 grid, 12053 plane
-// waves, 16 CG columns, FP32 3.64 -> 2.32 ms, FP64 15.8 -> 12.5 ms; 45^3, 2007
+// waves, 16 CG columns, FP32 3.64 -> 2.21 ms, FP64 15.8 -> 11.3 ms; 45^3, 2007
 // plane waves, 22 complex columns 11.7 -> 4.1 ms; 32^3, 2109 plane waves, 69
-// rows, 1104 complex columns 398 -> 92 ms; 64^3, 38401 plane waves, 64 rows,
-// 256 complex columns 1082 -> 553 ms.
+// rows, 1104 complex columns 398 -> 79 ms; 64^3, 38401 plane waves, 64 rows,
+// 256 complex columns 1082 -> 492 ms.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -63,8 +68,12 @@ namespace cgr = cooperative_groups;
 constexpr int kTPB = 512;
 constexpr int kNW = kTPB / 32;
 constexpr size_t kSmemMax = 226 * 1024;
-constexpr int kNearWait = 32;        // SQMR iterations granted within a factor 2 of the target norm (see below)
-constexpr int kQmrWindow = 1000;     // SQMR stagnation window (as the multi-launch solver's)
+// SQMR stagnation: iterations without a halving of the quasi-residual norm.
+// FP32: the recurrence goes no further than about 1e-5 of the right-hand side,
+// now and then 1.5 to 3 times the target; a plateau below 1e-4 is that floor.
+constexpr int kQmrWindow = 1000;     // anywhere (as the multi-launch solver's)
+constexpr int kQmrWindowFloor = 64;  // FP32, once the norm has dropped 1e4 times
+constexpr int kNearWait = 32;        // iterations granted within a factor 2 of the target norm
 
 template <typename T> struct alignas(16) V4 { T x, y, z, w; };
 
@@ -104,6 +113,33 @@ __device__ __forceinline__ double shx_(double a, int o) { return __shfl_xor_sync
 __device__ __forceinline__ float2 shx_(float2 a, int o) {
   return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
 }
+__device__ __forceinline__ float shx_(float a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ double shi_(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
+__device__ __forceinline__ float2 shi_(float2 a, int l) {
+  return make_float2(__shfl_sync(0xffffffffu, a.x, l), __shfl_sync(0xffffffffu, a.y, l));
+}
+__device__ __forceinline__ float add_(float a, float b) { return a + b; }
+
+// Warp sums of M values per lane (M a power of 2, at most 32) by recursive
+// halving: M - 1 + log2(32 / M) additions instead of 5 M.  Lane l returns the
+// sum of value l / (32 / M), the same bits in all its lanes.
+template <int M, typename A> __device__ __forceinline__ A warp_sums(A* v) {
+  const int lane = threadIdx.x & 31;
+  int o = 16;
+#pragma unroll
+  for (int n = M / 2; n >= 1; n >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < n; ++k) {
+      const A keep = up ? v[n + k] : v[k], give = up ? v[k] : v[n + k];
+      v[k] = add_(keep, shx_(give, o));
+    }
+  }
+#pragma unroll
+  for (int q = 16 / M; q >= 1; q >>= 1) v[0] = add_(v[0], shx_(v[0], q));
+  return v[0];
+}
+__host__ __device__ constexpr int pow2_up(int n) { int p = 1; while (p < n) p *= 2; return p; }
 
 // --- R-point transforms in registers
 template <typename T, int S> __device__ __forceinline__ cpx<T> rot(cpx<T> a, T c, T s) {   // a (c + S i s)
@@ -196,24 +232,36 @@ template <class F> __device__ __forceinline__ void radix2(int r, F f) {
 
 // --- shared memory of one CTA (byte offsets)
 struct Lay {
-  size_t Z, R, T, X, C, K, kin, hpos, rt, own, zm, zs, tw, coefp, coef, sc, total;
+  size_t Z, R, T, X, C, V, K, kin, hpos, rt, own, zm, zs, tw, cp, coefp, coef, part, sc, total;
 };
 __host__ __device__ inline size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
-__host__ __device__ inline int splits(int nproj) { return nproj >= kNW ? 1 : (nproj > 0 ? kNW / nproj : 1); }
+// Projector rows a warp takes at a time (their products with one load of the
+// vectors), and the parts the entries are cut into so that all warps work.
+__host__ __device__ inline int row_group(int nproj, bool f32) {
+  if (nproj < 8) return nproj < 4 ? 1 : 2;
+  if (!f32 || nproj <= 4 * kNW) return 4;
+  return nproj <= 5 * kNW ? 5 : nproj <= 6 * kNW ? 6 : 4;
+}
+__host__ __device__ inline int splits(int nproj, int rg, int nhl) {
+  const int g = (nproj + rg - 1) / rg, s = g > 0 ? kNW / g : 1, m = (nhl + 31) / 32;
+  return s < 1 ? 1 : s > m ? m : s;
+}
 
 template <typename T>
 __host__ __device__ inline Lay layout(int kind, const ColShape& sh, int N, int P, int npair, int ldz, int nhl,
                                       int nproj) {
   const size_t sv = sizeof(cpx<T>), s4 = 4 * sizeof(T);
   const int Q = 1 << sh.lq, nzl = (N + Q - 1) / Q, nv = kind == COL_CG_PAIR ? 4 : 2;
-  const size_t tile = (size_t)sh.nsb * N * (N | 1) * sv, temp = (size_t)nhl * s4;
+  const int rg = row_group(nproj, sizeof(T) == 4);
+  const size_t tile = (size_t)sh.nsb * N * (N | 1) * sv, temp = (size_t)nhl * s4 * (kind == COL_CG_PAIR ? 2 : 1);
   Lay L;
   L.Z = 0;
   L.R = up16(L.Z + (size_t)N * ldz * sv);
-  L.T = up16(L.R + (size_t)nzl * (2 * npair) * sv);
+  L.T = up16(L.R + (Q > 1 ? (size_t)nzl * (2 * npair) * sv : 0));
   L.X = up16(L.T + (tile > temp ? tile : temp));
   L.C = up16(L.X + (sh.vec_smem ? 4 * (size_t)nhl * s4 : 0));
-  L.K = up16(L.C + (sh.c_smem ? (size_t)nproj * nhl * sv : 0));
+  L.V = up16(L.C + (sh.c_smem ? (size_t)nproj * nhl * sv : 0));
+  L.K = up16(L.V + (sh.v_smem ? (size_t)nzl * N * N * sizeof(T) : 0));
   L.kin = up16(L.K + (size_t)nhl * (kind == COL_QMR ? 1 : 2) * sizeof(T));
   L.hpos = up16(L.kin + (size_t)nhl * sizeof(T));
   L.rt = up16(L.hpos + (size_t)nhl * sizeof(unsigned));
@@ -221,21 +269,23 @@ __host__ __device__ inline Lay layout(int kind, const ColShape& sh, int N, int P
   L.zm = up16(L.own + (size_t)2 * npair);
   L.zs = up16(L.zm + (size_t)ldz);
   L.tw = up16(L.zs + (size_t)N);
-  L.coefp = up16(L.tw + (size_t)N * sv);
-  L.coef = up16(L.coefp + (size_t)Q * splits(nproj) * nproj * nv * sizeof(T));
-  L.sc = up16(L.coef + (size_t)nproj * nv * sizeof(T));
-  L.total = up16(L.sc + (size_t)3 * Q * kNW * 4 * sizeof(Acc<T>));
+  L.cp = up16(L.tw + (size_t)N * sv);
+  L.coefp = up16(L.cp + (size_t)splits(nproj, rg, nhl) * nproj * nv * sizeof(T));
+  L.coef = up16(L.coefp + (size_t)Q * nproj * nv * sizeof(T));
+  L.part = up16(L.coef + (size_t)nproj * nv * sizeof(T));
+  L.sc = up16(L.part + (size_t)kNW * 4 * sizeof(Acc<T>));
+  L.total = up16(L.sc + (size_t)3 * Q * 4 * sizeof(Acc<T>));
   return L;
 }
 
 // Per-column state of the recurrences (every CTA keeps its own equal copy).
 template <typename T> struct CgCol {
-  T gam, gprev, alpha, stop, rmin, rbest, al, bt;
+  T gam, gdiv, alpha, stop, rmin, rbest, al, bt;
   int it, itb, active, flag;
 };
 struct QmrCol {
   double2 rho, alpha, beta, qc;
-  double dc, theta, tau, stop, qbest;
+  double dc, theta2, tau2, stop, qbest, rr0;         // theta^2, tau^2
   int it, itb, near, active, flag, upd;
 };
 
@@ -266,12 +316,13 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     return;
   }
   const int N = a.N, N1 = a.N1, N2 = a.N2, P = a.P, LD = N | 1, ldz = a.ldz, ldr = 2 * a.npair;
-  const int nproj = a.nproj, nsplit = splits(nproj);
+  const int nproj = a.nproj, rgrp = row_group(nproj, sizeof(T) == 4), nsplit = splits(nproj, rgrp, a.nhl);
   const Lay L = layout<T>(KIND, a.sh, N, P, a.npair, ldz, a.nhl, nproj);
   V* Z = reinterpret_cast<V*>(sm + L.Z);          // [N][ldz] own pencils
   V* R = reinterpret_cast<V*>(sm + L.R);          // [nzl][ldr] own slabs, disc values
   V* Tt = reinterpret_cast<V*>(sm + L.T);         // [nsb][N][LD] slab tiles
-  W4* Tm = reinterpret_cast<W4*>(sm + L.T);       // [nhl] A u (shares the tiles' place)
+  W4* Tm = reinterpret_cast<W4*>(sm + L.T);       // [nhl] A u, CG then u (share the tiles' place)
+  T* Vs = reinterpret_cast<T*>(sm + L.V);         // [nzl][N][N] V / N_g of the own slabs (v_smem)
   T* Kt = reinterpret_cast<T*>(sm + L.K);
   T* kin = reinterpret_cast<T*>(sm + L.kin);
   unsigned* hpos = reinterpret_cast<unsigned*>(sm + L.hpos);
@@ -280,10 +331,11 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   signed char* zm = reinterpret_cast<signed char*>(sm + L.zm);
   unsigned char* zs = sm + L.zs;
   V* stw = reinterpret_cast<V*>(sm + L.tw);
-  T* coefp = reinterpret_cast<T*>(sm + L.coefp);  // [Q][nsplit][nproj][NV]
+  T* cp = reinterpret_cast<T*>(sm + L.cp);        // [nsplit][nproj][NV] this CTA's coefficients in parts
+  T* coefp = reinterpret_cast<T*>(sm + L.coefp);  // [Q][nproj][NV]
   T* coef = reinterpret_cast<T*>(sm + L.coef);    // [nproj][NV]
-  SA* sc = reinterpret_cast<SA*>(sm + L.sc);      // [3][Q][kNW][4]
-  const int nsc = Q * kNW * 4;
+  SA* part = reinterpret_cast<SA*>(sm + L.part);  // [kNW][4] scalar sums of the warps
+  SA* sc = reinterpret_cast<SA*>(sm + L.sc);      // [3][Q][4] of the CTAs
 
   auto at = [&](auto* p, int q) { return Q > 1 ? cl.map_shared_rank(p, q) : p; };
   auto csync = [&]() { if (Q > 1) cl.sync(); else __syncthreads(); };
@@ -337,6 +389,10 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       for (int e = lane; e < nh; e += 32) Cs[(size_t)v * a.nhl + e] = C[(size_t)v * ldc + e];
     C = Cs;
     ldc = (size_t)a.nhl;
+  }
+  if (a.sh.v_smem) {
+    const T* v = a.Vp + (size_t)z0 * N * N;
+    for (int k = tid; k < nsl * N * N; k += kTPB) Vs[k] = v[k];
   }
   for (int e = tid; e < nh; e += kTPB) {
     const int h = h0 + e;
@@ -397,7 +453,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   };
 
   // z-IFFT of the own pencils, sent to the slab owners
-  auto z_inverse = [&]() {
+  auto z_step1 = [&]() {
     radix1(N1, [&](auto RR) {
       constexpr int R1 = decltype(RR)::value;
       for (int t = tid; t < nrl * N2; t += kTPB) {
@@ -415,6 +471,9 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         for (int k = 0; k < R1; ++k) Z[(k * N2 + n2) * ldz + row] = v[k];
       }
     });
+  };
+  auto z_inverse_send = [&]() {
+    z_step1();
     __syncthreads();
     radix2(N2, [&](auto RR) {
       constexpr int R2 = decltype(RR)::value;
@@ -433,6 +492,25 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       }
     });
   };
+  // Q = 1: the same, left in the pencils (i2 at slot zs[i2])
+  auto z_inverse_local = [&]() {
+    z_step1();
+    __syncthreads();
+    radix2(N2, [&](auto RR) {
+      constexpr int R2 = decltype(RR)::value;
+      for (int t = tid; t < nrl * N1; t += kTPB) {
+        const int k1 = dnr.div(t), row = t - k1 * nrl;
+        V v[R2];
+#pragma unroll
+        for (int k = 0; k < R2; ++k) v[k] = Z[(k1 * R2 + k) * ldz + row];
+        dft<T, 1, R2>(v);
+#pragma unroll
+        for (int k = 0; k < R2; ++k) Z[(k1 * R2 + k) * ldz + row] = v[k];
+      }
+    });
+  };
+
+  auto z_inverse = [&]() { if (Q > 1) z_inverse_send(); else z_inverse_local(); };
 
   // the slabs: returns true when the unit has stopped (CG: decided while the
   // first step runs)
@@ -444,7 +522,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         constexpr int R1 = decltype(RR)::value;
         for (int t = tid; t < ns * N2 * P; t += kTPB) {
           const int q = a.dP.div(t), p = t - q * P, s = a.dN2.div(q), n2 = q - s * N2;
-          const V* src = R + (size_t)(sb + s) * ldr;
+          const V* src = Q > 1 ? R + (size_t)(sb + s) * ldr : Z + zs[sb + s] * ldz;
           V v[R1];
 #pragma unroll
           for (int n1 = 0; n1 < R1; ++n1) {
@@ -491,22 +569,41 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
           for (int k = 0; k < R1; ++k) d[k * N2 * LD] = v[k];
         }
       });
-      __syncthreads();
       radix2(N2, [&](auto RR) {
         constexpr int R2 = decltype(RR)::value;
-        for (int t = tid; t < ns * N1 * N; t += kTPB) {
+        // FP32: the potential of a thread's next task is loaded ahead, of the
+        // first before the barrier, of the others before the second transform
+        // of the last (in FP64 the registers would spill, and the FP64 pipe,
+        // not latency, is the bound)
+        constexpr bool ahead = sizeof(T) == 4;
+        const int tasks = ns * N1 * N;
+        T pot[R2];
+        auto load = [&](int t) {
+          if (t >= tasks) return;
+          const int q = a.dN.div(t), y = t - q * N, s = a.dN1.div(q), k1 = q - s * N1;
+          if (a.sh.v_smem) {
+            const T* vp = Vs + ((sb + s) * N + k1) * N + y;
+#pragma unroll
+            for (int k = 0; k < R2; ++k) pot[k] = vp[k * N1 * N];
+          } else {
+            const T* vp = a.Vp + ((size_t)(z0 + sb + s) * N + k1) * N + y;
+#pragma unroll
+            for (int k = 0; k < R2; ++k) pot[k] = __ldg(vp + k * N1 * N);
+          }
+        };
+        if (ahead) load(tid);
+        __syncthreads();
+        for (int t = tid; t < tasks; t += kTPB) {
           const int q = a.dN.div(t), y = t - q * N, s = a.dN1.div(q), k1 = q - s * N1;
           V* d = Tt + (s * N + k1 * R2) * LD + y;
-          const T* vp = a.Vp + ((size_t)(z0 + sb + s) * N + k1) * N + y;
-          T pot[R2];
           V v[R2];
-#pragma unroll
-          for (int k = 0; k < R2; ++k) pot[k] = vp[k * N1 * N];
 #pragma unroll
           for (int k = 0; k < R2; ++k) v[k] = d[k * LD];
           dft<T, 1, R2>(v);
+          if (!ahead) load(t);
 #pragma unroll
           for (int k = 0; k < R2; ++k) v[k] = mk<T>(v[k].x * pot[k], v[k].y * pot[k]);
+          if (ahead) load(t + kTPB);
           dft<T, -1, R2>(v);
           twid<T, -1, R2>(v, stw, k1);
 #pragma unroll
@@ -555,7 +652,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 #pragma unroll
           for (int k = 0; k < R1; ++k) v[k] = d[k * N2];
           dft<T, -1, R1>(v);
-          const int z = z0 + sb + s;
+          const int z = zs[z0 + sb + s];
 #pragma unroll
           for (int n1 = 0; n1 < R1; ++n1) {
             const unsigned row = rt[(n1 * N2 + n2) * P + p];
@@ -571,22 +668,8 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     return false;
   };
 
-  // z-FFT of the own pencils, in place (frequency z at slot zs[z])
+  // z-FFT of the own pencils, from slot order to natural order, in place
   auto z_forward = [&]() {
-    radix1(N1, [&](auto RR) {
-      constexpr int R1 = decltype(RR)::value;
-      for (int t = tid; t < nrl * N2; t += kTPB) {
-        const int n2 = dnr.div(t), row = t - n2 * nrl;
-        V v[R1];
-#pragma unroll
-        for (int n1 = 0; n1 < R1; ++n1) v[n1] = Z[(n1 * N2 + n2) * ldz + row];
-        dft<T, -1, R1>(v);
-        twid<T, -1, R1>(v, stw, n2);
-#pragma unroll
-        for (int k = 0; k < R1; ++k) Z[(k * N2 + n2) * ldz + row] = v[k];
-      }
-    });
-    __syncthreads();
     radix2(N2, [&](auto RR) {
       constexpr int R2 = decltype(RR)::value;
       for (int t = tid; t < nrl * N1; t += kTPB) {
@@ -595,8 +678,26 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 #pragma unroll
         for (int k = 0; k < R2; ++k) v[k] = Z[(k1 * R2 + k) * ldz + row];
         dft<T, -1, R2>(v);
+        twid<T, -1, R2>(v, stw, k1);
 #pragma unroll
         for (int k = 0; k < R2; ++k) Z[(k1 * R2 + k) * ldz + row] = v[k];
+      }
+    });
+    __syncthreads();
+    radix1(N1, [&](auto RR) {
+      constexpr int R1 = decltype(RR)::value;
+      for (int t = tid; t < nrl * N2; t += kTPB) {
+        const int n2 = dnr.div(t), row = t - n2 * nrl;
+        const int zmx = zm[row];
+        V v[R1];
+#pragma unroll
+        for (int k = 0; k < R1; ++k) v[k] = Z[(k * N2 + n2) * ldz + row];
+        dft<T, -1, R1>(v);
+#pragma unroll
+        for (int n1 = 0; n1 < R1; ++n1) {
+          const int z = n1 * N2 + n2;
+          if (z <= zmx || z >= N - zmx) Z[z * ldz + row] = v[n1];
+        }
       }
     });
     __syncthreads();
@@ -606,7 +707,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   auto gather = [&](int e, const W4& u) {
     const unsigned hp = hpos[e];
     const int j = (int)(hp >> 8), z = (int)(hp & 255u);
-    const V y1 = Z[zs[z] * ldz + (j - p0)], y2 = Z[zs[(N - z) % N] * ldz + mirror_row(j)];
+    const V y1 = Z[z * ldz + (j - p0)], y2 = Z[(N - z) % N * ldz + mirror_row(j)];
     const T k = kin[e];
     W4 t;
     if (PAIR) {
@@ -624,89 +725,117 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     }
     return t;
   };
-  // the four real vectors whose products with Re C and Im C are the coefficients
-  auto abcd = [&](int e, const W4& y) {
-    if (PAIR) {
-      const T f = (h0 + e == 0) ? one : two;
-      return W4{f * y.x, f * y.y, f * y.z, f * y.w};
-    }
-    return W4{y.x + y.z, y.y - y.w, y.y + y.w, y.z - y.x};
-  };
-
-  // projector coefficients of Tm (and, CG, of u = K r): partial sums over the
-  // own entries to every CTA; a warp takes RG rows (and one of the nsplit parts
-  // of the entries) at a time
+  // Projector coefficients of Tm (and, CG, of u): a warp takes RG rows and one
+  // of the nsplit parts of the own entries.  PAIR: sum_h f Re conj(c) y with
+  // f = 2, 1 at G = 0 (summed with 1 and 1/2, doubled at the end); complex:
+  // sum_h conj(c) y(G) + c y(-G) = Re c (y + y') + i Im c (y' - y).
   auto dots_rows = [&](auto RR) {
     constexpr int RG = decltype(RR)::value;
+    constexpr int M = pow2_up(RG * NV);
     const int ngr = (nproj + RG - 1) / RG;
     for (int w = warp; w < ngr * nsplit; w += kNW) {
-      const int gr = w / nsplit, part = w - gr * nsplit, v0 = gr * RG;
-      T acc[RG][NV];
+      const int gr = w / nsplit, prt = w - gr * nsplit, v0 = gr * RG;
+      const V* Cr[RG];
 #pragma unroll
-      for (int q = 0; q < RG; ++q)
+      for (int q = 0; q < RG; ++q) Cr[q] = C + (size_t)min(v0 + q, nproj - 1) * ldc;
+      T acc[M];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) acc[q][k] = (T)0;
+      for (int k = 0; k < M; ++k) acc[k] = (T)0;
 #pragma unroll 2
-      for (int e = lane + 32 * part; e < nh; e += 32 * nsplit) {
+      for (int e = lane + 32 * prt; e < nh; e += 32 * nsplit) {
         V c[RG];
 #pragma unroll
-        for (int q = 0; q < RG; ++q) c[q] = C[(size_t)min(v0 + q, nproj - 1) * ldc + e];
-        const W4 y = abcd(e, Tm[e]);
-        W4 u = {(T)0, (T)0, (T)0, (T)0};
-        if (CG) {
-          const W4 r = X[e];
-          const T k0 = Kt[2 * e], k1 = Kt[2 * e + 1];
-          u = abcd(e, W4{k0 * r.x, k0 * r.y, k1 * r.z, k1 * r.w});
+        for (int q = 0; q < RG; ++q) c[q] = Cr[q][e];
+        W4 y = Tm[e];
+        if (PAIR) {
+          if (h0 + e == 0) { y.x *= (T)0.5; y.z *= (T)0.5; }
+        } else {
+          y = W4{y.x + y.z, y.y - y.w, y.y + y.w, y.z - y.x};
         }
 #pragma unroll
         for (int q = 0; q < RG; ++q) {
-          acc[q][0] += c[q].x * y.x + c[q].y * y.y;
-          acc[q][1] += c[q].x * y.z + c[q].y * y.w;
-          if (CG) {
-            acc[q][NV - 2] += c[q].x * u.x + c[q].y * u.y;
-            acc[q][NV - 1] += c[q].x * u.z + c[q].y * u.w;
+          acc[q * NV] += c[q].x * y.x + c[q].y * y.y;
+          acc[q * NV + 1] += c[q].x * y.z + c[q].y * y.w;
+        }
+        if (CG) {
+          W4 u = Tm[a.nhl + e];
+          if (h0 + e == 0) { u.x *= (T)0.5; u.z *= (T)0.5; }
+#pragma unroll
+          for (int q = 0; q < RG; ++q) {
+            acc[q * NV + NV - 2] += c[q].x * u.x + c[q].y * u.y;
+            acc[q * NV + NV - 1] += c[q].x * u.z + c[q].y * u.w;
           }
         }
       }
-#pragma unroll
-      for (int q = 0; q < RG; ++q)
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) acc[q][k] += __shfl_xor_sync(0xffffffffu, acc[q][k], o);
-      if (lane < Q) {
-        T* d = at(coefp, lane);
-#pragma unroll
-        for (int q = 0; q < RG; ++q)
-          if (v0 + q < nproj)
-#pragma unroll
-            for (int k = 0; k < NV; ++k)
-              d[((size_t)(rank * nsplit + part) * nproj + v0 + q) * NV + k] = acc[q][k];
-      }
+      const T t = warp_sums<M, T>(acc);
+      const int k = lane / (32 / M), q = k / NV;
+      if (lane % (32 / M) == 0 && q < RG && v0 + q < nproj)
+        cp[((size_t)prt * nproj + v0 + q) * NV + (k - q * NV)] = PAIR ? (T)2 * t : t;
     }
   };
   auto dots = [&]() {
-    if (nproj >= 4 * kNW) dots_rows(IC<4>());
-    else if (nproj >= 2 * kNW) dots_rows(IC<2>());
-    else dots_rows(IC<1>());
-  };
-  auto coef_sum = [&](int first) {                // threads from `first` on
-    for (int j = tid - first; j >= 0 && j < nproj * NV; j += kTPB - first) {
-      T s = (T)0;
-      for (int q = 0; q < Q * nsplit; ++q) s += coefp[(size_t)q * nproj * NV + j];
-      coef[j] = s;
+    switch (rgrp) {
+      case 1: dots_rows(IC<1>()); break;
+      case 2: dots_rows(IC<2>()); break;
+      case 5: if constexpr (sizeof(T) == 4) dots_rows(IC<5>()); break;
+      case 6: if constexpr (sizeof(T) == 4) dots_rows(IC<6>()); break;
+      default: dots_rows(IC<4>());
     }
+  };
+  // the parts added, to every CTA
+  auto send_coef = [&]() {
+    const int n = nproj * NV;
+    for (int t = tid; t < (n << a.sh.lq); t += kTPB) {
+      const int q = t / n, j = t - q * n;
+      T v = cp[j];
+      for (int p = 1; p < nsplit; ++p) v += cp[p * n + j];
+      at(coefp, q)[rank * n + j] = v;
+    }
+  };
+  auto coef_of = [&](int j) {
+    T v = coefp[j];
+    for (int q = 1; q < Q; ++q) v += coefp[q * nproj * NV + j];
+    return v;
+  };
+  auto coef_sum = [&]() {
+    for (int j = tid; j < nproj * NV; j += kTPB) coef[j] = coef_of(j);
+  };
+  // Up to four scalar sums.  put: this thread's values into the warp's part;
+  // after a barrier one warp adds the parts and sends them to every CTA (slot);
+  // after the cluster barrier take gives value (lane & 3) in every lane.
+  auto put_sums = [&](auto NN, SA* v) {
+    constexpr int NS = decltype(NN)::value;
+    const SA t = warp_sums<NS, SA>(v);
+    if (lane % (32 / NS) == 0) part[warp * 4 + lane / (32 / NS)] = t;
+  };
+  auto send_sums = [&](int ns, int slot) {        // one warp
+    const int k = lane & 3;
+    SA t = of_((T)0);
+    if (k < ns)
+      for (int w = lane >> 2; w < kNW; w += 8) t = add_(t, part[w * 4 + k]);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) t = add_(t, shx_(t, o));
+    if (k < ns)
+      for (int q = lane >> 2; q < Q; q += 8) at(sc, q)[((slot << a.sh.lq) + rank) * 4 + k] = t;
+  };
+  auto take_sums = [&](int slot) {                // one warp
+    SA t = of_((T)0);
+    for (int q = lane >> 2; q < Q; q += 8) t = add_(t, sc[((slot << a.sh.lq) + q) * 4 + (lane & 3)]);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) t = add_(t, shx_(t, o));
+    return t;
   };
   // y - sum_v C_v coef_v at one half entry
   auto project = [&](int e, W4 y) {
     T a1 = (T)0, a2 = (T)0, a3 = (T)0, a4 = (T)0;
+    constexpr int U = sizeof(T) == 4 ? 16 : 8;    // rows in flight
     int v = 0;
-    for (; v + 8 <= nproj; v += 8) {
-      V c[8];
+    for (; v + U <= nproj; v += U) {
+      V c[U];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) c[q] = C[(size_t)(v + q) * ldc + e];
+      for (int q = 0; q < U; ++q) c[q] = C[(size_t)(v + q) * ldc + e];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
+      for (int q = 0; q < U; ++q) {
         const T k0 = coef[(v + q) * NV], k1 = coef[(v + q) * NV + 1];
         a1 += c[q].x * k0;
         a4 += c[q].y * k0;
@@ -731,88 +860,162 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     return y;
   };
 
-  // NS sums of this thread's values to every CTA (slot k), and their ordered
-  // total in every lane of the calling warp after the cluster barrier
-  auto send_sums = [&](auto NN, SA* v, int slot) {
-    constexpr int NS = decltype(NN)::value;
-#pragma unroll
-    for (int k = 0; k < NS; ++k)
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v[k] = add_(v[k], shx_(v[k], o));
-    if (lane < Q) {
-      SA* d = at(sc, lane) + slot * nsc + (rank * kNW + warp) * 4;
-#pragma unroll
-      for (int k = 0; k < NS; ++k) d[k] = v[k];
-    }
-  };
-  auto take_sum = [&](int slot, int k) {          // one warp
-    const SA* s = sc + slot * nsc + k;
-    SA t = of_((T)0);
-    for (int q = lane; q < Q * kNW; q += 32) t = add_(t, s[q * 4]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t = add_(t, shx_(t, o));
-    return t;
-  };
-
   if constexpr (CG) {
     // Chronopoulos and Gear's one-reduction form (see kernels_cg.cu): u = K r,
-    // w = P_c (H - E) u, gamma = r^H u, delta = u^H w
-    for (int k = 0;; ++k) {
-      // r after k updates: u into the pencils, gamma and |r|^2
-      SA v4[4] = {of_((T)0), of_((T)0), of_((T)0), of_((T)0)};
-      {
-        T g0 = (T)0, r0 = (T)0, g1 = (T)0, r1 = (T)0;
-        const T al0 = s_cg[0].al, al1 = s_cg[1].al, bt0 = s_cg[0].bt, bt1 = s_cg[1].bt;
-        const bool a0 = k == 0 || s_cg[0].active, a1 = k == 0 || s_cg[1].active;
-        for (int e = tid; e < nh; e += kTPB) {
-          const T k0 = Kt[2 * e], k1 = Kt[2 * e + 1];
-          W4 r = X[e];
-          if (k > 0) {
-            W4 p = X[xs + e], s = X[2 * xs + e], x = X[3 * xs + e];
-            const W4 w = project(e, Tm[e]);
-            if (a0) {
-              p.x = k0 * r.x + bt0 * p.x; p.y = k0 * r.y + bt0 * p.y;
-              s.x = w.x + bt0 * s.x;      s.y = w.y + bt0 * s.y;
-              x.x += al0 * p.x;           x.y += al0 * p.y;
-              r.x -= al0 * s.x;           r.y -= al0 * s.y;
-            }
-            if (a1) {
-              p.z = k1 * r.z + bt1 * p.z; p.w = k1 * r.w + bt1 * p.w;
-              s.z = w.z + bt1 * s.z;      s.w = w.w + bt1 * s.w;
-              x.z += al1 * p.z;           x.w += al1 * p.w;
-              r.z -= al1 * s.z;           r.w -= al1 * s.w;
-            }
-            X[e] = r;
-            X[xs + e] = p;
-            X[2 * xs + e] = s;
-            X[3 * xs + e] = x;
+    // w = P_c (H - E) u, gamma = r^H u, delta = u^H w.  The four real
+    // components of a half entry (Re, Im of both columns) are independent but
+    // for the packing: one thread each while that fills no more than the CTA
+    // (latency counts: 16^3 FP64, update 9.6k -> 4.0k cycles), else one thread
+    // per entry (a quarter of the loads: 48^3 FP32, 7.4k -> 3.2k cycles).
+    T* XT = reinterpret_cast<T*>(X);
+    T* TT = reinterpret_cast<T*>(Tm);
+    T* ZT = reinterpret_cast<T*>(Z);
+    const T* CT = reinterpret_cast<const T*>(C);
+    const bool quads = 4 * a.nhl <= kTPB;
+    // r after k updates: u into the pencils, gamma and |r|^2
+    auto update1 = [&](int k, SA* v4) {
+      T g0 = (T)0, r0 = (T)0, g1 = (T)0, r1 = (T)0;
+      const T al0 = s_cg[0].al, al1 = s_cg[1].al, bt0 = s_cg[0].bt, bt1 = s_cg[1].bt;
+      const bool a0 = k == 0 || s_cg[0].active, a1 = k == 0 || s_cg[1].active;
+      for (int e = tid; e < nh; e += kTPB) {
+        const T k0 = Kt[2 * e], k1 = Kt[2 * e + 1];
+        W4 r = X[e];
+        if (k > 0) {
+          W4 p = X[xs + e], sv = X[2 * xs + e], x = X[3 * xs + e];
+          const W4 w = project(e, Tm[e]);
+          if (a0) {
+            p.x = k0 * r.x + bt0 * p.x; p.y = k0 * r.y + bt0 * p.y;
+            sv.x = w.x + bt0 * sv.x;    sv.y = w.y + bt0 * sv.y;
+            x.x += al0 * p.x;           x.y += al0 * p.y;
+            r.x -= al0 * sv.x;          r.y -= al0 * sv.y;
           }
-          const T f = (h0 + e == 0) ? one : two;
-          const T n0 = f * (r.x * r.x + r.y * r.y), n1 = f * (r.z * r.z + r.w * r.w);
-          r0 += n0;
-          g0 += k0 * n0;
-          r1 += n1;
-          g1 += k1 * n1;
-          W4 u = {(T)0, (T)0, (T)0, (T)0};
-          if (a0) { u.x = k0 * r.x; u.y = k0 * r.y; }
-          if (a1) { u.z = k1 * r.z; u.w = k1 * r.w; }
-          scatter(e, u);
+          if (a1) {
+            p.z = k1 * r.z + bt1 * p.z; p.w = k1 * r.w + bt1 * p.w;
+            sv.z = w.z + bt1 * sv.z;    sv.w = w.w + bt1 * sv.w;
+            x.z += al1 * p.z;           x.w += al1 * p.w;
+            r.z -= al1 * sv.z;          r.w -= al1 * sv.w;
+          }
+          X[e] = r;
+          X[xs + e] = p;
+          X[2 * xs + e] = sv;
+          X[3 * xs + e] = x;
         }
-        v4[0] = of_(g0); v4[1] = of_(r0); v4[2] = of_(g1); v4[3] = of_(r1);
+        const T f = (h0 + e == 0) ? one : two;
+        const T n0 = f * (r.x * r.x + r.y * r.y), n1 = f * (r.z * r.z + r.w * r.w);
+        r0 += n0;
+        g0 += k0 * n0;
+        r1 += n1;
+        g1 += k1 * n1;
+        W4 u = {(T)0, (T)0, (T)0, (T)0};
+        if (a0) { u.x = k0 * r.x; u.y = k0 * r.y; }
+        if (a1) { u.z = k1 * r.z; u.w = k1 * r.w; }
+        scatter(e, u);
       }
-      send_sums(IC<4>(), v4, 0);
+      v4[0] = of_(g0); v4[1] = of_(r0); v4[2] = of_(g1); v4[3] = of_(r1);
+    };
+    const int cmp = tid & 3, cc = cmp >> 1;       // component x, y (column 0), z, w (column 1)
+    const int im = (cmp == 1 || cmp == 2) ? 1 : 0;
+    auto update4 = [&](int k, SA* v4) {
+      T gs = (T)0, rs = (T)0, u = (T)0;
+      const int t = tid, e = t >> 2;              // 4 nh <= kTPB: one round
+      if (e < nh) {
+        const T kc = Kt[2 * e + cc];
+        T r = XT[t];
+        const bool act = k == 0 || s_cg[cc].active;
+        if (k > 0 && act) {
+          const T al = s_cg[cc].al, bt = s_cg[cc].bt;
+          T w = TT[t], p = XT[4 * xs + t], sv = XT[8 * xs + t], x = XT[12 * xs + t];
+          const T* c = CT + 2 * e + (cmp & 1);
+          const T* kf = coef + cc;
+          T acc = (T)0;
+          int v = 0;
+          for (; v + 8 <= nproj; v += 8) {
+            T cv[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) cv[q] = c[2 * (size_t)(v + q) * ldc];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) acc += cv[q] * kf[(v + q) * NV];
+          }
+          for (; v < nproj; ++v) acc += c[2 * (size_t)v * ldc] * kf[v * NV];
+          w -= acc;
+          p = kc * r + bt * p;
+          sv = w + bt * sv;
+          x += al * p;
+          r -= al * sv;
+          XT[t] = r;
+          XT[4 * xs + t] = p;
+          XT[8 * xs + t] = sv;
+          XT[12 * xs + t] = x;
+        }
+        rs = (h0 + e == 0) ? r * r : two * r * r;
+        gs = kc * rs;
+        if (act) u = kc * r;
+      }
+      // pair packing: x - w, y + z at G; x + w, z - y at -G
+      const T o = shx_(u, 3);
+      if (e < nh) {
+        const unsigned hp = hpos[e];
+        const int j = (int)(hp >> 8), z = (int)(hp & 255u);
+        if (cmp < 2) ZT[2 * (z * ldz + (j - p0)) + im] = cmp ? u + o : u - o;
+        else if (h0 + e != 0) ZT[2 * ((N - z) % N * ldz + mirror_row(j)) + im] = cmp == 2 ? u - o : u + o;
+      }
+      v4[0] = of_(cc ? (T)0 : gs); v4[1] = of_(cc ? (T)0 : rs);
+      v4[2] = of_(cc ? gs : (T)0); v4[3] = of_(cc ? rs : (T)0);
+    };
+    // w and u, and u^H w before the projector
+    auto gather1 = [&](SA* v2) {
+      T d0 = (T)0, d1 = (T)0;
+      for (int e = tid; e < nh; e += kTPB) {
+        const T k0 = Kt[2 * e], k1 = Kt[2 * e + 1];
+        const W4 r = X[e];
+        const W4 u = {k0 * r.x, k0 * r.y, k1 * r.z, k1 * r.w};
+        const W4 w = gather(e, u);
+        Tm[e] = w;
+        Tm[a.nhl + e] = u;
+        const T f = (h0 + e == 0) ? one : two;
+        d0 += f * (u.x * w.x + u.y * w.y);
+        d1 += f * (u.z * w.z + u.w * w.w);
+      }
+      v2[0] = of_(d0);
+      v2[1] = of_(d1);
+    };
+    auto gather4 = [&](SA* v2) {
+      T ds = (T)0;
+      const int t = tid, e = t >> 2;
+      if (e < nh) {
+        const unsigned hp = hpos[e];
+        const int j = (int)(hp >> 8), z = (int)(hp & 255u);
+        const T y1 = ZT[2 * (z * ldz + (j - p0)) + im], y2 = ZT[2 * ((N - z) % N * ldz + mirror_row(j)) + im];
+        const T u = Kt[2 * e + cc] * XT[t];
+        const T fv = (T)0.5 * (cmp == 1 ? y1 - y2 : cmp == 3 ? y2 - y1 : y1 + y2);
+        const T w = fv + (kin[e] - Ex[cc]) * u;
+        TT[t] = w;
+        TT[4 * a.nhl + t] = u;
+        ds = ((h0 + e == 0) ? one : two) * u * w;
+      }
+      v2[0] = of_(cc ? (T)0 : ds);
+      v2[1] = of_(cc ? ds : (T)0);
+    };
+    const bool decide = warp == kNW - 1;
+    for (int k = 0;; ++k) {
+      {
+        SA v4[4];
+        if (quads) update4(k, v4);
+        else update1(k, v4);
+        put_sums(IC<4>(), v4);
+      }
       __syncthreads();
+      if (decide) send_sums(4, 0);
       z_inverse();
       csync();
       // while the slabs' first step runs: gamma, |r|^2 and the stopping tests
-      if (warp == 0) {
-        SA g[2], q[2];
-#pragma unroll
-        for (int c = 0; c < 2; ++c) { g[c] = take_sum(0, 2 * c); q[c] = take_sum(0, 2 * c + 1); }
+      if (decide) {
+        const SA tot = take_sums(0);
+        const SA g = shi_(tot, (2 * lane) & 3), q = shi_(tot, (2 * lane + 1) & 3);
         int act = 0;
         if (lane < 2) {
           CgCol<T>& st = s_cg[lane];
-          const T gam = val_(lane ? g[1] : g[0]), rr = val_(lane ? q[1] : q[0]);
+          const T gam = val_(g), rr = val_(q);
           if (k == 0) {
             const T s1 = (T)a.tol2 * rr, s2 = (a.rr_abs && lane < nc) ? (T)a.rr_abs[c0 + lane] : (T)0;
             st.stop = s1 > s2 ? s1 : s2;
@@ -830,7 +1033,9 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
             else if (k >= a.maxit) { st.flag = 1; stop = 1; }
             else if (k - st.itb > max(kCgStagWindow, 2 * st.itb)) { st.flag = 4; stop = 1; }
             st.it = k;
-            st.gprev = st.gam;
+            // beta, and gamma / alpha_prev for the denominator of alpha
+            st.bt = k > 0 ? gam / st.gam : (T)0;
+            st.gdiv = k > 0 ? gam / st.alpha : (T)0;
             st.gam = gam;
             if (stop) st.active = 0;
           }
@@ -843,55 +1048,46 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       csync();
       z_forward();
       {
-        T d0 = (T)0, d1 = (T)0;
-        for (int e = tid; e < nh; e += kTPB) {
-          const T k0 = Kt[2 * e], k1 = Kt[2 * e + 1];
-          const W4 r = X[e];
-          const W4 u = {k0 * r.x, k0 * r.y, k1 * r.z, k1 * r.w};
-          const W4 w = gather(e, u);
-          Tm[e] = w;
-          const T f = (h0 + e == 0) ? one : two;
-          d0 += f * (u.x * w.x + u.y * w.y);
-          d1 += f * (u.z * w.z + u.w * w.w);
-        }
-        v4[0] = of_(d0);
-        v4[1] = of_(d1);
+        SA v2[2];
+        if (quads) gather4(v2);
+        else gather1(v2);
+        put_sums(IC<2>(), v2);
       }
-      send_sums(IC<2>(), v4, 1);
       __syncthreads();
       dots();
-      csync();
-      coef_sum(32);
-      SA uw0 = of_((T)0), uw1 = of_((T)0);
-      if (warp == 0) { uw0 = take_sum(1, 0); uw1 = take_sum(1, 1); }
       __syncthreads();
-      if (warp == 0) {
-        // delta = u^H w - sum_v <C_v|u> <C_v|w>, alpha, beta
-        SA t0 = of_((T)0), t1 = of_((T)0);
+      send_coef();
+      if (decide) send_sums(2, 1);
+      csync();
+      coef_sum();
+      if (decide) {
+        // delta = u^H w - sum_v <C_v|u> <C_v|w>, alpha
+        const SA tot = take_sums(1);
+        SA t2[2] = {of_((T)0), of_((T)0)};
         for (int v = lane; v < nproj; v += 32) {
-          const T* c = coef + v * NV;
-          t0 = add_(t0, of_(c[0] * c[NV - 2]));
-          t1 = add_(t1, of_(c[1] * c[NV - 1]));
+          const W4* c4 = reinterpret_cast<const W4*>(coefp) + v;
+          W4 c = c4[0];
+          for (int q = 1; q < Q; ++q) {
+            const W4 d = c4[q * nproj];
+            c.x += d.x; c.y += d.y; c.z += d.z; c.w += d.w;
+          }
+          t2[0] = add_(t2[0], of_(c.x * c.z));
+          t2[1] = add_(t2[1], of_(c.y * c.w));
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) { t0 = add_(t0, shx_(t0, o)); t1 = add_(t1, shx_(t1, o)); }
+        const SA tv = warp_sums<2, SA>(t2);
+        const SA t = shi_(tv, (lane & 1) * 16), uw = shi_(tot, lane & 1);
         int act = 0;
         if (lane < 2) {
           CgCol<T>& st = s_cg[lane];
           if (st.active) {
-            const T delta = val_(add_(lane ? uw1 : uw0, scale_(lane ? t1 : t0, (T)-1)));
-            T den = delta, bt = (T)0;
-            if (k > 0) {
-              bt = st.gam / st.gprev;
-              den = delta - bt * st.gam / st.alpha;
-            }
+            const T delta = val_(add_(uw, scale_(t, (T)-1)));
+            const T den = k > 0 ? delta - st.bt * st.gdiv : delta;
             if (!(den > (T)0) || !isfinite(den) || !(st.gam > (T)0)) {
               st.flag = 2;
               st.active = 0;
             } else {
               st.alpha = st.gam / den;
               st.al = st.alpha;
-              st.bt = bt;
             }
           }
           act = st.active;
@@ -929,24 +1125,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         }
       }
     };
-    // totals of the four slots of `norms` for column c: |r|^2, rho
-    auto take_norms = [&](int slot, int c, double* rr, double2* rho) {
-      if (PAIR) {
-        const double a0 = dbl_(take_sum(slot, 0)), a1 = dbl_(take_sum(slot, 1));
-        const double b0 = dbl_(take_sum(slot, 2)), b1 = dbl_(take_sum(slot, 3));
-        *rr = c ? a1 : a0;
-        *rho = make_double2(c ? b1 : b0, 0.0);
-      } else {
-        *rr = dbl_(take_sum(slot, 0));
-        const double x = dbl_(take_sum(slot, 1));
-        *rho = make_double2(x, dbl_(take_sum(slot, 2)));
-      }
-    };
-    auto cdiv_ = [](double2 p, double2 q) {
-      if (PAIR) return make_double2(p.x / q.x, 0.0);
-      const double den = q.x * q.x + q.y * q.y;
-      return make_double2((p.x * q.x + p.y * q.y) / den, (p.y * q.x - p.x * q.y) / den);
-    };
+    const bool decide = warp == kNW - 1;
     {
       SA v[4] = {of_((T)0), of_((T)0), of_((T)0), of_((T)0)};
       for (int e = tid; e < nh; e += kTPB) {
@@ -957,19 +1136,21 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         X[xs + e] = q;
         scatter(e, q);
       }
-      send_sums(IC<4>(), v, 0);
+      put_sums(IC<4>(), v);
+      __syncthreads();
+      if (decide) send_sums(4, 0);
       csync();
-      if (warp == 0) {
-        double rr;
-        double2 rho;
-        take_norms(0, lane, &rr, &rho);
+      if (decide) {
+        const double t = dbl_(take_sums(0));
+        const double rr = shi_(t, PAIR ? lane & 1 : 0), rx = shi_(t, PAIR ? 2 + (lane & 1) : 1), ry = shi_(t, 2);
         int act = 0;
         if (lane < nc) {
           QmrCol& st = s_q[lane];
-          st.tau = sqrt(rr);
-          st.rho = rho;
+          st.tau2 = rr;
+          st.rho = make_double2(rx, PAIR ? 0.0 : ry);
           st.stop = fmax(a.tol2 * rr, a.rr_abs ? a.rr_abs[c0 + lane] : 0.0);
           st.qbest = rr;
+          st.rr0 = rr;
           st.near = -1;
           st.active = act = (on[lane] && rr > 0.0) ? 1 : 0;
         }
@@ -987,8 +1168,10 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       for (int e = tid; e < nh; e += kTPB) Tm[e] = gather(e, X[xs + e]);
       __syncthreads();
       dots();
+      __syncthreads();
+      send_coef();
       csync();
-      coef_sum(0);
+      coef_sum();
       __syncthreads();
       // t = P_c t and [q, t]
       SA v[4] = {of_((T)0), of_((T)0), of_((T)0), of_((T)0)};
@@ -1008,23 +1191,26 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
           fma_(v[1], q.z, t.y); fma_(v[1], q.w, t.x); fma_(v[1], q.x, t.w); fma_(v[1], q.y, t.z);
         }
       }
-      send_sums(IC<2>(), v, 1);
+      put_sums(IC<2>(), v);
+      __syncthreads();
+      if (decide) send_sums(2, 1);
       csync();
-      if (warp == 0) {
-        const double s0 = dbl_(take_sum(1, 0)), s1 = dbl_(take_sum(1, 1));
-        if (lane < nc) {
-          QmrCol& st = s_q[lane];
-          const double2 sg = PAIR ? make_double2(lane ? s1 : s0, 0.0) : make_double2(s0, s1);
-          const double2 rho = st.rho;
-          if (!st.active) {
-            // a stopped column of a pair: q = 0, nothing to update
-          } else if (!(sg.x * sg.x + sg.y * sg.y > 1e-300 * (rho.x * rho.x + rho.y * rho.y)) || !isfinite(sg.x) ||
-              !isfinite(sg.y)) {
-            st.alpha = make_double2(0.0, 0.0);
-            st.flag = 2;                          // serious breakdown: [q, A q] = 0
-          } else {
-            st.alpha = cdiv_(rho, sg);
-          }
+      if (decide) {
+        // alpha = rho / [q, t]: one division in the lanes of Re and Im (PAIR: of the columns)
+        const double t = dbl_(take_sums(1));
+        const double sx = shi_(t, PAIR ? lane & 1 : 0), sy = PAIR ? 0.0 : shi_(t, 1);
+        QmrCol& st = s_q[PAIR ? lane & 1 : 0];
+        const double2 rho = st.rho;
+        const double num = PAIR ? rho.x : (lane & 1) ? rho.y * sx - rho.x * sy : rho.x * sx + rho.y * sy;
+        const double s2 = sx * sx + sy * sy;
+        const double al = num / (PAIR ? sx : s2);
+        const bool bad = !(s2 > 1e-300 * (rho.x * rho.x + rho.y * rho.y)) || !isfinite(sx) || !isfinite(sy);
+        __syncwarp();
+        // a stopped column of a pair has q = 0 and keeps its flag
+        if (lane < 2 && (!PAIR || (lane < nc && st.active))) {
+          if (bad) st.flag = 2;                   // serious breakdown: [q, A q] = 0
+          double* d = &st.alpha.x + (PAIR ? 0 : lane);
+          *d = bad ? 0.0 : al;
         }
       }
       __syncthreads();
@@ -1050,40 +1236,53 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
           norms(e, r, v);
         }
       }
-      send_sums(IC<4>(), v, 2);
+      put_sums(IC<4>(), v);
+      __syncthreads();
+      if (decide) send_sums(4, 2);
       csync();
-      if (warp == 0) {
-        double rr;
-        double2 rn;
-        take_norms(2, lane, &rr, &rn);
+      if (decide) {
+        // theta^2 = |r|^2 / tau^2, c^2 = 1 / (1 + theta^2) = tau^2 / (tau^2 + |r|^2),
+        // tau'^2 = tau^2 theta^2 c^2 = |r|^2 c^2, beta = rho' / rho: one division,
+        // the quotients in lanes 0, 1 .. (PAIR: two lanes each)
+        const double t = dbl_(take_sums(2));
+        const int c = PAIR ? lane & 1 : 0, w = PAIR ? lane >> 1 : lane;
+        const double rr = shi_(t, PAIR ? c : 0), rx = shi_(t, PAIR ? 2 + c : 1), ry = PAIR ? 0.0 : shi_(t, 2);
+        const double tau2 = s_q[c].tau2;
+        const double2 rho = s_q[c].rho;
+        const double rho2 = PAIR ? rho.x : rho.x * rho.x + rho.y * rho.y;
+        double num = w == 0 ? rr : w == 1 ? tau2 : rx, den = w == 0 ? tau2 : w == 1 ? tau2 + rr : rho2;
+        if (!PAIR && w == 2) num = rx * rho.x + ry * rho.y;
+        if (!PAIR && w == 3) num = ry * rho.x - rx * rho.y;
+        const double quo = num / den;
+        const double th2 = shi_(quo, c), c2 = shi_(quo, PAIR ? 2 + c : 1);
+        const double bx = shi_(quo, PAIR ? 4 + c : 2), by = PAIR ? 0.0 : shi_(quo, 3);
+        __syncwarp();
         int act = 0;
         if (lane < nc) {
           QmrCol& st = s_q[lane];
+          const double2 rn = make_double2(rx, ry);
           st.upd = st.active;
           if (st.active) {
-            const double th = sqrt(rr) / st.tau;
-            const double c2 = 1.0 / (1.0 + th * th);
-            st.dc = c2 * st.theta * st.theta;
+            st.dc = c2 * st.theta2;
             st.qc = make_double2(c2 * st.alpha.x, c2 * st.alpha.y);
-            st.tau = st.tau * th * sqrt(c2);
-            st.theta = th;
-            const double2 rho = st.rho;
-            st.beta = (rho.x * rho.x + rho.y * rho.y > 0.0) ? cdiv_(rn, rho) : make_double2(0.0, 0.0);
+            st.tau2 = rr * c2;
+            st.theta2 = th2;
+            st.beta = rho2 != 0.0 ? make_double2(bx, by) : make_double2(0.0, 0.0);
             st.rho = rn;
             const int it = ++st.it;
-            const double qb = st.tau * st.tau;
+            const double qb = st.tau2;
             if (qb < 0.25 * st.qbest) { st.qbest = qb; st.itb = it; }
             if (st.near < 0 && qb <= 4.0 * st.stop) st.near = it;
             bool stop = false;
-            if (st.flag == 2 || !isfinite(st.tau)) { st.flag = 2; stop = true; }
+            if (st.flag == 2 || !isfinite(st.tau2)) { st.flag = 2; stop = true; }
             else if (qb <= st.stop) { st.flag = 0; stop = true; }
             else if (!(rn.x * rn.x + rn.y * rn.y > 0.0)) { st.flag = 2; stop = true; }
             else if (it >= a.maxit) { st.flag = 1; stop = true; }
             else if (it - st.itb > max(kQmrWindow, 2 * st.itb)) { st.flag = 4; stop = true; }
-            // tau never grows; within a factor 2 of the target and still short
-            // of it after kNearWait iterations, it has reached the floor of
-            // the working precision (FP32 passes stop a little above 1e-5
-            // now and then): the FP64 residual of the refinement decides
+            else if (sizeof(T) == 4 && qb <= 1e-8 * st.rr0 && it - st.itb > kQmrWindowFloor) { st.flag = 4; stop = true; }
+            // tau never grows: short of the target after this, the FP64 residual of
+            // the refinement decides (1104 columns on 32^3: one or two of them kept
+            // the pass going for 1000 iterations after the others' 190)
             else if (st.near >= 0 && it - st.near > kNearWait) { st.flag = 4; stop = true; }
             if (stop) st.active = 0;
           }
@@ -1225,7 +1424,8 @@ bool col_shape(const ColPlan& p, int kind, int N, int nproj, int nunit, int cta_
   // with it the last bits, depends on Q: FP64 results do not depend on how many
   // contexts share the GPU, so there Q does not either.
   const bool f32 = sizeof(T) == 4;
-  const double share = f32 ? std::max(cta_div, 1) : 1.0;
+  // (contexts that share the GPU keep it busy about half the time each)
+  const double share = f32 ? std::max(0.5 * cta_div, 1.0) : 1.0;
   const double fixed = f32 ? 11.0 : 27.0;
   const double work = (f32 ? 1.0e-3 : 1.5e-2) * N * N * N + (f32 ? 0.9e-3 : 1.66e-2) * nproj * p.nh;
   double best = 1e300;
@@ -1235,21 +1435,37 @@ bool col_shape(const ColPlan& p, int kind, int N, int nproj, int nunit, int cta_
     ColShape s;
     s.lq = lq;
     const int nzl = (N + Q - 1) / Q;
-    auto fits = [&](int nsb, bool vec, bool c) {
+    auto fits = [&](int nsb, bool vec, bool c, bool v = false) {
       s.nsb = nsb;
       s.vec_smem = vec;
       s.c_smem = c;
+      s.v_smem = v;
       s.smem = col::layout<T>(kind, s, N, p.P, p.npair, ldz, nhl, nproj).total;
       return s.smem <= col::kSmemMax;
     };
-    // slabs together first (threads busy), then the vectors, then the rows
-    int nsb = nzl;
-    while (nsb > 1 && !fits(nsb, false, false)) --nsb;
-    if (!fits(nsb, false, false)) continue;
-    while (nsb > 1 && !fits(nsb, true, false) && (size_t)(nsb - 1) * N * N >= 8 * (size_t)col::kTPB) --nsb;
-    const bool vec = fits(nsb, true, false);
-    const bool c = fits(nsb, vec, true);
-    fits(nsb, vec, c);
+    // slabs together: the fewest rounds of the CTA's threads (FP64: of a warp
+    // per scheduler) over the passes of all batches; then the rows and the
+    // potential where room is left
+    auto rounds_of = [&](int nsb) {
+      const int unit = sizeof(T) == 4 ? col::kTPB : 128;
+      auto r = [&](long tasks) { return (double)((tasks + unit - 1) / unit); };
+      double t = 0.0;
+      for (int sb = 0; sb < nzl; sb += nsb) {
+        const long ns = std::min(nsb, nzl - sb);
+        t += 2.0 * (r(ns * p.N2 * p.P) + r(ns * p.N1 * p.P) + r(ns * p.N2 * N)) + 1.6 * r(ns * p.N1 * N) + 2.0;
+      }
+      return t;
+    };
+    int nsb = 0;
+    bool vec = true;
+    for (int pass = 0; pass < 2 && nsb == 0; ++pass) {
+      vec = pass == 0;
+      for (int n = 1; n <= nzl; ++n)
+        if (fits(n, vec, false) && (nsb == 0 || rounds_of(n) < rounds_of(nsb))) nsb = n;
+    }
+    if (nsb == 0) continue;
+    const bool c = fits(nsb, vec, true), v = fits(nsb, vec, c, true);
+    fits(nsb, vec, c, v);
     s.vec_elems = vec ? 0 : 16 * (size_t)p.nh;
     const int act = col::active_clusters<T>(kind, lq, s.smem);
     if (act < 1) continue;
