@@ -20,7 +20,8 @@ constexpr int kColNQ = 5;                          // cluster sizes 1, 2, 4, 8, 
 // -G (in the second); h = 0 is G = 0.  The CTA of rank r in a cluster of Q owns
 // the pairs split[lq][r] .. split[lq][r + 1] (lq = log2 Q) and their entries.
 struct ColPlan {
-  bool ok = false;
+  bool half = false;                               // the entry tables (gp, gm, nh) are set
+  bool ok = false;                                 // and the column solver has radices for N
   int N1 = 0, N2 = 0, P = 0, nm = 0;               // planes |n0| <= nm: P = 2 nm + 1
   int npair = 0, nh = 0;
   int maxpair[kColNQ] = {0}, maxh[kColNQ] = {0};   // per CTA, by log2 Q
@@ -78,6 +79,22 @@ struct ColArgs {
   int* iters;                    // [ncol]
   int* flags;                    // [ncol]
 };
+
+// FP64 projector and residual on half entries (kernels_half.cu); rows are
+// ColPrec<double>::Ch, real: columns real in real space.  launch_gram_half
+// leaves the coefficients <C|Y> in partial sums (half_part_elems) and returns
+// the number of parts for the kernels that use them:
+//   launch_proj_half      Y -= C coef
+//   launch_residual_half  r -= C coef; out[3][ncol] = |r|^2, |b|^2, |x|^2
+size_t half_part_elems(int nrow, int nh, int ncol);
+size_t half_sum_elems(int nh, int ncol);
+int launch_gram_half(cudaStream_t s, bool real, const ColPlan& p, const double2* Ch, int nrow, const double2* Y,
+                     int npw, int ncol, const int* active, double* part);
+void launch_proj_half(cudaStream_t s, bool real, const ColPlan& p, const double2* Ch, int nrow, double2* Y, int npw,
+                      int ncol, const int* active, int nchunk, const double* part);
+void launch_residual_half(cudaStream_t s, bool real, const ColPlan& p, const double2* Ch, int nrow, double2* r,
+                          const double2* b, const double2* x, int npw, int ncol, const int* active, int nchunk,
+                          const double* part, double* sums, unsigned* cnt, double* out);
 
 // The fastest shape for nunit units on 1 / cta_div of the GPU (false: no
 // cluster size fits).

@@ -1456,15 +1456,19 @@ bool col_shape(const ColPlan& p, int kind, int N, int nproj, int nunit, int cta_
       }
       return t;
     };
+    // the projector rows (read twice an iteration) before the vectors (read
+    // and written once) where the rows are the larger traffic
+    const bool rows_first = 2 * nproj * sizeof(cpx<T>) > 9 * 4 * sizeof(T);
     int nsb = 0;
-    bool vec = true;
-    for (int pass = 0; pass < 2 && nsb == 0; ++pass) {
-      vec = pass == 0;
+    bool vec = false, c = false, v = false;
+    for (int pass = 0; pass < 4 && nsb == 0; ++pass) {
+      vec = pass == 0 || pass == (rows_first ? 2 : 1);
+      c = pass == 0 || pass == (rows_first ? 1 : 2);
       for (int n = 1; n <= nzl; ++n)
-        if (fits(n, vec, false) && (nsb == 0 || rounds_of(n) < rounds_of(nsb))) nsb = n;
+        if (fits(n, vec, c) && (nsb == 0 || rounds_of(n) < rounds_of(nsb))) nsb = n;
     }
     if (nsb == 0) continue;
-    const bool c = fits(nsb, vec, true), v = fits(nsb, vec, c, true);
+    v = fits(nsb, vec, c, true);
     fits(nsb, vec, c, v);
     s.vec_elems = vec ? 0 : 16 * (size_t)p.nh;
     const int act = col::active_clusters<T>(kind, lq, s.smem);

@@ -63,8 +63,10 @@ struct gw_ctx {
   unsigned long long wait_limit = 1ull << 24;   // spins of one device wait before GW_E_TIMEOUT
   long long pcg_iters = 0;      // iterations run by persistent launches
   int pcg_launch_blocks = 0;
-  int* pcg_pin = nullptr;       // pinned read-back of the last persistent launch: iterations, flags, error
-  size_t pcg_pin_n = 0;
+  double* sv_pin = nullptr;     // pinned read-back of a refinement pass ("sv_out")
+  size_t sv_pin_n = 0;
+  int *pcg_iters_d = nullptr, *pcg_flags_d = nullptr;   // in "sv_out": iterations and flags of a one-launch pass
+  unsigned* pcg_err = nullptr;  // pinned error word of the last persistent launch
   struct PcgPending {           // that launch, until the caller's next synchronisation (pcg_finish)
     bool on = false;
     int ncol = 0, used = 0, tune_tpb = 0;
@@ -319,11 +321,11 @@ gw_status sqrtv(gw_ctx* ctx, const T* in, int nb, T* out, const T* sub) {
 }
 
 // ---------------------------------------------------------------------------
-// H applied to FP64 sphere vectors with shift: out = P_c? (H - E) x
+// H applied to FP64 sphere vectors with shift: out = (H - E) x, or sub - (H - E) x
 // ---------------------------------------------------------------------------
 template <typename T>
 gw_status h_apply(gw_ctx* ctx, cpx<T>* x, int ncol, const double2* E, const int* active, cpx<T>* out,
-                  const GatherDots* dots = nullptr) {
+                  const GatherDots* dots = nullptr, const cpx<T>* sub = nullptr) {
   cpx<T>* grid;
   TRY(getbuf(ctx, std::string("g_h") + tname<T>(), (size_t)ncol * ctx->N3, &grid));
   auto& P = prec_of<T>(ctx);
@@ -334,16 +336,17 @@ gw_status h_apply(gw_ctx* ctx, cpx<T>* x, int ncol, const double2* E, const int*
   launch_xpass_mul<T>(ctx->st, 1, 1, 1, g, P, ctx->plan, grid, P.vloc_s, active, ncol);
   launch_ypass<T>(ctx->st, 0, 0, 1, g, P, ctx->plan, grid, active, ncol, 0);
   launch_zpass<T>(ctx->st, Z_GATHER_FWD_H, g, P, ctx->plan, grid, out, nullptr, nullptr, x, E, active, nullptr,
-                  nullptr, ncol, dots);
+                  nullptr, ncol, dots, nullptr, 1, sub);
   return launch_check(ctx, "h_apply");
 }
 
 // (H - E) x in FP64 for columns that are real in real space, two per complex
 // transform (pack, the pruned passes, split through G and -G with the kinetic
 // part added); act: host mask of the columns wanted (a pair runs when one of
-// its columns is wanted, and both of its outputs are written).
+// its columns is wanted, and both of its outputs are written); with sub, sub -
+// (H - E) x.
 gw_status h_apply_sym(gw_ctx* ctx, const double2* x, int ncol, const double2* E, const std::vector<int>& act,
-                      double2* out) {
+                      double2* out, const double2* sub = nullptr) {
   const int npw = ctx->npw, npair = (ncol + 1) / 2;
   std::vector<int> ia(npair), ib(npair), pact(npair);
   for (int j = 0; j < npair; ++j) {
@@ -369,8 +372,24 @@ gw_status h_apply_sym(gw_ctx* ctx, const double2* x, int ncol, const double2* E,
   launch_ypass<double>(ctx->st, 0, 0, 1, g, P, ctx->plan, grid, dpact, npair, 0);
   launch_zpass<double>(ctx->st, Z_GATHER_FWD, g, P, ctx->plan, grid, yp, nullptr, nullptr, nullptr, nullptr, dpact,
                        nullptr, nullptr, npair);
-  launch_unpack_pairs(ctx->st, npw, npair, yp, g.sph_neg, dia, dib, dpact, P.kin, E, x, out);
+  launch_unpack_pairs(ctx->st, npw, npair, yp, g.sph_neg, dia, dib, dpact, P.kin, E, x, out, sub);
   return launch_check(ctx, "h_apply_sym");
+}
+
+// y = P_c y for FP64 columns (real: real in real space), on half the sphere
+// where the tables are there.
+gw_status proj64(gw_ctx* ctx, double2* Y, int ncol, bool real) {
+  if (ncol == 0 || ctx->nocc == 0) return GW_OK;
+  const ColPlan& p = ctx->col;
+  if (!p.half) {
+    launch_proj<double>(ctx->st, ctx->P64.C, ctx->nocc, ctx->npw, Y, ncol, nullptr, ctx->work, nullptr, nullptr, real);
+    return GW_OK;
+  }
+  double* part;
+  TRY(getbuf(ctx, "ph_part", half_part_elems(ctx->nocc, p.nh, ncol), &part));
+  const int n = launch_gram_half(ctx->st, real, p, ctx->col64.Ch, ctx->nocc, Y, ctx->npw, ncol, nullptr, part);
+  launch_proj_half(ctx->st, real, p, ctx->col64.Ch, ctx->nocc, Y, ctx->npw, ncol, nullptr, n, part);
+  return GW_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -488,21 +507,14 @@ gw_status cg_solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, 
   return GW_OK;
 }
 
-// Iteration counts, flags and the error word (if any) of a one-launch pass
-// come back into pinned memory and are read at the caller's next
-// synchronisation (pcg_finish): no stream synchronisation of its own per pass.
-gw_status pcg_read_back(gw_ctx* ctx, int ncol, const int* iters, const int* flags, const unsigned* ctl) {
-  if (ctx->pcg_pin_n < (size_t)(2 * ncol + 1)) {
-    if (ctx->pcg_pin) CK(cudaFreeHost(ctx->pcg_pin));
-    ctx->pcg_pin = nullptr;
-    ctx->pcg_pin_n = 0;
-    CK(cudaMallocHost(&ctx->pcg_pin, (size_t)(2 * ncol + 1) * sizeof(int)));
-    ctx->pcg_pin_n = (size_t)(2 * ncol + 1);
-  }
-  CK(cudaMemcpyAsync(ctx->pcg_pin, iters, ncol * sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-  CK(cudaMemcpyAsync(ctx->pcg_pin + ncol, flags, ncol * sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-  ctx->pcg_pin[2 * ncol] = 0;
-  if (ctl) CK(cudaMemcpyAsync(ctx->pcg_pin + 2 * ncol, ctl + 2, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->st));
+// A one-launch pass leaves its iteration counts and flags beside the norms of
+// the refinement (pcg_iters_d, pcg_flags_d in "sv_out"), which the caller
+// copies to sv_pin and reads after its own synchronisation (pcg_finish); the
+// error word of the task queue goes to pcg_err.
+gw_status pcg_pending(gw_ctx* ctx, int ncol, const unsigned* ctl) {
+  if (!ctx->pcg_err) CK(cudaMallocHost(&ctx->pcg_err, sizeof(unsigned)));
+  *ctx->pcg_err = 0;
+  if (ctl) CK(cudaMemcpyAsync(ctx->pcg_err, ctl + 2, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->st));
   ctx->pcg_pend.on = true;
   ctx->pcg_pend.ncol = ncol;
   return GW_OK;
@@ -535,12 +547,12 @@ gw_status col_solve(gw_ctx* ctx, int kind, int ncol, const double2* b64, const d
   a.tol2 = tol * tol;
   a.vecs = nullptr;
   if (a.sh.vec_elems) TRY(getbuf(ctx, "col_vecs" + t, a.sh.vec_elems * (size_t)a.nunit, &a.vecs));
-  TRY(getbuf(ctx, "pcg_iters", ncol, &a.iters));
-  TRY(getbuf(ctx, "pcg_flags", ncol, &a.flags));
+  a.iters = ctx->pcg_iters_d;
+  a.flags = ctx->pcg_flags_d;
   const int pa = prof_begin(ctx, kind == COL_CG_PAIR ? PC_PCG : PC_N);
   CK(launch_col_solve<T>(ctx->st, kind, a));
   prof_end(ctx, PC_PCG, pa);
-  TRY(pcg_read_back(ctx, ncol, a.iters, a.flags, nullptr));
+  TRY(pcg_pending(ctx, ncol, nullptr));
   ctx->pcg_pend.used = a.nunit << a.sh.lq;
   ctx->pcg_pend.fp64 = std::is_same<T, double>::value;
   ctx->pcg_pend.qmr = kind != COL_CG_PAIR;
@@ -566,11 +578,9 @@ gw_status cg_solve_persistent(gw_ctx* ctx, int ncol, const double2* b64, const d
   const int npw = ctx->npw;
   const std::string t = tname<T>();
   *ran = true;
-  int *iters, *flags;
+  int *iters = ctx->pcg_iters_d, *flags = ctx->pcg_flags_d;
   double* rr_out;
   TRY(getbuf(ctx, "pcg_rr", ncol, &rr_out));
-  TRY(getbuf(ctx, "pcg_iters", ncol, &iters));
-  TRY(getbuf(ctx, "pcg_flags", ncol, &flags));
   int used = 0;
   const int pa = prof_begin(ctx, PC_PCG);
   unsigned* ctl = nullptr;
@@ -631,7 +641,7 @@ gw_status cg_solve_persistent(gw_ctx* ctx, int ncol, const double2* b64, const d
   }
   CK(le);
   prof_end(ctx, PC_PCG, pa);
-  TRY(pcg_read_back(ctx, ncol, iters, flags, ctl));
+  TRY(pcg_pending(ctx, ncol, ctl));
   ctx->pcg_pend.used = used;
   ctx->pcg_pend.fp64 = std::is_same<T, double>::value;
   ctx->pcg_pend.qmr = false;
@@ -649,9 +659,9 @@ gw_status pcg_finish(gw_ctx* ctx, long long* it_sum, int* it_max) {
   if (!ctx->pcg_pend.on) return GW_OK;
   ctx->pcg_pend.on = false;
   const int ncol = ctx->pcg_pend.ncol;
-  const int* its = ctx->pcg_pin;
-  const int* fl = ctx->pcg_pin + ncol;
-  if (ctx->pcg_pin[2 * ncol]) return fail(ctx, GW_E_TIMEOUT, "persistent CG: a bounded device wait gave up");
+  const int* its = reinterpret_cast<const int*>(ctx->sv_pin + 3 * (size_t)ncol);
+  const int* fl = its + ncol;
+  if (*ctx->pcg_err) return fail(ctx, GW_E_TIMEOUT, "persistent CG: a bounded device wait gave up");
   int imax = 0;
   for (int c = 0; c < ncol; ++c) {
     *it_sum += its[c];
@@ -855,20 +865,38 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
   ctx->pcg_pend.on = false;
   const double tol = mixed ? ctx->tol_mixed : ctx->tol;
   const double tol_in = mixed ? ctx->tol_inner : std::max(1e2 * ctx->tol, 1e-11);
-  double2 *r64, *ax;
+  double2 *r64, *ax = nullptr;
   cpx<T>* d;
   int* oact;
   double *res2, *bb, *xx, *rra;
   TRY(getbuf(ctx, "sv_r64", (size_t)ncol * npw, &r64));
-  TRY(getbuf(ctx, "sv_ax", (size_t)ncol * npw, &ax));
   TRY(getbuf(ctx, std::string("sv_d") + tname<T>(), (size_t)ncol * npw, &d));
   TRY(getbuf(ctx, "sv_oact", ncol, &oact));
-  TRY(getbuf(ctx, "sv_res2", ncol, &res2));
-  TRY(getbuf(ctx, "sv_bb", ncol, &bb));
-  TRY(getbuf(ctx, "sv_xx", ncol, &xx));
-  double2 *cb, *cax;
-  TRY(getbuf(ctx, "sv_cb", (size_t)ctx->nocc * ncol, &cb));
-  TRY(getbuf(ctx, "sv_cax", (size_t)ctx->nocc * ncol, &cax));
+  // what the host reads after a pass, in one copy: |r|^2, |b|^2, |x|^2, then
+  // the iteration counts and flags of a one-launch inner pass
+  TRY(getbuf(ctx, "sv_out", (size_t)4 * ncol, &res2));
+  bb = res2 + ncol;
+  xx = bb + ncol;
+  ctx->pcg_iters_d = reinterpret_cast<int*>(xx + ncol);
+  ctx->pcg_flags_d = ctx->pcg_iters_d + ncol;
+  if (ctx->sv_pin_n < (size_t)4 * ncol) {
+    if (ctx->sv_pin) CK(cudaFreeHost(ctx->sv_pin));
+    ctx->sv_pin = nullptr;
+    ctx->sv_pin_n = 0;
+    CK(cudaMallocHost(&ctx->sv_pin, (size_t)4 * ncol * sizeof(double)));
+    ctx->sv_pin_n = (size_t)4 * ncol;
+  }
+  const bool half = ctx->col.half && !w2;      // residual and projector on half the sphere
+  double2 *cb = nullptr, *cax = nullptr;
+  double *part = nullptr, *sums = nullptr;
+  if (half) {
+    TRY(getbuf(ctx, "ph_part", half_part_elems(ctx->nocc, ctx->col.nh, ncol), &part));
+    TRY(getbuf(ctx, "ph_sums", half_sum_elems(ctx->col.nh, ncol), &sums));
+  } else {
+    TRY(getbuf(ctx, "sv_ax", (size_t)ncol * npw, &ax));
+    TRY(getbuf(ctx, "sv_cb", (size_t)ctx->nocc * ncol, &cb));
+    TRY(getbuf(ctx, "sv_cax", (size_t)ctx->nocc * ncol, &cax));
+  }
   TRY(ensure_work(ctx, ncol));
   double2* cdef = nullptr;
   double* edef = nullptr;
@@ -897,7 +925,7 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
     for (int c = 0; c < ncol; ++c) sym = sym && (hs[c] <= 1e-12 * hs[ncol + c]);
   }
   // C^H b (real coefficients for real-in-real-space columns: the occupied rows are too)
-  launch_gram<double>(ctx->st, ctx->P64.C, ctx->nocc, npw, b64, ncol, ctx->work, cb, sym);
+  if (!half) launch_gram<double>(ctx->st, ctx->P64.C, ctx->nocc, npw, b64, ncol, ctx->work, cb, sym);
   std::vector<int> act(ncol, 1);
   TRY(upload(ctx, "sv_oact", act, &oact));
   std::vector<double> hr(ncol, 0.0), hb(ncol, 0.0), hx(ncol, 0.0), habs(ncol, 0.0);
@@ -956,6 +984,17 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
       launch_sq_shift<double>(ctx->st, npw, ncol, ax, x64, w2, oact, ctx->work, nullptr);
       launch_gram<double>(ctx->st, ctx->P64.C, ctx->nocc, npw, ax, ncol, ctx->work, cax);
       prof_end(ctx, PC_REFINE, pa);
+    } else if (half) {
+      // r64 = b - (H - E) x in the last transform pass (two real columns per
+      // transform), then P_c and the norms
+      const int pa = prof_begin(ctx, PC_REFINE);
+      if (sym) TRY(h_apply_sym(ctx, x64, ncol, E, act, r64, b64));
+      else TRY(h_apply<double>(ctx, x64, ncol, E, oact, r64, nullptr, b64));
+      const double2* Ch = ctx->col64.Ch;
+      const int n = launch_gram_half(ctx->st, sym, ctx->col, Ch, ctx->nocc, r64, npw, ncol, oact, part);
+      launch_residual_half(ctx->st, sym, ctx->col, Ch, ctx->nocc, r64, b64, x64, npw, ncol, oact, n, part, sums,
+                           ctx->work.cnt_b, res2);
+      prof_end(ctx, PC_REFINE, pa);
     } else {
       const int pa = prof_begin(ctx, PC_REFINE);
       if (sym) {
@@ -974,13 +1013,19 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
       }
       prof_end(ctx, PC_REFINE, pa);
     }
-    launch_residual(ctx->st, npw, ncol, b64, ax, x64, oact, ctx->work, res2, bb, xx, ctx->P64.C, ctx->nocc, cb,
-                    cax, sym && !w2);
-    CK(cudaMemcpyAsync(r64, ax, (size_t)ncol * npw * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->st));
-    CK(cudaMemcpyAsync(hr.data(), res2, ncol * sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
-    CK(cudaMemcpyAsync(hb.data(), bb, ncol * sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
-    CK(cudaMemcpyAsync(hx.data(), xx, ncol * sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
+    if (!half) {
+      launch_residual(ctx->st, npw, ncol, b64, ax, x64, oact, ctx->work, res2, bb, xx, ctx->P64.C, ctx->nocc, cb,
+                      cax, sym && !w2);
+      CK(cudaMemcpyAsync(r64, ax, (size_t)ncol * npw * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->st));
+    }
+    CK(cudaMemcpyAsync(ctx->sv_pin, res2, (size_t)4 * ncol * sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
     TRY(sync(ctx, "solve"));
+    for (int c = 0; c < ncol; ++c) {
+      if (!act[c]) continue;                   // a column that has converged keeps its last norms
+      hr[c] = ctx->sv_pin[c];
+      hb[c] = ctx->sv_pin[ncol + c];
+      hx[c] = ctx->sv_pin[2 * ncol + c];
+    }
     TRY(pcg_finish(ctx, &it_sum, &it_max));
     if (hprev.empty()) hprev = hb;
     int nact = 0;
@@ -1017,7 +1062,7 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
   // The solution lies in P_c.  Inner passes in FP32 leave valence components
   // at the FP32 rounding level that the residual cannot see (P_c removes them
   // from A x) but the density reduction would: project them out in FP64.
-  launch_proj<double>(ctx->st, ctx->P64.C, ctx->nocc, npw, x64, ncol, nullptr, ctx->work, nullptr, nullptr, sym);
+  TRY(proj64(ctx, x64, ncol, sym));
   {
     double fin = 0.0;        // final relative FP64 residual |b - A x| / |b| over all columns
     for (int c = 0; c < ncol; ++c) fin = std::max(fin, hb[c] > 0 ? std::sqrt(hr[c] / hb[c]) : 0.0);
@@ -1122,89 +1167,62 @@ gw_status rhs_core(gw_ctx* ctx, const void* y, bool y_cplx, int nb, double2** ou
   // P_c once: psi_v* y has a large component along the occupied states (e.g.
   // <psi_v|y psi_v>) and one pass leaves |C C^H - 1| times it behind; the
   // solver's FP64 residual P_c (b - A x) removes that remnant
-  launch_proj<double>(ctx->st, ctx->P64.C, nocc, npw, rhs64, nr, nullptr, ctx->work, nullptr, nullptr, !y_cplx);
+  TRY(proj64(ctx, rhs64, nr, !y_cplx));
   *out = rhs64;
   return launch_check(ctx, "rhs");
 }
 
 // ---------------------------------------------------------------------------
-// The model operator (Sec. Dielectric model, Eq. model_eq), every step in
-// precision T: H -> T in Eq. P2a turns each Sternheimer solve into one
-// division by the kinetic denominators,
+// The model operator (Sec. Dielectric model, Eq. model_eq) in FP64: H -> T in
+// Eq. P2a turns each Sternheimer solve into one division by the kinetic
+// denominators,
 //   rhs_{b,v}  = P_c Sphere(FFT(conj(u_v) y_b))
 //   sol_{o,b,v} = P_c [ (pinv(|G|^2/2 - e_v - w_o) + pinv(|G|^2/2 - e_v + w_o)) rhs_{b,v} ]
 //   dn_{o,b}   = -(2/Omega) sum_v u_v IFFT(sol_{o,b,v})
 // (the two signs summed before the second projector, which is linear).
-// y: [nb][N_g] real or complex (interleaved) in T; dn: [nom][nb][N_g] in T.
+// y: [nb][N_g] real or complex (interleaved); dn: [nom][nb][N_g].  Real fields
+// share transforms in pairs on both ends (rhs_core, chi0_reduce): 48^3, 16
+// states 655 -> 430 us an application.
 // ---------------------------------------------------------------------------
-template <typename T>
-gw_status chi0_model_core(gw_ctx* ctx, const T* y, bool y_cplx, int nb, const std::vector<double2>& omega, T* dn,
-                          bool dn_cplx) {
+gw_status chi0_model_core(gw_ctx* ctx, const double* y, bool y_cplx, int nb, const std::vector<double2>& omega,
+                          double* dn, bool dn_cplx) {
   const int npw = ctx->npw, nocc = ctx->nocc;
   const int nom = (int)omega.size();
   const int nr = nocc * nb, nsol = nom * nr;
-  auto& P = prec_of<T>(ctx);
-  const Geometry& g = ctx->geo;
-  const std::string t = tname<T>();
-  std::vector<int> ca(nr), cy(nr), src(nsol), gstart(nom * nb + 1), colv(nsol);
+  std::vector<int> src(nsol);
   std::vector<double2> Em(nsol), Ep(nsol);
-  for (int b = 0; b < nb; ++b)
-    for (int v = 0; v < nocc; ++v) { ca[b * nocc + v] = v; cy[b * nocc + v] = b; }
   for (int o = 0; o < nom; ++o)
     for (int b = 0; b < nb; ++b)
       for (int v = 0; v < nocc; ++v) {
         const int j = (o * nb + b) * nocc + v;
         src[j] = b * nocc + v;
-        colv[j] = v;
         Em[j] = make_double2(ctx->eps[v] + omega[o].x, omega[o].y);     // T - e_v - w
         Ep[j] = make_double2(ctx->eps[v] - omega[o].x, -omega[o].y);    // T - e_v + w
       }
-  for (int j = 0; j <= nom * nb; ++j) gstart[j] = j * nocc;
-  int *dca, *dcy, *dsrc, *dgs, *dcv;
-  double2 *dEm, *dEp;
-  TRY(upload_table(ctx, "mod_ca", ca, &dca));
-  TRY(upload_table(ctx, "mod_cy", cy, &dcy));
+  int* dsrc;
+  double2 *dEm, *dEp, *rhs, *sol;
   TRY(upload_table(ctx, "mod_src", src, &dsrc));
   TRY(upload_table(ctx, "mod_em", Em, &dEm));
   TRY(upload_table(ctx, "mod_ep", Ep, &dEp));
-  TRY(upload_table(ctx, "mod_gs", gstart, &dgs));
-  TRY(upload_table(ctx, "mod_cv", colv, &dcv));
-  cpx<T> *grid, *rhs, *sol;
-  TRY(getbuf(ctx, "mod_grid" + t, (size_t)std::max(nr, nsol) * ctx->N3, &grid));
-  TRY(getbuf(ctx, "mod_rhs" + t, (size_t)nr * npw, &rhs));
-  TRY(getbuf(ctx, "mod_sol" + t, (size_t)nsol * npw, &sol));
+  TRY(getbuf(ctx, "mod_sol", (size_t)nsol * npw, &sol));
   TRY(ensure_work(ctx, std::max(nsol, 1)));
-  launch_xpass_prod_fwd<T>(ctx->st, g, P, ctx->plan, reinterpret_cast<const cpx<T>*>(y), y_cplx ? 1 : 0, P.U, 0,
-                           1, dca, dcy, grid, nr);
-  launch_ypass<T>(ctx->st, 0, 0, 1, g, P, ctx->plan, grid, nullptr, nr, 0);
-  launch_zpass<T>(ctx->st, Z_GATHER_FWD, g, P, ctx->plan, grid, rhs, nullptr, nullptr, nullptr, nullptr, nullptr,
-                  nullptr, nullptr, nr);
-  // real fields and realified states: real-in-real-space right-hand sides and,
-  // at real frequencies (denominators even in G), solutions: real coefficients
+  TRY(rhs_core(ctx, y, y_cplx, nb, &rhs));
+  launch_model_scale<double>(ctx->st, npw, nsol, ctx->P64.kin, rhs, dsrc, dEm, dEp, sol);
+  // real fields and realified states at real frequencies (denominators even in
+  // G): solutions real in real space
   bool real_w = !y_cplx;
   for (const double2& w : omega) real_w = real_w && w.y == 0.0;
-  launch_proj<T>(ctx->st, P.C, nocc, npw, rhs, nr, nullptr, ctx->work, nullptr, nullptr, !y_cplx);
-  launch_model_scale<T>(ctx->st, npw, nsol, P.kin, rhs, dsrc, dEm, dEp, sol);
-  launch_proj<T>(ctx->st, P.C, nocc, npw, sol, nsol, nullptr, ctx->work, nullptr, nullptr, real_w);
-  launch_zpass<T>(ctx->st, Z_SCATTER_INV, g, P, ctx->plan, grid, sol, nullptr, nullptr, nullptr, nullptr, nullptr,
-                  nullptr, nullptr, nsol);
-  launch_ypass<T>(ctx->st, 1, 1, 0, g, P, ctx->plan, grid, nullptr, nsol, 0);
-  cpx<T>* parts;
-  const size_t nparts = (size_t)kMaxReduceParts * ctx->N3;   // enough whenever a split pays (few groups)
-  TRY(getbuf(ctx, "mod_parts" + t, nparts, &parts));
-  launch_xpass_inv_reduce<T>(ctx->st, g, P, ctx->plan, grid, dgs, dcv, nom * nb, -2.0 / ctx->vol,
-                             dn_cplx ? nullptr : dn, dn_cplx ? reinterpret_cast<cpx<T>*>(dn) : nullptr, 0, parts,
-                             nparts, nocc);
+  TRY(proj64(ctx, sol, nsol, real_w));
   for (int i = 0; i < 6; ++i) ctx->stats[i] = 0;
-  return launch_check(ctx, "chi0 model");
+  return chi0_reduce(ctx, sol, nb, nom, dn, dn_cplx);
 }
 
 template <typename S>
 gw_status chi0_core(gw_ctx* ctx, const void* y, bool y_cplx, int nb, const std::vector<double2>& omega, void* dn,
                     bool dn_cplx) {
   if (ctx->op == GW_OP_MODEL)
-    return chi0_model_core<double>(ctx, reinterpret_cast<const double*>(y), y_cplx, nb, omega,
-                                   reinterpret_cast<double*>(dn), dn_cplx);
+    return chi0_model_core(ctx, reinterpret_cast<const double*>(y), y_cplx, nb, omega, reinterpret_cast<double*>(dn),
+                           dn_cplx);
   const int npw = ctx->npw, nocc = ctx->nocc;
   const int nom = (int)omega.size();
   double2* rhs64;
@@ -1228,7 +1246,10 @@ gw_status chi0_core(gw_ctx* ctx, const void* y, bool y_cplx, int nb, const std::
       if (squared(o) != (pass == 1)) continue;
       const bool zero = (omega[o].x == 0.0 && omega[o].y == 0.0);
       if (pass == 0) qmr |= !zero;
-      const int ns = (zero || pass == 1) ? 1 : 2;
+      // real fields at omega = i w: H and b are real in real space, so x^+ is the
+      // complex conjugate of x^- there, c^+(G) = conj c^-(-G): one solve
+      const bool mirror = pass == 0 && !zero && omega[o].x == 0.0 && !y_cplx && dn_cplx;
+      const int ns = (zero || pass == 1 || mirror) ? 1 : 2;
       for (int b = 0; b < nb; ++b)
         for (int v = 0; v < nocc; ++v) {
           const int k = (o * nb + b) * nocc + v;
@@ -1245,7 +1266,7 @@ gw_status chi0_core(gw_ctx* ctx, const void* y, bool y_cplx, int nb, const std::
             }
           }
           s0[k] = first;
-          s1[k] = ns == 2 ? first + 1 : -1;
+          s1[k] = ns == 2 ? first + 1 : mirror ? -2 : -1;
         }
     }
     if (pass == 0) nstd = (int)src.size();
@@ -1299,13 +1320,13 @@ gw_status chi0_core(gw_ctx* ctx, const void* y, bool y_cplx, int nb, const std::
     TRY(getbuf(ctx, "sq_hb", (size_t)nsq * npw, &hb));
     TRY(upload(ctx, "sq_w2", w2v, &dw2));
     TRY(h_apply<double>(ctx, bs, nsq, dE + nstd, nullptr, hb, nullptr));
-    launch_proj<double>(ctx->st, ctx->P64.C, nocc, npw, hb, nsq, nullptr, ctx->work, nullptr, nullptr);
+    TRY(proj64(ctx, hb, nsq, false));
     CK(cudaMemcpyAsync(bs, hb, (size_t)nsq * npw * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->st));
     SOFT(sv, (solve<S>(ctx, nsq, bs, dE + nstd, xcol + (size_t)nstd * npw, false, dtk ? dtk + nstd : nullptr, dw2,
                        w2max)));
   }
   // -- combine: x^- + x^+, or 2 x at omega = 0 (x^- = x^+) and on the squared route
-  launch_combine(ctx->st, npw, nsol, xcol, ds0, ds1, 1.0, 2.0, sol64);
+  launch_combine(ctx->st, npw, nsol, xcol, ds0, ds1, 1.0, 2.0, sol64, ctx->geo.sph_neg);
   TRY(chi0_reduce(ctx, sol64, nb, nom, dn, dn_cplx));
   return sv;
 }
@@ -1448,7 +1469,10 @@ gw_status eps_core(gw_ctx* ctx, const void* x, bool x_cplx, int nb, const std::v
     TRY(launch_check(ctx, "eps out"));
     return sv;
   }
-  // complex pipeline: promote a real input
+  // complex pipeline; a real field stays real up to the solves (its right-hand
+  // sides share transforms in pairs, and at i w one solve gives both signs)
+  double2* outr = reinterpret_cast<double2*>(out);
+  if (!x_cplx && chi0_only) return chi0_core<S>(ctx, x, false, nb, omega, outr, true);
   const double2* xc = reinterpret_cast<const double2*>(x);
   if (!x_cplx) {
     double2* tmp;
@@ -1464,9 +1488,11 @@ gw_status eps_core(gw_ctx* ctx, const void* x, bool x_cplx, int nb, const std::v
   double2 *y, *dn;
   TRY(getbuf(ctx, "eps_yc", (size_t)nb * N3, &y));
   TRY(getbuf(ctx, "eps_dnc", (size_t)nom * nb * N3, &dn));
-  TRY(sqrtv_c(ctx, xc, nb, y, nullptr));
+  const bool real_y = !x_cplx;
+  if (real_y) TRY(sqrtv<double>(ctx, reinterpret_cast<const double*>(x), nb, reinterpret_cast<double*>(y), nullptr));
+  else TRY(sqrtv_c(ctx, xc, nb, y, nullptr));
   gw_status sv = GW_OK;
-  SOFT(sv, (chi0_core<S>(ctx, y, true, nb, omega, dn, true)));
+  SOFT(sv, (chi0_core<S>(ctx, y, !real_y, nb, omega, dn, true)));
   for (int k = 0; k < nom; ++k)
     TRY(sqrtv_c(ctx, dn + (size_t)k * nb * N3, nb, outc + (size_t)k * nb * N3, xc));
   TRY(launch_check(ctx, "eps out"));
@@ -1821,8 +1847,8 @@ gw_status grad_from_basis(gw_ctx* ctx, const double* phi, const double* Q, const
                          nullptr, nullptr, nullptr, nocc);
   };
   sphere_of_product(P.U, 0, rhs);
-  launch_proj<double>(ctx->st, P.C, nocc, npw, rhs, nocc, nullptr, ctx->work, nullptr, nullptr);
-  launch_proj<double>(ctx->st, P.C, nocc, npw, rhs, nocc, nullptr, ctx->work, nullptr, nullptr);
+  TRY(proj64(ctx, rhs, nocc, false));
+  TRY(proj64(ctx, rhs, nocc, false));
   TRY(launch_check(ctx, "grad rhs"));
   TRY(solve<S>(ctx, nocc, rhs, dE, dC, false, dtk));
   // dC = -x  (dpsi coefficients); dU_v = IFFT(dC_v) on the grid
@@ -1859,8 +1885,8 @@ gw_status grad_from_basis(gw_ctx* ctx, const double* phi, const double* Q, const
                          nullptr, nullptr, nullptr, nocc);
     // eta_v -= sum_v' dC_v' W[v'][v]: the projector update with C := dC and coef[v' * ncol + v] = W[v'][v]
     launch_proj_update<double>(ctx->st, dC, nocc, npw, eta, nocc, nullptr, Wm, ctx->work, nullptr, nullptr);
-    launch_proj<double>(ctx->st, P.C, nocc, npw, eta, nocc, nullptr, ctx->work, nullptr, nullptr);
-    launch_proj<double>(ctx->st, P.C, nocc, npw, eta, nocc, nullptr, ctx->work, nullptr, nullptr);
+    TRY(proj64(ctx, eta, nocc, false));
+    TRY(proj64(ctx, eta, nocc, false));
   }
   TRY(launch_check(ctx, "grad eta"));
   TRY(solve<S>(ctx, nocc, eta, dE, lam, false, dtk));
@@ -1888,8 +1914,7 @@ gw_status build_col_plan(gw_ctx* ctx, const std::vector<int4>& pencils, const st
                          const std::vector<uint8_t>& disc, size_t nplanes) {
   ColPlan& p = ctx->col;
   const int N = ctx->N;
-  p.ok = false;
-  if (!col_radices(N, &p.N1, &p.N2)) return GW_OK;
+  p.half = p.ok = false;
   p.P = (int)nplanes;
   p.nm = p.P / 2;
   auto plane = [&](int i0) { return i0 <= p.nm ? i0 : i0 - (N - p.P); };
@@ -1934,6 +1959,10 @@ gw_status build_col_plan(gw_ctx* ctx, const std::vector<int4>& pencils, const st
   }
   p.nh = (int)gp.size();
   if (2 * p.nh - 1 != ctx->npw || gp[0] != gm[0]) return GW_OK;
+  TRY(upload(ctx, "col_gp", gp, &p.gp));
+  TRY(upload(ctx, "col_gm", gm, &p.gm));
+  p.half = true;
+  if (!col_radices(N, &p.N1, &p.N2)) return GW_OK;
   // equal shares of entries (solver vectors, projector) and pencils (transforms)
   std::vector<int> split(kColNQ * (kColMaxQ + 1), p.npair);
   auto cost = [&](int j) { return (long)hstart[j] + (long)j * N / 8; };
@@ -1956,8 +1985,6 @@ gw_status build_col_plan(gw_ctx* ctx, const std::vector<int4>& pencils, const st
   }
   TRY(upload(ctx, "col_split", split, &p.split));
   TRY(upload(ctx, "col_hstart", hstart, &p.hstart));
-  TRY(upload(ctx, "col_gp", gp, &p.gp));
-  TRY(upload(ctx, "col_gm", gm, &p.gm));
   TRY(upload(ctx, "col_hpos", hpos, &p.hpos));
   TRY(upload(ctx, "col_disc", dsc, &p.disc));
   TRY(upload(ctx, "col_zmax", zmax, &p.zmax));
@@ -2250,7 +2277,7 @@ gw_status upload_projector(gw_ctx* ctx, const std::vector<zc>& cdef) {
   }
   TRY(upload(ctx, "occ_C64", c64, &ctx->P64.C));
   TRY(upload(ctx, "occ_C32", c32, &ctx->P32.C));
-  if (ctx->col.ok) {
+  if (ctx->col.half) {
     const int r = (int)(n / ctx->npw);
     TRY(getbuf(ctx, "col_C64", (size_t)r * ctx->col.nh, &ctx->col64.Ch));
     TRY(getbuf(ctx, "col_C32", (size_t)r * ctx->col.nh, &ctx->col32.Ch));
@@ -2317,7 +2344,7 @@ gw_status recycle_core(gw_ctx* ctx, const double* F, int nl, const double* dw, i
   }
   TRY(h_apply<double>(ctx, bcp, nc, dE, nullptr, xc + (size_t)nc * npw));
   TRY(ensure_work(ctx, std::max(nx, nc)));
-  launch_proj<double>(ctx->st, P.C, nocc, npw, xc + (size_t)nc * npw, nc, nullptr, ctx->work, nullptr, nullptr);
+  TRY(proj64(ctx, xc + (size_t)nc * npw, nc, false));
   if (w0 > 0.0) {
     // x(i w0) = ((H - e_v)^2 + w0^2)^-1 (H - e_v) b (Eq. P2+), the right-hand
     // side being the high-frequency rows P_c (H - e_v) b just computed
@@ -2636,7 +2663,7 @@ gw_status sigma_c_core(gw_ctx* ctx, int e, double delta, double alpha, int nf, c
   TRY(getbuf(ctx, "sc_hp", (size_t)nl * npw, &hp));
   CK(cudaMemcpyAsync(bz, Z, (size_t)nl * npw * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->st));
   TRY(ensure_work(ctx, std::max(nl, 64)));
-  launch_proj<double>(ctx->st, ctx->P64.C, nocc, npw, bz, nl, nullptr, ctx->work, nullptr, nullptr);
+  TRY(proj64(ctx, bz, nl, false));
   std::vector<double2> Ea(nl, make_double2(c - alpha, 0.0));
   std::vector<double> tk(nl, ctx->tkin[e]);
   double2* dEa;
@@ -3529,7 +3556,8 @@ void gw_destroy(gw_ctx* ctx) {
     if (kv.second.first) cudaFree(kv.second.first);
   if (ctx->host_pin) cudaFreeHost(ctx->host_pin);
   if (ctx->stage) cudaFreeHost(ctx->stage);
-  if (ctx->pcg_pin) cudaFreeHost(ctx->pcg_pin);
+  if (ctx->sv_pin) cudaFreeHost(ctx->sv_pin);
+  if (ctx->pcg_err) cudaFreeHost(ctx->pcg_err);
   for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
   for (cudaEvent_t e : ctx->tune_ev)
     if (e) cudaEventDestroy(e);

@@ -741,11 +741,13 @@ void launch_pack_pairs(cudaStream_t s, int npw, int npair, const double2* x, con
 
 // The two parts of a packed transform Y_j = F(f_a) + i F(f_b) of real fields:
 //   out[ia[j]](G) = (Y_j(G) + conj Y_j(-G)) / 2,  out[ib[j]](G) = (Y_j(G) - conj Y_j(-G)) / 2i,
-// plus (kin(G) - E_c) x_c(G) when kin is given (the kinetic part of (H - E) x).
+// plus (kin(G) - E_c) x_c(G) when kin is given (the kinetic part of (H - E) x);
+// with sub given, sub - that (the residual b - (H - E) x).
 __global__ void k_unpack_pairs(size_t npw, const double2* __restrict__ Y, const int* __restrict__ neg,
                                const int* __restrict__ ia, const int* __restrict__ ib, const int* __restrict__ active,
                                const double* __restrict__ kin, const double2* __restrict__ E,
-                               const double2* __restrict__ x, double2* __restrict__ out) {
+                               const double2* __restrict__ x, double2* __restrict__ out,
+                               const double2* __restrict__ sub) {
   const int j = blockIdx.y;
   if (active && !active[j]) return;
   const int a = ia[j], b = ib[j];
@@ -766,6 +768,14 @@ __global__ void k_unpack_pairs(size_t npw, const double2* __restrict__ Y, const 
         o1.y += er * xb.y + ei * xb.x;
       }
     }
+    if (sub) {
+      const double2 s0 = sub[(size_t)a * npw + G];
+      o0 = make_double2(s0.x - o0.x, s0.y - o0.y);
+      if (b >= 0) {
+        const double2 s1 = sub[(size_t)b * npw + G];
+        o1 = make_double2(s1.x - o1.x, s1.y - o1.y);
+      }
+    }
     out[(size_t)a * npw + G] = o0;
     if (b >= 0) out[(size_t)b * npw + G] = o1;
   }
@@ -773,10 +783,10 @@ __global__ void k_unpack_pairs(size_t npw, const double2* __restrict__ Y, const 
 
 void launch_unpack_pairs(cudaStream_t s, int npw, int npair, const double2* Y, const int* neg, const int* ia,
                          const int* ib, const int* active, const double* kin, const double2* E, const double2* x,
-                         double2* out) {
+                         double2* out, const double2* sub) {
   dim3 g((npw + kLT - 1) / kLT, npair);
   ++g_launches;
-  k_unpack_pairs<<<g, kLT, 0, s>>>((size_t)npw, Y, neg, ia, ib, active, kin, E, x, out);
+  k_unpack_pairs<<<g, kLT, 0, s>>>((size_t)npw, Y, neg, ia, ib, active, kin, E, x, out, sub);
 }
 
 // out[c] = max_G |b(G) - conj b(-G)|, out[ncol + c] = max_G |b(G)| (one block per column)
@@ -906,9 +916,11 @@ void launch_defl_scale(cudaStream_t s, double2* coef, const double* eps, const d
 // ---------------------------------------------------------------------------
 // sphere-vector helpers
 // ---------------------------------------------------------------------------
-// out[j] = w_pair (in[src0[j]] + in[src1[j]])  or  w_single in[src0[j]] when src1[j] < 0
+// out[j] = w_pair (in[src0[j]] + in[src1[j]]),  w_single in[src0[j]] when src1[j] = -1,
+// and w_pair (in[src0[j]](G) + conj in[src0[j]](-G)) when src1[j] = -2
 __global__ void k_combine(int npw, const double2* __restrict__ in, const int* __restrict__ src0,
-                          const int* __restrict__ src1, double w_pair, double w_single, double2* __restrict__ out) {
+                          const int* __restrict__ src1, double w_pair, double w_single, double2* __restrict__ out,
+                          const int* __restrict__ neg) {
   const int j = blockIdx.y;
   const int a = src0[j], b = src1[j];
   for (int G = blockIdx.x * blockDim.x + threadIdx.x; G < npw; G += gridDim.x * blockDim.x) {
@@ -917,6 +929,10 @@ __global__ void k_combine(int npw, const double2* __restrict__ in, const int* __
       const double2 u = in[(size_t)b * npw + G];
       v.x = w_pair * (v.x + u.x);
       v.y = w_pair * (v.y + u.y);
+    } else if (b == -2) {
+      const double2 u = in[(size_t)a * npw + neg[G]];
+      v.x = w_pair * (v.x + u.x);
+      v.y = w_pair * (v.y - u.y);
     } else {
       v.x *= w_single;
       v.y *= w_single;
@@ -926,10 +942,10 @@ __global__ void k_combine(int npw, const double2* __restrict__ in, const int* __
 }
 
 void launch_combine(cudaStream_t s, int npw, int nout, const double2* in, const int* src0, const int* src1,
-                    double w_pair, double w_single, double2* out) {
+                    double w_pair, double w_single, double2* out, const int* neg) {
   dim3 g((npw + kLT - 1) / kLT, nout);
   ++g_launches;
-  k_combine<<<g, kLT, 0, s>>>(npw, in, src0, src1, w_pair, w_single, out);
+  k_combine<<<g, kLT, 0, s>>>(npw, in, src0, src1, w_pair, w_single, out, neg);
 }
 
 // Kinetic denominators of the model operator (Sec. Dielectric model, Eq.

@@ -104,7 +104,7 @@ void launch_pack_pairs(cudaStream_t s, int npw, int npair, const double2* x, con
                        const int* active, double2* out);
 void launch_unpack_pairs(cudaStream_t s, int npw, int npair, const double2* Y, const int* neg, const int* ia,
                          const int* ib, const int* active, const double* kin, const double2* E, const double2* x,
-                         double2* out);
+                         double2* out, const double2* sub = nullptr);
 // out[c] = max |b(G) - conj b(-G)|, out[ncol + c] = max |b(G)| per column
 void launch_sym_check(cudaStream_t s, int npw, int ncol, const double2* b, const int* neg, double* out);
 void launch_defl_scale(cudaStream_t s, double2* coef, const double* eps, const double2* E, int ndef, int ncol,
@@ -113,7 +113,7 @@ void launch_residual(cudaStream_t s, int npw, int ncol, const double2* b, double
                      const int* active, Work& w, double* res2, double* bb, double* xx, const double2* C = nullptr,
                      int nocc = 0, const double2* cb = nullptr, const double2* cax = nullptr, bool real = false);
 void launch_combine(cudaStream_t s, int npw, int nout, const double2* in, const int* src0, const int* src1,
-                    double w_pair, double w_single, double2* out);
+                    double w_pair, double w_single, double2* out, const int* neg = nullptr);
 // Eq. model_eq: out[j] = (pinv(T - Em_j) + pinv(T - Ep_j)) in[src_j] on the sphere
 template <typename T>
 void launch_model_scale(cudaStream_t s, int npw, int nout, const T* kin, const cpx<T>* in, const int* src,
