@@ -1571,23 +1571,22 @@ gw_status lanczos_core(gw_ctx* ctx, const double* x0, int K, const std::vector<d
   TRY(ensure_work(ctx, (size_t)width * (K + 1)));   // partial sums of the stacked length
   if (k0 == 0) {
     launch_dot(ctx->st, N3, x0, x0, wgt, 1, ctx->work, nrm);
-    launch_lz_axpy(ctx->st, N3, 2, nrm, const_cast<double*>(x0), nullptr, Q);
+    launch_lz_next(ctx->st, N3, nrm, x0, Q);
   }
   for (int k = k0; k < K; ++k) {
     double* qk = Q + (size_t)k * N3;
     TRY(eps_core<T>(ctx, qk, false, width, omega, w, false));
     if (done) *done = k + 1;
-    if (k > 0) launch_lz_axpy(ctx->st, N3, 0, beta + (k - 1), w, Q + (size_t)(k - 1) * N3, nullptr);
-    launch_dot(ctx->st, N3, qk, w, wgt, 0, ctx->work, alpha + k);
-    launch_lz_axpy(ctx->st, N3, 1, alpha + k, w, qk, nullptr);
-    for (int pass = 0; pass < 2; ++pass) {
-      launch_gemv_t(ctx->st, Q, N3, N3, w, wgt, k + 1, ctx->work, h);
-      launch_gemv_n(ctx->st, Q, N3, N3, h, k + 1, w);
-    }
+    // alpha; two Gram-Schmidt passes over all vectors, the first of w - alpha q_k; beta
+    launch_lz_alpha(ctx->st, N3, k > 0 ? beta + (k - 1) : nullptr, k > 0 ? Q + (size_t)(k - 1) * N3 : nullptr, w, qk,
+                    wgt, ctx->work, alpha + k);
+    launch_gemv_t(ctx->st, Q, N3, N3, w, wgt, k + 1, ctx->work, h, alpha + k, qk);
+    launch_gemv_n(ctx->st, Q, N3, N3, h, k + 1, w, alpha + k, qk);
+    launch_gemv_t(ctx->st, Q, N3, N3, w, wgt, k + 1, ctx->work, h);
+    launch_gemv_n(ctx->st, Q, N3, N3, h, k + 1, w, nullptr, nullptr, &ctx->work, wgt, k < K - 1 ? beta + k : nullptr);
     if (k == K - 1) break;
-    launch_dot(ctx->st, N3, w, w, wgt, 1, ctx->work, beta + k);
-    launch_lz_axpy(ctx->st, N3, 2, beta + k, w, nullptr, Q + (size_t)(k + 1) * N3);
-    double hb[2];
+    launch_lz_next(ctx->st, N3, beta + k, w, Q + (size_t)(k + 1) * N3);
+    double* hb = reinterpret_cast<double*>(ctx->host_pin);    // pinned: the copies queue like kernels
     CK(cudaMemcpyAsync(hb, beta + k, sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaMemcpyAsync(hb + 1, alpha + k, sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
     TRY(sync(ctx, "lanczos"));
@@ -1959,10 +1958,7 @@ gw_status build_col_plan(gw_ctx* ctx, const std::vector<int4>& pencils, const st
   }
   p.nh = (int)gp.size();
   if (2 * p.nh - 1 != ctx->npw || gp[0] != gm[0]) return GW_OK;
-  TRY(upload(ctx, "col_gp", gp, &p.gp));
-  TRY(upload(ctx, "col_gm", gm, &p.gm));
   p.half = true;
-  if (!col_radices(N, &p.N1, &p.N2)) return GW_OK;
   // equal shares of entries (solver vectors, projector) and pencils (transforms)
   std::vector<int> split(kColNQ * (kColMaxQ + 1), p.npair);
   auto cost = [&](int j) { return (long)hstart[j] + (long)j * N / 8; };
@@ -1983,12 +1979,29 @@ gw_status build_col_plan(gw_ctx* ctx, const std::vector<int4>& pencils, const st
       p.maxh[lq] = std::max(p.maxh[lq], hstart[s[r + 1]] - hstart[s[r]]);
     }
   }
-  TRY(upload(ctx, "col_split", split, &p.split));
-  TRY(upload(ctx, "col_hstart", hstart, &p.hstart));
-  TRY(upload(ctx, "col_hpos", hpos, &p.hpos));
-  TRY(upload(ctx, "col_disc", dsc, &p.disc));
-  TRY(upload(ctx, "col_zmax", zmax, &p.zmax));
-  p.ok = true;
+  // one allocation and one upload for all tables
+  std::vector<unsigned char> all;
+  auto put = [&](const void* v, size_t bytes) {
+    const size_t o = all.size();
+    all.resize((o + bytes + 255) & ~(size_t)255);
+    std::memcpy(all.data() + o, v, bytes);
+    return o;
+  };
+  const size_t o_gp = put(gp.data(), gp.size() * sizeof(int)), o_gm = put(gm.data(), gm.size() * sizeof(int)),
+               o_pos = put(hpos.data(), hpos.size() * sizeof(unsigned)),
+               o_sp = put(split.data(), split.size() * sizeof(int)),
+               o_hs = put(hstart.data(), hstart.size() * sizeof(int)),
+               o_ds = put(dsc.data(), dsc.size() * sizeof(unsigned short)), o_zm = put(zmax.data(), zmax.size());
+  unsigned char* d;
+  TRY(upload(ctx, "col_tables", all, &d));
+  p.gp = reinterpret_cast<int*>(d + o_gp);
+  p.gm = reinterpret_cast<int*>(d + o_gm);
+  p.hpos = reinterpret_cast<unsigned*>(d + o_pos);
+  p.split = reinterpret_cast<int*>(d + o_sp);
+  p.hstart = reinterpret_cast<int*>(d + o_hs);
+  p.disc = reinterpret_cast<unsigned short*>(d + o_ds);
+  p.zmax = d + o_zm;
+  p.ok = col_radices(N, &p.N1, &p.N2);
   return GW_OK;
 }
 
@@ -2108,8 +2121,8 @@ gw_status upload_prec(gw_ctx* ctx, const std::vector<double>& vloc, const std::v
   TRY(upload(ctx, "p_sqv" + t, sq, &P.sqv_s));
   if (ctx->col.ok) {
     auto& c = col_of<T>(ctx);
-    TRY(getbuf(ctx, "col_V" + t, (size_t)N3, &c.Vp));
-    TRY(getbuf(ctx, "col_kin" + t, (size_t)ctx->col.nh, &c.kin));
+    TRY(getbuf(ctx, "col_V" + t, (size_t)N3 + ctx->col.nh, &c.Vp));
+    c.kin = c.Vp + N3;
     CK(launch_col_permute<T>(ctx->st, ctx->col, N, ctx->npw, P.vloc_s, nullptr, 0, P.kin, c));
   }
   return GW_OK;

@@ -1057,67 +1057,113 @@ void launch_gather_rows(cudaStream_t s, int npw, int nout, const cpx<U>* in, con
 // ---------------------------------------------------------------------------
 // Lanczos vectors (real FP64 grid fields, weighted inner product)
 // ---------------------------------------------------------------------------
-// out[j] = wgt * sum_r Q[j][r] w[r], j < k; grid (nchunk, k)
+// Sum of n partial sums (stride apart) by the whole block: in thread 0.
+__device__ __forceinline__ double block_total(const double* p, int n, size_t stride) {
+  double t = 0.0;
+  for (int k = threadIdx.x; k < n; k += blockDim.x) t += p[(size_t)k * stride];
+  return block_sum(t);
+}
+
+// out[j] = wgt * sum_r Q[j][r] w'[r], j < k, with w' = w - alpha q (q given) or
+// w; grid (nchunk, k)
 __global__ void __launch_bounds__(kLT)
 k_gemv_t(const double* __restrict__ Q, size_t ld, int n, const double* __restrict__ w, double wgt,
-         double* __restrict__ partial, unsigned* __restrict__ cnt, double* __restrict__ out, int k) {
+         double* __restrict__ partial, unsigned* __restrict__ cnt, double* __restrict__ out, int k,
+         const double* __restrict__ alpha, const double* __restrict__ q) {
   const int j = blockIdx.y;
   const int g0 = blockIdx.x * kChunk, g1 = min(n, g0 + kChunk);
+  const double al = q ? *alpha : 0.0;
   double acc = 0.0;
-  for (int r = g0 + threadIdx.x; r < g1; r += blockDim.x) acc += Q[(size_t)j * ld + r] * w[r];
+  for (int r = g0 + threadIdx.x; r < g1; r += blockDim.x)
+    acc += Q[(size_t)j * ld + r] * (q ? w[r] - al * q[r] : w[r]);
   acc = block_sum(acc);
   if (threadIdx.x == 0) partial[(size_t)blockIdx.x * k + j] = acc;
   if (!last_block(&cnt[j], gridDim.x)) return;
-  if (threadIdx.x == 0) {
-    double s;
-    sum_records<1>(partial + j, gridDim.x, k, &s);
-    out[j] = wgt * s;
-  }
+  const double s = block_total(partial + j, gridDim.x, k);
+  if (threadIdx.x == 0) out[j] = wgt * s;
 }
 
-// w[r] -= sum_j Q[j][r] h[j]
-__global__ void k_gemv_n(const double* __restrict__ Q, size_t ld, int n, const double* __restrict__ h, int k,
-                         double* __restrict__ w) {
+// w[r] -= sum_j Q[j][r] h[j] (and alpha q[r], q given); norm (optional)
+// = sqrt(wgt |w|^2)
+__global__ void __launch_bounds__(kLT)
+k_gemv_n(const double* __restrict__ Q, size_t ld, int n, const double* __restrict__ h, int k, double* __restrict__ w,
+         const double* __restrict__ alpha, const double* __restrict__ q, double* __restrict__ partial,
+         unsigned* __restrict__ cnt, double wgt, double* __restrict__ norm) {
   extern __shared__ double sh[];
   for (int j = threadIdx.x; j < k; j += blockDim.x) sh[j] = h[j];
   __syncthreads();
+  const double al = q ? *alpha : 0.0;
+  double nn = 0.0;
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-    double acc = 0.0;
+    double acc = q ? al * q[r] : 0.0;
     for (int j = 0; j < k; ++j) acc += Q[(size_t)j * ld + r] * sh[j];
-    w[r] -= acc;
+    const double x = w[r] - acc;
+    w[r] = x;
+    nn += x * x;
   }
+  if (!norm) return;
+  nn = block_sum(nn);
+  if (threadIdx.x == 0) partial[blockIdx.x] = nn;
+  if (!last_block(cnt, gridDim.x)) return;
+  const double s = block_total(partial, gridDim.x, 1);
+  if (threadIdx.x == 0) *norm = sqrt(wgt * s);
 }
 
 void launch_gemv_t(cudaStream_t s, const double* Q, size_t ld, int n, const double* w, double wgt, int k,
-                   Work& wk, double* out) {
+                   Work& wk, double* out, const double* alpha, const double* q) {
   dim3 g((n + kChunk - 1) / kChunk, k);
   ++g_launches;
-  k_gemv_t<<<g, kLT, 0, s>>>(Q, ld, n, w, wgt, wk.part1, wk.cnt_c, out, k);
+  k_gemv_t<<<g, kLT, 0, s>>>(Q, ld, n, w, wgt, wk.part1, wk.cnt_c, out, k, alpha, q);
 }
 
-void launch_gemv_n(cudaStream_t s, const double* Q, size_t ld, int n, const double* h, int k, double* w) {
+void launch_gemv_n(cudaStream_t s, const double* Q, size_t ld, int n, const double* h, int k, double* w,
+                   const double* alpha, const double* q, Work* wk, double wgt, double* norm) {
   const int nb = (n + kLT - 1) / kLT;
   ++g_launches;
-  k_gemv_n<<<nb, kLT, k * sizeof(double), s>>>(Q, ld, n, h, k, w);
+  k_gemv_n<<<nb, kLT, k * sizeof(double), s>>>(Q, ld, n, h, k, w, alpha, q, wk ? wk->part1 : nullptr,
+                                               wk ? wk->cnt_c : nullptr, wgt, norm);
 }
 
-// Lanczos scalar steps on device:
-//   op 0: w -= beta[k-1] * qprev                          (k > 0)
-//   op 1: w -= alpha[k] * q
-//   op 2: q_next = w / beta[k]
-__global__ void k_lz_axpy(int n, int op, const double* __restrict__ sc, double* __restrict__ w,
-                          const double* __restrict__ q, double* __restrict__ qn) {
-  const double a = *sc;
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-    if (op == 2) qn[r] = w[r] / a;
-    else w[r] -= a * q[r];
+// w -= beta qprev (qprev given), alpha = wgt <q|w>
+__global__ void __launch_bounds__(kLT)
+k_lz_alpha(int n, const double* __restrict__ beta, const double* __restrict__ qprev, double* __restrict__ w,
+           const double* __restrict__ q, double wgt, double* __restrict__ partial, unsigned* __restrict__ cnt,
+           double* __restrict__ alpha) {
+  const int g0 = blockIdx.x * kChunk, g1 = min(n, g0 + kChunk);
+  const double b = qprev ? *beta : 0.0;
+  double acc = 0.0;
+  for (int r = g0 + threadIdx.x; r < g1; r += blockDim.x) {
+    double x = w[r];
+    if (qprev) {
+      x -= b * qprev[r];
+      w[r] = x;
+    }
+    acc += q[r] * x;
   }
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) partial[blockIdx.x] = acc;
+  if (!last_block(cnt, gridDim.x)) return;
+  const double s = block_total(partial, gridDim.x, 1);
+  if (threadIdx.x == 0) *alpha = wgt * s;
 }
 
-void launch_lz_axpy(cudaStream_t s, int n, int op, const double* sc, double* w, const double* q, double* qn) {
+void launch_lz_alpha(cudaStream_t s, int n, const double* beta, const double* qprev, double* w, const double* q,
+                     double wgt, Work& wk, double* alpha) {
+  ++g_launches;
+  k_lz_alpha<<<(n + kChunk - 1) / kChunk, kLT, 0, s>>>(n, beta, qprev, w, q, wgt, wk.part1, wk.cnt_c, alpha);
+}
+
+// qn = w / beta
+__global__ void k_lz_next(int n, const double* __restrict__ beta, const double* __restrict__ w,
+                          double* __restrict__ qn) {
+  const double a = *beta;
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) qn[r] = w[r] / a;
+}
+
+void launch_lz_next(cudaStream_t s, int n, const double* beta, const double* w, double* qn) {
   const int nb = min((n + kLT - 1) / kLT, 4 * 152);
   ++g_launches;
-  k_lz_axpy<<<nb, kLT, 0, s>>>(n, op, sc, w, q, qn);
+  k_lz_next<<<nb, kLT, 0, s>>>(n, beta, w, qn);
 }
 
 // out = wgt * sum x*y (sqrt if want_sqrt); single block reduce over a grid of blocks
@@ -1130,12 +1176,8 @@ k_dot(int n, const double* __restrict__ x, const double* __restrict__ y, double 
   acc = block_sum(acc);
   if (threadIdx.x == 0) partial[blockIdx.x] = acc;
   if (!last_block(cnt, gridDim.x)) return;
-  if (threadIdx.x == 0) {
-    double s;
-    sum_records<1>(partial, gridDim.x, 1, &s);
-    s *= wgt;
-    *out = want_sqrt ? sqrt(s) : s;
-  }
+  const double s = wgt * block_total(partial, gridDim.x, 1);
+  if (threadIdx.x == 0) *out = want_sqrt ? sqrt(s) : s;
 }
 
 void launch_dot(cudaStream_t s, int n, const double* x, const double* y, double wgt, int want_sqrt, Work& w,

@@ -125,10 +125,16 @@ void launch_split_form(cudaStream_t s, int m, int k, int km, const double* a, co
 void launch_to_cplx(cudaStream_t s, size_t n, const double* x, double2* y);
 template <typename T, typename U>
 void launch_gather_rows(cudaStream_t s, int npw, int nout, const cpx<U>* in, const int* idx, cpx<T>* out);
+// out[j] = wgt Q_j^T (w - alpha q), w -= alpha q + Q h (q null: without alpha q); norm = sqrt(wgt |w|^2)
 void launch_gemv_t(cudaStream_t s, const double* Q, size_t ld, int n, const double* w, double wgt, int k,
-                   Work& wk, double* out);
-void launch_gemv_n(cudaStream_t s, const double* Q, size_t ld, int n, const double* h, int k, double* w);
-void launch_lz_axpy(cudaStream_t s, int n, int op, const double* sc, double* w, const double* q, double* qn);
+                   Work& wk, double* out, const double* alpha = nullptr, const double* q = nullptr);
+void launch_gemv_n(cudaStream_t s, const double* Q, size_t ld, int n, const double* h, int k, double* w,
+                   const double* alpha = nullptr, const double* q = nullptr, Work* wk = nullptr, double wgt = 0.0,
+                   double* norm = nullptr);
+// w -= beta qprev (qprev null: not), alpha = wgt <q|w>;  qn = w / beta
+void launch_lz_alpha(cudaStream_t s, int n, const double* beta, const double* qprev, double* w, const double* q,
+                     double wgt, Work& wk, double* alpha);
+void launch_lz_next(cudaStream_t s, int n, const double* beta, const double* w, double* qn);
 void launch_dot(cudaStream_t s, int n, const double* x, const double* y, double wgt, int want_sqrt, Work& w,
                 double* out);
 void launch_tridiag_inv(cudaStream_t s, int K, const double* alpha, const double* beta, double* d, double* l,
