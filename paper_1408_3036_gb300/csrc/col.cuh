@@ -56,9 +56,9 @@ struct ColShape {
 template <typename T>
 struct ColArgs {
   ColShape sh;
-  int N, N1, N2, P, nm, npair, nh, npw, nproj, ncol, nunit, maxit;
+  int N, P, nm, npair, nh, npw, nproj, ncol, nunit, maxit;
   int ldz, nhl;                  // rows of Z (2 maxpair), entries per CTA (maxh)
-  FastDiv dN, dP, dN1, dN2, dnz;
+  FastDiv dP, dnz;               // by P and by the slabs per CTA
   const cpx<T>* tw;
   const T* Vp;
   const cpx<T>* Ch;

@@ -50,13 +50,7 @@
 
 #include <cooperative_groups.h>
 
-#include <algorithm>
-#include <cmath>
-#include <map>
-#include <mutex>
-#include <tuple>
-
-#include "col.cuh"
+#include "col_layout.cuh"
 #include "fft.cuh"
 #include "linalg.cuh"
 
@@ -65,9 +59,6 @@ namespace col {
 
 namespace cgr = cooperative_groups;
 
-constexpr int kTPB = 512;
-constexpr int kNW = kTPB / 32;
-constexpr size_t kSmemMax = 226 * 1024;
 // SQMR stagnation: iterations without a halving of the quasi-residual norm.
 // FP32: the recurrence goes no further than about 1e-5 of the right-hand side,
 // now and then 1.5 to 3 times the target; a plateau below 1e-4 is that floor.
@@ -77,11 +68,7 @@ constexpr int kNearWait = 32;        // iterations granted within a factor 2 of 
 
 template <typename T> struct alignas(16) V4 { T x, y, z, w; };
 
-// --- scalar sums: FP64, or a float pair whose additions are error-free
-// transformations (Knuth's TwoSum; products split through an FMA)
-template <typename T> struct AccOf { using type = double; };
-template <> struct AccOf<float> { using type = float2; };
-template <typename T> using Acc = typename AccOf<T>::type;
+// sums of Acc values (col_layout.cuh)
 __device__ __forceinline__ double add_(double a, double b) { return a + b; }
 __device__ __forceinline__ float2 add_(float2 a, float2 b) {
   const float s = __fadd_rn(a.x, b.x);
@@ -210,73 +197,6 @@ template <typename T, int S, int R> __device__ __forceinline__ void twid(cpx<T>*
   }
 }
 template <int R> struct IC { static constexpr int value = R; };
-template <class F> __device__ __forceinline__ void radix1(int r, F f) {
-  switch (r) {
-    case 3: f(IC<3>()); break;
-    case 4: f(IC<4>()); break;
-    case 5: f(IC<5>()); break;
-    case 6: f(IC<6>()); break;
-    default: f(IC<8>());
-  }
-}
-template <class F> __device__ __forceinline__ void radix2(int r, F f) {
-  switch (r) {
-    case 4: f(IC<4>()); break;
-    case 5: f(IC<5>()); break;
-    case 6: f(IC<6>()); break;
-    case 8: f(IC<8>()); break;
-    case 9: f(IC<9>()); break;
-    default: f(IC<10>());
-  }
-}
-
-// --- shared memory of one CTA (byte offsets)
-struct Lay {
-  size_t Z, R, T, X, C, V, K, kin, hpos, rt, own, zm, zs, tw, cp, coefp, coef, part, sc, total;
-};
-__host__ __device__ inline size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
-// Projector rows a warp takes at a time (their products with one load of the
-// vectors), and the parts the entries are cut into so that all warps work.
-__host__ __device__ inline int row_group(int nproj, bool f32) {
-  if (nproj < 8) return nproj < 4 ? 1 : 2;
-  if (!f32 || nproj <= 4 * kNW) return 4;
-  return nproj <= 5 * kNW ? 5 : nproj <= 6 * kNW ? 6 : 4;
-}
-__host__ __device__ inline int splits(int nproj, int rg, int nhl) {
-  const int g = (nproj + rg - 1) / rg, s = g > 0 ? kNW / g : 1, m = (nhl + 31) / 32;
-  return s < 1 ? 1 : s > m ? m : s;
-}
-
-template <typename T>
-__host__ __device__ inline Lay layout(int kind, const ColShape& sh, int N, int P, int npair, int ldz, int nhl,
-                                      int nproj) {
-  const size_t sv = sizeof(cpx<T>), s4 = 4 * sizeof(T);
-  const int Q = 1 << sh.lq, nzl = (N + Q - 1) / Q, nv = kind == COL_CG_PAIR ? 4 : 2;
-  const int rg = row_group(nproj, sizeof(T) == 4);
-  const size_t tile = (size_t)sh.nsb * N * (N | 1) * sv, temp = (size_t)nhl * s4 * (kind == COL_CG_PAIR ? 2 : 1);
-  Lay L;
-  L.Z = 0;
-  L.R = up16(L.Z + (size_t)N * ldz * sv);
-  L.T = up16(L.R + (Q > 1 ? (size_t)nzl * (2 * npair) * sv : 0));
-  L.X = up16(L.T + (tile > temp ? tile : temp));
-  L.C = up16(L.X + (sh.vec_smem ? 4 * (size_t)nhl * s4 : 0));
-  L.V = up16(L.C + (sh.c_smem ? (size_t)nproj * nhl * sv : 0));
-  L.K = up16(L.V + (sh.v_smem ? (size_t)nzl * N * N * sizeof(T) : 0));
-  L.kin = up16(L.K + (size_t)nhl * (kind == COL_QMR ? 1 : 2) * sizeof(T));
-  L.hpos = up16(L.kin + (size_t)nhl * sizeof(T));
-  L.rt = up16(L.hpos + (size_t)nhl * sizeof(unsigned));
-  L.own = up16(L.rt + (size_t)N * P * sizeof(unsigned short));
-  L.zm = up16(L.own + (size_t)2 * npair);
-  L.zs = up16(L.zm + (size_t)ldz);
-  L.tw = up16(L.zs + (size_t)N);
-  L.cp = up16(L.tw + (size_t)N * sv);
-  L.coefp = up16(L.cp + (size_t)splits(nproj, rg, nhl) * nproj * nv * sizeof(T));
-  L.coef = up16(L.coefp + (size_t)Q * nproj * nv * sizeof(T));
-  L.part = up16(L.coef + (size_t)nproj * nv * sizeof(T));
-  L.sc = up16(L.part + (size_t)kNW * 4 * sizeof(Acc<T>));
-  L.total = up16(L.sc + (size_t)3 * Q * 4 * sizeof(Acc<T>));
-  return L;
-}
 
 // Per-column state of the recurrences (every CTA keeps its own equal copy).
 template <typename T> struct CgCol {
@@ -289,7 +209,7 @@ struct QmrCol {
   int it, itb, near, active, flag, upd;
 };
 
-template <typename T, int KIND>
+template <typename T, int KIND, int N1, int N2>
 __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   using V = cpx<T>;
   using W4 = V4<T>;
@@ -298,6 +218,9 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   constexpr bool CG = KIND == COL_CG_PAIR;
   constexpr int NV = CG ? 4 : 2;
   constexpr int NC = PAIR ? 2 : 1;
+  constexpr int N = N1 * N2, LD = N | 1;
+  constexpr IC<N1> R1_{};
+  constexpr IC<N2> R2_{};
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int s_pb[kColMaxQ + 1];
   __shared__ CgCol<T> s_cg[2];
@@ -315,7 +238,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     if (rank == 0 && tid < nc) { a.iters[c0 + tid] = 0; a.flags[c0 + tid] = 0; }
     return;
   }
-  const int N = a.N, N1 = a.N1, N2 = a.N2, P = a.P, LD = N | 1, ldz = a.ldz, ldr = 2 * a.npair;
+  const int P = a.P, nm = a.nm, ldz = a.ldz, ldr = 2 * a.npair;
   const int nproj = a.nproj, rgrp = row_group(nproj, sizeof(T) == 4), nsplit = splits(nproj, rgrp, a.nhl);
   const Lay L = layout<T>(KIND, a.sh, N, P, a.npair, ldz, a.nhl, nproj);
   V* Z = reinterpret_cast<V*>(sm + L.Z);          // [N][ldz] own pencils
@@ -434,6 +357,9 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   csync();                                        // every CTA of the cluster has started
 
   const T one = (T)1, two = (T)2;
+  // |n| <= m for index k of N (one comparison; m = -1: none)
+  auto inside = [&](int k, int m) { return (unsigned)(k - m - 1) >= (unsigned)(N - 2 * m - 1); };
+  auto present = [&](int x) { return inside(x, nm); };
   auto mirror_row = [&](int j) { return j == 0 ? 0 : npl + (j - p0); };   // local row of a pair's second pencil
 
   // u (both halves of the pair, or the complex column) into the own pencils
@@ -454,7 +380,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 
   // z-IFFT of the own pencils, sent to the slab owners
   auto z_step1 = [&]() {
-    radix1(N1, [&](auto RR) {
+    ([&](auto RR) {
       constexpr int R1 = decltype(RR)::value;
       for (int t = tid; t < nrl * N2; t += kTPB) {
         const int n2 = dnr.div(t), row = t - n2 * nrl;
@@ -463,19 +389,19 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 #pragma unroll
         for (int n1 = 0; n1 < R1; ++n1) {
           const int z = n1 * N2 + n2;
-          v[n1] = (z <= zmx || z >= N - zmx) ? Z[z * ldz + row] : mk<T>(0, 0);
+          v[n1] = inside(z, zmx) ? Z[z * ldz + row] : mk<T>(0, 0);
         }
         dft<T, 1, R1>(v);
         twid<T, 1, R1>(v, stw, n2);
 #pragma unroll
         for (int k = 0; k < R1; ++k) Z[(k * N2 + n2) * ldz + row] = v[k];
       }
-    });
+    })(R1_);
   };
   auto z_inverse_send = [&]() {
     z_step1();
     __syncthreads();
-    radix2(N2, [&](auto RR) {
+    ([&](auto RR) {
       constexpr int R2 = decltype(RR)::value;
       for (int t = tid; t < nrl * N1; t += kTPB) {
         const int k1 = dnr.div(t), row = t - k1 * nrl;
@@ -490,13 +416,13 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
           at(R, o)[(z - o * nzl) * ldr + 2 * p0 + row] = v[k];
         }
       }
-    });
+    })(R2_);
   };
   // Q = 1: the same, left in the pencils (i2 at slot zs[i2])
   auto z_inverse_local = [&]() {
     z_step1();
     __syncthreads();
-    radix2(N2, [&](auto RR) {
+    ([&](auto RR) {
       constexpr int R2 = decltype(RR)::value;
       for (int t = tid; t < nrl * N1; t += kTPB) {
         const int k1 = dnr.div(t), row = t - k1 * nrl;
@@ -507,7 +433,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 #pragma unroll
         for (int k = 0; k < R2; ++k) Z[(k1 * R2 + k) * ldz + row] = v[k];
       }
-    });
+    })(R2_);
   };
 
   auto z_inverse = [&]() { if (Q > 1) z_inverse_send(); else z_inverse_local(); };
@@ -518,10 +444,10 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     const int absent = N - P;                     // planes without entries: nm < i0 < N - nm
     for (int sb = 0; sb < max(nsl, 1); sb += a.sh.nsb) {
       const int ns = min(a.sh.nsb, nsl - sb);
-      radix1(N1, [&](auto RR) {
+      ([&](auto RR) {
         constexpr int R1 = decltype(RR)::value;
         for (int t = tid; t < ns * N2 * P; t += kTPB) {
-          const int q = a.dP.div(t), p = t - q * P, s = a.dN2.div(q), n2 = q - s * N2;
+          const int q = a.dP.div(t), p = t - q * P, s = (int)((unsigned)q / N2), n2 = q - s * N2;
           const V* src = Q > 1 ? R + (size_t)(sb + s) * ldr : Z + zs[sb + s] * ldz;
           V v[R1];
 #pragma unroll
@@ -531,18 +457,18 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
           }
           dft<T, 1, R1>(v);
           twid<T, 1, R1>(v, stw, n2);
-          V* d = Tt + (s * N + (p <= a.nm ? p : p + absent)) * LD + n2;
+          V* d = Tt + (s * N + (p <= nm ? p : p + absent)) * LD + n2;
 #pragma unroll
           for (int k = 0; k < R1; ++k) d[k * N2] = v[k];
         }
-      });
+      })(R1_);
       __syncthreads();
       if (check && sb == 0 && !s_any) return true;
-      radix2(N2, [&](auto RR) {
+      ([&](auto RR) {
         constexpr int R2 = decltype(RR)::value;
         for (int t = tid; t < ns * N1 * P; t += kTPB) {
-          const int q = a.dP.div(t), p = t - q * P, s = a.dN1.div(q), k1 = q - s * N1;
-          V* d = Tt + (s * N + (p <= a.nm ? p : p + absent)) * LD + k1 * R2;
+          const int q = a.dP.div(t), p = t - q * P, s = (int)((unsigned)q / N1), k1 = q - s * N1;
+          V* d = Tt + (s * N + (p <= nm ? p : p + absent)) * LD + k1 * R2;
           V v[R2];
 #pragma unroll
           for (int k = 0; k < R2; ++k) v[k] = d[k];
@@ -550,26 +476,26 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 #pragma unroll
           for (int k = 0; k < R2; ++k) d[k] = v[k];
         }
-      });
+      })(R2_);
       __syncthreads();
-      radix1(N1, [&](auto RR) {
+      ([&](auto RR) {
         constexpr int R1 = decltype(RR)::value;
         for (int t = tid; t < ns * N2 * N; t += kTPB) {
-          const int q = a.dN.div(t), y = t - q * N, s = a.dN2.div(q), n2 = q - s * N2;
+          const int q = (int)((unsigned)t / N), y = t - q * N, s = (int)((unsigned)q / N2), n2 = q - s * N2;
           V* d = Tt + (s * N + n2) * LD + y;
           V v[R1];
 #pragma unroll
           for (int n1 = 0; n1 < R1; ++n1) {
             const int x = n1 * N2 + n2;
-            v[n1] = (x <= a.nm || x >= N - a.nm) ? d[n1 * N2 * LD] : mk<T>(0, 0);
+            v[n1] = present(x) ? d[n1 * N2 * LD] : mk<T>(0, 0);
           }
           dft<T, 1, R1>(v);
           twid<T, 1, R1>(v, stw, n2);
 #pragma unroll
           for (int k = 0; k < R1; ++k) d[k * N2 * LD] = v[k];
         }
-      });
-      radix2(N2, [&](auto RR) {
+      })(R1_);
+      ([&](auto RR) {
         constexpr int R2 = decltype(RR)::value;
         // FP32: the potential of a thread's next task is loaded ahead, of the
         // first before the barrier, of the others before the second transform
@@ -580,7 +506,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         T pot[R2];
         auto load = [&](int t) {
           if (t >= tasks) return;
-          const int q = a.dN.div(t), y = t - q * N, s = a.dN1.div(q), k1 = q - s * N1;
+          const int q = (int)((unsigned)t / N), y = t - q * N, s = (int)((unsigned)q / N1), k1 = q - s * N1;
           if (a.sh.v_smem) {
             const T* vp = Vs + ((sb + s) * N + k1) * N + y;
 #pragma unroll
@@ -594,7 +520,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         if (ahead) load(tid);
         __syncthreads();
         for (int t = tid; t < tasks; t += kTPB) {
-          const int q = a.dN.div(t), y = t - q * N, s = a.dN1.div(q), k1 = q - s * N1;
+          const int q = (int)((unsigned)t / N), y = t - q * N, s = (int)((unsigned)q / N1), k1 = q - s * N1;
           V* d = Tt + (s * N + k1 * R2) * LD + y;
           V v[R2];
 #pragma unroll
@@ -609,12 +535,12 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 #pragma unroll
           for (int k = 0; k < R2; ++k) d[k * LD] = v[k];
         }
-      });
+      })(R2_);
       __syncthreads();
-      radix1(N1, [&](auto RR) {
+      ([&](auto RR) {
         constexpr int R1 = decltype(RR)::value;
         for (int t = tid; t < ns * N2 * N; t += kTPB) {
-          const int q = a.dN.div(t), y = t - q * N, s = a.dN2.div(q), n2 = q - s * N2;
+          const int q = (int)((unsigned)t / N), y = t - q * N, s = (int)((unsigned)q / N2), n2 = q - s * N2;
           V* d = Tt + (s * N + n2) * LD + y;
           V v[R1];
 #pragma unroll
@@ -623,16 +549,16 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 #pragma unroll
           for (int n1 = 0; n1 < R1; ++n1) {
             const int x = n1 * N2 + n2;
-            if (x <= a.nm || x >= N - a.nm) d[n1 * N2 * LD] = v[n1];
+            if (present(x)) d[n1 * N2 * LD] = v[n1];
           }
         }
-      });
+      })(R1_);
       __syncthreads();
-      radix2(N2, [&](auto RR) {
+      ([&](auto RR) {
         constexpr int R2 = decltype(RR)::value;
         for (int t = tid; t < ns * N1 * P; t += kTPB) {
-          const int q = a.dP.div(t), p = t - q * P, s = a.dN1.div(q), k1 = q - s * N1;
-          V* d = Tt + (s * N + (p <= a.nm ? p : p + absent)) * LD + k1 * R2;
+          const int q = a.dP.div(t), p = t - q * P, s = (int)((unsigned)q / N1), k1 = q - s * N1;
+          V* d = Tt + (s * N + (p <= nm ? p : p + absent)) * LD + k1 * R2;
           V v[R2];
 #pragma unroll
           for (int k = 0; k < R2; ++k) v[k] = d[k];
@@ -641,13 +567,13 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 #pragma unroll
           for (int k = 0; k < R2; ++k) d[k] = v[k];
         }
-      });
+      })(R2_);
       __syncthreads();
-      radix1(N1, [&](auto RR) {
+      ([&](auto RR) {
         constexpr int R1 = decltype(RR)::value;
         for (int t = tid; t < ns * N2 * P; t += kTPB) {
-          const int q = a.dP.div(t), p = t - q * P, s = a.dN2.div(q), n2 = q - s * N2;
-          const V* d = Tt + (s * N + (p <= a.nm ? p : p + absent)) * LD + n2;
+          const int q = a.dP.div(t), p = t - q * P, s = (int)((unsigned)q / N2), n2 = q - s * N2;
+          const V* d = Tt + (s * N + (p <= nm ? p : p + absent)) * LD + n2;
           V v[R1];
 #pragma unroll
           for (int k = 0; k < R1; ++k) v[k] = d[k * N2];
@@ -662,7 +588,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
             }
           }
         }
-      });
+      })(R1_);
       __syncthreads();
     }
     return false;
@@ -670,7 +596,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 
   // z-FFT of the own pencils, from slot order to natural order, in place
   auto z_forward = [&]() {
-    radix2(N2, [&](auto RR) {
+    ([&](auto RR) {
       constexpr int R2 = decltype(RR)::value;
       for (int t = tid; t < nrl * N1; t += kTPB) {
         const int k1 = dnr.div(t), row = t - k1 * nrl;
@@ -682,9 +608,9 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 #pragma unroll
         for (int k = 0; k < R2; ++k) Z[(k1 * R2 + k) * ldz + row] = v[k];
       }
-    });
+    })(R2_);
     __syncthreads();
-    radix1(N1, [&](auto RR) {
+    ([&](auto RR) {
       constexpr int R1 = decltype(RR)::value;
       for (int t = tid; t < nrl * N2; t += kTPB) {
         const int n2 = dnr.div(t), row = t - n2 * nrl;
@@ -696,10 +622,10 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 #pragma unroll
         for (int n1 = 0; n1 < R1; ++n1) {
           const int z = n1 * N2 + n2;
-          if (z <= zmx || z >= N - zmx) Z[z * ldz + row] = v[n1];
+          if (inside(z, zmx)) Z[z * ldz + row] = v[n1];
         }
       }
-    });
+    })(R1_);
     __syncthreads();
   };
 
@@ -735,9 +661,9 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     const int ngr = (nproj + RG - 1) / RG;
     for (int w = warp; w < ngr * nsplit; w += kNW) {
       const int gr = w / nsplit, prt = w - gr * nsplit, v0 = gr * RG;
-      const V* Cr[RG];
+      unsigned row[RG];
 #pragma unroll
-      for (int q = 0; q < RG; ++q) Cr[q] = C + (size_t)min(v0 + q, nproj - 1) * ldc;
+      for (int q = 0; q < RG; ++q) row[q] = (unsigned)min(v0 + q, nproj - 1) * (unsigned)ldc;
       T acc[M];
 #pragma unroll
       for (int k = 0; k < M; ++k) acc[k] = (T)0;
@@ -745,7 +671,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       for (int e = lane + 32 * prt; e < nh; e += 32 * nsplit) {
         V c[RG];
 #pragma unroll
-        for (int q = 0; q < RG; ++q) c[q] = Cr[q][e];
+        for (int q = 0; q < RG; ++q) c[q] = C[row[q] + (unsigned)e];
         W4 y = Tm[e];
         if (PAIR) {
           if (h0 + e == 0) { y.x *= (T)0.5; y.z *= (T)0.5; }
@@ -833,7 +759,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     for (; v + U <= nproj; v += U) {
       V c[U];
 #pragma unroll
-      for (int q = 0; q < U; ++q) c[q] = C[(size_t)(v + q) * ldc + e];
+      for (int q = 0; q < U; ++q) c[q] = C[(unsigned)(v + q) * (unsigned)ldc + (unsigned)e];
 #pragma unroll
       for (int q = 0; q < U; ++q) {
         const T k0 = coef[(v + q) * NV], k1 = coef[(v + q) * NV + 1];
@@ -1356,195 +1282,15 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   csync();                                        // no CTA leaves while others may reach its memory
 }
 
-template <typename T, int KIND> struct Fn { static const void* get() { return (const void*)k_col_solve<T, KIND>; } };
-
-template <typename T> const void* kernel_of(int kind) {
-  if (kind == COL_CG_PAIR) return Fn<T, COL_CG_PAIR>::get();
-  if (kind == COL_QMR) return Fn<T, COL_QMR>::get();
-  return Fn<T, COL_QMR_PAIR>::get();
-}
-
-inline cudaLaunchConfig_t config(cudaLaunchAttribute* at, int q, int grid, size_t smem, cudaStream_t s) {
-  cudaLaunchConfig_t c = {};
-  c.gridDim = dim3(grid);
-  c.blockDim = dim3(kTPB);
-  c.dynamicSmemBytes = smem;
-  c.stream = s;
-  at->id = cudaLaunchAttributeClusterDimension;
-  at->val.clusterDim.x = q;
-  at->val.clusterDim.y = 1;
-  at->val.clusterDim.z = 1;
-  c.attrs = at;
-  c.numAttrs = 1;
-  return c;
-}
-
-// Kernel attributes (once per function and process) and the clusters of size q
-// that run at once (0: this size does not run here).
-template <typename T> int active_clusters(int kind, int lq, size_t smem) {
-  static std::mutex mu;
-  static std::map<std::tuple<int, int, size_t>, int> known;
-  static bool ready[3] = {false, false, false};
-  std::lock_guard<std::mutex> lock(mu);
-  const void* f = kernel_of<T>(kind);
-  if (!ready[kind]) {
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess ||
-        cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-      cudaGetLastError();
-      return 0;
-    }
-    ready[kind] = true;
-  }
-  auto it = known.find({kind, lq, smem});
-  if (it != known.end()) return it->second;
-  cudaLaunchAttribute at;
-  const cudaLaunchConfig_t c = config(&at, 1 << lq, 1 << lq, smem, nullptr);
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, f, &c) != cudaSuccess) {
-    cudaGetLastError();
-    n = 0;
-  }
-  known[{kind, lq, smem}] = n;
-  return n;
+template <typename T, int A, int B> const void* kernel_ptr(int kind) {
+  if (kind == COL_CG_PAIR) return (const void*)k_col_solve<T, COL_CG_PAIR, A, B>;
+  if (kind == COL_QMR) return (const void*)k_col_solve<T, COL_QMR, A, B>;
+  return (const void*)k_col_solve<T, COL_QMR_PAIR, A, B>;
 }
 
 }  // namespace col
-
-template <typename T>
-bool col_shape(const ColPlan& p, int kind, int N, int nproj, int nunit, int cta_div, ColShape* out) {
-  if (!p.ok || nunit < 1 || nproj > kMaxOcc) return false;
-  // An iteration of one unit takes a fixed time (barriers, reductions, scalar
-  // steps) and its work over Q CTAs; microseconds, fitted to sweeps over Q
-  // (45^3 grid, 11 rows, FP32 SQMR: 107, 57, 38, 26, 25 for Q = 1 .. 16; 48^3,
-  // 16 rows, CG pair: 55, 30, 22 for Q = 4 .. 16, FP64 424, 222 for Q = 8, 16;
-  // 16^3, 4 rows, FP64: 88, 57, 42, 35, 36).  Units beyond the clusters that
-  // run at once wait for a free one: whole rounds for CG (columns alike, but the
-  // last few pairs of a cell are its fastest); for SQMR the slowest columns,
-  // which start first, take about twice the mean.  The order of the sums, and
-  // with it the last bits, depends on Q: FP64 results do not depend on how many
-  // contexts share the GPU, so there Q does not either.
-  const bool f32 = sizeof(T) == 4;
-  // (contexts that share the GPU keep it busy about half the time each)
-  const double share = f32 ? std::max(0.5 * cta_div, 1.0) : 1.0;
-  const double fixed = f32 ? 11.0 : 27.0;
-  const double work = (f32 ? 1.0e-3 : 1.5e-2) * N * N * N + (f32 ? 0.9e-3 : 1.66e-2) * nproj * p.nh;
-  double best = 1e300;
-  for (int lq = 0; lq < kColNQ; ++lq) {
-    const int Q = 1 << lq, ldz = 2 * p.maxpair[lq], nhl = p.maxh[lq];
-    if (Q > N || Q > p.npair) continue;
-    ColShape s;
-    s.lq = lq;
-    const int nzl = (N + Q - 1) / Q;
-    auto fits = [&](int nsb, bool vec, bool c, bool v = false) {
-      s.nsb = nsb;
-      s.vec_smem = vec;
-      s.c_smem = c;
-      s.v_smem = v;
-      s.smem = col::layout<T>(kind, s, N, p.P, p.npair, ldz, nhl, nproj).total;
-      return s.smem <= col::kSmemMax;
-    };
-    // slabs together: the fewest rounds of the CTA's threads (FP64: of a warp
-    // per scheduler) over the passes of all batches; then the rows and the
-    // potential where room is left
-    auto rounds_of = [&](int nsb) {
-      const int unit = sizeof(T) == 4 ? col::kTPB : 128;
-      auto r = [&](long tasks) { return (double)((tasks + unit - 1) / unit); };
-      double t = 0.0;
-      for (int sb = 0; sb < nzl; sb += nsb) {
-        const long ns = std::min(nsb, nzl - sb);
-        t += 2.0 * (r(ns * p.N2 * p.P) + r(ns * p.N1 * p.P) + r(ns * p.N2 * N)) + 1.6 * r(ns * p.N1 * N) + 2.0;
-      }
-      return t;
-    };
-    // the projector rows (read twice an iteration) before the vectors (read
-    // and written once) where the rows are the larger traffic
-    const bool rows_first = 2 * nproj * sizeof(cpx<T>) > 9 * 4 * sizeof(T);
-    int nsb = 0;
-    bool vec = false, c = false, v = false;
-    for (int pass = 0; pass < 4 && nsb == 0; ++pass) {
-      vec = pass == 0 || pass == (rows_first ? 2 : 1);
-      c = pass == 0 || pass == (rows_first ? 1 : 2);
-      for (int n = 1; n <= nzl; ++n)
-        if (fits(n, vec, c) && (nsb == 0 || rounds_of(n) < rounds_of(nsb))) nsb = n;
-    }
-    if (nsb == 0) continue;
-    v = fits(nsb, vec, c, true);
-    fits(nsb, vec, c, v);
-    s.vec_elems = vec ? 0 : 16 * (size_t)p.nh;
-    const int act = col::active_clusters<T>(kind, lq, s.smem);
-    if (act < 1) continue;
-    const double load = (double)nunit * share / act;
-    const double rounds = kind != COL_CG_PAIR ? std::max(1.0, 0.5 * load)
-                                              : load <= 1.25 ? std::max(1.0, load) : std::ceil(load);
-    const double t = rounds * (fixed + lq + work / Q);
-    if (t < best) { best = t; *out = s; }
-  }
-  return best < 1e300;
-}
-
-template <typename T>
-cudaError_t launch_col_solve(cudaStream_t s, int kind, const ColArgs<T>& a) {
-  const int Q = 1 << a.sh.lq;
-  if (col::active_clusters<T>(kind, a.sh.lq, a.sh.smem) < 1) return cudaErrorNotSupported;
-  cudaLaunchAttribute at;
-  const cudaLaunchConfig_t c = col::config(&at, Q, a.nunit * Q, a.sh.smem, s);
-  ColArgs<T> arg = a;
-  void* args[] = {&arg};
-  ++g_launches;
-  return cudaLaunchKernelExC(&c, col::kernel_of<T>(kind), args);
-}
-
-namespace col {
-template <typename T>
-__global__ void k_col_perm_v(int N, int N1, int N2, const T* __restrict__ v, T* __restrict__ out) {
-  const int n = N * N * N;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const int c = i % N, x = (i / N) % N, z = i / (N * N);
-    const int y = c / N2 + N1 * (c % N2);
-    out[i] = v[((size_t)x * N + y) * N + z];
-  }
-}
-template <typename T>
-__global__ void k_col_perm_rows(int nh, int npw, int rows, const int* __restrict__ gp, const cpx<T>* __restrict__ C,
-                                cpx<T>* __restrict__ out) {
-  const size_t n = (size_t)nh * rows;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const size_t v = i / nh;
-    out[i] = C[v * npw + gp[i - v * nh]];
-  }
-}
-template <typename T>
-__global__ void k_col_perm_kin(int nh, const int* __restrict__ gp, const T* __restrict__ kin, T* __restrict__ out) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nh; i += gridDim.x * blockDim.x) out[i] = kin[gp[i]];
-}
-}  // namespace col
-
-// vloc_s / kin (fixed per cell) and C (per occupied block) in the solver's
-// orders; a null input leaves that part alone.
-template <typename T>
-cudaError_t launch_col_permute(cudaStream_t s, const ColPlan& p, int N, int npw, const T* vloc_s, const cpx<T>* C,
-                               int nproj, const T* kin, ColPrec<T>& out) {
-  if (vloc_s) {
-    ++g_launches;
-    col::k_col_perm_v<T><<<std::min((N * N * N + 255) / 256, 152 * 8), 256, 0, s>>>(N, p.N1, p.N2, vloc_s, out.Vp);
-  }
-  if (kin) {
-    ++g_launches;
-    col::k_col_perm_kin<T><<<(p.nh + 255) / 256, 256, 0, s>>>(p.nh, p.gp, kin, out.kin);
-  }
-  if (C && nproj > 0) {
-    const size_t n = (size_t)p.nh * nproj;
-    ++g_launches;
-    col::k_col_perm_rows<T><<<(int)std::min<size_t>((n + 255) / 256, 152 * 16), 256, 0, s>>>(p.nh, npw, nproj, p.gp, C,
-                                                                                              out.Ch);
-  }
-  return cudaGetLastError();
-}
-
-#define GW_COL_INST(T)                                                                                     \
-  template bool col_shape<T>(const ColPlan&, int, int, int, int, int, ColShape*);                               \
-  template cudaError_t launch_col_solve<T>(cudaStream_t, int, const ColArgs<T>&);                          \
-  template cudaError_t launch_col_permute<T>(cudaStream_t, const ColPlan&, int, int, const T*, const cpx<T>*, int, \
-                                             const T*, ColPrec<T>&);
-
 }  // namespace gw
+
+#define GW_COL_SIZE(A, B)                                       \
+  template const void* gw::col::kernel_ptr<float, A, B>(int);   \
+  template const void* gw::col::kernel_ptr<double, A, B>(int);

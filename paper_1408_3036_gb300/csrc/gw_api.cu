@@ -535,12 +535,13 @@ gw_status col_solve(gw_ctx* ctx, int kind, int ncol, const double2* b64, const d
   if (!col_shape<T>(p, kind, ctx->N, nproj(ctx), a.nunit, ctx->cta_div, &a.sh)) return GW_OK;
   auto& P = prec_of<T>(ctx);
   auto& c = col_of<T>(ctx);
-  a.N = ctx->N; a.N1 = p.N1; a.N2 = p.N2; a.P = p.P; a.nm = p.nm; a.npair = p.npair; a.nh = p.nh;
+  a.N = ctx->N; a.P = p.P; a.nm = p.nm; a.npair = p.npair; a.nh = p.nh;
   a.npw = ctx->npw; a.nproj = nproj(ctx); a.ncol = ncol; a.maxit = ctx->max_iter;
   a.ldz = 2 * p.maxpair[a.sh.lq];
   a.nhl = p.maxh[a.sh.lq];
   const int nzl = (a.N + (1 << a.sh.lq) - 1) >> a.sh.lq;
-  a.dN.set(a.N); a.dP.set(a.P); a.dN1.set(a.N1); a.dN2.set(a.N2); a.dnz.set(nzl);
+  a.dP.set(a.P);
+  a.dnz.set(nzl);
   a.tw = P.tw; a.Vp = c.Vp; a.Ch = c.Ch; a.kin = c.kin;
   a.split = p.split; a.hstart = p.hstart; a.gp = p.gp; a.gm = p.gm; a.hpos = p.hpos; a.disc = p.disc; a.zmax = p.zmax;
   a.b64 = b64; a.x64 = x64; a.outer_active = outer_active; a.E = E; a.rr_abs = rr_abs; a.tk = tk; a.order = nullptr;
