@@ -423,9 +423,11 @@ gw_status gw_set_cg_kernel(gw_ctx* ctx, int kind, long long wait_limit);
 
 /*
  * gw_set_precond -- preconditioner of the Sternheimer solvers (CG and SQMR):
- *   1 (default)  kinetic preconditioner of Teter, Payne and Allan, diagonal in
- *                G, with the kinetic energy of the column's occupied state as
- *                reference (symmetric, also in the bilinear form)
+ *   1 (default)  kinetic, diagonal in G and symmetric, also in the bilinear form:
+ *                the column solver takes the kinetic denominators of the
+ *                column's own shift, |G|^2/2 - E kept away from zero; the
+ *                other kernels the form of Teter, Payne and Allan, with the
+ *                kinetic energy of the column's occupied state as reference
  *   0            none, as in the paper (Sec. Avoiding summations: SQMR without
  *                preconditioning)
  * Both solve the same equations to the same tolerance; the preconditioner

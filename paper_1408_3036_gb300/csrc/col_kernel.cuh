@@ -30,6 +30,17 @@
 // and half entry for either kind, half of what the full sphere takes, and half
 // of the rows' bytes.
 //
+// Preconditioner.  The kinetic denominators of the column's own shift (those of
+// the model operator), kept away from zero: with d = |G|^2/2 - Re E,
+//   real shift     K = 1 / sqrt(d^2 + 0.03^2)   (positive, as CG needs)
+//   complex shift  K = 1 / (d - i (Im E + 0.2 sgn Im E))
+// K(-G) = K(G), so it is symmetric in the bilinear form too.  The
+// Teter-Payne-Allan form of the other kernels knows the kinetic energy of the
+// occupied state but not the shift.  Iterations to 1e-5 (FP64), then and now:
+// 32^3, 2109 plane waves, 0.957 + 0.1 i: 170 -> 46 for the slow sign, 11 -> 7
+// for the other; 45^3, 0.3 + 0.1 i 55 -> 35 and 15 -> 10; static 32^3 10 -> 7,
+// 48^3 29 -> 25 (slowest column) and 10 -> 7 (fastest).
+//
 // Scalars of the recurrences come from ordered sums that every CTA of the
 // cluster forms from the same partial sums: all CTAs decide alike.
 //
@@ -41,11 +52,13 @@
 // cycles and scheduler here, so sums are halved across the lanes instead of
 // repeated in them, and scalar steps share one division).
 // Measured on a GB300, one application, before (launches per step, or the
-// grid-wide task queue of kernels_cg.cu) and after: 48^3 grid, 12053 plane
-// waves, 16 CG columns, FP32 3.64 -> 2.21 ms, FP64 15.8 -> 11.3 ms; 45^3, 2007
-// plane waves, 22 complex columns 11.7 -> 4.1 ms; 32^3, 2109 plane waves, 69
-// rows, 1104 complex columns 398 -> 79 ms; 64^3, 38401 plane waves, 64 rows,
-// 256 complex columns 1082 -> 492 ms.
+// grid-wide task queue of kernels_cg.cu, with the Teter-Payne-Allan form) and
+// after, of which the preconditioner alone in brackets: 48^3 grid, 12053 plane
+// waves, 16 CG columns, FP32 3.70 -> 1.58 ms (1.65 -> 1.58), FP64 15.8 -> 9.8 ms
+// (10.9 -> 9.8); 45^3, 2007 plane waves, 22 complex columns 11.7 -> 2.29 ms
+// (3.2 -> 2.29); 32^3, 2109 plane waves, 69 rows, 1104 complex columns 400 ->
+// 30.5 ms (58 -> 30.5); 64^3, 38401 plane waves, 64 rows, 256 complex columns
+// 1051 -> 113 ms (386 -> 113).
 #pragma once
 
 #include <cooperative_groups.h>
@@ -59,11 +72,17 @@ namespace col {
 
 namespace cgr = cooperative_groups;
 
-// SQMR stagnation: iterations without a halving of the quasi-residual norm.
-// FP32: the recurrence goes no further than about 1e-5 of the right-hand side,
-// now and then 1.5 to 3 times the target; a plateau below 1e-4 is that floor.
+// Smoothing of the preconditioner's denominators (Ha), by scans of 0.02 .. 0.8
+// over static, real, imaginary and complex frequencies on 16^3 .. 48^3 cells.
+constexpr double kPreReal = 0.03, kPreImag = 0.2;
+// SQMR stagnation: iterations without a halving of the quasi-residual norm tau.
+// FP32: rounding errors scale with the largest residual of the pass (it peaks
+// in the first steps), so tau goes no further than some 30 ulp of that, now and
+// then 1.5 to 10 times the target; past it the recurrence comes apart, |r|
+// grows to 1e2 .. 1e5 times tau and tau stays.
 constexpr int kQmrWindow = 1000;     // anywhere (as the multi-launch solver's)
-constexpr int kQmrWindowFloor = 64;  // FP32, once the norm has dropped 1e4 times
+constexpr int kQmrWindowFloor = 48;  // FP32, tau below 1e-4 |b| or 2e-6 max |r|
+constexpr int kApartWait = 16;       // FP32, iterations in a row with |r| > 100 tau
 constexpr int kNearWait = 32;        // iterations granted within a factor 2 of the target norm
 
 template <typename T> struct alignas(16) V4 { T x, y, z, w; };
@@ -205,8 +224,8 @@ template <typename T> struct CgCol {
 };
 struct QmrCol {
   double2 rho, alpha, beta, qc;
-  double dc, theta2, tau2, stop, qbest, rr0;         // theta^2, tau^2
-  int it, itb, near, active, flag, upd;
+  double dc, theta2, tau2, stop, qbest, rr0, rmax;         // theta^2, tau^2
+  int it, itb, near, apart, active, flag, upd;
 };
 
 template <typename T, int KIND, int N1, int N2>
@@ -246,7 +265,8 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   V* Tt = reinterpret_cast<V*>(sm + L.T);         // [nsb][N][LD] slab tiles
   W4* Tm = reinterpret_cast<W4*>(sm + L.T);       // [nhl] A u, CG then u (share the tiles' place)
   T* Vs = reinterpret_cast<T*>(sm + L.V);         // [nzl][N][N] V / N_g of the own slabs (v_smem)
-  T* Kt = reinterpret_cast<T*>(sm + L.K);
+  T* Kt = reinterpret_cast<T*>(sm + L.K);         // preconditioner: one real value per column,
+  V* KC = reinterpret_cast<V*>(sm + L.K);         // COL_QMR one complex value
   T* kin = reinterpret_cast<T*>(sm + L.kin);
   unsigned* hpos = reinterpret_cast<unsigned*>(sm + L.hpos);
   unsigned short* rt = reinterpret_cast<unsigned short*>(sm + L.rt);
@@ -293,13 +313,14 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     const int j = p0 + (k < npl ? k : k - npl);
     zm[k] = (signed char)((j == 0 && k >= npl) ? -1 : (int)a.zmax[j]);
   }
-  T rtk[2] = {(T)0, (T)0};
+  bool pre[2] = {false, false};
   T Ex[2] = {(T)0, (T)0}, Ey = (T)0;
   for (int c = 0; c < nc; ++c) {
-    rtk[c] = (a.tk && a.tk[c0 + c] != 0.0) ? (T)(1.0 / a.tk[c0 + c]) : (T)0;
+    pre[c] = a.tk && a.tk[c0 + c] != 0.0;
     Ex[c] = (T)a.E[c0 + c].x;
     if (!PAIR) Ey = (T)a.E[c0].y;
   }
+  auto precond_real = [](T d) { return (T)1 / sqrt(d * d + (T)(kPreReal * kPreReal)); };
   // solver vectors: CG r, p, s, x; SQMR r, q, d, x
   const size_t xs = a.sh.vec_smem ? (size_t)a.nhl : (size_t)a.nh;
   W4* X = a.sh.vec_smem ? reinterpret_cast<W4*>(sm + L.X)
@@ -323,10 +344,16 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     kin[e] = k;
     hpos[e] = a.hpos[h];
     if (PAIR) {
-      Kt[2 * e] = (rtk[0] != (T)0) ? tpa<T>(k * rtk[0]) : (T)1;
-      Kt[2 * e + 1] = (rtk[1] != (T)0) ? tpa<T>(k * rtk[1]) : (T)1;
+      Kt[2 * e] = pre[0] ? precond_real(k - Ex[0]) : (T)1;
+      Kt[2 * e + 1] = pre[1] ? precond_real(k - Ex[1]) : (T)1;
     } else {
-      Kt[e] = (rtk[0] != (T)0) ? tpa<T>(k * rtk[0]) : (T)1;
+      const T dr = k - Ex[0], di = Ey > (T)0 ? Ey + (T)kPreImag : Ey - (T)kPreImag;
+      V kc = mk<T>((T)1, (T)0);
+      if (pre[0]) {
+        if (Ey == (T)0) kc.x = precond_real(dr);
+        else { const T d = (T)1 / (dr * dr + di * di); kc = mk<T>(dr * d, di * d); }
+      }
+      KC[e] = kc;
     }
     const int g = a.gp[h], m = a.gm[h];
     W4 r = {(T)0, (T)0, (T)0, (T)0};
@@ -1028,26 +1055,33 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     // simplified QMR (kernels_linalg.cu has the recurrences):
     //   t = P_c (H - E) q; alpha = rho / [q, t]; r -= alpha t;
     //   theta, tau from |r|; d = dc d + qc q; x += d; rho' = [r, K r]; q = K r + beta q
-    auto kk = [&](int e, int c) { return PAIR ? Kt[2 * e + c] : Kt[e]; };
+    // K r
+    auto apply_k = [&](int e, const W4& r) {
+      if (PAIR) {
+        const T k0 = Kt[2 * e], k1 = Kt[2 * e + 1];
+        return W4{k0 * r.x, k0 * r.y, k1 * r.z, k1 * r.w};
+      }
+      const V k = KC[e];
+      return W4{k.x * r.x - k.y * r.y, k.x * r.y + k.y * r.x, k.x * r.z - k.y * r.w, k.x * r.w + k.y * r.z};
+    };
     // r^H r and [r, K r] of one entry into v (PAIR: rr0, rr1, rho0, rho1; else rr, rho)
     auto norms = [&](int e, const W4& r, SA* v) {
       if (PAIR) {
         const T f = (h0 + e == 0) ? one : two;
-        const T k0 = f * kk(e, 0), k1 = f * kk(e, 1);
+        const T k0 = f * Kt[2 * e], k1 = f * Kt[2 * e + 1];
         fma_(v[0], f * r.x, r.x); fma_(v[0], f * r.y, r.y);
         fma_(v[1], f * r.z, r.z); fma_(v[1], f * r.w, r.w);
         fma_(v[2], k0 * r.x, r.x); fma_(v[2], k0 * r.y, r.y);
         fma_(v[3], k1 * r.z, r.z); fma_(v[3], k1 * r.w, r.w);
       } else {
-        const T k = kk(e, 0);
+        const W4 u = apply_k(e, r);
         fma_(v[0], r.x, r.x); fma_(v[0], r.y, r.y); fma_(v[0], r.z, r.z); fma_(v[0], r.w, r.w);
         if (h0 + e == 0) {
-          fma_(v[1], k * r.x, r.x); fma_(v[1], -k * r.y, r.y);
-          fma_(v[2], two * k * r.x, r.y);
+          fma_(v[1], u.x, r.x); fma_(v[1], -u.y, r.y);
+          fma_(v[2], u.x, r.y); fma_(v[2], u.y, r.x);
         } else {
-          const T k2 = two * k;
-          fma_(v[1], k2 * r.x, r.z); fma_(v[1], -k2 * r.y, r.w);
-          fma_(v[2], k2 * r.x, r.w); fma_(v[2], k2 * r.y, r.z);
+          fma_(v[1], two * u.x, r.z); fma_(v[1], -two * u.y, r.w);
+          fma_(v[2], two * u.x, r.w); fma_(v[2], two * u.y, r.z);
         }
       }
     };
@@ -1057,8 +1091,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       for (int e = tid; e < nh; e += kTPB) {
         const W4 r = X[e];
         norms(e, r, v);
-        const T k0 = kk(e, 0), k1 = kk(e, NC - 1);
-        const W4 q = {k0 * r.x, k0 * r.y, k1 * r.z, k1 * r.w};
+        const W4 q = apply_k(e, r);
         X[xs + e] = q;
         scatter(e, q);
       }
@@ -1077,6 +1110,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
           st.stop = fmax(a.tol2 * rr, a.rr_abs ? a.rr_abs[c0 + lane] : 0.0);
           st.qbest = rr;
           st.rr0 = rr;
+          st.rmax = rr;
           st.near = -1;
           st.active = act = (on[lane] && rr > 0.0) ? 1 : 0;
         }
@@ -1199,16 +1233,21 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
             const double qb = st.tau2;
             if (qb < 0.25 * st.qbest) { st.qbest = qb; st.itb = it; }
             if (st.near < 0 && qb <= 4.0 * st.stop) st.near = it;
+            st.rmax = fmax(st.rmax, rr);
+            st.apart = rr > 1e4 * qb ? st.apart + 1 : 0;
             bool stop = false;
             if (st.flag == 2 || !isfinite(st.tau2)) { st.flag = 2; stop = true; }
             else if (qb <= st.stop) { st.flag = 0; stop = true; }
             else if (!(rn.x * rn.x + rn.y * rn.y > 0.0)) { st.flag = 2; stop = true; }
             else if (it >= a.maxit) { st.flag = 1; stop = true; }
             else if (it - st.itb > max(kQmrWindow, 2 * st.itb)) { st.flag = 4; stop = true; }
-            else if (sizeof(T) == 4 && qb <= 1e-8 * st.rr0 && it - st.itb > kQmrWindowFloor) { st.flag = 4; stop = true; }
+            else if (sizeof(T) == 4 && qb <= fmax(1e-8 * st.rr0, 4e-12 * st.rmax) && it - st.itb > kQmrWindowFloor) {
+              st.flag = 4;
+              stop = true;
+            } else if (sizeof(T) == 4 && st.apart > kApartWait) { st.flag = 4; stop = true; }
             // tau never grows: short of the target after this, the FP64 residual of
-            // the refinement decides (1104 columns on 32^3: one or two of them kept
-            // the pass going for 1000 iterations after the others' 190)
+            // the refinement decides (1104 columns on 32^3, 256 on 64^3: one or two
+            // kept the pass going for 1000 iterations after the others' 80)
             else if (st.near >= 0 && it - st.near > kNearWait) { st.flag = 4; stop = true; }
             if (stop) st.active = 0;
           }
@@ -1227,7 +1266,6 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         const T bx = (T)s_q[0].beta.x, by = (T)(PAIR ? s_q[1].beta.x : s_q[0].beta.y);
         for (int e = tid; e < nh; e += kTPB) {
           W4 q = X[xs + e], d = X[2 * xs + e], x = X[3 * xs + e];
-          const T k0 = kk(e, 0), k1 = kk(e, NC - 1);
           if (PAIR) {
             if (u0) { d.x = d0 * d.x + qx * q.x; d.y = d0 * d.y + qx * q.y; x.x += d.x; x.y += d.y; }
             if (u1) { d.z = d1 * d.z + qy * q.z; d.w = d1 * d.w + qy * q.w; x.z += d.z; x.w += d.w; }
@@ -1241,15 +1279,15 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
           X[2 * xs + e] = d;
           X[3 * xs + e] = x;
           if (!any) continue;
-          const W4 r = X[e];
+          const W4 z = apply_k(e, X[e]);
           if (PAIR) {
-            q.x = a0 ? k0 * r.x + bx * q.x : (T)0;
-            q.y = a0 ? k0 * r.y + bx * q.y : (T)0;
-            q.z = a1 ? k1 * r.z + by * q.z : (T)0;
-            q.w = a1 ? k1 * r.w + by * q.w : (T)0;
+            q.x = a0 ? z.x + bx * q.x : (T)0;
+            q.y = a0 ? z.y + bx * q.y : (T)0;
+            q.z = a1 ? z.z + by * q.z : (T)0;
+            q.w = a1 ? z.w + by * q.w : (T)0;
           } else {
-            q = W4{k0 * r.x + bx * q.x - by * q.y, k0 * r.y + bx * q.y + by * q.x,
-                   k0 * r.z + bx * q.z - by * q.w, k0 * r.w + bx * q.w + by * q.z};
+            q = W4{z.x + bx * q.x - by * q.y, z.y + bx * q.y + by * q.x,
+                   z.z + bx * q.z - by * q.w, z.w + bx * q.w + by * q.z};
           }
           X[xs + e] = q;
           scatter(e, q);

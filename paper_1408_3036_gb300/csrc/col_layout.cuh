@@ -49,7 +49,7 @@ __host__ __device__ inline Lay layout(int kind, const ColShape& sh, int N, int P
   L.C = up16(L.X + (sh.vec_smem ? 4 * (size_t)nhl * s4 : 0));
   L.V = up16(L.C + (sh.c_smem ? (size_t)nproj * nhl * sv : 0));
   L.K = up16(L.V + (sh.v_smem ? (size_t)nzl * N * N * sizeof(T) : 0));
-  L.kin = up16(L.K + (size_t)nhl * (kind == COL_QMR ? 1 : 2) * sizeof(T));
+  L.kin = up16(L.K + (size_t)nhl * 2 * sizeof(T));
   L.hpos = up16(L.kin + (size_t)nhl * sizeof(T));
   L.rt = up16(L.hpos + (size_t)nhl * sizeof(unsigned));
   L.own = up16(L.rt + (size_t)N * P * sizeof(unsigned short));

@@ -90,3 +90,21 @@ def test_full_sphere_and_complex_fields():
         a, b = both_routes(c, gap, f, om, gw.GW_FP64)
         c.close()
         assert rel(a, b) < TOL[0]
+
+
+@pytest.mark.parametrize("om", [0.957 + 0.1j, -0.957 - 0.1j, 0.05 - 0.02j, 3.0 + 0.5j, 0.5j])
+def test_preconditioner_of_the_shift(om):
+    """Denominators around zero (real parts inside the kinetic spectrum, either
+    sign of the imaginary part) against the solver without a preconditioner:
+    |Im| >= 0.02 and |H - E| < 15 Ha keep the condition number below 2e3.  A
+    single-precision pass ends with its columns, not with the 1000 iterations
+    of the stagnation window."""
+    for prec in (gw.GW_FP64, gw.GW_MIXED):
+        c, _ = cell_of(20, 8.0, 4.0, 5)
+        f = W.random_fields(8, 4, 20 ** 3, complex_=True)
+        a = c.apply_chi0(f, [om], prec)
+        assert c.stats()["max_iter"] < 900
+        c.set_precond(0)
+        b = c.apply_chi0(f, [om], prec)
+        c.close()
+        assert rel(a, b) < TOL[prec]
