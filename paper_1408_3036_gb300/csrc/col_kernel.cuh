@@ -44,21 +44,25 @@
 // Scalars of the recurrences come from ordered sums that every CTA of the
 // cluster forms from the same partial sums: all CTAs decide alike.
 //
-// What bounds it: the latency of one unit's iteration (barriers of the
-// cluster, shared-memory passes of the transforms; FP64 the FP64 pipe).
-// FP32 at 48^3, 16 rows, Q = 16: 41k cycles an iteration, of which the slabs'
-// seven passes 19k, z passes 6k, projector 6k, three cluster barriers 4k;
-// FP64 390k, of which the transforms 280k (FP64 instructions issue once in 64
-// cycles and scheduler here, so sums are halved across the lanes instead of
-// repeated in them, and scalar steps share one division).
+// What bounds it: FP32 the latency of one unit's iteration (48^3, 16 rows, Q =
+// 16: 39k cycles, of which the slabs' seven passes 13k, z passes 4k, update 4k,
+// projector 5k, three cluster barriers and scalar steps the rest), and the
+// occupied rows where they don't fit beside the vectors: 69 rows of 1055
+// entries, read twice an iteration by every SM at about 12 TB/s out of L2, 31k
+// of 110k cycles.  FP64 the FP64 pipe, which takes one warp instruction in 64
+// cycles and scheduler here: sums are halved across the lanes instead of
+// repeated in them, scalar steps share one division, products are accumulated
+// in chains of fused multiply-adds (a += x y + z w is three instructions, not
+// two) and the transforms keep the fewest operations (dft in fft.cuh).
 // Measured on a GB300, one application, before (launches per step, or the
 // grid-wide task queue of kernels_cg.cu, with the Teter-Payne-Allan form) and
-// after, of which the preconditioner alone in brackets: 48^3 grid, 12053 plane
-// waves, 16 CG columns, FP32 3.70 -> 1.58 ms (1.65 -> 1.58), FP64 15.8 -> 9.8 ms
-// (10.9 -> 9.8); 45^3, 2007 plane waves, 22 complex columns 11.7 -> 2.29 ms
-// (3.2 -> 2.29); 32^3, 2109 plane waves, 69 rows, 1104 complex columns 400 ->
-// 30.5 ms (58 -> 30.5); 64^3, 38401 plane waves, 64 rows, 256 complex columns
-// 1051 -> 113 ms (386 -> 113).
+// after; in brackets what the preconditioner, then the multiply-adds and
+// transforms took off: 48^3 grid, 12053 plane waves, 16 CG columns, FP32 3.70 ->
+// 1.55 ms (1.65, 1.57, 1.55), FP64 15.8 -> 8.9 ms (10.9, 9.8, 8.9); 45^3, 2007
+// plane waves, 22 complex columns 11.7 -> 2.24 ms (3.2, 2.29, 2.24); 32^3, 2109
+// plane waves, 69 rows, 1104 complex columns 400 -> 29.1 ms (58, 30.5, 29.1);
+// 64^3, 38401 plane waves, 64 rows, 256 complex columns 1051 -> 108 ms (386, 113,
+// 108; of the last step the coefficient sums of kernels_half.cu are the most).
 #pragma once
 
 #include <cooperative_groups.h>
@@ -147,65 +151,7 @@ template <int M, typename A> __device__ __forceinline__ A warp_sums(A* v) {
 }
 __host__ __device__ constexpr int pow2_up(int n) { int p = 1; while (p < n) p *= 2; return p; }
 
-// --- R-point transforms in registers
-template <typename T, int S> __device__ __forceinline__ cpx<T> rot(cpx<T> a, T c, T s) {   // a (c + S i s)
-  return S > 0 ? mk<T>(a.x * c - a.y * s, a.y * c + a.x * s) : mk<T>(a.x * c + a.y * s, a.y * c - a.x * s);
-}
-template <typename T, int S, int R> __device__ __forceinline__ void dft(cpx<T>* v) {
-  using V = cpx<T>;
-  if constexpr (R <= 5) {
-    if constexpr (R > 1) butterfly<T, S>(v, R);
-  } else if constexpr (R == 9) {
-    const T c1 = (T)0.76604444311897803520, s1 = (T)0.64278760968653932632;   // exp(2 pi i / 9)
-    const T c2 = (T)0.17364817766693034885, s2 = (T)0.98480775301220805937;
-    const T c4 = (T)-0.93969262078590838405, s4 = (T)0.34202014332566873304;
-    V a[3][3];
-#pragma unroll
-    for (int n2 = 0; n2 < 3; ++n2) {
-#pragma unroll
-      for (int n1 = 0; n1 < 3; ++n1) a[n2][n1] = v[3 * n1 + n2];
-      butterfly<T, S>(a[n2], 3);
-    }
-    a[1][1] = rot<T, S>(a[1][1], c1, s1);
-    a[1][2] = rot<T, S>(a[1][2], c2, s2);
-    a[2][1] = rot<T, S>(a[2][1], c2, s2);
-    a[2][2] = rot<T, S>(a[2][2], c4, s4);
-#pragma unroll
-    for (int k1 = 0; k1 < 3; ++k1) {
-      V b[3] = {a[0][k1], a[1][k1], a[2][k1]};
-      butterfly<T, S>(b, 3);
-#pragma unroll
-      for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = b[k2];
-    }
-  } else {                                   // 6, 8, 10: two interleaved transforms of R / 2 points
-    constexpr int H = R / 2;
-    V e[H], o[H];
-#pragma unroll
-    for (int k = 0; k < H; ++k) { e[k] = v[2 * k]; o[k] = v[2 * k + 1]; }
-    butterfly<T, S>(e, H);
-    butterfly<T, S>(o, H);
-    if constexpr (R == 6) {
-      const T h = (T)0.86602540378443864676;
-      o[1] = rot<T, S>(o[1], (T)0.5, h);
-      o[2] = rot<T, S>(o[2], (T)-0.5, h);
-    } else if constexpr (R == 8) {
-      const T h = (T)0.70710678118654752440;
-      const V p = o[1], q = o[3];
-      o[1] = S > 0 ? mk<T>((p.x - p.y) * h, (p.x + p.y) * h) : mk<T>((p.x + p.y) * h, (p.y - p.x) * h);
-      o[2] = mul_i(o[2], S);
-      o[3] = S > 0 ? mk<T>(-(q.x + q.y) * h, (q.x - q.y) * h) : mk<T>((q.y - q.x) * h, -(q.x + q.y) * h);
-    } else {
-      const T c1 = (T)0.80901699437494742410, s1 = (T)0.58778525229247312917;   // exp(2 pi i / 10)
-      const T c2 = (T)0.30901699437494742410, s2 = (T)0.95105651629515357212;
-      o[1] = rot<T, S>(o[1], c1, s1);
-      o[2] = rot<T, S>(o[2], c2, s2);
-      o[3] = rot<T, S>(o[3], -c2, s2);
-      o[4] = rot<T, S>(o[4], -c1, s1);
-    }
-#pragma unroll
-    for (int k = 0; k < H; ++k) { v[k] = cadd(e[k], o[k]); v[k + H] = csub(e[k], o[k]); }
-  }
-}
+// --- R-point transforms in registers: dft (fft.cuh)
 // v[k] *= w_N^(S k m)  (stw holds exp(-2 pi i k / N); k m < N)
 template <typename T, int S, int R> __device__ __forceinline__ void twid(cpx<T>* v, const cpx<T>* stw, int m) {
 #pragma unroll
@@ -707,16 +653,16 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         }
 #pragma unroll
         for (int q = 0; q < RG; ++q) {
-          acc[q * NV] += c[q].x * y.x + c[q].y * y.y;
-          acc[q * NV + 1] += c[q].x * y.z + c[q].y * y.w;
+          acc[q * NV] = fma(c[q].y, y.y, fma(c[q].x, y.x, acc[q * NV]));
+          acc[q * NV + 1] = fma(c[q].y, y.w, fma(c[q].x, y.z, acc[q * NV + 1]));
         }
         if (CG) {
           W4 u = Tm[a.nhl + e];
           if (h0 + e == 0) { u.x *= (T)0.5; u.z *= (T)0.5; }
 #pragma unroll
           for (int q = 0; q < RG; ++q) {
-            acc[q * NV + NV - 2] += c[q].x * u.x + c[q].y * u.y;
-            acc[q * NV + NV - 1] += c[q].x * u.z + c[q].y * u.w;
+            acc[q * NV + NV - 2] = fma(c[q].y, u.y, fma(c[q].x, u.x, acc[q * NV + NV - 2]));
+            acc[q * NV + NV - 1] = fma(c[q].y, u.w, fma(c[q].x, u.z, acc[q * NV + NV - 1]));
           }
         }
       }
@@ -1187,10 +1133,10 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
             if (a0) { r.x -= ax * t.x; r.y -= ax * t.y; }
             if (a1) { r.z -= ay * t.z; r.w -= ay * t.w; }
           } else {
-            r.x -= ax * t.x - ay * t.y;
-            r.y -= ax * t.y + ay * t.x;
-            r.z -= ax * t.z - ay * t.w;
-            r.w -= ax * t.w + ay * t.z;
+            r.x = fma(ay, t.y, fma(-ax, t.x, r.x));
+            r.y = fma(-ay, t.x, fma(-ax, t.y, r.y));
+            r.z = fma(ay, t.w, fma(-ax, t.z, r.z));
+            r.w = fma(-ay, t.z, fma(-ax, t.w, r.w));
           }
           X[e] = r;
           norms(e, r, v);
