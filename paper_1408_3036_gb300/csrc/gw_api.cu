@@ -54,7 +54,8 @@ struct gw_ctx {
                                       // by one, -1 the column solver where it fits, else replayed
   int imag_route = GW_IMAG_SQMR;      // solver of purely imaginary frequencies (gw_set_imaginary_route)
   double recycle_w0 = 0.0;            // > 0: recycled bases augmented with x(i w0)
-  bool use_tc = false;                // tensor-core projector coefficients where they apply (opt-in)
+  int use_tc = -1;                    // SQMR projector coefficients: -1 the column solver's, 0 / 1 those of the
+                                      // launches per step on the CUDA cores / on the tensor cores where they apply
   bool tune = true;                   // launch shapes picked by timing (tune.cu)
   int pcg_tpb = 0;                    // CTA width of the last persistent CG launch
   bool tc_ok = false;                 // the split occupied rows and their tensor maps are ready
@@ -732,7 +733,7 @@ gw_status qmr_solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E,
   dots.coef = ctx->work.coef;
   // Mixed path with many columns: the projector coefficients <C_v|t> on the
   // tensor cores (kernels_tc.cu) instead of the dots fused into the gather
-  const bool tc = std::is_same<T, float>::value && ctx->use_tc && ctx->tc_ok && ncol >= kTcMinCols;
+  const bool tc = std::is_same<T, float>::value && ctx->use_tc > 0 && ctx->tc_ok && ncol >= kTcMinCols;
   float* tc_part = nullptr;
   int* tc_err = nullptr;
   if (tc) {
@@ -833,7 +834,7 @@ template <typename U>
 gw_status inner_solve(gw_ctx* ctx, bool qmr, int ncol, const double2* r64, const double2* E, const int* oact,
                       cpx<U>* d, double2* x64, double tol_in, const double* rra, const double* tk, bool sym,
                       bool real_shift, long long* it_sum, int* it_max, const double* w2 = nullptr) {
-  const bool col = !w2 && (qmr ? ctx->use_graphs < 0 && !ctx->use_tc
+  const bool col = !w2 && (qmr ? ctx->use_graphs < 0 && ctx->use_tc < 0
                                : sym && (ctx->cg_kernel < 0 || ctx->cg_kernel == GW_CG_CLUSTER));
   bool ran = false;
   if (col) {
@@ -3244,7 +3245,7 @@ gw_status gw_set_autotune(gw_ctx* ctx, int on) {
 
 gw_status gw_set_tensor_cores(gw_ctx* ctx, int on) {
   if (!ctx) return GW_E_ARG;
-  ctx->use_tc = (on != 0);
+  ctx->use_tc = (on != 0) ? 1 : 0;
   return GW_OK;
 }
 
