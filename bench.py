@@ -677,8 +677,9 @@ def run_gpu(args):
             X0 = bw.starts[0]
             kb = args.block_freq_steps
             rows = []
-            for tc_on in (0, 1):
-                bcell.set_tensor_cores(tc_on)
+            for tc_on in (None, 1):            # the default route, then the tensor-core projector
+                if tc_on is not None:
+                    bcell.set_tensor_cores(tc_on)
                 flush.fill_(1.0)
                 e0 = torch.cuda.Event(enable_timing=True)
                 e1 = torch.cuda.Event(enable_timing=True)
@@ -691,7 +692,6 @@ def run_gpu(args):
                                  applies_per_s=kb * X0.shape[0] / (e0.elapsed_time(e1) / 1e3),
                                  sqmr_mean_iter=stb["mean_iter"], sqmr_max_iter=stb["max_iter"],
                                  sqmr_columns=stb["columns"], graph_replays=stb["graph_replays"]))
-            bcell.set_tensor_cores(0)
             bfl = dict(workload="L=24 bohr, 64^3, 15 Ha (%d PW), 24 wells, N_occ=64, block 8, omega=%.4f+0.1i"
                        % (bcell.npw, om.real), block_steps=kb, precision=args.prec, runs=rows,
                        unit="eps~ applications (block columns) per second")
@@ -726,16 +726,18 @@ def run_gpu(args):
         t_prep = time.perf_counter() - t_prep
         bst = [x[0] for x in bw.starts]
         rows = []
-        for graphs in (1, 0):
+        for graphs in (None, 1, 0):        # the default route, then the launches per step
             for i in range(len(bw.cells)):
-                bt.cell(i).set_graphs(graphs)
+                if graphs is not None:
+                    bt.cell(i).set_graphs(graphs)
             torch.cuda.synchronize()
             t0 = time.perf_counter()
             bt.lanczos(bst, args.batch_k, bom, prec)
             torch.cuda.synchronize()
             dt = time.perf_counter() - t0
             replays = sum(gw.gw_stats(bt.cell(i).ctx)["graph_replays"] for i in range(len(bw.cells)))
-            rows.append(dict(cuda_graphs=bool(graphs), s=dt,
+            rows.append(dict(route="default" if graphs is None else "launches per step",
+                             cuda_graphs=bool(graphs), s=dt,
                              applies_per_s=len(bw.cells) * bom.shape[1] * args.batch_k / dt,
                              status_ok=int((bt.last_status == 0).sum()),
                              graph_replays_last_solve=int(replays)))
