@@ -73,7 +73,6 @@ struct ColArgs {
   const double2* E;              // [ncol]
   const double* rr_abs;          // [ncol] or null
   const double* tk;              // [ncol] or null
-  const int* order;              // [nunit] launch order of the units, or null
   double tol2;
   T* vecs;                       // [nunit][vec_elems]
   int* iters;                    // [ncol]

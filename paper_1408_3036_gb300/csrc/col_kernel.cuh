@@ -194,8 +194,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   cgr::cluster_group cl = cgr::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int Q = 1 << a.sh.lq, rank = Q > 1 ? (int)cl.block_rank() : 0;
-  int unit = blockIdx.x >> a.sh.lq;
-  if (a.order) unit = a.order[unit];
+  const int unit = blockIdx.x >> a.sh.lq;
   const int c0 = PAIR ? 2 * unit : unit, nc = min(NC, a.ncol - c0);
   bool on[2] = {false, false};
   for (int c = 0; c < nc; ++c) on[c] = !a.outer_active || a.outer_active[c0 + c];

@@ -987,8 +987,6 @@ void launch_model_scale(cudaStream_t s, int npw, int nout, const T* kin, const c
 }
 template void launch_model_scale<double>(cudaStream_t, int, int, const double*, const double2*, const int*,
                                          const double2*, const double2*, double2*);
-template void launch_model_scale<float>(cudaStream_t, int, int, const float*, const float2*, const int*,
-                                        const double2*, const double2*, float2*);
 
 // precision changes at the boundary of an FP32 pipeline; out = x - z (FP64 result)
 // Eq. subs_epsilon in the two bases: out[i][j] = sum_ab a_ia (Ti_ab - (M^-1)_ab) a_jb
