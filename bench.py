@@ -301,18 +301,18 @@ def model_bytes(N, npw, nocc, s):
 
 def src_hash():
     h = hashlib.sha256()
-    for f in ("fft.cuh", "kernels_fft.cu", "kernels_linalg.cu", "gw_common.cuh", "kernels_cg.cu", "col.cuh", "col_kernel.cuh"):
+    for f in ("fft.cuh", "gw_common.cuh", "linalg.cuh", "col.cuh", "col_layout.cuh", "col_kernel.cuh", "kernels_col.cu"):
         with open(os.path.join(ROOT, "paper_1408_3036_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
 
 def ncu_traffic(kernel_class):
-    """DRAM bytes per column-iteration of the persistent CG kernel from the
-    committed ncu summary, if it was taken on the current kernel sources."""
+    """DRAM bytes per column-iteration of the CG passes from the committed ncu
+    summary, if it was taken on the current kernel sources."""
     if kernel_class != "persistent_cg":
         return None
-    p = os.path.join(ROOT, "profiles", "k_cg_persistent_molecule.md")
+    p = os.path.join(ROOT, "profiles", "k_col_solve_molecule.md")
     try:
         with open(p) as f:
             for line in f:
