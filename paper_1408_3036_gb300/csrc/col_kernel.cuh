@@ -191,6 +191,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   __shared__ CgCol<T> s_cg[2];
   __shared__ QmrCol s_q[2];
   __shared__ int s_any;
+  __shared__ int s_top[2];                        // FP32: high word of the columns' largest component
   cgr::cluster_group cl = cgr::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int Q = 1 << a.sh.lq, rank = Q > 1 ? (int)cl.block_rank() : 0;
@@ -230,6 +231,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 
   // ---- tables
   if (tid <= Q) s_pb[tid] = a.split[a.sh.lq * (kColMaxQ + 1) + tid];
+  if (tid < 2) s_top[tid] = 0;
   __syncthreads();
   const int p0 = s_pb[rank], npl = s_pb[rank + 1] - p0, nrl = 2 * npl;
   const int h0 = a.hstart[p0], nh = a.hstart[p0 + npl] - h0;
@@ -283,6 +285,40 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     const T* v = a.Vp + (size_t)z0 * N * N;
     for (int k = tid; k < nsl * N * N; k += kTPB) Vs[k] = v[k];
   }
+  // FP32 passes run on the right-hand side times the power of two that brings
+  // its largest component to 1 .. 2 (exact; nothing else depends on the size of
+  // b): unscaled, products of its entries leave the range below 1e-22 and their
+  // rounding errors below 3e-16, where a refinement's later passes arrive.
+  int ex[2] = {0, 0};
+  if constexpr (sizeof(T) == 4) {
+    int top[2] = {0, 0};
+    auto hi = [](double x) { return __double2hiint(x) & 0x7fffffff; };
+    for (int e = tid; e < nh; e += kTPB) {
+      const int g = a.gp[h0 + e], m = a.gm[h0 + e];
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+        if (on[c]) {
+          const double2 u = a.b64[(size_t)(c0 + c) * a.npw + g], w = a.b64[(size_t)(c0 + c) * a.npw + m];
+          top[c] = max(max(top[c], max(hi(u.x), hi(u.y))), max(hi(w.x), hi(w.y)));
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      top[c] = __reduce_max_sync(0xffffffffu, top[c]);
+      if (lane == 0) atomicMax(&s_top[c], top[c]);
+    }
+    csync();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      int t = 0;
+      for (int q = 0; q < Q; ++q) t = max(t, *at(&s_top[c], q));
+      ex[c] = min(max((t >> 20) - 1023, -1021), 1022);
+    }
+  }
+  // 2^-ex of column c, and back
+  auto scale_in = [&](int c) { return sizeof(T) == 4 ? __hiloint2double((1023 - (c ? ex[1] : ex[0])) << 20, 0) : 1.0; };
+  auto scale_out = [&](int c) { return sizeof(T) == 4 ? __hiloint2double((1023 + (c ? ex[1] : ex[0])) << 20, 0) : 1.0; };
+  auto stop_abs = [&](int c) { return a.rr_abs ? a.rr_abs[c0 + c] * scale_in(c) * scale_in(c) : 0.0; };
   for (int e = tid; e < nh; e += kTPB) {
     const int h = h0 + e;
     const T k = a.kin[h];
@@ -308,12 +344,13 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       for (int c = 0; c < 2; ++c)
         if (on[c]) {
           const double2 u = a.b64[(size_t)(c0 + c) * a.npw + g], w = a.b64[(size_t)(c0 + c) * a.npw + m];
-          b[c] = make_double2(0.5 * (u.x + w.x), 0.5 * (u.y - w.y));
+          b[c] = make_double2(0.5 * scale_in(c) * (u.x + w.x), 0.5 * scale_in(c) * (u.y - w.y));
         }
       r = {(T)b[0].x, (T)b[0].y, (T)b[1].x, (T)b[1].y};
     } else {
       const double2 u = a.b64[(size_t)c0 * a.npw + g], w = a.b64[(size_t)c0 * a.npw + m];
-      r = {(T)u.x, (T)u.y, (T)w.x, (T)w.y};
+      const double f = scale_in(0);
+      r = {(T)(f * u.x), (T)(f * u.y), (T)(f * w.x), (T)(f * w.y)};
       if (h == 0) r.z = r.w = (T)0;
     }
     const W4 zero = {(T)0, (T)0, (T)0, (T)0};
@@ -915,7 +952,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
           CgCol<T>& st = s_cg[lane];
           const T gam = val_(g), rr = val_(q);
           if (k == 0) {
-            const T s1 = (T)a.tol2 * rr, s2 = (a.rr_abs && lane < nc) ? (T)a.rr_abs[c0 + lane] : (T)0;
+            const T s1 = (T)a.tol2 * rr, s2 = lane < nc ? (T)stop_abs(lane) : (T)0;
             st.stop = s1 > s2 ? s1 : s2;
             st.rmin = rr;
             st.rbest = rr;
@@ -1052,7 +1089,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
           QmrCol& st = s_q[lane];
           st.tau2 = rr;
           st.rho = make_double2(rx, PAIR ? 0.0 : ry);
-          st.stop = fmax(a.tol2 * rr, a.rr_abs ? a.rr_abs[c0 + lane] : 0.0);
+          st.stop = fmax(a.tol2 * rr, stop_abs(lane));
           st.qbest = rr;
           st.rr0 = rr;
           st.rmax = rr;
@@ -1250,12 +1287,13 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     for (int c = 0; c < NC; ++c) {
       if (c >= nc || !on[c]) continue;
       double2* o = a.x64 + (size_t)(c0 + c) * a.npw;
-      const double ux = c ? (double)x.z : (double)x.x, uy = c ? (double)x.w : (double)x.y;
+      const double f = scale_out(c);
+      const double ux = f * (c ? (double)x.z : (double)x.x), uy = f * (c ? (double)x.w : (double)x.y);
       double2 y = o[g];
       o[g] = make_double2(y.x + ux, y.y + uy);
       if (h == 0) continue;
       y = o[m];
-      o[m] = PAIR ? make_double2(y.x + ux, y.y - uy) : make_double2(y.x + (double)x.z, y.y + (double)x.w);
+      o[m] = PAIR ? make_double2(y.x + ux, y.y - uy) : make_double2(y.x + f * (double)x.z, y.y + f * (double)x.w);
     }
   }
   if (rank == 0 && tid < nc) {

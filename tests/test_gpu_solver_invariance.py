@@ -1,0 +1,63 @@
+"""What a Sternheimer solve must not depend on, whatever route it takes."""
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import pw
+from tests.conftest import rel
+
+pytestmark = pytest.mark.gpu
+
+gw = pytest.importorskip("paper_1408_3036_gb300")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_1408_3036_gb300 import _build
+    _build.build()
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+@pytest.fixture(scope="module")
+def system():
+    """16^3, 179 plane waves, 6 states: gap 0.052 Ha, |H - E| < 12 Ha."""
+    L, N, ecut = 8.0, 16, 4.0
+    rng = np.random.default_rng(1604)
+    v = W.gaussian_wells(L, N, rng.uniform(0.0, L, size=(3, 3)), -2.0, 1.0)
+    gs = pw.ground_state_dense(pw.Sphere(L, N, ecut), v, 6)
+    gap = float(gs.eps_all[6] - gs.eps_all[5])
+    assert gap > 0.05
+    return L, N, ecut, v, gs, gap
+
+
+def cell_of(system, shift=0.0):
+    L, N, ecut, v, gs, _ = system
+    c = gw.Cell(L, N, ecut, v + shift)
+    c.set_occupied(gs.C_all[:6], gs.eps_all[:6] + shift)
+    return c
+
+
+def omega_of(om, gap):
+    return 0.4 * gap if om == "real" else om
+
+
+# |H - E| < 12 Ha and shifts 0.03 Ha or more from a transition: condition below
+# 400.  Two solutions of backward error tol (10 tol where the refinement
+# stagnates) differ by less than 2 10 tol 400, so 1e-6 and 1e-8 for 1e-10, 1e-12.
+@pytest.mark.parametrize("tol,err", [(1e-10, 1e-6), (1e-12, 1e-8)])
+@pytest.mark.parametrize("om", [0.0, "real", 0.3 + 0.1j])
+def test_amplitude_of_the_field(system, om, tol, err):
+    """chi0 is linear: a small field takes the passes of a large one, and the
+    mixed path reaches the same accuracy."""
+    c = cell_of(system)
+    c.set_solver(tol=tol)
+    f = W.random_fields(3, 2, system[1] ** 3)
+    om = omega_of(om, system[5])
+    one = c.apply_chi0(f, [om], gw.GW_MIXED)
+    passes = c.stats()["outer"]
+    for s in (1e-12, 1e-16, 1e-20, 1e-30, 1e20):
+        assert rel(c.apply_chi0(s * f, [om], gw.GW_MIXED) / s, one) < err
+        assert c.stats()["outer"] <= passes + 1
+    c.close()
