@@ -77,6 +77,7 @@ struct ColArgs {
   T* vecs;                       // [nunit][vec_elems]
   int* iters;                    // [ncol]
   int* flags;                    // [ncol]
+  double* xmax;                  // [ncol] largest component of x64 (to a factor 2), for the pairs of the residual
 };
 
 // FP64 projector and residual on half entries (kernels_half.cu); rows are

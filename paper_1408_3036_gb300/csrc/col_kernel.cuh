@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   __shared__ CgCol<T> s_cg[2];
   __shared__ QmrCol s_q[2];
   __shared__ int s_any;
-  __shared__ int s_top[2];                        // FP32: high word of the columns' largest component
+  __shared__ int s_top[2], s_xtop[2];             // high words of the columns' largest components: b, x
   cgr::cluster_group cl = cgr::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int Q = 1 << a.sh.lq, rank = Q > 1 ? (int)cl.block_rank() : 0;
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 
   // ---- tables
   if (tid <= Q) s_pb[tid] = a.split[a.sh.lq * (kColMaxQ + 1) + tid];
-  if (tid < 2) s_top[tid] = 0;
+  if (tid < 2) s_top[tid] = s_xtop[tid] = 0;
   __syncthreads();
   const int p0 = s_pb[rank], npl = s_pb[rank + 1] - p0, nrl = 2 * npl;
   const int h0 = a.hstart[p0], nh = a.hstart[p0 + npl] - h0;
@@ -285,14 +285,16 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     const T* v = a.Vp + (size_t)z0 * N * N;
     for (int k = tid; k < nsl * N * N; k += kTPB) Vs[k] = v[k];
   }
-  // FP32 passes run on the right-hand side times the power of two that brings
-  // its largest component to 1 .. 2 (exact; nothing else depends on the size of
-  // b): unscaled, products of its entries leave the range below 1e-22 and their
-  // rounding errors below 3e-16, where a refinement's later passes arrive.
+  // FP32 passes and pairs run on the right-hand side times the power of two that
+  // brings its largest component to 1 .. 2 (exact; nothing else depends on the
+  // size of b).  Unscaled, products of FP32 entries leave the range below 1e-22
+  // and their rounding errors below 3e-16, where a refinement's later passes
+  // arrive; and the rounding errors of one column of a pair land in the other.
+  constexpr bool SCALED = sizeof(T) == 4 || PAIR;
+  auto hi = [](double x) { return __double2hiint(x) & 0x7fffffff; };
   int ex[2] = {0, 0};
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (SCALED) {
     int top[2] = {0, 0};
-    auto hi = [](double x) { return __double2hiint(x) & 0x7fffffff; };
     for (int e = tid; e < nh; e += kTPB) {
       const int g = a.gp[h0 + e], m = a.gm[h0 + e];
 #pragma unroll
@@ -312,12 +314,12 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     for (int c = 0; c < NC; ++c) {
       int t = 0;
       for (int q = 0; q < Q; ++q) t = max(t, *at(&s_top[c], q));
-      ex[c] = min(max((t >> 20) - 1023, -1021), 1022);
+      ex[c] = pow2_exp(__hiloint2double(t, 0));
     }
   }
   // 2^-ex of column c, and back
-  auto scale_in = [&](int c) { return sizeof(T) == 4 ? __hiloint2double((1023 - (c ? ex[1] : ex[0])) << 20, 0) : 1.0; };
-  auto scale_out = [&](int c) { return sizeof(T) == 4 ? __hiloint2double((1023 + (c ? ex[1] : ex[0])) << 20, 0) : 1.0; };
+  auto scale_in = [&](int c) { return SCALED ? pow2_in(c ? ex[1] : ex[0]) : 1.0; };
+  auto scale_out = [&](int c) { return SCALED ? pow2_out(c ? ex[1] : ex[0]) : 1.0; };
   auto stop_abs = [&](int c) { return a.rr_abs ? a.rr_abs[c0 + c] * scale_in(c) * scale_in(c) : 0.0; };
   for (int e = tid; e < nh; e += kTPB) {
     const int h = h0 + e;
@@ -1280,6 +1282,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   }
 
   // ---- the solution of the pass, added to x64 (own entries)
+  int xt[2] = {0, 0};
   for (int e = tid; e < nh; e += kTPB) {
     const int h = h0 + e, g = a.gp[h], m = a.gm[h];
     const W4 x = X[3 * xs + e];
@@ -1290,7 +1293,9 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       const double f = scale_out(c);
       const double ux = f * (c ? (double)x.z : (double)x.x), uy = f * (c ? (double)x.w : (double)x.y);
       double2 y = o[g];
-      o[g] = make_double2(y.x + ux, y.y + uy);
+      y = make_double2(y.x + ux, y.y + uy);
+      o[g] = y;
+      xt[c] = max(xt[c], max(hi(y.x), hi(y.y)));
       if (h == 0) continue;
       y = o[m];
       o[m] = PAIR ? make_double2(y.x + ux, y.y - uy) : make_double2(y.x + f * (double)x.z, y.y + f * (double)x.w);
@@ -1300,7 +1305,15 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     a.iters[c0 + tid] = CG ? s_cg[tid].it : s_q[tid].it;
     a.flags[c0 + tid] = CG ? s_cg[tid].flag : s_q[tid].flag;
   }
+  if (PAIR) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      xt[c] = __reduce_max_sync(0xffffffffu, xt[c]);
+      if (lane == 0) atomicMax(at(&s_xtop[c], 0), xt[c]);
+    }
+  }
   csync();                                        // no CTA leaves while others may reach its memory
+  if (PAIR && rank == 0 && tid < nc && (tid ? on[1] : on[0])) a.xmax[c0 + tid] = __hiloint2double(s_xtop[tid], 0);
 }
 
 template <typename T, int A, int B> const void* kernel_ptr(int kind) {

@@ -344,10 +344,10 @@ gw_status h_apply(gw_ctx* ctx, cpx<T>* x, int ncol, const double2* E, const int*
 // (H - E) x in FP64 for columns that are real in real space, two per complex
 // transform (pack, the pruned passes, split through G and -G with the kinetic
 // part added); act: host mask of the columns wanted (a pair runs when one of
-// its columns is wanted, and both of its outputs are written); with sub, sub -
-// (H - E) x.
+// its columns is wanted, and both of its outputs are written); xmax: the
+// columns' largest components; with sub, sub - (H - E) x.
 gw_status h_apply_sym(gw_ctx* ctx, const double2* x, int ncol, const double2* E, const std::vector<int>& act,
-                      double2* out, const double2* sub = nullptr) {
+                      const double* xmax, double2* out, const double2* sub = nullptr) {
   const int npw = ctx->npw, npair = (ncol + 1) / 2;
   std::vector<int> ia(npair), ib(npair), pact(npair);
   for (int j = 0; j < npair; ++j) {
@@ -365,7 +365,7 @@ gw_status h_apply_sym(gw_ctx* ctx, const double2* x, int ncol, const double2* E,
   TRY(getbuf(ctx, "g_hs", (size_t)npair * ctx->N3, &grid));
   auto& P = ctx->P64;
   const Geometry& g = ctx->geo;
-  launch_pack_pairs(ctx->st, npw, npair, x, dia, dib, dpact, xp);
+  launch_pack_pairs(ctx->st, npw, npair, x, dia, dib, dpact, xp, xmax);
   launch_zpass<double>(ctx->st, Z_SCATTER_INV, g, P, ctx->plan, grid, xp, nullptr, nullptr, nullptr, nullptr, dpact,
                        nullptr, nullptr, npair);
   launch_ypass<double>(ctx->st, 1, 1, 0, g, P, ctx->plan, grid, dpact, npair, 0);
@@ -373,7 +373,7 @@ gw_status h_apply_sym(gw_ctx* ctx, const double2* x, int ncol, const double2* E,
   launch_ypass<double>(ctx->st, 0, 0, 1, g, P, ctx->plan, grid, dpact, npair, 0);
   launch_zpass<double>(ctx->st, Z_GATHER_FWD, g, P, ctx->plan, grid, yp, nullptr, nullptr, nullptr, nullptr, dpact,
                        nullptr, nullptr, npair);
-  launch_unpack_pairs(ctx->st, npw, npair, yp, g.sph_neg, dia, dib, dpact, P.kin, E, x, out, sub);
+  launch_unpack_pairs(ctx->st, npw, npair, yp, g.sph_neg, dia, dib, dpact, P.kin, E, x, out, sub, xmax);
   return launch_check(ctx, "h_apply_sym");
 }
 
@@ -527,7 +527,7 @@ gw_status pcg_pending(gw_ctx* ctx, int ncol, const unsigned* ctl) {
 // there or no cluster holds a unit.
 template <typename T>
 gw_status col_solve(gw_ctx* ctx, int kind, int ncol, const double2* b64, const double2* E, const int* outer_active,
-                    double2* x64, double tol, const double* rr_abs, const double* tk, bool* ran) {
+                    double2* x64, double* xmax, double tol, const double* rr_abs, const double* tk, bool* ran) {
   *ran = false;
   const ColPlan& p = ctx->col;
   if (!p.ok) return GW_OK;
@@ -552,6 +552,7 @@ gw_status col_solve(gw_ctx* ctx, int kind, int ncol, const double2* b64, const d
   if (a.sh.vec_elems) TRY(getbuf(ctx, "col_vecs" + t, a.sh.vec_elems * (size_t)a.nunit, &a.vecs));
   a.iters = ctx->pcg_iters_d;
   a.flags = ctx->pcg_flags_d;
+  a.xmax = xmax;
   const int pa = prof_begin(ctx, kind == COL_CG_PAIR ? PC_PCG : PC_N);
   CK(launch_col_solve<T>(ctx->st, kind, a));
   prof_end(ctx, PC_PCG, pa);
@@ -827,20 +828,21 @@ gw_status qmr_solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E,
 // states).  Each inner solve stops at tol_inner relative to its own right-hand
 // side, or at a tenth of the final target, whichever is larger.
 // ---------------------------------------------------------------------------
-// One inner solve in precision U, its solution added to x64: the column solver
+// One inner solve in precision U, its solution added to x64 (and, sym, the
+// columns' largest components left in xmax[ncol ..]): the column solver
 // where it takes the unit (real columns in pairs; complex columns with
 // simplified QMR), else the persistent or the multi-launch kernels through the
 // buffer d.
 template <typename U>
 gw_status inner_solve(gw_ctx* ctx, bool qmr, int ncol, const double2* r64, const double2* E, const int* oact,
-                      cpx<U>* d, double2* x64, double tol_in, const double* rra, const double* tk, bool sym,
-                      bool real_shift, long long* it_sum, int* it_max, const double* w2 = nullptr) {
+                      cpx<U>* d, double2* x64, double* xmax, double tol_in, const double* rra, const double* tk,
+                      bool sym, bool real_shift, long long* it_sum, int* it_max, const double* w2 = nullptr) {
   const bool col = !w2 && (qmr ? ctx->use_graphs < 0 && ctx->use_tc < 0
                                : sym && (ctx->cg_kernel < 0 || ctx->cg_kernel == GW_CG_CLUSTER));
   bool ran = false;
   if (col) {
     const int kind = !qmr ? COL_CG_PAIR : sym && real_shift ? COL_QMR_PAIR : COL_QMR;
-    TRY(col_solve<U>(ctx, kind, ncol, r64, E, oact, x64, tol_in, rra, tk, &ran));
+    TRY(col_solve<U>(ctx, kind, ncol, r64, E, oact, x64, xmax + ncol, tol_in, rra, tk, &ran));
     if (ran) return GW_OK;
   }
   if (w2) {
@@ -852,8 +854,12 @@ gw_status inner_solve(gw_ctx* ctx, bool qmr, int ncol, const double2* r64, const
       TRY(cg_solve_persistent<U>(ctx, ncol, r64, E, oact, d, tol_in, rra, tk, sym, it_sum, it_max, &ran));
     if (!ran) TRY(cg_solve<U>(ctx, ncol, r64, E, oact, d, tol_in, rra, tk, it_sum, it_max));
   }
-  if (sym) launch_add_conv_sym<U>(ctx->st, ctx->npw, ncol, d, x64, oact, ctx->geo.sph_neg);
-  else launch_add_conv<U>(ctx->st, ctx->npw, ncol, d, x64, oact);
+  if (sym) {
+    launch_add_conv_sym<U>(ctx->st, ctx->npw, ncol, d, x64, oact, ctx->geo.sph_neg);
+    launch_sym_check(ctx->st, ctx->npw, ncol, x64, ctx->geo.sph_neg, xmax);
+  } else {
+    launch_add_conv<U>(ctx->st, ctx->npw, ncol, d, x64, oact);
+  }
   return GW_OK;
 }
 
@@ -876,12 +882,13 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
   TRY(getbuf(ctx, std::string("sv_d") + tname<T>(), (size_t)ncol * npw, &d));
   TRY(getbuf(ctx, "sv_oact", ncol, &oact));
   // what the host reads after a pass, in one copy: |r|^2, |b|^2, |x|^2, then
-  // the iteration counts and flags of a one-launch inner pass
-  TRY(getbuf(ctx, "sv_out", (size_t)4 * ncol, &res2));
+  // the iteration counts and flags of a one-launch inner pass; behind them xmax
+  TRY(getbuf(ctx, "sv_out", (size_t)6 * ncol, &res2));
   bb = res2 + ncol;
   xx = bb + ncol;
   ctx->pcg_iters_d = reinterpret_cast<int*>(xx + ncol);
   ctx->pcg_flags_d = ctx->pcg_iters_d + ncol;
+  double* xmax = res2 + (size_t)4 * ncol;
   if (ctx->sv_pin_n < (size_t)4 * ncol) {
     if (ctx->sv_pin) CK(cudaFreeHost(ctx->sv_pin));
     ctx->sv_pin = nullptr;
@@ -957,15 +964,17 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
     }
     if (esc) {
       if (!d64) TRY(getbuf(ctx, "sv_d64", (size_t)ncol * npw, &d64));
-      TRY(inner_solve<double>(ctx, qmr, ncol, r64, E, oact, reinterpret_cast<cpx<double>*>(d64), x64,
+      TRY(inner_solve<double>(ctx, qmr, ncol, r64, E, oact, reinterpret_cast<cpx<double>*>(d64), x64, xmax,
                               std::max(1e2 * ctx->tol, 1e-11), rra, tk, sym, real_shift, &it_sum, &it_max, w2));
     } else {
-      TRY(inner_solve<T>(ctx, qmr, ncol, r64, E, oact, d, x64, tol_in, rra, tk, sym, real_shift, &it_sum, &it_max,
-                         w2));
+      TRY(inner_solve<T>(ctx, qmr, ncol, r64, E, oact, d, x64, xmax, tol_in, rra, tk, sym, real_shift, &it_sum,
+                         &it_max, w2));
     }
-    if (ctx->ndef > 0)                // the deflated components, exactly
+    if (ctx->ndef > 0) {              // the deflated components, exactly
       launch_proj_update<double>(ctx->st, ctx->P64.C + (size_t)ctx->nocc * npw, ctx->ndef, npw, x64, ncol, oact,
                                  cdef, ctx->work, nullptr, nullptr);
+      if (sym) launch_sym_check(ctx->st, npw, ncol, x64, ctx->geo.sph_neg, xmax);
+    }
     // r64 = P_c (b - (H - E) x64): C^H (H - E) x64 from the dots fused into the
     // last transform pass, C^H b computed once per solve
     if (w2) {
@@ -991,7 +1000,7 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
       // r64 = b - (H - E) x in the last transform pass (two real columns per
       // transform), then P_c and the norms
       const int pa = prof_begin(ctx, PC_REFINE);
-      if (sym) TRY(h_apply_sym(ctx, x64, ncol, E, act, r64, b64));
+      if (sym) TRY(h_apply_sym(ctx, x64, ncol, E, act, xmax + ncol, r64, b64));
       else TRY(h_apply<double>(ctx, x64, ncol, E, oact, r64, nullptr, b64));
       const double2* Ch = ctx->col64.Ch;
       const int n = launch_gram_half(ctx->st, sym, ctx->col, Ch, ctx->nocc, r64, npw, ncol, oact, part);
@@ -1002,7 +1011,7 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
       const int pa = prof_begin(ctx, PC_REFINE);
       if (sym) {
         // two real-in-real-space columns per FP64 transform
-        TRY(h_apply_sym(ctx, x64, ncol, E, act, ax));
+        TRY(h_apply_sym(ctx, x64, ncol, E, act, xmax + ncol, ax));
         launch_gram<double>(ctx->st, ctx->P64.C, ctx->nocc, npw, ax, ncol, ctx->work, cax, true);
       } else {
         GatherDots dots;

@@ -78,6 +78,16 @@ struct FftPlan {
 };
 bool make_plan(int N, FftPlan* p);
 
+#ifdef __CUDACC__
+// Scaling by powers of two (exact): e = floor(log2 |x|), kept where 2^e and
+// 2^-e are normal numbers; x 2^-e is 1 .. 2 in size.
+__device__ __forceinline__ int pow2_exp(double x) {
+  return min(max(((__double2hiint(x) & 0x7fffffff) >> 20) - 1023, -1021), 1022);
+}
+__device__ __forceinline__ double pow2_in(int e) { return __hiloint2double((1023 - e) << 20, 0); }
+__device__ __forceinline__ double pow2_out(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+#endif
+
 // kernel launches issued by this library since it was loaded (host counter)
 extern std::atomic<unsigned long long> g_launches;
 

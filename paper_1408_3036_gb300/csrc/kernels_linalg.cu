@@ -720,42 +720,49 @@ void launch_add_conv_sym(cudaStream_t s, int npw, int ncol, const cpx<T>* d, dou
 
 // Two columns that are real in real space in one complex vector:
 //   out[j](G) = x[ia[j]](G) + i x[ib[j]](G)   (ib[j] < 0: the first alone)
+// With xmax (the columns' largest components) each times the power of two that
+// brings it to 1 .. 2 (exact): the rounding errors of one column land in the
+// other, so a column 1e-4 of its partner would lose four digits, one of 1e-16 all.
 __global__ void k_pack_pairs(size_t npw, const double2* __restrict__ x, const int* __restrict__ ia,
-                             const int* __restrict__ ib, const int* __restrict__ active, double2* __restrict__ out) {
+                             const int* __restrict__ ib, const int* __restrict__ active, double2* __restrict__ out,
+                             const double* __restrict__ xmax) {
   const int j = blockIdx.y;
   if (active && !active[j]) return;
   const int a = ia[j], b = ib[j];
+  const double sa = xmax ? pow2_in(pow2_exp(xmax[a])) : 1.0, sb = xmax && b >= 0 ? pow2_in(pow2_exp(xmax[b])) : 1.0;
   for (size_t G = blockIdx.x * (size_t)blockDim.x + threadIdx.x; G < npw; G += (size_t)gridDim.x * blockDim.x) {
     const double2 u = x[(size_t)a * npw + G];
     const double2 v = (b >= 0) ? x[(size_t)b * npw + G] : make_double2(0.0, 0.0);
-    out[(size_t)j * npw + G] = make_double2(u.x - v.y, u.y + v.x);
+    out[(size_t)j * npw + G] = make_double2(sa * u.x - sb * v.y, sa * u.y + sb * v.x);
   }
 }
 
 void launch_pack_pairs(cudaStream_t s, int npw, int npair, const double2* x, const int* ia, const int* ib,
-                       const int* active, double2* out) {
+                       const int* active, double2* out, const double* xmax) {
   dim3 g((npw + kLT - 1) / kLT, npair);
   ++g_launches;
-  k_pack_pairs<<<g, kLT, 0, s>>>((size_t)npw, x, ia, ib, active, out);
+  k_pack_pairs<<<g, kLT, 0, s>>>((size_t)npw, x, ia, ib, active, out, xmax);
 }
 
 // The two parts of a packed transform Y_j = F(f_a) + i F(f_b) of real fields:
 //   out[ia[j]](G) = (Y_j(G) + conj Y_j(-G)) / 2,  out[ib[j]](G) = (Y_j(G) - conj Y_j(-G)) / 2i,
 // plus (kin(G) - E_c) x_c(G) when kin is given (the kinetic part of (H - E) x);
-// with sub given, sub - that (the residual b - (H - E) x).
+// with sub given, sub - that (the residual b - (H - E) x); xmax as it was packed.
 __global__ void k_unpack_pairs(size_t npw, const double2* __restrict__ Y, const int* __restrict__ neg,
                                const int* __restrict__ ia, const int* __restrict__ ib, const int* __restrict__ active,
                                const double* __restrict__ kin, const double2* __restrict__ E,
                                const double2* __restrict__ x, double2* __restrict__ out,
-                               const double2* __restrict__ sub) {
+                               const double2* __restrict__ sub, const double* __restrict__ xmax) {
   const int j = blockIdx.y;
   if (active && !active[j]) return;
   const int a = ia[j], b = ib[j];
+  const double ha = xmax ? 0.5 * pow2_out(pow2_exp(xmax[a])) : 0.5;
+  const double hb = xmax && b >= 0 ? 0.5 * pow2_out(pow2_exp(xmax[b])) : 0.5;
   for (size_t G = blockIdx.x * (size_t)blockDim.x + threadIdx.x; G < npw; G += (size_t)gridDim.x * blockDim.x) {
     const double2 y1 = Y[(size_t)j * npw + G];
     const double2 yn = Y[(size_t)j * npw + neg[G]];
-    double2 o0 = make_double2(0.5 * (y1.x + yn.x), 0.5 * (y1.y - yn.y));
-    double2 o1 = make_double2(0.5 * (y1.y + yn.y), -0.5 * (y1.x - yn.x));
+    double2 o0 = make_double2(ha * (y1.x + yn.x), ha * (y1.y - yn.y));
+    double2 o1 = make_double2(hb * (y1.y + yn.y), -hb * (y1.x - yn.x));
     if (kin) {
       const double2 xa = x[(size_t)a * npw + G];
       const double dr = kin[G] - E[a].x, di = -E[a].y;
@@ -783,10 +790,10 @@ __global__ void k_unpack_pairs(size_t npw, const double2* __restrict__ Y, const 
 
 void launch_unpack_pairs(cudaStream_t s, int npw, int npair, const double2* Y, const int* neg, const int* ia,
                          const int* ib, const int* active, const double* kin, const double2* E, const double2* x,
-                         double2* out, const double2* sub) {
+                         double2* out, const double2* sub, const double* xmax) {
   dim3 g((npw + kLT - 1) / kLT, npair);
   ++g_launches;
-  k_unpack_pairs<<<g, kLT, 0, s>>>((size_t)npw, Y, neg, ia, ib, active, kin, E, x, out, sub);
+  k_unpack_pairs<<<g, kLT, 0, s>>>((size_t)npw, Y, neg, ia, ib, active, kin, E, x, out, sub, xmax);
 }
 
 // out[c] = max_G |b(G) - conj b(-G)|, out[ncol + c] = max_G |b(G)| (one block per column)

@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 import workloads as W
-from oracle import pw
+from oracle import pw, response
 from tests.conftest import rel
 
 pytestmark = pytest.mark.gpu
@@ -61,3 +61,39 @@ def test_amplitude_of_the_field(system, om, tol, err):
         assert rel(c.apply_chi0(s * f, [om], gw.GW_MIXED) / s, one) < err
         assert c.stats()["outer"] <= passes + 1
     c.close()
+
+
+# FP64: backward error 1e-13 (1e-12), condition below 400: 2 1e-12 400
+@pytest.mark.parametrize("prec,tol,err", [(gw.GW_FP64, 1e-13, 1e-9), (gw.GW_MIXED, 1e-10, 1e-6),
+                                          (gw.GW_MIXED, 1e-12, 1e-8)])
+@pytest.mark.parametrize("om", [0.0, "real", 0.3 + 0.1j])
+def test_fields_of_different_size_in_one_call(system, om, prec, tol, err):
+    """Columns that are real in real space run in pairs, two to a complex
+    transform: the large one's rounding errors stay out of the small one."""
+    c = cell_of(system)
+    c.set_solver(tol=tol)
+    om = omega_of(om, system[5])
+    f = W.random_fields(4, 3, system[1] ** 3)
+    one = c.apply_chi0(f, [om], prec)[0]
+    size = np.array([1.0, 1e-6, 1e-18])
+    two = c.apply_chi0(f * size[:, None], [om], prec)[0]
+    c.close()
+    for b in range(3):
+        assert rel(two[b] / size[b], one[b]) < err
+
+
+@pytest.mark.parametrize("d", [1e-4, 1e-6])
+def test_fp64_next_to_a_transition(system, d):
+    """A real frequency d Ha above the second-lowest transition: one column's
+    solution is 1e4 .. 1e6 times its partners'.  Backward error 1e-13 and
+    |H - E| < 12 Ha: 2 1e-13 12 / d of that column (and the transition energy
+    itself is known to 1e-14 / d)."""
+    gs = system[4]
+    t = np.sort((gs.eps_all[6:, None] - gs.eps_all[None, :6]).ravel())
+    assert np.abs(t[:8] - t[1] - d).min() > 0.9 * d
+    c = cell_of(system)
+    f = W.random_fields(5, 2, system[1] ** 3)
+    a = c.apply_chi0(f, [float(t[1] + d)], gw.GW_FP64)[0]
+    c.close()
+    for b in range(2):
+        assert rel(a[b], np.real(response.chi0_sos(gs, f[b], float(t[1] + d)))) < 4e-12 / d
