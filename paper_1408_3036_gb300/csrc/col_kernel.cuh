@@ -83,7 +83,7 @@ constexpr double kPreReal = 0.03, kPreImag = 0.2;
 // FP32: rounding errors scale with the largest residual of the pass (it peaks
 // in the first steps), so tau goes no further than some 30 ulp of that, now and
 // then 1.5 to 10 times the target; past it the recurrence comes apart, |r|
-// grows to 1e2 .. 1e5 times tau and tau stays.
+// grows to 1e2 .. 1e5 times tau and tau stays (kApartWait: within 10 of it).
 constexpr int kQmrWindow = 1000;     // anywhere (as the multi-launch solver's)
 constexpr int kQmrWindowFloor = 48;  // FP32, tau below 1e-4 |b| or 2e-6 max |r|
 constexpr int kApartWait = 16;       // FP32, iterations in a row with |r| > 100 tau
@@ -1218,14 +1218,17 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
             if (qb < 0.25 * st.qbest) { st.qbest = qb; st.itb = it; }
             if (st.near < 0 && qb <= 4.0 * st.stop) st.near = it;
             st.rmax = fmax(st.rmax, rr);
-            st.apart = rr > 1e4 * qb ? st.apart + 1 : 0;
+            // (a large |r| over a flat tau is ordinary far from the floor: an
+            // eigenvalue close to the shift)
+            const double floor2 = fmax(1e-8 * st.rr0, 4e-12 * st.rmax);
+            st.apart = rr > 1e4 * qb && qb <= 100.0 * floor2 ? st.apart + 1 : 0;
             bool stop = false;
             if (st.flag == 2 || !isfinite(st.tau2)) { st.flag = 2; stop = true; }
             else if (qb <= st.stop) { st.flag = 0; stop = true; }
             else if (!(rn.x * rn.x + rn.y * rn.y > 0.0)) { st.flag = 2; stop = true; }
             else if (it >= a.maxit) { st.flag = 1; stop = true; }
             else if (it - st.itb > max(kQmrWindow, 2 * st.itb)) { st.flag = 4; stop = true; }
-            else if (sizeof(T) == 4 && qb <= fmax(1e-8 * st.rr0, 4e-12 * st.rmax) && it - st.itb > kQmrWindowFloor) {
+            else if (sizeof(T) == 4 && qb <= floor2 && it - st.itb > kQmrWindowFloor) {
               st.flag = 4;
               stop = true;
             } else if (sizeof(T) == 4 && st.apart > kApartWait) { st.flag = 4; stop = true; }

@@ -74,6 +74,7 @@ struct gw_ctx {
     bool fp64 = false, qmr = false;
     std::string tune_key;
   } pcg_pend;
+  std::vector<int> pass_flags;  // its columns' flags (empty: another solver ran)
   int pcg_cluster = 0;          // cluster size of the last persistent launch (0: grid-wide kernel)
   int cta_div = 1;              // contexts sharing the GPU concurrently (batch mode)
   int precond = 1;              // 1: kinetic (TPA) preconditioner in the Sternheimer solvers; 0: none
@@ -660,11 +661,13 @@ gw_status cg_solve_persistent(gw_ctx* ctx, int ncol, const double2* b64, const d
 // synchronised: a bounded wait that gave up (GW_E_TIMEOUT), an FP64 breakdown,
 // the iteration statistics and the autotuner's sample.
 gw_status pcg_finish(gw_ctx* ctx, long long* it_sum, int* it_max) {
+  ctx->pass_flags.clear();
   if (!ctx->pcg_pend.on) return GW_OK;
   ctx->pcg_pend.on = false;
   const int ncol = ctx->pcg_pend.ncol;
   const int* its = reinterpret_cast<const int*>(ctx->sv_pin + 3 * (size_t)ncol);
   const int* fl = its + ncol;
+  ctx->pass_flags.assign(fl, fl + ncol);
   if (*ctx->pcg_err) return fail(ctx, GW_E_TIMEOUT, "persistent CG: a bounded device wait gave up");
   int imax = 0;
   for (int c = 0; c < ncol; ++c) {
@@ -944,10 +947,11 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
   int it_max = 0, outer = 0;
   bool done = false;
   double prev_worst = 1e300;
-  // Mixed path: a pass in which some column far from convergence does not
-  // drop its residual by 10x means the FP32 recurrence cannot resolve that
-  // system (a nearly singular, indefinite shift close to a transition); the
-  // remaining passes then run the inner solver in FP64.
+  // Mixed path: a pass in which some column far from convergence, or one whose
+  // recurrence stagnated (flag 4 of a one-launch pass), does not drop its
+  // residual by 10x means the FP32 recurrence cannot resolve that system (a
+  // nearly singular, indefinite shift close to a transition); the remaining
+  // passes then run the inner solver in FP64.
   bool esc = false;
   double2* d64 = nullptr;
   std::vector<double> hprev;
@@ -1050,7 +1054,8 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
       habs[c] = 0.01 * tol * tol * scale * scale;
       if (be > tol) {
         ++nact;
-        if (mixed && be > 1e3 * tol && hr[c] > 1e-2 * hprev[c]) esc = true;
+        const bool stuck = be > 1e3 * tol || (!ctx->pass_flags.empty() && ctx->pass_flags[c] == 4);
+        if (mixed && stuck && hr[c] > 1e-2 * hprev[c]) esc = true;
       } else {
         act[c] = 0;
       }

@@ -97,3 +97,30 @@ def test_fp64_next_to_a_transition(system, d):
     c.close()
     for b in range(2):
         assert rel(a[b], np.real(response.chi0_sos(gs, f[b], float(t[1] + d)))) < 4e-12 / d
+
+
+@pytest.mark.parametrize("im", [0.0, 1e-4])
+def test_mixed_next_to_transitions(system, im):
+    """Real frequencies all over the spectrum and 1e-3 .. 1e-6 Ha next to its
+    transitions: an indefinite column holds a large residual over a flat
+    quasi-residual for a while, which must not end its pass.  Five passes suffice (as many as
+    the solver of one launch per step takes for these); backward error 1e-10,
+    10 times that where the refinement stagnates, |H - E| < 12 Ha."""
+    gs = system[4]
+    t = np.sort((gs.eps_all[6:, None] - gs.eps_all[None, :6]).ravel())
+    rng = np.random.default_rng(5)
+    oms = np.concatenate([rng.uniform(0.05, 2.5, 60), t[rng.integers(0, 500, 60)]
+                          + rng.choice([-1, 1], 60) * 10 ** rng.uniform(-6, -3, 60)])
+    c = cell_of(system)
+    f = W.random_fields(3, 2, system[1] ** 3)
+    passes = []
+    for om in oms:
+        w = complex(om, im) if im else float(om)
+        a = c.apply_chi0(f, [w], gw.GW_MIXED)[0]
+        passes.append(c.stats()["outer"])
+        d = max(np.abs(t - om).min(), im)
+        for b in range(2):
+            ref = response.chi0_sos(gs, f[b], w)
+            assert rel(a[b], ref if im else np.real(ref)) < 2 * 10 * 1e-10 * 12 / d
+    c.close()
+    assert max(passes) <= 5
