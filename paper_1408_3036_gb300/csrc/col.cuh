@@ -74,6 +74,7 @@ struct ColArgs {
   const double* rr_abs;          // [ncol] or null
   const double* tk;              // [ncol] or null
   double tol2;
+  double v0;                     // level of V in the outer parts of the cell (two thirds lie below it)
   T* vecs;                       // [nunit][vec_elems]
   int* iters;                    // [ncol]
   int* flags;                    // [ncol]

@@ -30,10 +30,15 @@
 // and half entry for either kind, half of what the full sphere takes, and half
 // of the rows' bytes.
 //
-// Preconditioner.  The kinetic denominators of the column's own shift (those of
-// the model operator), kept away from zero: with d = |G|^2/2 - Re E,
+// Preconditioner.  The diagonal of H - E at the column's own shift, kept away
+// from zero: with V0 the level below which V lies in two thirds of the cell and
+// d = |G|^2/2 + V0 - Re E,
 //   real shift     K = 1 / sqrt(d^2 + 0.03^2)   (positive, as CG needs)
 //   complex shift  K = 1 / (d - i (Im E + 0.2 sgn Im E))
+// V0 because a constant in V and the energies changes nothing (without it 16^3,
+// 179 plane waves, V + 3 Ha: static 20 -> 166 iterations, 0.957 + 0.1 i 32 ->
+// 174); not the mean, the diagonal's own, because P_c takes away the states of
+// the wells (mean: 24^3, 619 plane waves, static 18 -> 25 iterations).
 // K(-G) = K(G), so it is symmetric in the bilinear form too.  The
 // Teter-Payne-Allan form of the other kernels knows the kinetic energy of the
 // occupied state but not the shift.  Iterations to 1e-5 (FP64), then and now:
@@ -77,7 +82,11 @@ namespace col {
 namespace cgr = cooperative_groups;
 
 // Smoothing of the preconditioner's denominators (Ha), by scans of 0.02 .. 0.8
-// over static, real, imaginary and complex frequencies on 16^3 .. 48^3 cells.
+// over static, real, imaginary and complex frequencies on 16^3 .. 48^3 cells, wells
+// and barriers, dense and sparse (mean of V -0.76 .. +0.14 Ha).  Of the levels of V
+// tried there (mean, 1/2, 3/5, 2/3, 3/4, 9/10, largest) that of 2/3 is the best or
+// within a tenth of it everywhere: higher ones cost barriers (3/4: 108 -> 145
+// iterations), lower ones dense wells (1/2: 110 -> 125).
 constexpr double kPreReal = 0.03, kPreImag = 0.2;
 // SQMR stagnation: iterations without a halving of the quasi-residual norm tau.
 // FP32: rounding errors scale with the largest residual of the pass (it peaks
@@ -261,10 +270,11 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     zm[k] = (signed char)((j == 0 && k >= npl) ? -1 : (int)a.zmax[j]);
   }
   bool pre[2] = {false, false};
-  T Ex[2] = {(T)0, (T)0}, Ey = (T)0;
+  T Ex[2] = {(T)0, (T)0}, Ep[2] = {(T)0, (T)0}, Ey = (T)0;   // Ep: of the preconditioner
   for (int c = 0; c < nc; ++c) {
     pre[c] = a.tk && a.tk[c0 + c] != 0.0;
     Ex[c] = (T)a.E[c0 + c].x;
+    Ep[c] = (T)(a.E[c0 + c].x - a.v0);
     if (!PAIR) Ey = (T)a.E[c0].y;
   }
   auto precond_real = [](T d) { return (T)1 / sqrt(d * d + (T)(kPreReal * kPreReal)); };
@@ -327,10 +337,10 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     kin[e] = k;
     hpos[e] = a.hpos[h];
     if (PAIR) {
-      Kt[2 * e] = pre[0] ? precond_real(k - Ex[0]) : (T)1;
-      Kt[2 * e + 1] = pre[1] ? precond_real(k - Ex[1]) : (T)1;
+      Kt[2 * e] = pre[0] ? precond_real(k - Ep[0]) : (T)1;
+      Kt[2 * e + 1] = pre[1] ? precond_real(k - Ep[1]) : (T)1;
     } else {
-      const T dr = k - Ex[0], di = Ey > (T)0 ? Ey + (T)kPreImag : Ey - (T)kPreImag;
+      const T dr = k - Ep[0], di = Ey > (T)0 ? Ey + (T)kPreImag : Ey - (T)kPreImag;
       V kc = mk<T>((T)1, (T)0);
       if (pre[0]) {
         if (Ey == (T)0) kc.x = precond_real(dr);

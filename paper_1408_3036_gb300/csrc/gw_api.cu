@@ -82,6 +82,7 @@ struct gw_ctx {
   std::vector<double> tkin;     // kinetic energy of each occupied state (preconditioner reference)
   bool ptime_init = false;
   double vmax = 0.0;            // max |V_loc|
+  double vlevel = 0.0;          // V_loc is below it in two thirds of the cell (column solver's preconditioner)
   int max_iter = 20000, max_outer = 12;
   double stats[6] = {0, 0, 0, 0, 0, 0};
   int* host_pin = nullptr;      // pinned scratch for small read-backs
@@ -549,6 +550,7 @@ gw_status col_solve(gw_ctx* ctx, int kind, int ncol, const double2* b64, const d
   a.split = p.split; a.hstart = p.hstart; a.gp = p.gp; a.gm = p.gm; a.hpos = p.hpos; a.disc = p.disc; a.zmax = p.zmax;
   a.b64 = b64; a.x64 = x64; a.outer_active = outer_active; a.E = E; a.rr_abs = rr_abs; a.tk = tk;
   a.tol2 = tol * tol;
+  a.v0 = ctx->vlevel;
   a.vecs = nullptr;
   if (a.sh.vec_elems) TRY(getbuf(ctx, "col_vecs" + t, a.sh.vec_elems * (size_t)a.nunit, &a.vecs));
   a.iters = ctx->pcg_iters_d;
@@ -2143,6 +2145,18 @@ gw_status upload_prec(gw_ctx* ctx, const std::vector<double>& vloc, const std::v
   return GW_OK;
 }
 
+// Level that two thirds of v lie below, to 1/4096 of its range (a histogram)
+double upper_third(const std::vector<double>& v) {
+  const auto mm = std::minmax_element(v.begin(), v.end());
+  const double lo = *mm.first, step = (*mm.second - lo) / 4096.0;
+  if (!(step > 0.0) || !std::isfinite(step)) return lo;
+  std::vector<size_t> n(4097, 0);
+  for (double x : v) ++n[(size_t)((x - lo) / step)];
+  size_t k = 0;
+  for (size_t below = n[0]; below * 3 < 2 * v.size(); below += n[++k]) {}
+  return lo + ((double)k + 0.5) * step;
+}
+
 // complex helpers on the host
 using zc = std::complex<double>;
 
@@ -2798,6 +2812,7 @@ gw_status gw_setup(gw_ctx** out, double L, int n_grid, double ecut, const double
   const double gg = 2.0 * M_PI / L, Rc = 0.5 * L;
   std::vector<double> v(vloc, vloc + ctx->N3), sqv(ctx->N3);
   for (double x : v) ctx->vmax = std::max(ctx->vmax, std::fabs(x));
+  ctx->vlevel = upper_third(v);
   for (int i0 = 0; i0 < N; ++i0)
     for (int i1 = 0; i1 < N; ++i1)
       for (int i2 = 0; i2 < N; ++i2) {

@@ -124,3 +124,23 @@ def test_mixed_next_to_transitions(system, im):
             assert rel(a[b], ref if im else np.real(ref)) < 2 * 10 * 1e-10 * 12 / d
     c.close()
     assert max(passes) <= 5
+
+
+# Shifting V rounds V - E by up to 10 Ha 2^-53 (FP32 passes: 2^-24, corrected by
+# the refinement) and the target by |A| in it: the errors of the solves as above.
+@pytest.mark.parametrize("prec,err", [(gw.GW_FP64, 1e-9), (gw.GW_MIXED, 1e-6)])
+@pytest.mark.parametrize("om", [0.0, "real", 0.3 + 0.1j, 0.957 + 0.1j, 0.4j])
+def test_zero_of_the_potential(system, om, prec, err):
+    """V + c with the energies + c is the same system: the same answer in the
+    same number of iterations (within a few, for the roundings)."""
+    om = omega_of(om, system[5])
+    f = W.random_fields(3, 2, system[1] ** 3)
+    c = cell_of(system)
+    one, its = c.apply_chi0(f, [om], prec), c.stats()["mean_iter"]
+    c.close()
+    for shift in (-5.0, 1.0, 3.0, 10.0):
+        c = cell_of(system, shift)
+        two, its2 = c.apply_chi0(f, [om], prec), c.stats()["mean_iter"]
+        c.close()
+        assert rel(two, one) < err
+        assert its2 <= 1.25 * its + 2
