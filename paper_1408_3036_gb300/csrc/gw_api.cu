@@ -557,8 +557,13 @@ gw_status col_solve(gw_ctx* ctx, int kind, int ncol, const double2* b64, const d
   a.flags = ctx->pcg_flags_d;
   a.xmax = xmax;
   const int pa = prof_begin(ctx, kind == COL_CG_PAIR ? PC_PCG : PC_N);
-  CK(launch_col_solve<T>(ctx->st, kind, a));
+  const cudaError_t le = launch_col_solve<T>(ctx->st, kind, a);
   prof_end(ctx, PC_PCG, pa);
+  if (le == cudaErrorNotSupported || le == cudaErrorInvalidConfiguration) {
+    cudaGetLastError();               // nothing ran: the other kernels take the pass
+    return GW_OK;
+  }
+  CK(le);
   TRY(pcg_pending(ctx, ncol, nullptr));
   ctx->pcg_pend.used = a.nunit << a.sh.lq;
   ctx->pcg_pend.fp64 = std::is_same<T, double>::value;

@@ -53,8 +53,7 @@
 #include <algorithm>
 #include <cstdio>
 
-#include <mutex>
-
+#include "device_cache.h"
 #include "fft.cuh"
 #include "gw_common.cuh"
 #include "linalg.cuh"
@@ -1120,20 +1119,17 @@ template <typename T, int TPB>
 static cudaError_t launch_pcg_tpb(cudaStream_t s, const PcgArgs<T>& a0, size_t sm, int cta_div, int per_it,
                                   int* grid_used) {
   cudaError_t e = cudaSuccess;
-  {
-    // The attribute is per function and per process: only ever raise it, so a
-    // context on another host thread never sees its limit lowered under it.
-    static std::mutex mu;
-    static size_t raised = 0;
-    std::lock_guard<std::mutex> lock(mu);
-    if (sm > raised) {
-      e = cudaFuncSetAttribute(k_cg_persistent<T, TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      if (e != cudaSuccess) return e;
-      raised = sm;
-    }
-  }
   int dev = 0, nsm = 0, per = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  {
+    // The attribute is per function and device: only ever raise it, so a
+    // context on another host thread never sees its limit lowered under it.
+    static DeviceCache<int, size_t> limit;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    e = (cudaError_t)limit.raise(dev, 0, sm, [](size_t v) {
+      return (int)cudaFuncSetAttribute(k_cg_persistent<T, TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v);
+    });
+    if (e != cudaSuccess) return e;
+  }
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cg_persistent<T, TPB>, TPB, sm)) != cudaSuccess)
     return e;

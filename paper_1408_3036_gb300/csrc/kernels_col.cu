@@ -2,12 +2,10 @@
 // (col_kernel.cuh has the kernel; kernels_col_*.cu its instances).
 #include <algorithm>
 #include <cmath>
-#include <map>
-#include <mutex>
-#include <set>
 #include <tuple>
 
 #include "col_layout.cuh"
+#include "device_cache.h"
 #include "linalg.cuh"
 
 namespace gw {
@@ -42,32 +40,24 @@ inline cudaLaunchConfig_t config(cudaLaunchAttribute* at, int q, int grid, size_
   return c;
 }
 
-// Kernel attributes (once per function and process) and the clusters of size q
-// that run at once (0: this size does not run here).
+// Kernel attributes (once per function and device) and the clusters of size q
+// that run at once on the current device (0: this size does not run here).
 int active_clusters(const void* f, int lq, size_t smem) {
-  static std::mutex mu;
-  static std::map<std::tuple<const void*, int, size_t>, int> known;
-  static std::set<const void*> ready;
-  std::lock_guard<std::mutex> lock(mu);
-  if (!ready.count(f)) {
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess ||
-        cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-      cudaGetLastError();
-      return 0;
-    }
-    ready.insert(f);
-  }
-  auto it = known.find({f, lq, smem});
-  if (it != known.end()) return it->second;
-  cudaLaunchAttribute at;
-  const cudaLaunchConfig_t c = config(&at, 1 << lq, 1 << lq, smem, nullptr);
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, f, &c) != cudaSuccess) {
-    cudaGetLastError();
-    n = 0;
-  }
-  known[{f, lq, smem}] = n;
-  return n;
+  static DeviceCache<const void*, bool> ready;
+  static DeviceCache<std::tuple<const void*, int, size_t>, int> known;
+  int dev = 0, n = 0;
+  bool set = false;
+  const bool ok =
+      cudaGetDevice(&dev) == cudaSuccess && ready.get(dev, f, &set, [&](bool* s) {
+        return *s = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) == cudaSuccess &&
+                    cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+      }) && known.get(dev, {f, lq, smem}, &n, [&](int* c) {
+        cudaLaunchAttribute at;
+        const cudaLaunchConfig_t cfg = config(&at, 1 << lq, 1 << lq, smem, nullptr);
+        return cudaOccupancyMaxActiveClusters(c, f, &cfg) == cudaSuccess;
+      });
+  if (!ok) cudaGetLastError();
+  return ok ? n : 0;
 }
 
 }  // namespace col

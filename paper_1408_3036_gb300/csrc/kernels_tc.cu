@@ -46,6 +46,7 @@
 #include <mutex>
 #include <vector>
 
+#include "device_cache.h"
 #include "gw_common.cuh"
 #include "linalg.cuh"
 
@@ -381,12 +382,13 @@ size_t tc_part_elems(int npw, int ncol) {
 }
 
 cudaError_t tc_prepare() {
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(k_tc_dots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
+  static DeviceCache<int, size_t> limit;
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return (cudaError_t)limit.raise(dev, 0, (size_t)kTcSmem, [](size_t v) {
+    return (int)cudaFuncSetAttribute(k_tc_dots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v);
   });
-  return attr;
 }
 
 cudaError_t launch_tc_dots(cudaStream_t s, const TcMaps& maps, const float2* Y, int npw, int ncol, int nocc,
