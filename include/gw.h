@@ -334,8 +334,9 @@ gw_status gw_proj_coef(gw_ctx* ctx, const float* y, int ncol, double* coef, int 
 /* gw_set_tensor_cores -- projector coefficients of the mixed simplified-QMR
    solver that runs one launch per step.  1: the tensor cores (gw_proj_coef
    kernel 1) when it has at least 256 columns and at most 64 projector rows;
-   0: its CUDA-core dots, the solver to compare with.  A context on which it was
-   never called takes the column solver, where it fits, with CUDA-core dots.
+   0: its CUDA-core dots, the solver to compare with.  Both concern only the
+   passes that 1 would change.  -1 (default): the column solver, where it fits,
+   with CUDA-core dots.
    The tensor-core coefficients carry about 2e-6 relative error (the FP32
    accumulation in tensor memory) against about 1e-7 for the CUDA-core FP32
    dots, and on the 64^3 cell with 64 occupied states the solver then needs
@@ -372,13 +373,13 @@ typedef enum {
 gw_status gw_set_imaginary_route(gw_ctx* ctx, int route);
 
 /*
- * gw_set_graphs -- 1: the ten launches of one simplified-QMR iteration (the
+ * gw_set_graphs -- 1 (any other positive value): the ten launches of one simplified-QMR iteration (the
  * transform passes of H, the projector, the four update steps) are captured
  * once per solve into a CUDA graph and replayed every iteration; 0: launched
  * one by one.  Same arithmetic either way; a stream that cannot be captured
- * falls back to direct launches.  A context on which it was never called runs
- * a whole simplified-QMR pass in one launch, one thread-block cluster per
- * column, where that fits, and replays graphs elsewhere.
+ * falls back to direct launches.  -1 (default; any negative value): a whole
+ * simplified-QMR pass in one launch, one thread-block cluster per column, where
+ * that fits, and graphs elsewhere.
  */
 gw_status gw_set_graphs(gw_ctx* ctx, int on);
 
@@ -396,13 +397,12 @@ gw_status gw_set_graphs(gw_ctx* ctx, int on);
  */
 gw_status gw_set_solver(gw_ctx* ctx, double tol, double tol_inner, int max_iter, int max_outer);
 
-/* Kernel of the CG passes at omega = 0 (gw_set_cg_kernel).  A context on which
- * it was never called takes the cluster form where it fits. */
+/* Kernel of the CG passes at omega = 0 (gw_set_cg_kernel). */
 typedef enum {
   GW_CG_PERSISTENT = 0,    /* one cooperative persistent launch per pass */
   GW_CG_MULTI_LAUNCH = 1,  /* one launch per transform pass, projector and update, per iteration */
-  GW_CG_CLUSTER = 2        /* one thread-block cluster per pair of columns that are real in real
-                              space (the persistent kernel for other columns, and when the grid
+  GW_CG_CLUSTER = 2        /* default: one thread-block cluster per pair of columns that are real in
+                              real space (the persistent kernel for other columns, and when the grid
                               size has no radices there or a pair does not fit in a cluster) */
 } gw_cg_kernel;
 

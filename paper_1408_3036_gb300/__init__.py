@@ -355,6 +355,8 @@ def gw_proj_coef(ctx, y, coef, kernel=1):
 
 
 def gw_set_tensor_cores(ctx, on):
+    """Tensor-core projector coefficients where they apply (1), launches per step with
+    CUDA-core dots there (0), or the column solver as everywhere else (-1, default)."""
     _check(ctx, load().gw_set_tensor_cores(ctx, int(on)))
 
 
@@ -369,7 +371,8 @@ def gw_set_imaginary_route(ctx, route):
 
 
 def gw_set_graphs(ctx, on):
-    """SQMR iterations replayed from a captured CUDA graph (1, default) or launched one by one (0)."""
+    """SQMR iterations replayed from a captured CUDA graph (1), launched one by one (0), or
+    whole passes in one launch where they fit (-1, default)."""
     _check(ctx, load().gw_set_graphs(ctx, int(on)))
 
 
@@ -390,8 +393,8 @@ def gw_set_precond(ctx, kind):
 
 
 def gw_set_cg_kernel(ctx, kind, wait_limit=0):
-    """GW_CG_PERSISTENT, GW_CG_MULTI_LAUNCH or GW_CG_CLUSTER, and the bound on the
-    persistent kernel's device waits (0 keeps it)."""
+    """GW_CG_PERSISTENT, GW_CG_MULTI_LAUNCH or GW_CG_CLUSTER (default), and the bound on
+    the persistent kernel's device waits (0 keeps it)."""
     _check(ctx, load().gw_set_cg_kernel(ctx, int(kind), int(wait_limit)))
 
 

@@ -45,7 +45,7 @@ struct gw_ctx {
   size_t work_cols = 0;
   double tol = 1e-13, tol_mixed = 1e-10, tol_inner = 1e-5;   // backward errors (FP64 / mixed), inner
   double anorm = 1.0;           // bound on |H - E| used by the backward error
-  int cg_kernel = -1;                 // kernel of the CG passes (gw_set_cg_kernel; -1: chosen by size)
+  int cg_kernel = GW_CG_CLUSTER;      // kernel of the CG passes (gw_set_cg_kernel)
   ColPlan col;                        // column solver (col_kernel.cuh): tables, and the data in its orders
   ColPrec<double> col64;
   ColPrec<float> col32;
@@ -54,8 +54,8 @@ struct gw_ctx {
                                       // by one, -1 the column solver where it fits, else replayed
   int imag_route = GW_IMAG_SQMR;      // solver of purely imaginary frequencies (gw_set_imaginary_route)
   double recycle_w0 = 0.0;            // > 0: recycled bases augmented with x(i w0)
-  int use_tc = -1;                    // SQMR projector coefficients: -1 the column solver's, 0 / 1 those of the
-                                      // launches per step on the CUDA cores / on the tensor cores where they apply
+  int use_tc = -1;                    // SQMR passes that the tensor cores apply to (tc_applies): -1 as any other,
+                                      // 0 / 1 launches per step with coefficients of the CUDA / tensor cores
   bool tune = true;                   // launch shapes picked by timing (tune.cu)
   int pcg_tpb = 0;                    // CTA width of the last persistent CG launch
   bool tc_ok = false;                 // the split occupied rows and their tensor maps are ready
@@ -699,6 +699,11 @@ gw_status pcg_finish(gw_ctx* ctx, long long* it_sum, int* it_max) {
 // ---------------------------------------------------------------------------
 // batched simplified QMR on P_c (H - E) P_c x = b (complex or indefinite shifts)
 // ---------------------------------------------------------------------------
+// Passes that take their projector coefficients from the tensor cores when asked
+template <typename T> bool tc_applies(const gw_ctx* ctx, int ncol) {
+  return std::is_same<T, float>::value && ctx->tc_ok && ncol >= kTcMinCols;
+}
+
 template <typename T>
 gw_status qmr_solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, const int* outer_active,
                     cpx<T>* x, double tol, const double* rr_abs, const double* tk, long long* it_sum, int* it_max) {
@@ -745,7 +750,7 @@ gw_status qmr_solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E,
   dots.coef = ctx->work.coef;
   // Mixed path with many columns: the projector coefficients <C_v|t> on the
   // tensor cores (kernels_tc.cu) instead of the dots fused into the gather
-  const bool tc = std::is_same<T, float>::value && ctx->use_tc > 0 && ctx->tc_ok && ncol >= kTcMinCols;
+  const bool tc = ctx->use_tc > 0 && tc_applies<T>(ctx, ncol);
   float* tc_part = nullptr;
   int* tc_err = nullptr;
   if (tc) {
@@ -847,8 +852,8 @@ template <typename U>
 gw_status inner_solve(gw_ctx* ctx, bool qmr, int ncol, const double2* r64, const double2* E, const int* oact,
                       cpx<U>* d, double2* x64, double* xmax, double tol_in, const double* rra, const double* tk,
                       bool sym, bool real_shift, long long* it_sum, int* it_max, const double* w2 = nullptr) {
-  const bool col = !w2 && (qmr ? ctx->use_graphs < 0 && ctx->use_tc < 0
-                               : sym && (ctx->cg_kernel < 0 || ctx->cg_kernel == GW_CG_CLUSTER));
+  const bool col = !w2 && (qmr ? ctx->use_graphs < 0 && (ctx->use_tc < 0 || !tc_applies<U>(ctx, ncol))
+                               : sym && ctx->cg_kernel == GW_CG_CLUSTER);
   bool ran = false;
   if (col) {
     const int kind = !qmr ? COL_CG_PAIR : sym && real_shift ? COL_QMR_PAIR : COL_QMR;
@@ -3278,7 +3283,7 @@ gw_status gw_set_autotune(gw_ctx* ctx, int on) {
 
 gw_status gw_set_tensor_cores(gw_ctx* ctx, int on) {
   if (!ctx) return GW_E_ARG;
-  ctx->use_tc = (on != 0) ? 1 : 0;
+  ctx->use_tc = on < 0 ? -1 : on != 0;
   return GW_OK;
 }
 
@@ -3326,7 +3331,7 @@ gw_status gw_set_imaginary_route(gw_ctx* ctx, int route) {
 
 gw_status gw_set_graphs(gw_ctx* ctx, int on) {
   if (!ctx) return GW_E_ARG;
-  ctx->use_graphs = (on != 0);
+  ctx->use_graphs = on < 0 ? -1 : on != 0;
   return GW_OK;
 }
 
