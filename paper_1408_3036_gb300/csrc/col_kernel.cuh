@@ -100,45 +100,6 @@ constexpr int kNearWait = 32;        // iterations granted within a factor 2 of 
 
 template <typename T> struct alignas(16) V4 { T x, y, z, w; };
 
-// sums of Acc values (col_layout.cuh)
-__device__ __forceinline__ double add_(double a, double b) { return a + b; }
-__device__ __forceinline__ float2 add_(float2 a, float2 b) {
-  const float s = __fadd_rn(a.x, b.x);
-  const float bb = __fsub_rn(s, a.x);
-  const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
-  const float t = __fadd_rn(e, __fadd_rn(a.y, b.y));
-  const float h = __fadd_rn(s, t);
-  return make_float2(h, __fsub_rn(t, __fsub_rn(h, s)));
-}
-__device__ __forceinline__ double scale_(double a, double c) { return a * c; }
-__device__ __forceinline__ float2 scale_(float2 a, float c) {
-  const float p = __fmul_rn(a.x, c);
-  const float e = fmaf(a.y, c, fmaf(a.x, c, -p));
-  const float h = __fadd_rn(p, e);
-  return make_float2(h, __fsub_rn(e, __fsub_rn(h, p)));
-}
-__device__ __forceinline__ void fma_(double& acc, double a, double b) { acc += a * b; }
-__device__ __forceinline__ void fma_(float2& acc, float a, float b) {
-  const float p = __fmul_rn(a, b);
-  acc = add_(acc, make_float2(p, fmaf(a, b, -p)));
-}
-__device__ __forceinline__ double of_(double x) { return x; }
-__device__ __forceinline__ float2 of_(float x) { return make_float2(x, 0.f); }
-__device__ __forceinline__ double val_(double a) { return a; }
-__device__ __forceinline__ float val_(float2 a) { return __fadd_rn(a.x, a.y); }
-__device__ __forceinline__ double dbl_(double a) { return a; }
-__device__ __forceinline__ double dbl_(float2 a) { return (double)a.x + (double)a.y; }
-__device__ __forceinline__ double shx_(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
-__device__ __forceinline__ float2 shx_(float2 a, int o) {
-  return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
-}
-__device__ __forceinline__ float shx_(float a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
-__device__ __forceinline__ double shi_(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
-__device__ __forceinline__ float2 shi_(float2 a, int l) {
-  return make_float2(__shfl_sync(0xffffffffu, a.x, l), __shfl_sync(0xffffffffu, a.y, l));
-}
-__device__ __forceinline__ float add_(float a, float b) { return a + b; }
-
 // Warp sums of M values per lane (M a power of 2, at most 32) by recursive
 // halving: M - 1 + log2(32 / M) additions instead of 5 M.  Lane l returns the
 // sum of value l / (32 / M), the same bits in all its lanes.
@@ -151,11 +112,11 @@ template <int M, typename A> __device__ __forceinline__ A warp_sums(A* v) {
 #pragma unroll
     for (int k = 0; k < n; ++k) {
       const A keep = up ? v[n + k] : v[k], give = up ? v[k] : v[n + k];
-      v[k] = add_(keep, shx_(give, o));
+      v[k] = acc_add(keep, acc_shfl(give, o));
     }
   }
 #pragma unroll
-  for (int q = 16 / M; q >= 1; q >>= 1) v[0] = add_(v[0], shx_(v[0], q));
+  for (int q = 16 / M; q >= 1; q >>= 1) v[0] = acc_add(v[0], acc_shfl(v[0], q));
   return v[0];
 }
 __host__ __device__ constexpr int pow2_up(int n) { int p = 1; while (p < n) p *= 2; return p; }
@@ -187,7 +148,8 @@ template <typename T, int KIND, int N1, int N2>
 __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   using V = cpx<T>;
   using W4 = V4<T>;
-  using SA = Acc<T>;
+  using SA = ScalarAcc<T, KIND>;
+  using CA = CoefAcc<T, KIND>;
   constexpr bool PAIR = KIND != COL_QMR;
   constexpr bool CG = KIND == COL_CG_PAIR;
   constexpr int NV = CG ? 4 : 2;
@@ -229,8 +191,8 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   signed char* zm = reinterpret_cast<signed char*>(sm + L.zm);
   unsigned char* zs = sm + L.zs;
   V* stw = reinterpret_cast<V*>(sm + L.tw);
-  T* cp = reinterpret_cast<T*>(sm + L.cp);        // [nsplit][nproj][NV] this CTA's coefficients in parts
-  T* coefp = reinterpret_cast<T*>(sm + L.coefp);  // [Q][nproj][NV]
+  CA* cp = reinterpret_cast<CA*>(sm + L.cp);      // [nsplit][nproj][NV] this CTA's coefficients in parts
+  CA* coefp = reinterpret_cast<CA*>(sm + L.coefp);   // [Q][nproj][NV]
   T* coef = reinterpret_cast<T*>(sm + L.coef);    // [nproj][NV]
   SA* part = reinterpret_cast<SA*>(sm + L.part);  // [kNW][4] scalar sums of the warps
   SA* sc = reinterpret_cast<SA*>(sm + L.sc);      // [3][Q][4] of the CTAs
@@ -378,6 +340,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   csync();                                        // every CTA of the cluster has started
 
   const T one = (T)1, two = (T)2;
+  auto of = [](T x) { return AccFrom<SA>::of(x); };
   // |n| <= m for index k of N (one comparison; m = -1: none)
   auto inside = [&](int k, int m) { return (unsigned)(k - m - 1) >= (unsigned)(N - 2 * m - 1); };
   auto present = [&](int x) { return inside(x, nm); };
@@ -686,10 +649,13 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
 #pragma unroll
       for (int q = 0; q < RG; ++q) row[q] = (unsigned)min(v0 + q, nproj - 1) * (unsigned)ldc;
       T acc[M];
+      CA sum[M];
 #pragma unroll
-      for (int k = 0; k < M; ++k) acc[k] = (T)0;
-#pragma unroll 2
-      for (int e = lane + 32 * prt; e < nh; e += 32 * nsplit) {
+      for (int k = 0; k < M; ++k) {
+        acc[k] = (T)0;
+        sum[k] = AccFrom<CA>::of((T)0);
+      }
+      auto entry = [&](int e) {
         V c[RG];
 #pragma unroll
         for (int q = 0; q < RG; ++q) c[q] = C[row[q] + (unsigned)e];
@@ -713,11 +679,37 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
             acc[q * NV + NV - 1] = fma(c[q].y, u.w, fma(c[q].x, u.z, acc[q * NV + NV - 1]));
           }
         }
+      };
+      if constexpr (std::is_same<CA, T>::value) {
+#pragma unroll 2
+        for (int e = lane + 32 * prt; e < nh; e += 32 * nsplit) entry(e);
+#pragma unroll
+        for (int k = 0; k < M; ++k) sum[k] = acc[k];
+      } else {
+        // 8 entries (16 products) in plain FP32
+        auto take = [&]() {
+#pragma unroll
+          for (int k = 0; k < RG * NV; ++k) {
+            acc_in(sum[k], acc[k]);
+            acc[k] = (T)0;
+          }
+        };
+        const int st = 32 * nsplit;
+        int e = lane + 32 * prt;
+        for (; e + 7 * st < nh; e += 8 * st) {
+#pragma unroll 2
+          for (int k = 0; k < 8; ++k) entry(e + k * st);
+          take();
+        }
+#pragma unroll 2
+        for (; e < nh; e += st) entry(e);
+        take();
       }
-      const T t = warp_sums<M, T>(acc);
+      CA t = warp_sums<M, CA>(sum);
+      if (PAIR) t = acc_add(t, t);
       const int k = lane / (32 / M), q = k / NV;
       if (lane % (32 / M) == 0 && q < RG && v0 + q < nproj)
-        cp[((size_t)prt * nproj + v0 + q) * NV + (k - q * NV)] = PAIR ? (T)2 * t : t;
+        cp[((size_t)prt * nproj + v0 + q) * NV + (k - q * NV)] = t;
     }
   };
   auto dots = [&]() {
@@ -734,15 +726,15 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
     const int n = nproj * NV;
     for (int t = tid; t < (n << a.sh.lq); t += kTPB) {
       const int q = t / n, j = t - q * n;
-      T v = cp[j];
-      for (int p = 1; p < nsplit; ++p) v += cp[p * n + j];
+      CA v = cp[j];
+      for (int p = 1; p < nsplit; ++p) v = acc_add(v, cp[p * n + j]);
       at(coefp, q)[rank * n + j] = v;
     }
   };
   auto coef_of = [&](int j) {
-    T v = coefp[j];
-    for (int q = 1; q < Q; ++q) v += coefp[q * nproj * NV + j];
-    return v;
+    CA v = coefp[j];
+    for (int q = 1; q < Q; ++q) v = acc_add(v, coefp[q * nproj * NV + j]);
+    return acc_val(v);
   };
   auto coef_sum = [&]() {
     for (int j = tid; j < nproj * NV; j += kTPB) coef[j] = coef_of(j);
@@ -757,19 +749,19 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
   };
   auto send_sums = [&](int ns, int slot) {        // one warp
     const int k = lane & 3;
-    SA t = of_((T)0);
+    SA t = of((T)0);
     if (k < ns)
-      for (int w = lane >> 2; w < kNW; w += 8) t = add_(t, part[w * 4 + k]);
+      for (int w = lane >> 2; w < kNW; w += 8) t = acc_add(t, part[w * 4 + k]);
 #pragma unroll
-    for (int o = 4; o < 32; o <<= 1) t = add_(t, shx_(t, o));
+    for (int o = 4; o < 32; o <<= 1) t = acc_add(t, acc_shfl(t, o));
     if (k < ns)
       for (int q = lane >> 2; q < Q; q += 8) at(sc, q)[((slot << a.sh.lq) + rank) * 4 + k] = t;
   };
   auto take_sums = [&](int slot) {                // one warp
-    SA t = of_((T)0);
-    for (int q = lane >> 2; q < Q; q += 8) t = add_(t, sc[((slot << a.sh.lq) + q) * 4 + (lane & 3)]);
+    SA t = of((T)0);
+    for (int q = lane >> 2; q < Q; q += 8) t = acc_add(t, sc[((slot << a.sh.lq) + q) * 4 + (lane & 3)]);
 #pragma unroll
-    for (int o = 4; o < 32; o <<= 1) t = add_(t, shx_(t, o));
+    for (int o = 4; o < 32; o <<= 1) t = acc_add(t, acc_shfl(t, o));
     return t;
   };
   // y - sum_v C_v coef_v at one half entry
@@ -858,7 +850,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         if (a1) { u.z = k1 * r.z; u.w = k1 * r.w; }
         scatter(e, u);
       }
-      v4[0] = of_(g0); v4[1] = of_(r0); v4[2] = of_(g1); v4[3] = of_(r1);
+      v4[0] = of(g0); v4[1] = of(r0); v4[2] = of(g1); v4[3] = of(r1);
     };
     const int cmp = tid & 3, cc = cmp >> 1;       // component x, y (column 0), z, w (column 1)
     const int im = (cmp == 1 || cmp == 2) ? 1 : 0;
@@ -899,15 +891,15 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         if (act) u = kc * r;
       }
       // pair packing: x - w, y + z at G; x + w, z - y at -G
-      const T o = shx_(u, 3);
+      const T o = acc_shfl(u, 3);
       if (e < nh) {
         const unsigned hp = hpos[e];
         const int j = (int)(hp >> 8), z = (int)(hp & 255u);
         if (cmp < 2) ZT[2 * (z * ldz + (j - p0)) + im] = cmp ? u + o : u - o;
         else if (h0 + e != 0) ZT[2 * ((N - z) % N * ldz + mirror_row(j)) + im] = cmp == 2 ? u - o : u + o;
       }
-      v4[0] = of_(cc ? (T)0 : gs); v4[1] = of_(cc ? (T)0 : rs);
-      v4[2] = of_(cc ? gs : (T)0); v4[3] = of_(cc ? rs : (T)0);
+      v4[0] = of(cc ? (T)0 : gs); v4[1] = of(cc ? (T)0 : rs);
+      v4[2] = of(cc ? gs : (T)0); v4[3] = of(cc ? rs : (T)0);
     };
     // w and u, and u^H w before the projector
     auto gather1 = [&](SA* v2) {
@@ -923,8 +915,8 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         d0 += f * (u.x * w.x + u.y * w.y);
         d1 += f * (u.z * w.z + u.w * w.w);
       }
-      v2[0] = of_(d0);
-      v2[1] = of_(d1);
+      v2[0] = of(d0);
+      v2[1] = of(d1);
     };
     auto gather4 = [&](SA* v2) {
       T ds = (T)0;
@@ -940,8 +932,8 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         TT[4 * a.nhl + t] = u;
         ds = ((h0 + e == 0) ? one : two) * u * w;
       }
-      v2[0] = of_(cc ? (T)0 : ds);
-      v2[1] = of_(cc ? ds : (T)0);
+      v2[0] = of(cc ? (T)0 : ds);
+      v2[1] = of(cc ? ds : (T)0);
     };
     const bool decide = warp == kNW - 1;
     for (int k = 0;; ++k) {
@@ -958,11 +950,11 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       // while the slabs' first step runs: gamma, |r|^2 and the stopping tests
       if (decide) {
         const SA tot = take_sums(0);
-        const SA g = shi_(tot, (2 * lane) & 3), q = shi_(tot, (2 * lane + 1) & 3);
+        const SA g = acc_lane(tot, (2 * lane) & 3), q = acc_lane(tot, (2 * lane + 1) & 3);
         int act = 0;
         if (lane < 2) {
           CgCol<T>& st = s_cg[lane];
-          const T gam = val_(g), rr = val_(q);
+          const T gam = acc_val(g), rr = acc_val(q);
           if (k == 0) {
             const T s1 = (T)a.tol2 * rr, s2 = lane < nc ? (T)stop_abs(lane) : (T)0;
             st.stop = s1 > s2 ? s1 : s2;
@@ -1010,7 +1002,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       if (decide) {
         // delta = u^H w - sum_v <C_v|u> <C_v|w>, alpha
         const SA tot = take_sums(1);
-        SA t2[2] = {of_((T)0), of_((T)0)};
+        SA t2[2] = {of((T)0), of((T)0)};
         for (int v = lane; v < nproj; v += 32) {
           const W4* c4 = reinterpret_cast<const W4*>(coefp) + v;
           W4 c = c4[0];
@@ -1018,16 +1010,16 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
             const W4 d = c4[q * nproj];
             c.x += d.x; c.y += d.y; c.z += d.z; c.w += d.w;
           }
-          t2[0] = add_(t2[0], of_(c.x * c.z));
-          t2[1] = add_(t2[1], of_(c.y * c.w));
+          t2[0] = acc_add(t2[0], of(c.x * c.z));
+          t2[1] = acc_add(t2[1], of(c.y * c.w));
         }
         const SA tv = warp_sums<2, SA>(t2);
-        const SA t = shi_(tv, (lane & 1) * 16), uw = shi_(tot, lane & 1);
+        const SA t = acc_lane(tv, (lane & 1) * 16), uw = acc_lane(tot, lane & 1);
         int act = 0;
         if (lane < 2) {
           CgCol<T>& st = s_cg[lane];
           if (st.active) {
-            const T delta = val_(add_(uw, scale_(t, (T)-1)));
+            const T delta = acc_val(acc_add(uw, acc_scale(t, (T)-1)));
             const T den = k > 0 ? delta - st.bt * st.gdiv : delta;
             if (!(den > (T)0) || !isfinite(den) || !(st.gam > (T)0)) {
               st.flag = 2;
@@ -1063,25 +1055,25 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       if (PAIR) {
         const T f = (h0 + e == 0) ? one : two;
         const T k0 = f * Kt[2 * e], k1 = f * Kt[2 * e + 1];
-        fma_(v[0], f * r.x, r.x); fma_(v[0], f * r.y, r.y);
-        fma_(v[1], f * r.z, r.z); fma_(v[1], f * r.w, r.w);
-        fma_(v[2], k0 * r.x, r.x); fma_(v[2], k0 * r.y, r.y);
-        fma_(v[3], k1 * r.z, r.z); fma_(v[3], k1 * r.w, r.w);
+        acc_fma(v[0], f * r.x, r.x); acc_fma(v[0], f * r.y, r.y);
+        acc_fma(v[1], f * r.z, r.z); acc_fma(v[1], f * r.w, r.w);
+        acc_fma(v[2], k0 * r.x, r.x); acc_fma(v[2], k0 * r.y, r.y);
+        acc_fma(v[3], k1 * r.z, r.z); acc_fma(v[3], k1 * r.w, r.w);
       } else {
         const W4 u = apply_k(e, r);
-        fma_(v[0], r.x, r.x); fma_(v[0], r.y, r.y); fma_(v[0], r.z, r.z); fma_(v[0], r.w, r.w);
+        acc_fma(v[0], r.x, r.x); acc_fma(v[0], r.y, r.y); acc_fma(v[0], r.z, r.z); acc_fma(v[0], r.w, r.w);
         if (h0 + e == 0) {
-          fma_(v[1], u.x, r.x); fma_(v[1], -u.y, r.y);
-          fma_(v[2], u.x, r.y); fma_(v[2], u.y, r.x);
+          acc_fma(v[1], u.x, r.x); acc_fma(v[1], -u.y, r.y);
+          acc_fma(v[2], u.x, r.y); acc_fma(v[2], u.y, r.x);
         } else {
-          fma_(v[1], two * u.x, r.z); fma_(v[1], -two * u.y, r.w);
-          fma_(v[2], two * u.x, r.w); fma_(v[2], two * u.y, r.z);
+          acc_fma(v[1], two * u.x, r.z); acc_fma(v[1], -two * u.y, r.w);
+          acc_fma(v[2], two * u.x, r.w); acc_fma(v[2], two * u.y, r.z);
         }
       }
     };
     const bool decide = warp == kNW - 1;
     {
-      SA v[4] = {of_((T)0), of_((T)0), of_((T)0), of_((T)0)};
+      SA v[4] = {of((T)0), of((T)0), of((T)0), of((T)0)};
       for (int e = tid; e < nh; e += kTPB) {
         const W4 r = X[e];
         norms(e, r, v);
@@ -1094,8 +1086,8 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       if (decide) send_sums(4, 0);
       csync();
       if (decide) {
-        const double t = dbl_(take_sums(0));
-        const double rr = shi_(t, PAIR ? lane & 1 : 0), rx = shi_(t, PAIR ? 2 + (lane & 1) : 1), ry = shi_(t, 2);
+        const double t = acc_dbl(take_sums(0));
+        const double rr = acc_lane(t, PAIR ? lane & 1 : 0), rx = acc_lane(t, PAIR ? 2 + (lane & 1) : 1), ry = acc_lane(t, 2);
         int act = 0;
         if (lane < nc) {
           QmrCol& st = s_q[lane];
@@ -1128,21 +1120,21 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       coef_sum();
       __syncthreads();
       // t = P_c t and [q, t]
-      SA v[4] = {of_((T)0), of_((T)0), of_((T)0), of_((T)0)};
+      SA v[4] = {of((T)0), of((T)0), of((T)0), of((T)0)};
       for (int e = tid; e < nh; e += kTPB) {
         const W4 t = project(e, Tm[e]);
         Tm[e] = t;
         const W4 q = X[xs + e];
         if (PAIR) {
           const T f = (h0 + e == 0) ? one : two;
-          fma_(v[0], f * q.x, t.x); fma_(v[0], f * q.y, t.y);
-          fma_(v[1], f * q.z, t.z); fma_(v[1], f * q.w, t.w);
+          acc_fma(v[0], f * q.x, t.x); acc_fma(v[0], f * q.y, t.y);
+          acc_fma(v[1], f * q.z, t.z); acc_fma(v[1], f * q.w, t.w);
         } else if (h0 + e == 0) {
-          fma_(v[0], q.x, t.x); fma_(v[0], -q.y, t.y);
-          fma_(v[1], q.x, t.y); fma_(v[1], q.y, t.x);
+          acc_fma(v[0], q.x, t.x); acc_fma(v[0], -q.y, t.y);
+          acc_fma(v[1], q.x, t.y); acc_fma(v[1], q.y, t.x);
         } else {
-          fma_(v[0], q.z, t.x); fma_(v[0], -q.w, t.y); fma_(v[0], q.x, t.z); fma_(v[0], -q.y, t.w);
-          fma_(v[1], q.z, t.y); fma_(v[1], q.w, t.x); fma_(v[1], q.x, t.w); fma_(v[1], q.y, t.z);
+          acc_fma(v[0], q.z, t.x); acc_fma(v[0], -q.w, t.y); acc_fma(v[0], q.x, t.z); acc_fma(v[0], -q.y, t.w);
+          acc_fma(v[1], q.z, t.y); acc_fma(v[1], q.w, t.x); acc_fma(v[1], q.x, t.w); acc_fma(v[1], q.y, t.z);
         }
       }
       put_sums(IC<2>(), v);
@@ -1151,8 +1143,8 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
       csync();
       if (decide) {
         // alpha = rho / [q, t]: one division in the lanes of Re and Im (PAIR: of the columns)
-        const double t = dbl_(take_sums(1));
-        const double sx = shi_(t, PAIR ? lane & 1 : 0), sy = PAIR ? 0.0 : shi_(t, 1);
+        const double t = acc_dbl(take_sums(1));
+        const double sx = acc_lane(t, PAIR ? lane & 1 : 0), sy = PAIR ? 0.0 : acc_lane(t, 1);
         QmrCol& st = s_q[PAIR ? lane & 1 : 0];
         const double2 rho = st.rho;
         const double num = PAIR ? rho.x : (lane & 1) ? rho.y * sx - rho.x * sy : rho.x * sx + rho.y * sy;
@@ -1173,7 +1165,7 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         const bool a0 = s_q[0].active, a1 = PAIR ? s_q[1].active : a0;
         const T ax = (T)s_q[0].alpha.x, ay = (T)(PAIR ? s_q[1].alpha.x : s_q[0].alpha.y);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = of_((T)0);
+        for (int q = 0; q < 4; ++q) v[q] = of((T)0);
         for (int e = tid; e < nh; e += kTPB) {
           W4 r = X[e];
           const W4 t = Tm[e];
@@ -1198,9 +1190,9 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         // theta^2 = |r|^2 / tau^2, c^2 = 1 / (1 + theta^2) = tau^2 / (tau^2 + |r|^2),
         // tau'^2 = tau^2 theta^2 c^2 = |r|^2 c^2, beta = rho' / rho: one division,
         // the quotients in lanes 0, 1 .. (PAIR: two lanes each)
-        const double t = dbl_(take_sums(2));
+        const double t = acc_dbl(take_sums(2));
         const int c = PAIR ? lane & 1 : 0, w = PAIR ? lane >> 1 : lane;
-        const double rr = shi_(t, PAIR ? c : 0), rx = shi_(t, PAIR ? 2 + c : 1), ry = PAIR ? 0.0 : shi_(t, 2);
+        const double rr = acc_lane(t, PAIR ? c : 0), rx = acc_lane(t, PAIR ? 2 + c : 1), ry = PAIR ? 0.0 : acc_lane(t, 2);
         const double tau2 = s_q[c].tau2;
         const double2 rho = s_q[c].rho;
         const double rho2 = PAIR ? rho.x : rho.x * rho.x + rho.y * rho.y;
@@ -1208,8 +1200,8 @@ __global__ void __launch_bounds__(kTPB, 1) k_col_solve(ColArgs<T> a) {
         if (!PAIR && w == 2) num = rx * rho.x + ry * rho.y;
         if (!PAIR && w == 3) num = ry * rho.x - rx * rho.y;
         const double quo = num / den;
-        const double th2 = shi_(quo, c), c2 = shi_(quo, PAIR ? 2 + c : 1);
-        const double bx = shi_(quo, PAIR ? 4 + c : 2), by = PAIR ? 0.0 : shi_(quo, 3);
+        const double th2 = acc_lane(quo, c), c2 = acc_lane(quo, PAIR ? 2 + c : 1);
+        const double bx = acc_lane(quo, PAIR ? 4 + c : 2), by = PAIR ? 0.0 : acc_lane(quo, 3);
         __syncwarp();
         int act = 0;
         if (lane < nc) {

@@ -1,7 +1,10 @@
 // Column solver: shared-memory layout of one CTA (kernel and launch).
 #pragma once
 
+#include <type_traits>
+
 #include "col.cuh"
+#include "sums.cuh"
 
 namespace gw {
 namespace col {
@@ -11,11 +14,15 @@ namespace col {
 constexpr int kTPB = 512;
 constexpr int kNW = kTPB / 32;
 constexpr size_t kSmemMax = 226 * 1024;
-// Scalar sums: FP64, or a float pair whose additions are error-free
-// transformations (Knuth's TwoSum; products split through an FMA)
-template <typename T> struct AccOf { using type = double; };
-template <> struct AccOf<float> { using type = float2; };
-template <typename T> using Acc = typename AccOf<T>::type;
+// Sums over entries, as exact as those of the solvers they stand for (sums.cuh).
+// FP64 throughout in FP64.  FP32 CG: scalars in two floats, projector
+// coefficients in one, as the persistent CG.  FP32 SQMR: scalars in three floats
+// (the launches per step sum in FP64), coefficients in plain FP32 over 8 entries
+// of a lane, then two floats (launches per step: FP32 within a tile of 16
+// pencils, FP64 over the tiles; the FP32 part decides).
+template <typename T, int KIND>
+using ScalarAcc = typename std::conditional<KIND == COL_CG_PAIR, Acc<T>, Acc3<T>>::type;
+template <typename T, int KIND> using CoefAcc = typename std::conditional<KIND == COL_CG_PAIR, T, Acc<T>>::type;
 
 // Shared memory of one CTA (byte offsets)
 struct Lay {
@@ -40,6 +47,9 @@ __host__ __device__ inline Lay layout(int kind, const ColShape& sh, int N, int P
   const size_t sv = sizeof(cpx<T>), s4 = 4 * sizeof(T);
   const int Q = 1 << sh.lq, nzl = (N + Q - 1) / Q, nv = kind == COL_CG_PAIR ? 4 : 2;
   const int rg = row_group(nproj, sizeof(T) == 4);
+  const bool cg = kind == COL_CG_PAIR;
+  const size_t sc = cg ? sizeof(CoefAcc<T, COL_CG_PAIR>) : sizeof(CoefAcc<T, COL_QMR>);
+  const size_t ss = cg ? sizeof(ScalarAcc<T, COL_CG_PAIR>) : sizeof(ScalarAcc<T, COL_QMR>);
   const size_t tile = (size_t)sh.nsb * N * (N | 1) * sv, temp = (size_t)nhl * s4 * (kind == COL_CG_PAIR ? 2 : 1);
   Lay L;
   L.Z = 0;
@@ -57,11 +67,11 @@ __host__ __device__ inline Lay layout(int kind, const ColShape& sh, int N, int P
   L.zs = up16(L.zm + (size_t)ldz);
   L.tw = up16(L.zs + (size_t)N);
   L.cp = up16(L.tw + (size_t)N * sv);
-  L.coefp = up16(L.cp + (size_t)splits(nproj, rg, nhl) * nproj * nv * sizeof(T));
-  L.coef = up16(L.coefp + (size_t)Q * nproj * nv * sizeof(T));
+  L.coefp = up16(L.cp + (size_t)splits(nproj, rg, nhl) * nproj * nv * sc);
+  L.coef = up16(L.coefp + (size_t)Q * nproj * nv * sc);
   L.part = up16(L.coef + (size_t)nproj * nv * sizeof(T));
-  L.sc = up16(L.part + (size_t)kNW * 4 * sizeof(Acc<T>));
-  L.total = up16(L.sc + (size_t)3 * Q * 4 * sizeof(Acc<T>));
+  L.sc = up16(L.part + (size_t)kNW * 4 * ss);
+  L.total = up16(L.sc + (size_t)3 * Q * 4 * ss);
   return L;
 }
 
