@@ -57,6 +57,7 @@
 #include "fft.cuh"
 #include "gw_common.cuh"
 #include "linalg.cuh"
+#include "sums.cuh"
 
 namespace gw {
 
@@ -103,40 +104,10 @@ template <typename V> __device__ __forceinline__ V ldcg(const V* p);
 template <> __device__ __forceinline__ float2 ldcg<float2>(const float2* p) { return __ldcg(p); }
 template <> __device__ __forceinline__ double2 ldcg<double2>(const double2* p) { return __ldcg(p); }
 
-// Scalar sums of the CG (inner products, |r|^2, the plane records): FP64 in
-// the FP64 kernel; in the FP32 kernel a pair of floats hi + lo whose
-// additions are error-free transformations (Knuth's TwoSum, then a
-// renormalising FastTwoSum; products by Dekker's splitting through an FMA),
-// which keeps the sums close to FP64 accuracy with FP32 instructions only --
-// this GPU runs FP64 at a small fraction of its FP32 rate.
-template <typename T> struct AccOf { using type = double; };
-template <> struct AccOf<float> { using type = float2; };
-template <typename T> using Acc = typename AccOf<T>::type;
-
-__device__ __forceinline__ double acc_add(double a, double b) { return a + b; }
-__device__ __forceinline__ float2 acc_add(float2 a, float2 b) {
-  const float s = __fadd_rn(a.x, b.x);
-  const float bb = __fsub_rn(s, a.x);
-  const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
-  const float t = __fadd_rn(e, __fadd_rn(a.y, b.y));
-  const float h = __fadd_rn(s, t);
-  return make_float2(h, __fsub_rn(t, __fsub_rn(h, s)));
-}
-__device__ __forceinline__ double acc_scale(double a, double c) { return a * c; }
-__device__ __forceinline__ float2 acc_scale(float2 a, float c) {
-  const float p = __fmul_rn(a.x, c);
-  const float e = fmaf(a.y, c, fmaf(a.x, c, -p));
-  const float h = __fadd_rn(p, e);
-  return make_float2(h, __fsub_rn(e, __fsub_rn(h, p)));
-}
+// Scalar sums of the CG (inner products, |r|^2, the plane records): FP64 in the
+// FP64 kernel, a pair of floats in the FP32 kernel (sums.cuh).
 __device__ __forceinline__ double acc_of(double x) { return x; }
 __device__ __forceinline__ float2 acc_of(float x) { return make_float2(x, 0.f); }
-__device__ __forceinline__ double acc_val(double a) { return a; }
-__device__ __forceinline__ float acc_val(float2 a) { return __fadd_rn(a.x, a.y); }
-__device__ __forceinline__ double acc_shfl(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
-__device__ __forceinline__ float2 acc_shfl(float2 a, int o) {
-  return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
-}
 __device__ __forceinline__ double acc_ldcg(const double* p) { return __ldcg(p); }
 __device__ __forceinline__ float2 acc_ldcg(const float2* p) { return __ldcg(p); }
 
