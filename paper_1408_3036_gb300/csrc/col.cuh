@@ -20,8 +20,7 @@ constexpr int kColNQ = 5;                          // cluster sizes 1, 2, 4, 8, 
 // -G (in the second); h = 0 is G = 0.  The CTA of rank r in a cluster of Q owns
 // the pairs split[lq][r] .. split[lq][r + 1] (lq = log2 Q) and their entries.
 struct ColPlan {
-  bool half = false;                               // the entry tables (gp, gm, nh) are set
-  bool ok = false;                                 // and the column solver has radices for N
+  bool ok = false;                                 // the column solver has radices for N
   int N1 = 0, N2 = 0, P = 0, nm = 0;               // planes |n0| <= nm: P = 2 nm + 1
   int npair = 0, nh = 0;
   int maxpair[kColNQ] = {0}, maxh[kColNQ] = {0};   // per CTA, by log2 Q

@@ -379,16 +379,10 @@ gw_status h_apply_sym(gw_ctx* ctx, const double2* x, int ncol, const double2* E,
   return launch_check(ctx, "h_apply_sym");
 }
 
-// y = P_c y for FP64 columns (real: real in real space), on half the sphere
-// where the tables are there.
+// y = P_c y for FP64 columns (real: real in real space), on half the sphere.
 gw_status proj64(gw_ctx* ctx, double2* Y, int ncol, bool real) {
   if (ncol == 0 || ctx->nocc == 0) return GW_OK;
   const ColPlan& p = ctx->col;
-  if (!p.half) {
-    TRY(ensure_work(ctx, ncol));
-    launch_proj<double>(ctx->st, ctx->P64.C, ctx->nocc, ctx->npw, Y, ncol, nullptr, ctx->work, nullptr, nullptr, real);
-    return GW_OK;
-  }
   double* part;
   TRY(getbuf(ctx, "ph_part", half_part_elems(ctx->nocc, p.nh, ncol), &part));
   const int n = launch_gram_half(ctx->st, real, p, ctx->col64.Ch, ctx->nocc, Y, ctx->npw, ncol, nullptr, part);
@@ -911,10 +905,9 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
     CK(cudaMallocHost(&ctx->sv_pin, (size_t)4 * ncol * sizeof(double)));
     ctx->sv_pin_n = (size_t)4 * ncol;
   }
-  const bool half = ctx->col.half && !w2;      // residual and projector on half the sphere
   double2 *cb = nullptr, *cax = nullptr;
   double *part = nullptr, *sums = nullptr;
-  if (half) {
+  if (!w2) {
     TRY(getbuf(ctx, "ph_part", half_part_elems(ctx->nocc, ctx->col.nh, ncol), &part));
     TRY(getbuf(ctx, "ph_sums", half_sum_elems(ctx->col.nh, ncol), &sums));
   } else {
@@ -949,8 +942,8 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
     sym = true;
     for (int c = 0; c < ncol; ++c) sym = sym && (hs[c] <= 1e-12 * hs[ncol + c]);
   }
-  // C^H b (real coefficients for real-in-real-space columns: the occupied rows are too)
-  if (!half) launch_gram<double>(ctx->st, ctx->P64.C, ctx->nocc, npw, b64, ncol, ctx->work, cb, sym);
+  // squared system: C^H b (real coefficients for real-in-real-space columns: the occupied rows are too)
+  if (w2) launch_gram<double>(ctx->st, ctx->P64.C, ctx->nocc, npw, b64, ncol, ctx->work, cb, sym);
   std::vector<int> act(ncol, 1);
   TRY(upload(ctx, "sv_oact", act, &oact));
   std::vector<double> hr(ncol, 0.0), hb(ncol, 0.0), hx(ncol, 0.0), habs(ncol, 0.0);
@@ -991,10 +984,9 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
                                  cdef, ctx->work, nullptr, nullptr);
       if (sym) launch_sym_check(ctx->st, npw, ncol, x64, ctx->geo.sph_neg, xmax);
     }
-    // r64 = P_c (b - (H - E) x64): C^H (H - E) x64 from the dots fused into the
-    // last transform pass, C^H b computed once per solve
     if (w2) {
-      // Eq. P2+ residual in FP64: ax = P_c (H - E) P_c (H - E) x + w2 x
+      // Eq. P2+ residual in FP64: ax = P_c (H - E) P_c (H - E) x + w2 x, the
+      // coefficients from the dots fused into the last transform pass
       const int pa = prof_begin(ctx, PC_REFINE);
       double2* ax1;
       TRY(getbuf(ctx, "sv_ax1", (size_t)ncol * npw, &ax1));
@@ -1012,7 +1004,10 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
       launch_sq_shift<double>(ctx->st, npw, ncol, ax, x64, w2, oact, ctx->work, nullptr);
       launch_gram<double>(ctx->st, ctx->P64.C, ctx->nocc, npw, ax, ncol, ctx->work, cax);
       prof_end(ctx, PC_REFINE, pa);
-    } else if (half) {
+      launch_residual(ctx->st, npw, ncol, b64, ax, x64, oact, ctx->work, res2, bb, xx, ctx->P64.C, ctx->nocc, cb,
+                      cax);
+      CK(cudaMemcpyAsync(r64, ax, (size_t)ncol * npw * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->st));
+    } else {
       // r64 = b - (H - E) x in the last transform pass (two real columns per
       // transform), then P_c and the norms
       const int pa = prof_begin(ctx, PC_REFINE);
@@ -1023,28 +1018,6 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
       launch_residual_half(ctx->st, sym, ctx->col, Ch, ctx->nocc, r64, b64, x64, npw, ncol, oact, n, part, sums,
                            ctx->work.cnt_b, res2);
       prof_end(ctx, PC_REFINE, pa);
-    } else {
-      const int pa = prof_begin(ctx, PC_REFINE);
-      if (sym) {
-        // two real-in-real-space columns per FP64 transform
-        TRY(h_apply_sym(ctx, x64, ncol, E, act, xmax + ncol, ax));
-        launch_gram<double>(ctx->st, ctx->P64.C, ctx->nocc, npw, ax, ncol, ctx->work, cax, true);
-      } else {
-        GatherDots dots;
-        dots.C = ctx->P64.C;
-        dots.nocc = ctx->nocc;
-        dots.ncol = ncol;
-        dots.part = ctx->work.part_d;
-        dots.cnt = ctx->work.cnt_d;
-        dots.coef = cax;
-        TRY(h_apply<double>(ctx, x64, ncol, E, oact, ax, &dots));
-      }
-      prof_end(ctx, PC_REFINE, pa);
-    }
-    if (!half) {
-      launch_residual(ctx->st, npw, ncol, b64, ax, x64, oact, ctx->work, res2, bb, xx, ctx->P64.C, ctx->nocc, cb,
-                      cax, sym && !w2);
-      CK(cudaMemcpyAsync(r64, ax, (size_t)ncol * npw * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->st));
     }
     CK(cudaMemcpyAsync(ctx->sv_pin, res2, (size_t)4 * ncol * sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
     TRY(sync(ctx, "solve"));
@@ -1234,7 +1207,7 @@ gw_status chi0_model_core(gw_ctx* ctx, const double* y, bool y_cplx, int nb, con
   TRY(upload_table(ctx, "mod_ep", Ep, &dEp));
   TRY(getbuf(ctx, "mod_sol", (size_t)nsol * npw, &sol));
   TRY(rhs_core(ctx, y, y_cplx, nb, &rhs));
-  launch_model_scale<double>(ctx->st, npw, nsol, ctx->P64.kin, rhs, dsrc, dEm, dEp, sol);
+  launch_model_scale(ctx->st, npw, nsol, ctx->P64.kin, rhs, dsrc, dEm, dEp, sol);
   // real fields and realified states at real frequencies (denominators even in
   // G): solutions real in real space
   bool real_w = !y_cplx;
@@ -1932,21 +1905,23 @@ gw_status grad_from_basis(gw_ctx* ctx, const double* phi, const double* Q, const
   return launch_check(ctx, "grad");
 }
 
-// host sphere, pencils, planes
-// Tables of the column solver: the disc pencils as mirror pairs in the order
-// (n1, then n0 as the planes are counted), the half entries in that order.
+// Tables of the column solver and of the FP64 projector: the disc pencils as
+// mirror pairs in the order (n1, then n0 as the planes are counted), the half
+// entries in that order.  The sphere |G|^2/2 <= ecut has every -G and whole
+// pencils (build_geometry refuses one that its grid cuts).
 gw_status build_col_plan(gw_ctx* ctx, const std::vector<int4>& pencils, const std::vector<int>& i2s,
                          const std::vector<int>& pen, const std::vector<int>& negs,
                          const std::vector<uint8_t>& disc, size_t nplanes) {
   ColPlan& p = ctx->col;
   const int N = ctx->N;
-  p.half = p.ok = false;
+  p.ok = false;
+  auto odd = [&]() { return fail(ctx, GW_E_ARG, "the sphere has no mirror symmetry"); };
   p.P = (int)nplanes;
   p.nm = p.P / 2;
   auto plane = [&](int i0) { return i0 <= p.nm ? i0 : i0 - (N - p.P); };
   for (const int4& q : pencils) {           // the planes are |n0| <= nm
     const int n0 = 2 * q.x < N ? q.x : q.x - N;
-    if (std::abs(n0) > p.nm) return GW_OK;
+    if (std::abs(n0) > p.nm) return odd();
   }
   std::vector<int> where(N * N, -1);
   for (size_t k = 0; k < pencils.size(); ++k) where[pencils[k].x * N + pencils[k].y] = (int)k;
@@ -1959,7 +1934,7 @@ gw_status build_col_plan(gw_ctx* ctx, const std::vector<int4>& pencils, const st
       if (i1 == 0 && (q == 0 || q > p.nm)) continue;
       if (disc[i0 * N + i1]) rep.push_back(where[i0 * N + i1]);
     }
-  if (2 * rep.size() - 1 != pencils.size()) return GW_OK;
+  if (2 * rep.size() - 1 != pencils.size()) return odd();
   p.npair = (int)rep.size();
   std::vector<int> hstart(1, 0), gp, gm;
   std::vector<unsigned> hpos;
@@ -1979,13 +1954,12 @@ gw_status build_col_plan(gw_ctx* ctx, const std::vector<int4>& pencils, const st
       gm.push_back(negs[s]);
       hpos.push_back((unsigned)j << 8 | (unsigned)z);
     }
-    if (2 * zm + 1 != q.w) return GW_OK;       // the pencil's entries are |n2| <= zm
+    if (2 * zm + 1 != q.w) return odd();       // the pencil's entries are |n2| <= zm
     zmax[j] = (unsigned char)zm;
     hstart.push_back((int)gp.size());
   }
   p.nh = (int)gp.size();
-  if (2 * p.nh - 1 != ctx->npw || gp[0] != gm[0]) return GW_OK;
-  p.half = true;
+  if (2 * p.nh - 1 != ctx->npw || gp[0] != gm[0]) return odd();
   // equal shares of entries (solver vectors, projector) and pencils (transforms)
   std::vector<int> split(kColNQ * (kColMaxQ + 1), p.npair);
   auto cost = [&](int j) { return (long)hstart[j] + (long)j * N / 8; };
@@ -2032,6 +2006,7 @@ gw_status build_col_plan(gw_ctx* ctx, const std::vector<int4>& pencils, const st
   return GW_OK;
 }
 
+// host sphere, pencils, planes
 gw_status build_geometry(gw_ctx* ctx) {
   const int N = ctx->N;
   const double gg = 2.0 * M_PI / ctx->L;
@@ -2329,18 +2304,15 @@ gw_status upload_projector(gw_ctx* ctx, const std::vector<zc>& cdef) {
   }
   TRY(upload(ctx, "occ_C64", c64, &ctx->P64.C));
   TRY(upload(ctx, "occ_C32", c32, &ctx->P32.C));
-  if (ctx->col.half) {
-    const int r = (int)(n / ctx->npw);
-    TRY(getbuf(ctx, "col_C64", (size_t)r * ctx->col.nh, &ctx->col64.Ch));
-    TRY(getbuf(ctx, "col_C32", (size_t)r * ctx->col.nh, &ctx->col32.Ch));
-    CK(launch_col_permute<double>(ctx->st, ctx->col, ctx->N, ctx->npw, nullptr, ctx->P64.C, r, nullptr, ctx->col64));
-    CK(launch_col_permute<float>(ctx->st, ctx->col, ctx->N, ctx->npw, nullptr, ctx->P32.C, r, nullptr, ctx->col32));
-  }
+  const int rows = (int)(n / std::max(ctx->npw, 1));
+  TRY(getbuf(ctx, "col_C64", (size_t)rows * ctx->col.nh, &ctx->col64.Ch));
+  TRY(getbuf(ctx, "col_C32", (size_t)rows * ctx->col.nh, &ctx->col32.Ch));
+  CK(launch_col_permute<double>(ctx->st, ctx->col, ctx->N, ctx->npw, nullptr, ctx->P64.C, rows, nullptr, ctx->col64));
+  CK(launch_col_permute<float>(ctx->st, ctx->col, ctx->N, ctx->npw, nullptr, ctx->P32.C, rows, nullptr, ctx->col32));
   // the rows split into TF32 hi / lo parts for the tensor-core projector
   // coefficients (up to 64 rows); without a tensor-map encoder the CUDA-core
   // dots remain
   ctx->tc_ok = false;
-  const int rows = (int)(n / std::max(ctx->npw, 1));
   if (rows >= 1 && rows <= 64 && tc_prepare() == cudaSuccess) {
     std::vector<float> hi, lo;
     tc_split_rows(c64, rows, ctx->npw, &hi, &lo);

@@ -96,7 +96,7 @@ k_proj_dots(const cpx<T>* __restrict__ C, int nocc, int npw, const cpx<T>* __res
 
 // (b) Y[b] -= sum_v C[v] coef[v][b] (precision T); optionally pap[b] = Re <P[b]|Y[b]> (new Y),
 // accumulated in FP64.  grid (nchunk, ncol)
-template <typename T, bool REAL>
+template <typename T>
 __global__ void __launch_bounds__(kLT)
 k_proj_update(const cpx<T>* __restrict__ C, int nocc, int npw, cpx<T>* __restrict__ Y, int ncol,
               const int* __restrict__ active, const double2* __restrict__ coef,
@@ -114,13 +114,8 @@ k_proj_update(const cpx<T>* __restrict__ C, int nocc, int npw, cpx<T>* __restric
     for (int v = 0; v < nocc; ++v) {
       const cpx<T> c = C[(size_t)v * npw + G];
       const cpx<T> a = sc[v];
-      if (REAL) {                   // real coefficient
-        y.x -= c.x * a.x;
-        y.y -= c.y * a.x;
-      } else {
-        y.x -= c.x * a.x - c.y * a.y;
-        y.y -= c.x * a.y + c.y * a.x;
-      }
+      y.x -= c.x * a.x - c.y * a.y;
+      y.y -= c.x * a.y + c.y * a.x;
     }
     Y[(size_t)b * npw + G] = y;
     if (Pv) {
@@ -137,18 +132,6 @@ k_proj_update(const cpx<T>* __restrict__ C, int nocc, int npw, cpx<T>* __restric
     sum_records<1>(partial + b, gridDim.x, ncol, &s);
     pap[b] = s;
   }
-}
-
-template <typename T>
-void launch_proj(cudaStream_t s, const cpx<T>* C, int nocc, int npw, cpx<T>* Y, int ncol, const int* active,
-                 Work& w, const cpx<T>* Pv, double* pap, bool real) {
-  if (ncol == 0 || nocc == 0) return;
-  const int nchunk = (npw + kChunkP - 1) / kChunkP;
-  dim3 g1(nchunk, (ncol + kCT - 1) / kCT);
-  ++g_launches;
-  if (real) k_proj_dots<T, true><<<g1, kLT, 0, s>>>(C, nocc, npw, Y, ncol, active, w.part2, w.cnt_a, w.coef);
-  else k_proj_dots<T, false><<<g1, kLT, 0, s>>>(C, nocc, npw, Y, ncol, active, w.part2, w.cnt_a, w.coef);
-  launch_proj_update<T>(s, C, nocc, npw, Y, ncol, active, w.coef, w, Pv, pap, real);
 }
 
 // Gram matrix only: coef[v * ncol + b] = sum_G conj(C[v][G]) Y[b][G]
@@ -282,13 +265,12 @@ void launch_sq_shift(cudaStream_t s, int npw, int ncol, cpx<T>* Ap, const cpx<T>
 
 template <typename T>
 void launch_proj_update(cudaStream_t s, const cpx<T>* C, int nocc, int npw, cpx<T>* Y, int ncol,
-                        const int* active, const double2* coef, Work& w, const cpx<T>* Pv, double* pap, bool real) {
+                        const int* active, const double2* coef, Work& w, const cpx<T>* Pv, double* pap) {
   if (ncol == 0 || nocc == 0) return;
   const int nchunk = (npw + kChunk - 1) / kChunk;
   dim3 g2(nchunk, ncol);
   ++g_launches;
-  if (real) k_proj_update<T, true><<<g2, kLT, 0, s>>>(C, nocc, npw, Y, ncol, active, coef, Pv, w.part1, w.cnt_b, pap);
-  else k_proj_update<T, false><<<g2, kLT, 0, s>>>(C, nocc, npw, Y, ncol, active, coef, Pv, w.part1, w.cnt_b, pap);
+  k_proj_update<T><<<g2, kLT, 0, s>>>(C, nocc, npw, Y, ncol, active, coef, Pv, w.part1, w.cnt_b, pap);
 }
 
 // ---------------------------------------------------------------------------
@@ -833,7 +815,7 @@ k_residual(int npw, const double2* __restrict__ b, double2* __restrict__ ax, con
            const int* __restrict__ active, double* __restrict__ partial, unsigned* __restrict__ cnt,
            double* __restrict__ res2, double* __restrict__ bb, double* __restrict__ xx, int ncol,
            const double2* __restrict__ C, int nocc, const double2* __restrict__ cb,
-           const double2* __restrict__ cax, int real) {
+           const double2* __restrict__ cax) {
   __shared__ double2 sc[kMaxOcc];
   const int c = blockIdx.y;
   if (active && !active[c]) return;
@@ -852,14 +834,7 @@ k_residual(int npw, const double2* __restrict__ b, double2* __restrict__ ax, con
     double2 r = ax[i];
     r.x = bv.x - r.x;
     r.y = bv.y - r.y;
-    if (C && real) {               // real coefficients (real-in-real-space columns)
-      for (int v = 0; v < nocc; ++v) {
-        const double2 cv = C[(size_t)v * npw + G];
-        const double k = sc[v].x;
-        r.x -= cv.x * k;
-        r.y -= cv.y * k;
-      }
-    } else if (C) {
+    if (C) {
       for (int v = 0; v < nocc; ++v) {
         const double2 cv = C[(size_t)v * npw + G], k = sc[v];
         r.x -= cv.x * k.x - cv.y * k.y;
@@ -891,11 +866,11 @@ k_residual(int npw, const double2* __restrict__ b, double2* __restrict__ ax, con
 
 void launch_residual(cudaStream_t s, int npw, int ncol, const double2* b, double2* ax, const double2* x,
                      const int* active, Work& w, double* res2, double* bb, double* xx, const double2* C, int nocc,
-                     const double2* cb, const double2* cax, bool real) {
+                     const double2* cb, const double2* cax) {
   dim3 g((npw + kChunk - 1) / kChunk, ncol);
   ++g_launches;
   k_residual<<<g, kLT, 0, s>>>(npw, b, ax, x, active, reinterpret_cast<double*>(w.part2), w.cnt_b, res2, bb,
-                                xx, ncol, C, nocc, cb, cax, real ? 1 : 0);
+                                xx, ncol, C, nocc, cb, cax);
 }
 
 // Deflated components of a Sternheimer pass: coef[d][c] = <D_d|r_c> on entry;
@@ -960,40 +935,33 @@ void launch_combine(cudaStream_t s, int npw, int nout, const double2* in, const 
 // with Em = e_v + omega, Ep = e_v - omega (complex).  A reciprocal whose
 // denominator is exactly zero is taken as 0 (the pseudo-inverse of the
 // diagonal; such an entry of a projected right-hand side is zero).
-template <typename T>
-__device__ __forceinline__ cpx<T> pinv_shift(T t, cpx<T> e) {
-  const T dr = t - e.x, di = -e.y;
-  const T d2 = dr * dr + di * di;
-  if (d2 == (T)0) return mk<T>(0, 0);
-  const T r = (T)1 / d2;
-  return mk<T>(dr * r, -di * r);
+__device__ __forceinline__ double2 pinv_shift(double t, double2 e) {
+  const double dr = t - e.x, di = -e.y;
+  const double d2 = dr * dr + di * di;
+  if (d2 == 0.0) return make_double2(0, 0);
+  const double r = 1.0 / d2;
+  return make_double2(dr * r, -di * r);
 }
 
-// (in the precision T of the vectors)
-template <typename T>
-__global__ void k_model_scale(int npw, const T* __restrict__ kin, const cpx<T>* __restrict__ in,
+__global__ void k_model_scale(int npw, const double* __restrict__ kin, const double2* __restrict__ in,
                               const int* __restrict__ src, const double2* __restrict__ Em,
-                              const double2* __restrict__ Ep, cpx<T>* __restrict__ out) {
+                              const double2* __restrict__ Ep, double2* __restrict__ out) {
   const int j = blockIdx.y;
   const int a = src[j];
-  const cpx<T> em = from_d<T>(Em[j]), ep = from_d<T>(Ep[j]);
+  const double2 em = Em[j], ep = Ep[j];
   for (int G = blockIdx.x * blockDim.x + threadIdx.x; G < npw; G += gridDim.x * blockDim.x) {
-    const T t = kin[G];
-    const cpx<T> w = cadd(pinv_shift<T>(t, em), pinv_shift<T>(t, ep));
-    out[(size_t)j * npw + G] = cmul(w, in[(size_t)a * npw + G]);
+    const double t = kin[G];
+    out[(size_t)j * npw + G] = cmul(cadd(pinv_shift(t, em), pinv_shift(t, ep)), in[(size_t)a * npw + G]);
   }
 }
 
-template <typename T>
-void launch_model_scale(cudaStream_t s, int npw, int nout, const T* kin, const cpx<T>* in, const int* src,
-                        const double2* Em, const double2* Ep, cpx<T>* out) {
+void launch_model_scale(cudaStream_t s, int npw, int nout, const double* kin, const double2* in, const int* src,
+                        const double2* Em, const double2* Ep, double2* out) {
   if (nout == 0) return;
   dim3 g((npw + kLT - 1) / kLT, nout);
   ++g_launches;
-  k_model_scale<T><<<g, kLT, 0, s>>>(npw, kin, in, src, Em, Ep, out);
+  k_model_scale<<<g, kLT, 0, s>>>(npw, kin, in, src, Em, Ep, out);
 }
-template void launch_model_scale<double>(cudaStream_t, int, int, const double*, const double2*, const int*,
-                                         const double2*, const double2*, double2*);
 
 // precision changes at the boundary of an FP32 pipeline; out = x - z (FP64 result)
 // Eq. subs_epsilon in the two bases: out[i][j] = sum_ab a_ia (Ti_ab - (M^-1)_ab) a_jb
@@ -1238,9 +1206,7 @@ void launch_tridiag_inv(cudaStream_t s, int K, const double* alpha, const double
   template void launch_gram<T>(cudaStream_t, const cpx<T>*, int, int, const cpx<T>*, int, Work&, double2*, \
                                bool);                                                                      \
   template void launch_proj_update<T>(cudaStream_t, const cpx<T>*, int, int, cpx<T>*, int, const int*,     \
-                                      const double2*, Work&, const cpx<T>*, double*, bool);                \
-  template void launch_proj<T>(cudaStream_t, const cpx<T>*, int, int, cpx<T>*, int, const int*, Work&,     \
-                               const cpx<T>*, double*, bool);                                              \
+                                      const double2*, Work&, const cpx<T>*, double*);                      \
   template void launch_cg_init<T, double>(cudaStream_t, int, int, const double2*, cpx<T>*, cpx<T>*,       \
                                           const int*, Work&, CgState, const T*, double, double);           \
   template void launch_cg_update<T>(cudaStream_t, int, int, cpx<T>*, cpx<T>*, const cpx<T>*,              \

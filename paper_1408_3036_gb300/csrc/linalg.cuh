@@ -63,9 +63,6 @@ struct QmrState {
   unsigned* cnt = nullptr;
 };
 
-template <typename T>
-void launch_proj(cudaStream_t s, const cpx<T>* C, int nocc, int npw, cpx<T>* Y, int ncol, const int* active,
-                 Work& w, const cpx<T>* Pv, double* pap, bool real = false);
 // step 0 init, 1 sigma/alpha, 2 residual, 3 d/x/rho/beta + stop test, 4 q update
 template <typename T>
 void launch_qmr(cudaStream_t s, int step, int npw, int ncol, const double2* b, cpx<T>* x, cpx<T>* r, cpx<T>* q,
@@ -73,7 +70,7 @@ void launch_qmr(cudaStream_t s, int step, int npw, int ncol, const double2* b, c
                 const T* kin, double tol_in2, int maxit);
 template <typename T>
 void launch_proj_update(cudaStream_t s, const cpx<T>* C, int nocc, int npw, cpx<T>* Y, int ncol,
-                        const int* active, const double2* coef, Work& w, const cpx<T>* Pv, double* pap, bool real = false);
+                        const int* active, const double2* coef, Work& w, const cpx<T>* Pv, double* pap);
 // Ap += w2[c] p per column; pap[c] = Re <p|Ap> when pap is given
 template <typename T>
 void launch_sq_shift(cudaStream_t s, int npw, int ncol, cpx<T>* Ap, const cpx<T>* p, const double* w2,
@@ -111,13 +108,12 @@ void launch_defl_scale(cudaStream_t s, double2* coef, const double* eps, const d
                        const int* active);
 void launch_residual(cudaStream_t s, int npw, int ncol, const double2* b, double2* ax, const double2* x,
                      const int* active, Work& w, double* res2, double* bb, double* xx, const double2* C = nullptr,
-                     int nocc = 0, const double2* cb = nullptr, const double2* cax = nullptr, bool real = false);
+                     int nocc = 0, const double2* cb = nullptr, const double2* cax = nullptr);
 void launch_combine(cudaStream_t s, int npw, int nout, const double2* in, const int* src0, const int* src1,
                     double w_pair, double w_single, double2* out, const int* neg = nullptr);
 // Eq. model_eq: out[j] = (pinv(T - Em_j) + pinv(T - Ep_j)) in[src_j] on the sphere
-template <typename T>
-void launch_model_scale(cudaStream_t s, int npw, int nout, const T* kin, const cpx<T>* in, const int* src,
-                        const double2* Em, const double2* Ep, cpx<T>* out);
+void launch_model_scale(cudaStream_t s, int npw, int nout, const double* kin, const double2* in, const int* src,
+                        const double2* Em, const double2* Ep, double2* out);
 // Eq. subs_epsilon: out[m][m] from the coefficients a [m][k], am [m][km] and the
 // inverses Ti (exact basis), Mi (model in the exact basis, complex), Tmi (model basis)
 void launch_split_form(cudaStream_t s, int m, int k, int km, const double* a, const double* Ti,
