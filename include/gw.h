@@ -572,8 +572,9 @@ gw_status gw_sigma_c(gw_ctx* ctx, int e, double delta, double alpha, int n_freq,
  * Classes (multi-launch CG): 0 scatter + inverse z pass (with the CG p update),
  * 1 inverse y pass, 2 x pass with V_loc (H), 3 forward y pass, 4 forward z pass
  * + gather + kinetic and shift, 5 projector P_c, 6 CG update; 7 FP64
- * refinement residual (H apply + P_c); 8 persistent CG launch (all phases);
- * 9 the persistent CG's tasks, timed inside the kernel (global timer): read
+ * refinement residual (H apply + P_c); 8 one-launch CG pass (column solver or
+ * persistent kernel; simplified QMR has no class); 9 the persistent CG's tasks
+ * (when gw_set_cg_kernel selects it), timed inside the kernel (global timer): read
  * back as entries 10..15 = task kind A busy, A waiting, B busy, B waiting,
  * C busy, C waiting (milliseconds summed over tasks; counts: tasks run for
  * "busy", tasks skipped for "waiting"), then 16..27 the busy time of four

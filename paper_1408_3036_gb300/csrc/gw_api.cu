@@ -865,7 +865,7 @@ gw_status inner_solve(gw_ctx* ctx, bool qmr, int ncol, const double2* r64, const
   }
   if (sym) {
     launch_add_conv_sym<U>(ctx->st, ctx->npw, ncol, d, x64, oact, ctx->geo.sph_neg);
-    launch_sym_check(ctx->st, ctx->npw, ncol, x64, ctx->geo.sph_neg, xmax);
+    if (!w2) launch_sym_check(ctx->st, ctx->npw, ncol, x64, ctx->geo.sph_neg, xmax);
   } else {
     launch_add_conv<U>(ctx->st, ctx->npw, ncol, d, x64, oact);
   }
@@ -982,7 +982,7 @@ gw_status solve(gw_ctx* ctx, int ncol, const double2* b64, const double2* E, dou
     if (ctx->ndef > 0) {              // the deflated components, exactly
       launch_proj_update<double>(ctx->st, ctx->P64.C + (size_t)ctx->nocc * npw, ctx->ndef, npw, x64, ncol, oact,
                                  cdef, ctx->work, nullptr, nullptr);
-      if (sym) launch_sym_check(ctx->st, npw, ncol, x64, ctx->geo.sph_neg, xmax);
+      if (sym && !w2) launch_sym_check(ctx->st, npw, ncol, x64, ctx->geo.sph_neg, xmax);
     }
     if (w2) {
       // Eq. P2+ residual in FP64: ax = P_c (H - E) P_c (H - E) x + w2 x, the
