@@ -252,7 +252,9 @@ def class_bytes(miller, N, npw, nocc, s):
     """Algorithmic bytes of the inner CG kernels per column-iteration, and per
     launch-iteration for data shared by all columns; s = bytes per complex value.
 
-    persistent_cg (one launch = one CG pass, four phases per iteration):
+    persistent_cg (one launch = one CG pass; bytes of the form that keeps its vectors
+    and planes in memory, four phases per iteration -- the column solver keeps
+    them in shared memory):
       A  read r, p, write p (3 N_PW s); write the planes of the sphere (P0 N^2 s)
       B  read + write those planes (2 P0 N^2 s); V shared (N^3 real)
       C  read the planes (P0 N^2 s); read p, write Ap (2 N_PW s); C_v shared (n_occ N_PW s)
@@ -301,7 +303,8 @@ def model_bytes(N, npw, nocc, s):
 
 def src_hash():
     h = hashlib.sha256()
-    for f in ("fft.cuh", "gw_common.cuh", "linalg.cuh", "col.cuh", "col_layout.cuh", "col_kernel.cuh", "kernels_col.cu"):
+    for f in ("fft.cuh", "gw_common.cuh", "linalg.cuh", "sums.cuh", "col.cuh", "col_layout.cuh", "col_kernel.cuh",
+              "kernels_col.cu"):
         with open(os.path.join(ROOT, "paper_1408_3036_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -438,11 +441,15 @@ def run_gpu(args):
     traffic = None
     if tr is not None and n_dom > 0:
         traffic = tr["dram_bytes_per_col_iter"] * it_cols / n_dom
-    roofline = dict(bound="hbm", kernel=dominant, achieved=achieved, peak=hbm, unit="GB/s",
+    roofline = dict(bound="hbm", kernel="cg_pass" if dominant == "persistent_cg" else dominant,
+                    achieved=achieved, peak=hbm, unit="GB/s",
                     frac=(achieved / hbm if achieved else None), peak_kind=hbm_kind,
                     traffic=traffic, alg_bytes_per_launch=alg_bytes / max(n_dom, 1),
                     alg_bytes_per_col_iter=b_it,
-                    byte_model="s (11 N_PW + 4 N_g) per column-iteration, s = bytes per complex value",
+                    byte_model="s (11 N_PW + 4 N_g) per column-iteration, s = bytes per complex value: what a solver "
+                               "with its vectors in memory moves; the column solver keeps them in shared memory, and "
+                               "traffic is what a pass takes from DRAM",
+                    frac_traffic=(traffic * n_dom / (ms_dom / 1e3) / 1e9 / hbm if traffic and ms_dom > 0 else None),
                     achieved_pruned_model=(pruned_bytes / (ms_dom / 1e3) / 1e9 if ms_dom > 0 else None),
                     kernel_ms_share=ms_dom / total_ms, launches=n_dom, column_iterations=it_cols,
                     launch_iterations=it_launch)
