@@ -61,13 +61,14 @@
 // two) and the transforms keep the fewest operations (dft in fft.cuh).
 // Measured on a GB300, one application, before (launches per step, or the
 // grid-wide task queue of kernels_cg.cu, with the Teter-Payne-Allan form) and
-// after; in brackets what the preconditioner, then the multiply-adds and
-// transforms took off: 48^3 grid, 12053 plane waves, 16 CG columns, FP32 3.70 ->
-// 1.55 ms (1.65, 1.57, 1.55), FP64 15.8 -> 8.9 ms (10.9, 9.8, 8.9); 45^3, 2007
-// plane waves, 22 complex columns 11.7 -> 2.24 ms (3.2, 2.29, 2.24); 32^3, 2109
-// plane waves, 69 rows, 1104 complex columns 400 -> 29.1 ms (58, 30.5, 29.1);
-// 64^3, 38401 plane waves, 64 rows, 256 complex columns 1051 -> 108 ms (386, 113,
-// 108; of the last step the coefficient sums of kernels_half.cu are the most).
+// after, both sides in one run: 48^3 grid, 12053 plane waves, 16 CG columns, FP32
+// 3.69 -> 1.58 ms, FP64 15.8 -> 8.9 ms; 45^3, 2007 plane waves, 22 complex columns
+// 11.7 -> 2.29 ms; 32^3, 2109 plane waves, 69 rows, 1104 complex columns 398 ->
+// 29.9 ms; 64^3, 38401 plane waves, 64 rows, 256 complex columns 1044 -> 111 ms
+// (of the last two, columns that stalled on the rounding floor took 120 .. 400 ms
+// before, more or fewer by the input: 232 and 837 ms at least).  What the scaling
+// of the columns costs of that: a second read of b and one barrier a pass, 0.5 to
+// 1%; the exact sums of FP32 SQMR: 2 to 3%.
 #pragma once
 
 #include <cooperative_groups.h>
