@@ -427,8 +427,9 @@ gw_status gw_set_cg_kernel(gw_ctx* ctx, int kind, long long wait_limit);
  *   1 (default)  kinetic, diagonal in G and symmetric, also in the bilinear form:
  *                the column solver takes the denominators of the column's own
  *                shift, |G|^2/2 + V0 - E kept away from zero (V0: the level that
- *                V_loc lies below in two thirds of the cell); the other kernels the form of Teter, Payne and Allan, with the
- *                kinetic energy of the column's occupied state as reference
+ *                V_loc lies below in two thirds of the cell); the other kernels
+ *                the form of Teter, Payne and Allan, with the kinetic energy of
+ *                the column's occupied state as reference
  *   0            none, as in the paper (Sec. Avoiding summations: SQMR without
  *                preconditioning)
  * Both solve the same equations to the same tolerance; the preconditioner
